@@ -1,19 +1,25 @@
-"""ctypes binding of the CAST C-ABI library (include/cast.h).
+"""Binding of the CAST C-ABI library (include/cast.h).
 
 Argument marshalling only: every function here has the name and the argument
 order of its C counterpart and passes device pointers of torch tensors plus
-sizes.  No step of the method runs in Python.  Loading fails loudly when the
-CUDA library has not been built; there is no fallback path.
+sizes.  No step of the method runs in Python.  Set-up calls and synchronising
+queries go through ctypes; the compute calls, of which a decoding step makes
+some forty, through the extension module _cast_calls (csrc/binding_calls.cpp).
+Loading fails loudly when either has not been built; there is no fallback path.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 from typing import Optional
 
 import torch
 
-_LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libcast_b200.so")
+_PKG = os.path.dirname(os.path.abspath(__file__))
+_LIB_PATH = os.path.join(_PKG, "libcast_b200.so")
+_CALLS_PATH = os.path.join(_PKG, "_cast_calls.so")
 
 CAST_OK = 0
 STATUS_NAMES = {
@@ -49,19 +55,24 @@ class CastError(RuntimeError):
 
 
 _lib = None
+_calls = None
 
 
 def load_library() -> C.CDLL:
-    """Loads libcast_b200.so (built in-tree by paper_2510_26577_b200/build.py)."""
-    global _lib
+    """Loads libcast_b200.so and _cast_calls.so (built in-tree by paper_2510_26577_b200/build.py)."""
+    global _lib, _calls
     if _lib is not None:
         return _lib
-    if not os.path.exists(_LIB_PATH):
-        raise ImportError(
-            f"{_LIB_PATH} is missing: build it with `python paper_2510_26577_b200/build.py` "
-            "(there is no CPU or PyTorch fallback for the CAST kernels)")
+    for path in (_LIB_PATH, _CALLS_PATH):
+        if not os.path.exists(path):
+            raise ImportError(
+                f"{path} is missing: build it with `python paper_2510_26577_b200/build.py` "
+                "(there is no CPU or PyTorch fallback for the CAST kernels)")
     lib = C.CDLL(_LIB_PATH)
-    vp, i32, i32p = C.c_void_p, C.c_int, C.c_void_p
+    loader = importlib.machinery.ExtensionFileLoader("_cast_calls", _CALLS_PATH)
+    _calls = importlib.util.module_from_spec(importlib.util.spec_from_file_location("_cast_calls", _CALLS_PATH, loader=loader))
+    loader.exec_module(_calls)
+    vp, i32 = C.c_void_p, C.c_int
     lib.cast_status_string.restype = C.c_char_p
     lib.cast_status_string.argtypes = [C.c_int]
     sig = {
@@ -70,20 +81,8 @@ def load_library() -> C.CDLL:
         "cast_set_cost_tables": [vp, i32, i32, i32, i32, vp, vp],
         "cast_state_export": [vp, vp, C.POINTER(C.c_size_t)],
         "cast_state_import": [vp, vp, C.c_size_t],
-        "cast_step_begin": [vp, i32, i32p, i32p, vp],
-        "cast_tree_expand": [vp, i32, vp, i32, i32p, i32p, i32p, vp],
-        "cast_select_nodes": [vp, i32p, i32p, i32p, vp, i32p, vp, i32p, vp],
         "cast_reserve_attention": [vp, i32, i32, i32, i32, i32, i32, i32],
         "cast_set_attention_early_reads": [vp, i32],
-        "cast_tree_attention": [vp, vp, vp, vp, i32, i32, i32, i32, i32, i32, i32p, i32, i32, i32p, vp, i32p,
-                                C.c_float, vp, vp],
-        "cast_tree_attention_rows": [vp, vp, vp, vp, i32, i32, i32, i32, i32, i32, i32p, i32, i32, i32p, vp, i32p,
-                                     i32p, C.c_float, vp, vp],
-        "cast_accept": [vp, vp, i32, i32, i32p, i32p, i32p, vp, i32p, i32p, i32p, i32p, vp],
-        "cast_compact_kv": [vp, vp, vp, i32, i32, i32, C.c_size_t, i32, i32, i32, i32p, i32, i32, i32p, i32p, i32p,
-                            vp],
-        "cast_accept_static": [vp, i32, i32, i32, i32, i32, i32p, i32p, i32p, i32p, i32p, i32p, vp],
-        "cast_accept_stochastic": [vp, vp, vp, i32, i32, C.c_double, i32p, i32p, i32p, vp, vp, i32p, i32p, i32p, vp],
         "cast_accept_stochastic_plan": [vp, i32, C.POINTER(C.c_int), C.POINTER(C.c_int)],
         "cast_poll_status": [vp, vp, C.POINTER(C.c_int), C.POINTER(C.c_int32)],
         "cast_step_info": [vp, vp, C.POINTER(C.c_int32)],
@@ -94,21 +93,6 @@ def load_library() -> C.CDLL:
         fn.argtypes = argtypes
     _lib = lib
     return lib
-
-
-def _ptr(t: Optional[torch.Tensor]):
-    if t is None:
-        return None
-    assert t.is_cuda and t.is_contiguous(), "device-resident contiguous tensor expected"
-    return t.data_ptr()
-
-
-def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float32:
-        return CAST_F32
-    if t.dtype == torch.bfloat16:
-        return CAST_BF16
-    raise CastError(4, "dtype")
 
 
 def _stream(stream) -> int:
@@ -126,10 +110,9 @@ def cast_accept_static(target_logits, B, n_cap, vocab, max_depth, tokens, parent
                        bonus_token, stream=None):
     """The acceptance step without a context and without any allocation (see include/cast.h): for callers
     that are handed device pointers but may not allocate.  Needs B * n_cap <= 2048."""
-    lib = load_library()
-    _check(lib.cast_accept_static(_ptr(target_logits), _dtype_code(target_logits), B, n_cap, vocab, max_depth,
-                                  _ptr(tokens), _ptr(parent), _ptr(n_tree), _ptr(accept_len), _ptr(accept_path),
-                                  _ptr(bonus_token), _stream(stream)), "cast_accept_static")
+    load_library()
+    _check(_calls.accept_static(target_logits, B, n_cap, vocab, max_depth, tokens, parent, n_tree, accept_len, accept_path,
+                                bonus_token, stream), "cast_accept_static")
 
 
 class CastContext:
@@ -142,7 +125,9 @@ class CastContext:
         self.cfg = CastConfig(C1, C2, C3, max_batch, vocab, top_k, max_depth, max_width, max_tree, total_token,
                               fifo_len, enable_bp, enable_dp, enable_dr, pool_mode, ctx_base_mode, rerank_per_row)
         self.handle = C.c_void_p()
+        self._ctx = 0  # the handle as the compute calls take it
         _check(self.lib.cast_create(C.byref(self.cfg), C.byref(self.handle)), "cast_create")
+        self._ctx = self.handle.value
         self.width = max_width if max_width > 0 else top_k
         self.words = (max_tree + 31) // 32
 
@@ -150,6 +135,7 @@ class CastContext:
         if getattr(self, "handle", None) and self.handle.value:
             self.lib.cast_destroy(self.handle)
             self.handle = C.c_void_p()
+            self._ctx = 0
 
     def __del__(self):
         try:
@@ -189,48 +175,44 @@ class CastContext:
 
     # --- compute calls (enqueue only) ----------------------------------------
     def cast_step_begin(self, B, root_token, kv_len, stream=None):
-        _check(self.lib.cast_step_begin(self.handle, B, _ptr(root_token), _ptr(kv_len), _stream(stream)),
-               "cast_step_begin")
+        _check(_calls.step_begin(self._ctx, B, root_token, kv_len, stream), "cast_step_begin")
 
     def cast_tree_expand(self, layer, draft_logits, next_tokens, next_parent_row, next_count, stream=None):
-        _check(self.lib.cast_tree_expand(self.handle, layer, _ptr(draft_logits), _dtype_code(draft_logits),
-                                         _ptr(next_tokens), _ptr(next_parent_row), _ptr(next_count),
-                                         _stream(stream)), "cast_tree_expand")
+        _check(_calls.tree_expand(self._ctx, layer, draft_logits, next_tokens, next_parent_row, next_count, stream),
+               "cast_tree_expand")
 
     def cast_select_nodes(self, tokens, parent, depth, anc_mask, pool_idx, scores, n_tree, stream=None):
-        _check(self.lib.cast_select_nodes(self.handle, _ptr(tokens), _ptr(parent), _ptr(depth), _ptr(anc_mask),
-                                          _ptr(pool_idx), _ptr(scores), _ptr(n_tree), _stream(stream)),
+        _check(_calls.select_nodes(self._ctx, tokens, parent, depth, anc_mask, pool_idx, scores, n_tree, stream),
                "cast_select_nodes")
 
     def cast_tree_attention(self, q, k_cache, v_cache, B, Hq, Hkv, D, page_size, page_table, seq_capacity,
                             num_pages, kv_len, anc_mask, n_tree, scale, out, stream=None):
-        _check(self.lib.cast_tree_attention(self.handle, _ptr(q), _ptr(k_cache), _ptr(v_cache), _dtype_code(q), B, Hq,
-                                            Hkv, D, page_size, _ptr(page_table), seq_capacity, num_pages,
-                                            _ptr(kv_len), _ptr(anc_mask), _ptr(n_tree), float(scale), _ptr(out),
-                                            _stream(stream)), "cast_tree_attention")
+        _check(_calls.tree_attention(self._ctx, q, k_cache, v_cache, B, Hq, Hkv, D, page_size, page_table, seq_capacity,
+                                     num_pages, kv_len, anc_mask, n_tree, scale, out, stream), "cast_tree_attention")
 
     def cast_tree_attention_rows(self, q, k_cache, v_cache, B, Hq, Hkv, D, page_size, page_table, seq_capacity,
                                  num_pages, kv_len, anc_mask, n_tree, first_row, scale, out, stream=None):
-        _check(self.lib.cast_tree_attention_rows(self.handle, _ptr(q), _ptr(k_cache), _ptr(v_cache), _dtype_code(q), B,
-                                                 Hq, Hkv, D, page_size, _ptr(page_table), seq_capacity, num_pages,
-                                                 _ptr(kv_len), _ptr(anc_mask), _ptr(n_tree), _ptr(first_row),
-                                                 float(scale), _ptr(out), _stream(stream)), "cast_tree_attention_rows")
+        _check(_calls.tree_attention_rows(self._ctx, q, k_cache, v_cache, B, Hq, Hkv, D, page_size, page_table,
+                                          seq_capacity, num_pages, kv_len, anc_mask, n_tree, first_row, scale, out, stream),
+               "cast_tree_attention_rows")
 
     def cast_accept(self, target_logits, B, tokens, parent, depth, anc_mask, n_tree, accept_len, accept_path,
                     bonus_token, stream=None):
-        _check(self.lib.cast_accept(self.handle, _ptr(target_logits), _dtype_code(target_logits), B, _ptr(tokens),
-                                    _ptr(parent), _ptr(depth), _ptr(anc_mask), _ptr(n_tree), _ptr(accept_len),
-                                    _ptr(accept_path), _ptr(bonus_token), _stream(stream)), "cast_accept")
+        _check(_calls.accept(self._ctx, target_logits, B, tokens, parent, depth, anc_mask, n_tree, accept_len, accept_path,
+                             bonus_token, stream), "cast_accept")
 
     def cast_accept_stochastic(self, target_logits, draft_logits, B, temperature, tokens, parent, n_tree, u_accept,
                                u_bonus, accept_len, accept_path, bonus_token, stream=None):
         assert draft_logits.dtype == target_logits.dtype and u_accept.dtype == torch.float64 and \
             u_bonus.dtype == torch.float64
-        _check(self.lib.cast_accept_stochastic(self.handle, _ptr(target_logits), _ptr(draft_logits),
-                                               _dtype_code(target_logits), B, float(temperature), _ptr(tokens),
-                                               _ptr(parent), _ptr(n_tree), _ptr(u_accept), _ptr(u_bonus),
-                                               _ptr(accept_len), _ptr(accept_path), _ptr(bonus_token),
-                                               _stream(stream)), "cast_accept_stochastic")
+        _check(_calls.accept_stochastic(self._ctx, target_logits, draft_logits, B, temperature, tokens, parent, n_tree,
+                                        u_accept, u_bonus, accept_len, accept_path, bonus_token, stream),
+               "cast_accept_stochastic")
+
+    def cast_compact_kv(self, k_cache, v_cache, B, n_layers, layer_stride_bytes, Hkv, D, page_size, page_table,
+                        seq_capacity, num_pages, accept_path, accept_len, kv_len, stream=None):
+        _check(_calls.compact_kv(self._ctx, k_cache, v_cache, B, n_layers, layer_stride_bytes, Hkv, D, page_size, page_table,
+                                 seq_capacity, num_pages, accept_path, accept_len, kv_len, stream), "cast_compact_kv")
 
     def cast_accept_stochastic_plan(self, dtype):
         """(cluster size, slices cached in shared memory?) for logits of torch dtype `dtype`."""
@@ -239,13 +221,6 @@ class CastContext:
         _check(self.lib.cast_accept_stochastic_plan(self.handle, code, C.byref(cs), C.byref(cached)),
                "cast_accept_stochastic_plan")
         return cs.value, bool(cached.value)
-
-    def cast_compact_kv(self, k_cache, v_cache, B, n_layers, layer_stride_bytes, Hkv, D, page_size, page_table,
-                        seq_capacity, num_pages, accept_path, accept_len, kv_len, stream=None):
-        _check(self.lib.cast_compact_kv(self.handle, _ptr(k_cache), _ptr(v_cache), _dtype_code(k_cache), B, n_layers,
-                                        layer_stride_bytes, Hkv, D, page_size, _ptr(page_table), seq_capacity,
-                                        num_pages, _ptr(accept_path), _ptr(accept_len), _ptr(kv_len),
-                                        _stream(stream)), "cast_compact_kv")
 
     # --- synchronising queries ------------------------------------------------
     def cast_poll_status(self, stream=None):

@@ -1,9 +1,12 @@
-"""Builds the CAST CUDA library in-tree: csrc/*.cu -> libcast_b200.so (sm_100a only)."""
+"""Builds the CAST CUDA library in-tree: csrc/*.cu -> libcast_b200.so (sm_100a only), and the native side of the
+Python binding: csrc/binding_calls.cpp -> _cast_calls.so."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -11,6 +14,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(ROOT, "build", "obj")
 LIB = os.path.join(PKG, "libcast_b200.so")
+CALLS = os.path.join(PKG, "_cast_calls.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -29,6 +33,24 @@ def _stale(target: str, deps) -> bool:
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _build_calls() -> None:
+    """The extension module the binding calls through (host code against torch's headers; links the CUDA library)."""
+    src = os.path.join(CSRC, "binding_calls.cpp")
+    if not _stale(CALLS, [src, os.path.join(ROOT, "include", "cast.h")]):
+        return
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    inc, lib = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    cmd = ["g++", "-shared", "-fPIC", "-O2", "-std=c++17", "-fvisibility=hidden", "-I", os.path.join(ROOT, "include"),
+           "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"), "-I", cuda,
+           "-I", sysconfig.get_paths()["include"], src, "-o", CALLS, "-L", lib, "-lc10", "-lc10_cuda", "-ltorch_cpu",
+           "-ltorch_python", "-L", PKG, "-lcast_b200", "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+        raise RuntimeError("g++ failed for binding_calls.cpp")
 
 
 def build(verbose: bool = False, force: bool = False) -> str:
@@ -63,6 +85,7 @@ def build(verbose: bool = False, force: bool = False) -> str:
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
+    _build_calls()
     return LIB
 
 
