@@ -7,6 +7,8 @@ using namespace cast;
 
 namespace {
 
+// One 16-byte vector of logits: its largest element, and the place of the first element equal to a value.
+// (NaN is dropped by the maxima, as by a comparison; -0 and +0 compare equal.)
 template <typename T> struct Vec;
 template <> struct Vec<float> {
   static constexpr int N = 4;
@@ -153,13 +155,13 @@ __global__ void __launch_bounds__(CAST_MAX_TREE) accept_walk_kernel(
 
 // ------------------------------------------------------------------ compaction
 constexpr int kCompactThreads = 256;
-constexpr int kCompactItems = 8;  // 16-byte pieces per thread
+constexpr int kMaxPath = CAST_MAX_DEPTH + 1;
 
 struct CompactParams {
   char* k;
   char* v;
   size_t layer_stride;
-  int Hkv, row_bytes, page_size, seq_capacity, num_pages, H1;
+  int row_bytes, page_size, seq_capacity, num_pages, H1;  // row_bytes: one position, all kv-heads
   const int32_t* page_table;
   const int32_t* accept_path;
   const int32_t* accept_len;
@@ -168,78 +170,74 @@ struct CompactParams {
   DevState* st;
 };
 
-__device__ __forceinline__ size_t cache_row_offset(const CompactParams& p, int b, int pos, int h, bool* bad) {
-  size_t slot;
-  if (p.page_size == 0) {
-    slot = (size_t)b * p.seq_capacity + pos;
-  } else {
-    const int page = p.page_table[(size_t)b * p.seq_capacity + pos / p.page_size];
-    if (page < 0 || page >= p.num_pages) {
-      *bad = true;
-      return 0;
-    }
-    slot = (size_t)page * p.page_size + pos % p.page_size;
-  }
-  return (slot * p.Hkv + h) * (size_t)p.row_bytes;
+// Slot of position `pos` of sequence b, or -1 for a page id out of range.
+__device__ __forceinline__ long long cache_slot(const CompactParams& p, int b, int pos) {
+  if (p.page_size == 0) return (long long)b * p.seq_capacity + pos;
+  const int page = p.page_table[(size_t)b * p.seq_capacity + pos / p.page_size];
+  return page < 0 || page >= p.num_pages ? -1 : (long long)page * p.page_size + pos % p.page_size;
 }
 
-// One CTA per (kv-head, layer, sequence). Every source row is in registers before the first
-// store, so a destination slot that is also a later source (path 0,2,3: slot 2) is safe.
+// One CTA per (layer, sequence, up to 256 16-byte columns of the position rows of K and V). A position's heads are
+// contiguous in memory, so a row is copied whole: with a CTA per kv-head, 4096 CTAs of a few hundred bytes each, the
+// launch of 32 layers at batch 16 took 28 us; this one is bound by three dependent round trips (lengths and path, page
+// ids, the rows). The destinations and sources of the sequence are worked out once per CTA, one path entry per
+// lane; a row that is already in place (path 0, 1, 2, ...: the usual case of the root) is not touched.
+// Column by column the copy is safe in any order of the stores: a path entry is no smaller than its place, so a
+// destination slot is never the source of a later entry, and all loads come before the stores.
 __global__ void __launch_bounds__(kCompactThreads) compact_kernel(const CompactParams p) {
-  const int h = blockIdx.x, layer = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+  __shared__ long long src_s[kMaxPath], dst_s[kMaxPath];
+  __shared__ int n_moves;
+  const int layer = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int L = p.kv_len[b];
-  int a = p.accept_len[b];
-  if (a < 0) a = 0;
-  if (a > p.H1 - 1) a = p.H1 - 1;
-  const int rows = a + 1, vpr = p.row_bytes / 16;
-  const int per = rows * vpr, items = 2 * per;
-  const int max_pos = p.page_size == 0 ? p.seq_capacity : p.seq_capacity * p.page_size;
-  uint4 buf[kCompactItems];
   bool bad = false;
-#pragma unroll
-  for (int it = 0; it < kCompactItems; ++it) {
-    const int i = it * kCompactThreads + tid;
-    if (i < items) {
-      const int which = i / per, rem = i % per, j = rem / vpr, vv = rem % vpr;
-      const int src = p.accept_path[b * p.H1 + j];
-      const int pos = L + src;
+  int a = 0;
+  if (tid < 32) {
+    a = p.accept_len[b];
+    const int src = tid < p.H1 ? p.accept_path[b * p.H1 + tid] : 0;
+    a = a < 0 ? 0 : (a > p.H1 - 1 ? p.H1 - 1 : a);
+    const int max_pos = p.page_size == 0 ? p.seq_capacity : p.seq_capacity * p.page_size;
+    long long from = 0, to = 0;
+    if (tid <= a) {
       // a path element is a tree index no smaller than its place on the path (parents precede children), so
       // the destination L + j never lies past the source; anything else is a malformed path
-      if (L < 0 || src < j || pos >= max_pos) {
-        bad = true;
-        continue;
+      bad = L < 0 || src < tid || L + src >= max_pos;
+      if (!bad) {
+        from = cache_slot(p, b, L + src);
+        to = cache_slot(p, b, L + tid);
+        bad = from < 0 || to < 0;
       }
-      const size_t off = cache_row_offset(p, b, pos, h, &bad);
-      char* base = (which ? p.v : p.k) + (size_t)layer * p.layer_stride;
-      if (!bad) buf[it] = *reinterpret_cast<const uint4*>(base + off + (size_t)vv * 16);
     }
+    const unsigned moves = __ballot_sync(0xffffffffu, tid <= a && from != to);
+    if (tid <= a && from != to) {
+      const int at = __popc(moves & ((1u << tid) - 1u));
+      src_s[at] = from;
+      dst_s[at] = to;
+    }
+    if (tid == 0) n_moves = __popc(moves);
   }
   const int any_bad = __syncthreads_or(bad ? 1 : 0);
-  if (any_bad) {
-    if (tid == 0) report(p.st, CAST_ERR_BAD_PAGE, b);
-  } else {
-#pragma unroll
-    for (int it = 0; it < kCompactItems; ++it) {
-      const int i = it * kCompactThreads + tid;
-      if (i < items) {
-        const int which = i / per, rem = i % per, j = rem / vpr, vv = rem % vpr;
-        bool bad2 = false;
-        const size_t off = cache_row_offset(p, b, L + j, h, &bad2);
-        char* base = (which ? p.v : p.k) + (size_t)layer * p.layer_stride;
-        if (!bad2) *reinterpret_cast<uint4*>(base + off + (size_t)vv * 16) = buf[it];
-      }
-    }
-  }
-  // the last CTA of the sequence (every CTA has read kv_len[b] by then) publishes the new length
-  __syncthreads();
   if (tid == 0) {
-    __threadfence();
+    if (any_bad) report(p.st, CAST_ERR_BAD_PAGE, b);
+    // every CTA of the sequence has read kv_len[b] once all have taken the ticket: the last one publishes the new length
+    // (the rows themselves are the next kernel's business, which starts after this grid)
     const int t = atomicAdd(&p.ticket[b], 1);
     if (t == (int)(gridDim.x * gridDim.y) - 1) {
       p.ticket[b] = 0;
       if (!any_bad) p.kv_len[b] = L + a + 1;
     }
   }
+  const int cols = p.row_bytes / 16;
+  const int i = blockIdx.x * kCompactThreads + tid, n = n_moves;
+  if (any_bad || i >= 2 * cols) return;
+  char* base = (i < cols ? p.k : p.v) + (size_t)layer * p.layer_stride + (size_t)(i < cols ? i : i - cols) * 16;
+  uint4 buf[kMaxPath];
+#pragma unroll
+  for (int j = 0; j < kMaxPath; ++j)
+    if (j < n) buf[j] = *reinterpret_cast<const uint4*>(base + src_s[j] * p.row_bytes);
+#pragma unroll
+  for (int j = 0; j < kMaxPath; ++j)
+    if (j < n) *reinterpret_cast<uint4*>(base + dst_s[j] * p.row_bytes) = buf[j];
 }
 
 }  // namespace
@@ -402,14 +400,26 @@ extern "C" cast_status cast_compact_kv(cast_ctx* c, void* k_cache, void* v_cache
   if (row_bytes % 16 != 0) return CAST_ERR_SHAPE;
   if (((uintptr_t)k_cache | (uintptr_t)v_cache | layer_stride_bytes) & 15) return CAST_ERR_SHAPE;
   const int H1 = c->cfg.max_depth + 1;
-  if (2 * H1 * (row_bytes / 16) > kCompactThreads * kCompactItems) return CAST_ERR_CAPACITY;
   c->tree_inputs_fresh = 1;  // kv_len and cache rows: an attention call that follows reads them after its dependency wait
   CompactParams p;
   p.k = (char*)k_cache; p.v = (char*)v_cache; p.layer_stride = layer_stride_bytes;
-  p.Hkv = Hkv; p.row_bytes = row_bytes; p.page_size = page_size; p.seq_capacity = seq_capacity;
+  p.row_bytes = Hkv * row_bytes; p.page_size = page_size; p.seq_capacity = seq_capacity;
   p.num_pages = num_pages; p.H1 = H1;
   p.page_table = page_table; p.accept_path = accept_path; p.accept_len = accept_len; p.kv_len = kv_len;
   p.ticket = c->compact_ticket; p.st = c->state;
-  compact_kernel<<<dim3(Hkv, n_layers, B), kCompactThreads, 0, (cudaStream_t)stream>>>(p);
-  return launch_status();
+  const int cols = 2 * (p.row_bytes / 16);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((cols + kCompactThreads - 1) / kCompactThreads, n_layers, B);
+  cfg.blockDim = dim3(kCompactThreads, 1, 1);
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // launched while the walk finishes; waits for it
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, compact_kernel, p) != cudaSuccess) {
+    cudaGetLastError();
+    return CAST_ERR_CUDA;
+  }
+  return CAST_OK;
 }
