@@ -1,6 +1,6 @@
 // cast_tree_attention: tree-masked verification attention.
 //
-// CUDA-core path (fp32 inputs, and any shape the tensor-core path does not take): a
+// CUDA-core path (fp32 inputs, and bf16 caches the tensor-core path does not take: pages below 8 or above 64 positions): a
 // flash-style kernel. One CTA owns (sequence, kv-head, block of 32 query rows, KV split); a
 // query row is a (tree token, head of the GQA group) pair, so a K/V tile fetched once serves
 // all tree tokens and all heads of the group. Tiles of 64 positions are converted to fp32 in

@@ -1,4 +1,8 @@
-// Tensor-core path of cast_tree_attention for bf16, head_dim 128 (sm_100a: tcgen05 + TMEM + TMA).
+// Tensor-core path of cast_tree_attention for bf16, head_dim 128 or 64 (sm_100a: tcgen05 + TMEM + TMA). The figures
+// below are those of 128 dims. 64 dims came to this path from the CUDA-core kernel, which keeps P and the partials of KV
+// splits in fp32: here P enters the product as two bf16 terms (hi + lo, 16 bits, two MMAs: the second product is half
+// as wide anyway) and the partials stay fp32, so the result is no less precise. Eight ragged sequences of
+// 512-2048 positions, 24-48 tokens, 32/8 heads of 64 dims: 340 -> 19 us per layer.
 //
 // One CTA owns (sequence b, kv-head, block of 128 query rows, KV split). A query row is a
 // (tree token, head of the GQA group) pair, so every K/V tile is fetched once for all tree
@@ -43,19 +47,31 @@ namespace {
 
 constexpr int kBM = 128;          // query rows per CTA (UMMA M)
 constexpr int kBN = 64;           // positions per tile
-constexpr int kHD = 128;          // head dim
-constexpr int kStagesK = 3;       // tiles in the K ring
-constexpr int kStagesV = 2;       // tiles in the V ring
 constexpr int kSoftmaxThreads = 128;               // one thread per query row
 constexpr int kThreadsTC = 256;  // 4 softmax warps, K producer, MMA issuer, V producer, 1 idle: registers are allotted per 4 warps
 constexpr int kRegionQ = kBM * 128;                // [128 rows][64] bf16, 128-byte rows: 16 KB
 constexpr int kRegionKV = kBN * 128;               // [64 positions][64] bf16: 8 KB
-constexpr int kTileKV = 2 * kRegionKV;             // a [64][128] K or V tile: 16 KB
-constexpr int kSmemQ = 0;                          // 2 regions (d 0-63, d 64-127)
-constexpr int kSmemK = 2 * kRegionQ;                 // kStagesK tiles
-constexpr int kSmemV = kSmemK + kStagesK * kTileKV;  // kStagesV tiles
-constexpr int kSmemBar = kSmemV + kStagesV * kTileKV;  // mbarriers and two words, 128 bytes
-constexpr int kSmemBytes = kSmemBar + 128;           // 112 KB + 128 B: two CTAs per SM
+constexpr int kPartRow = 256;                      // bytes of a partial output row: 128 halves or 64 floats
+
+// What depends on the head dimension. A region is 64 dims wide. 64-dim tiles are half as large, so the rings are deeper
+// (the same bytes in flight); their P goes to the tensor cores as two bf16 terms, and their partials stay fp32 (see Part).
+template <int HD>
+struct Geo {
+  static constexpr int kReg = HD / 64;
+  static constexpr bool kSplitP = HD == 64;
+  static constexpr int kStagesK = HD == 64 ? 4 : 3;      // tiles in the K ring
+  static constexpr int kStagesV = HD == 64 ? 4 : 2;      // tiles in the V ring
+  static constexpr int kTileKV = kReg * kRegionKV;       // a [64][HD] K or V tile: 16 KB at 128 dims
+  static constexpr int kSmemQ = 0;                       // kReg regions (d 0-63, d 64-127)
+  static constexpr int kSmemK = kReg * kRegionQ;         // kStagesK tiles
+  static constexpr int kSmemV = kSmemK + kStagesK * kTileKV;    // kStagesV tiles
+  static constexpr int kSmemBar = kSmemV + kStagesV * kTileKV;  // mbarriers and two words
+  static constexpr int kBars = 2 * kStagesK + 2 * kStagesV + 5;
+  static constexpr int kSmemBytes = kSmemBar + 256;      // 112 KB at 128 dims: two CTAs per SM
+  static constexpr int kStageStride = HD + 4;            // floats per staged output row: 16-byte accesses stay conflict-free
+  static_assert(kBM * kStageStride * 4 <= (kStagesK + kStagesV) * kTileKV, "staged rows fit in the rings");
+  static_assert(kBars * 8 + 8 <= 256, "barrier slots");
+};
 constexpr int kTmemCols = 256;                     // S0: [0,64), S1: [64,128), O: [128,256)
 constexpr long long kWaitCycles = 4000000000ll;    // about two seconds
 constexpr int kMaxSplit = 8;
@@ -74,7 +90,7 @@ struct TcParams {
   int cs;   // CTAs per cluster (1..8); 0: no clusters, splits sized on the device and merged through global memory
   int rpc;  // cluster mode: row blocks a cluster covers at most (cs is a multiple of it)
   int nsplit_max, num_sms, nrb;  // global-merge mode
-  __half* part_o;    // [B][Hq][Ncap][nsplit_max][D]: partial rows normalised by their own sum, half precision
+  unsigned char* part_o;  // [B][Hq][Ncap][nsplit_max] partial rows of kPartRow bytes, normalised by their own sum
   float* part_ml;    // [B][Hq][Ncap][nsplit_max][2]
   int32_t* ticket;   // [B][Hkv][nrb]
   const int32_t* page_table;
@@ -249,9 +265,18 @@ __device__ __forceinline__ void tmem_wait_ld_regs(uint32_t (&r)[32]) {
 }
 // One half tile (32 scores of this thread's row, in registers) of the single-pass softmax: P = 2^(s * scale -
 // m * scale) as bf16 pairs, the row sum as a packed pair of partial sums. kMasked: `vv` holds the 32 visibility bits.
-template <bool kMasked>
+// kSplit: `lo` receives what the bf16 rounding of P left over, again as bf16 pairs.
+__device__ __forceinline__ void pack_p(float p0, float p1, uint32_t& hi) {
+  const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
+  hi = *reinterpret_cast<const uint32_t*>(&pb);
+}
+__device__ __forceinline__ void pack_p(float p0, float p1, uint32_t& hi, uint32_t& lo) {
+  pack_p(p0, p1, hi);
+  pack_p(p0 - __uint_as_float(hi << 16), p1 - __uint_as_float(hi & 0xffff0000u), lo);
+}
+template <bool kMasked, bool kSplit>
 __device__ __forceinline__ void softmax_half(const uint32_t (&sr)[32], unsigned long long sc2, unsigned long long neg2,
-                                             uint32_t vv, unsigned long long& lacc, uint32_t (&pk)[16]) {
+                                             uint32_t vv, unsigned long long& lacc, uint32_t (&pk)[16], uint32_t (&lo)[16]) {
 #pragma unroll
   for (int e = 0; e < 16; ++e) {
     const int c = 2 * e;
@@ -263,8 +288,8 @@ __device__ __forceinline__ void softmax_half(const uint32_t (&sr)[32], unsigned 
       p1 = ((vv >> (c + 1)) & 1u) ? p1 : 0.f;
     }
     lacc = add_f2(lacc, pack_f2(p0, p1));
-    const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
-    pk[e] = *reinterpret_cast<const uint32_t*>(&pb);
+    if constexpr (kSplit) pack_p(p0, p1, pk[e], lo[e]);
+    else pack_p(p0, p1, pk[e]);
   }
 }
 
@@ -391,8 +416,40 @@ __device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr) {
   return v;
 }
 
-constexpr int kStageStride = kHD + 4;   // floats per staged output row: 16-byte accesses stay conflict-free
-constexpr int kStageStrideH = kHD + 8;  // halves per staged row of a cluster-merged partial (272 bytes)
+constexpr int kStageStrideP = kPartRow + 16;  // bytes per staged partial row (272)
+
+// Partial rows: 256 bytes, a lane owns 8 of them. 128 dims: halves (their rounding, 2^-11 relative, is a quarter of the
+// bf16 output's; half the bytes to move), four columns per lane. 64 dims: floats, two columns per lane.
+template <int HD> struct Part;
+template <> struct Part<128> {
+  static constexpr int NC = 4;
+  static __device__ __forceinline__ void add(float (&acc)[4], uint2 v, float w) {
+    const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&v.x));
+    const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
+    acc[0] += lo.x * w;
+    acc[1] += lo.y * w;
+    acc[2] += hi.x * w;
+    acc[3] += hi.y * w;
+  }
+  static __device__ __forceinline__ void store(__nv_bfloat16* row, int lane, const float (&acc)[4], float inv) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv), c = __floats2bfloat162_rn(acc[2] * inv, acc[3] * inv);
+    uint2 pk;
+    pk.x = *reinterpret_cast<const uint32_t*>(&a);
+    pk.y = *reinterpret_cast<const uint32_t*>(&c);
+    *reinterpret_cast<uint2*>(row + lane * 4) = pk;
+  }
+};
+template <> struct Part<64> {
+  static constexpr int NC = 2;
+  static __device__ __forceinline__ void add(float (&acc)[2], uint2 v, float w) {
+    acc[0] += __uint_as_float(v.x) * w;
+    acc[1] += __uint_as_float(v.y) * w;
+  }
+  static __device__ __forceinline__ void store(__nv_bfloat16* row, int lane, const float (&acc)[2], float inv) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv);
+    *reinterpret_cast<uint32_t*>(row + lane * 2) = *reinterpret_cast<const uint32_t*>(&a);
+  }
+};
 __device__ __forceinline__ uint2 ld_cluster_u2(uint32_t addr) {
   uint2 v;
   asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
@@ -405,7 +462,7 @@ __device__ __forceinline__ uint2 ld_cluster_u2(uint32_t addr) {
 // output's), and (max, sum) per row in its own shared memory. This CTA owns the rows rr with
 // rr % nsplit == split and reads them from all peers: split s weighs sum_s * e^(max_s - max).
 // Warp w takes owned rows w, w+8, ...; a lane owns 4 output columns; ROWS x SPL loads in flight.
-template <int ROWS, int SPL>
+template <int HD, int ROWS, int SPL>
 __device__ __forceinline__ void merge_rows(const TcParams& p, uint32_t stage_o_s, uint32_t stage_ml_s, int rank0,
                                            int b, int kvh, int row0, int rows_here, int nsplit, int split) {
   const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5, G = p.G;
@@ -419,7 +476,7 @@ __device__ __forceinline__ void merge_rows(const TcParams& p, uint32_t stage_o_s
       const int i2 = i0 + 8 * u;
       const int rr = split + nsplit * (i2 < owned ? i2 : i0);
       const int grow = row0 + rr, tt = grow / G, hh = kvh * G + grow % G;
-      orow[u] = (((size_t)b * p.Ncap + tt) * p.Hq + hh) * kHD;
+      orow[u] = (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD;
       float ms = -INFINITY, ls = 0.f;  // lane s holds split s's (max, sum)
       if (lane < nsplit) {
         const float2 ml = ld_cluster_f2(map_to_rank(stage_ml_s + (uint32_t)rr * 8u, (uint32_t)(rank0 + lane)));
@@ -428,7 +485,7 @@ __device__ __forceinline__ void merge_rows(const TcParams& p, uint32_t stage_o_s
       }
 #pragma unroll
       for (int s2 = 0; s2 < SPL; ++s2)
-        v[u][s2] = s2 < nsplit ? ld_cluster_u2(map_to_rank(stage_o_s + (uint32_t)(rr * kStageStrideH + lane * 4) * 2u,
+        v[u][s2] = s2 < nsplit ? ld_cluster_u2(map_to_rank(stage_o_s + (uint32_t)(rr * kStageStrideP + lane * 8),
                                                            (uint32_t)(rank0 + s2)))
                                : make_uint2(0u, 0u);
       float M = ms;
@@ -442,26 +499,16 @@ __device__ __forceinline__ void merge_rows(const TcParams& p, uint32_t stage_o_s
     }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float acc[Part<HD>::NC] = {};
 #pragma unroll
       for (int s2 = 0; s2 < SPL; ++s2) {
         const float w = __shfl_sync(0xffffffffu, wgt[u], s2);
         if (w > 0.f) {  // a split without visible positions staged nothing: its buffer may hold anything
-          const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&v[u][s2].x));
-          const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&v[u][s2].y));
-          acc.x += lo.x * w;
-          acc.y += lo.y * w;
-          acc.z += hi.x * w;
-          acc.w += hi.y * w;
+          Part<HD>::add(acc, v[u][s2], w);
         }
       }
       if (i0 + 8 * u < owned) {
-        const __nv_bfloat162 a = __floats2bfloat162_rn(acc.x * inv[u], acc.y * inv[u]),
-                             c2 = __floats2bfloat162_rn(acc.z * inv[u], acc.w * inv[u]);
-        uint2 pk;
-        pk.x = *reinterpret_cast<const uint32_t*>(&a);
-        pk.y = *reinterpret_cast<const uint32_t*>(&c2);
-        *reinterpret_cast<uint2*>(p.out + orow[u] + lane * 4) = pk;
+        Part<HD>::store(p.out + orow[u], lane, acc, inv[u]);
       }
     }
   }
@@ -598,7 +645,7 @@ __device__ __forceinline__ WorkItem decode_work_chunked(const TcParams& p, int i
 // Merge of the split partials of a row block, run by all 8 warps of the last CTA to finish it.
 // Warp w takes rows w, w+8, ...; a lane owns 4 output columns. ROWS rows x SPL splits = 16 loads are
 // in flight per lane: the merge is bound by L2 latency, not by bytes.
-template <int ROWS, int SPL>
+template <int HD, int ROWS, int SPL>
 __device__ __forceinline__ void merge_rows_global(const TcParams& p, int b, int kvh, int row0, int rows_here, int nsplit) {
   const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5, G = p.G;
   for (int rr = wv; rr < rows_here; rr += 8 * ROWS) {
@@ -612,7 +659,7 @@ __device__ __forceinline__ void merge_rows_global(const TcParams& p, int b, int 
       const int r2 = rr + 8 * u;
       const int grow = row0 + (r2 < rows_here ? r2 : rr), tt = grow / G, hh = kvh * G + grow % G;
       const size_t pr = (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max;
-      orow[u] = (((size_t)b * p.Ncap + tt) * p.Hq + hh) * kHD;
+      orow[u] = (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD;
       msv[u] = -INFINITY;  // lane s holds split s's (max, sum)
       lsv[u] = 0.f;
       if (lane < nsplit) {
@@ -622,7 +669,7 @@ __device__ __forceinline__ void merge_rows_global(const TcParams& p, int b, int 
       }
 #pragma unroll
       for (int s2 = 0; s2 < SPL; ++s2)
-        v[u][s2] = s2 < nsplit ? __ldcg(reinterpret_cast<const uint2*>(p.part_o + (pr + s2) * kHD + lane * 4))
+        v[u][s2] = s2 < nsplit ? __ldcg(reinterpret_cast<const uint2*>(p.part_o + (pr + s2) * kPartRow + lane * 8))
                                : make_uint2(0u, 0u);
     }
 #pragma unroll
@@ -639,26 +686,16 @@ __device__ __forceinline__ void merge_rows_global(const TcParams& p, int b, int 
     }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float acc[Part<HD>::NC] = {};
 #pragma unroll
       for (int s2 = 0; s2 < SPL; ++s2) {
         const float w = __shfl_sync(0xffffffffu, wgt[u], s2);
         if (w > 0.f) {  // a split without visible positions wrote zeros at best
-          const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&v[u][s2].x));
-          const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&v[u][s2].y));
-          acc.x += lo.x * w;
-          acc.y += lo.y * w;
-          acc.z += hi.x * w;
-          acc.w += hi.y * w;
+          Part<HD>::add(acc, v[u][s2], w);
         }
       }
       if (rr + 8 * u < rows_here) {
-        const __nv_bfloat162 a = __floats2bfloat162_rn(acc.x * inv[u], acc.y * inv[u]),
-                             c2 = __floats2bfloat162_rn(acc.z * inv[u], acc.w * inv[u]);
-        uint2 pk;
-        pk.x = *reinterpret_cast<const uint32_t*>(&a);
-        pk.y = *reinterpret_cast<const uint32_t*>(&c2);
-        *reinterpret_cast<uint2*>(p.out + orow[u] + lane * 4) = pk;
+        Part<HD>::store(p.out + orow[u], lane, acc, inv[u]);
       }
     }
   }
@@ -690,10 +727,14 @@ __global__ void __launch_bounds__(256) attn_worklist_kernel(const TcParams p, in
   if ((threadIdx.x & 31) == 0) store_item(list + (size_t)idx * 8, w);
 }
 
+template <int HD>
 __global__ void __launch_bounds__(kThreadsTC, 2)
 tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_q) {
   extern __shared__ __align__(1024) unsigned char smem[];  // no static shared memory: the base is 1 KB aligned
+  using GE = Geo<HD>;
+  constexpr int kStagesK = GE::kStagesK, kStagesV = GE::kStagesV, kTileKV = GE::kTileKV, kReg = GE::kReg;
+  constexpr int kSmemQ = GE::kSmemQ, kSmemK = GE::kSmemK, kSmemV = GE::kSmemV, kStageStride = GE::kStageStride;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cs = p.cs;
@@ -757,17 +798,15 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   const bool row_ok = warp < 4 && row < rows_total;
   const int t_tok = row_ok ? F + row / G : 0, h_q = kvh * G + (row_ok ? row % G : 0);
 
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kSmemBar);
-  static_assert(kStagesK <= 3 && kStagesV <= 2, "barrier slots");
-  uint64_t* bar_fullk = bars;          // [kStagesK]
-  uint64_t* bar_fullv = bars + 3;      // [kStagesV]
-  uint64_t* bar_freek = bars + 5;      // [kStagesK]
-  uint64_t* bar_freev = bars + 8;      // [kStagesV]
-  uint64_t* bar_s = bars + 10;         // [2]
-  uint64_t* bar_p = bars + 12;         // [2]: tile it uses bar_p[it & 1], phase it >> 1
-  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(bars + 14);
-  int* last_s = reinterpret_cast<int*>(bars + 14) + 1;
-  uint64_t* bar_q = bars + 15;         // the Q row block has landed (TMA)
+  uint64_t* bar_fullk = reinterpret_cast<uint64_t*>(smem + GE::kSmemBar);  // [kStagesK]
+  uint64_t* bar_fullv = bar_fullk + kStagesK;                              // [kStagesV]
+  uint64_t* bar_freek = bar_fullv + kStagesV;                              // [kStagesK]
+  uint64_t* bar_freev = bar_freek + kStagesK;                              // [kStagesV]
+  uint64_t* bar_s = bar_freev + kStagesV;                                  // [2]
+  uint64_t* bar_p = bar_s + 2;                                             // [2]: tile it uses bar_p[it & 1], phase it >> 1
+  uint64_t* bar_q = bar_p + 2;                                             // the Q row block has landed (TMA)
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(bar_q + 1);
+  int* last_s = reinterpret_cast<int*>(bar_q + 1) + 1;
 
   // ---- producer helper (warp 4; all 32 lanes call it): which = 0: K tile j, which = 1: V tile j
   // Paged caches: a producer warp reads the page table 32 entries at a time (one coalesced load, lane l keeps
@@ -790,8 +829,8 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
         pg_win0 = e0;
         pg_id = e0 + lane < p.seq_capacity ? p.page_table[(size_t)b * p.seq_capacity + e0 + lane] : 0;
       }
-      const int pg = __shfl_sync(0xffffffffu, pg_id, e0 - pg_win0 + (lane >> 1));
-      if (lane < npages * 2) {
+      const int pg = __shfl_sync(0xffffffffu, pg_id, e0 - pg_win0 + lane / kReg);
+      if (lane < npages * kReg) {
         page = pg;
         if (page < 0 || page >= p.num_pages) {
           report(p.st, CAST_ERR_BAD_PAGE, b);
@@ -803,12 +842,12 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     if (ps == 0) {
       if (lane == 0) mbar_expect_tx(full, kTileKV);
       __syncwarp();
-      if (lane < 2) tma_load_3d(map, dst + lane * kRegionKV, full, lane * 64, kvh, b * p.seq_capacity + pos0);
+      if (lane < kReg) tma_load_3d(map, dst + lane * kRegionKV, full, lane * 64, kvh, b * p.seq_capacity + pos0);
     } else {  // at most 8 pages per tile (page size >= 8): one (page, column half) per lane
-      if (lane == 0) mbar_expect_tx(full, (uint32_t)npages * ps * 128 * 2);
+      if (lane == 0) mbar_expect_tx(full, (uint32_t)npages * ps * 128 * kReg);
       __syncwarp();
-      if (lane < npages * 2) {
-        const int slot = lane >> 1, hsel = lane & 1;
+      if (lane < npages * kReg) {
+        const int slot = lane / kReg, hsel = lane % kReg;
         tma_load_4d(map, dst + hsel * kRegionKV + slot * ps * 128, full, hsel * 64, kvh, 0, page);
       }
     }
@@ -872,9 +911,9 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
       asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
     if (p.q_tma && ntile > 0) {  // (a split without tiles stages its empty partial in this region right away)
-      if (lane == 0) mbar_expect_tx(bar_q, 2 * kRegionQ);
+      if (lane == 0) mbar_expect_tx(bar_q, kReg * kRegionQ);
       __syncwarp();
-      if (lane < 2)
+      if (lane < kReg)
         tma_load_3d(&map_q, smem + kSmemQ + lane * kRegionQ, bar_q, lane * 64, kvh * G, b * p.Ncap + F + row0 / G);
     }
     // the first K tiles need no stage wait: the ring fills while Q is on its way
@@ -892,12 +931,12 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
         if (w < p.words) aw[w] = p.anc[((size_t)b * p.Ncap + t_tok) * p.words + w];
     }
     if (!p.q_tma) {
-      const __nv_bfloat16* qrow = p.q + (((size_t)b * p.Ncap + t_tok) * p.Hq + h_q) * kHD;
-      uint4 qv[16];
+      const __nv_bfloat16* qrow = p.q + (((size_t)b * p.Ncap + t_tok) * p.Hq + h_q) * HD;
+      uint4 qv[HD / 8];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) qv[c] = row_ok ? *reinterpret_cast<const uint4*>(qrow + c * 8) : make_uint4(0u, 0u, 0u, 0u);
+      for (int c = 0; c < HD / 8; ++c) qv[c] = row_ok ? *reinterpret_cast<const uint4*>(qrow + c * 8) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-      for (int c = 0; c < 16; ++c)
+      for (int c = 0; c < HD / 8; ++c)
         *reinterpret_cast<uint4*>(smem + kSmemQ + (c >> 3) * kRegionQ + swz(r, c & 7)) = qv[c];
       fence_proxy_async();
     }
@@ -922,7 +961,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   } else if (warp == 5) {
     // =========================== MMA issuer ===========================
     const uint32_t idesc_qk = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-    const uint32_t idesc_pv = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(kHD >> 3) << 17) |
+    const uint32_t idesc_pv = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(HD >> 3) << 17) |
                               ((uint32_t)(kBM >> 4) << 24);  // B operand (V) is MN-major, N = head dim
     // Everything the issue loop computes with is made warp-uniform in the compiler's eyes (a warp reduction
     // of values that are equal in all lanes anyway: the tile count comes from a load, the TMEM address from
@@ -937,7 +976,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     auto mma_qk = [&](int stage, int buf) {  // S[buf] = Q K^T; releases the K stage (all lanes, converged)
       const uint64_t dks = dk + (uint64_t)(stage * (kTileKV >> 4));
 #pragma unroll
-      for (int ks = 0; ks < kHD / 16; ++ks)
+      for (int ks = 0; ks < HD / 16; ++ks)
         umma_bf16(tmem_su + buf * kBN, dq + (uint64_t)((ks >> 2) * (kRegionQ >> 4) + (ks & 3) * 2),
                   dks + (uint64_t)((ks >> 2) * (kRegionKV >> 4) + (ks & 3) * 2), idesc_qk, ks > 0);
       umma_commit(&bar_s[buf]);
@@ -949,6 +988,11 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
       for (int ks = 0; ks < kBN / 16; ++ks)
         umma_bf16_ts(tmem_ou, tmem_su + buf * kBN + ks * 8, dvs + (uint64_t)(ks * (2048 >> 4)), idesc_pv,
                      (!first || ks > 0) ? 1u : 0u);
+      if constexpr (GE::kSplitP) {  // the second bf16 term of P lies in the upper half of the score buffer
+#pragma unroll
+        for (int ks = 0; ks < kBN / 16; ++ks)
+          umma_bf16_ts(tmem_ou, tmem_su + buf * kBN + kBN / 2 + ks * 8, dvs + (uint64_t)(ks * (2048 >> 4)), idesc_pv, 1u);
+      }
       umma_commit(&bar_freev[stage]);
     };
     // next scores first: Q K^T of tile it+1 runs while the softmax of tile `it` does; the other CTA on
@@ -999,8 +1043,8 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
         if (ok) {
           const int valid = total - pos0;
           unsigned char* vbase = smem + kSmemV + stage * kTileKV;
-          for (int i = tid; i < (kBN - valid) * 16; i += kSoftmaxThreads) {
-            const int rr = valid + (i >> 4), reg = (i >> 3) & 1, c = i & 7;
+          for (int i = tid; i < (kBN - valid) * 8 * kReg; i += kSoftmaxThreads) {
+            const int rr = valid + i / (8 * kReg), reg = (i >> 3) % kReg, c = i & 7;
             *reinterpret_cast<uint4*>(vbase + reg * kRegionKV + rr * 128 + c * 16) = make_uint4(0u, 0u, 0u, 0u);
           }
           fence_proxy_async();  // the MMA reads these rows through the async proxy
@@ -1062,7 +1106,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
         }
         // a row past the tree takes -inf: its P is 0 for every finite score, with no masking
         float neg_ms = row_ok ? -m_used * sc : -INFINITY;
-        uint32_t pk[2][16];
+        uint32_t pk[2][16], plo[2][16];  // P, and (64 dims) its second term
         unsigned long long lacc = pack_f2(0.f, 0.f);
         {
           const unsigned long long neg2 = pack_f2(neg_ms, neg_ms);
@@ -1072,11 +1116,11 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
           // top of five per pair), and all tiles but the last one or two are unmasked.
           tmem_wait_ld_regs(sra);
           tmem_ld32(tp + 32, srb);  // in flight while the first half is computed
-          if (plain) softmax_half<false>(sra, sc2, neg2, 0u, lacc, pk[0]);
-          else softmax_half<true>(sra, sc2, neg2, v0, lacc, pk[0]);
+          if (plain) softmax_half<false, GE::kSplitP>(sra, sc2, neg2, 0u, lacc, pk[0], plo[0]);
+          else softmax_half<true, GE::kSplitP>(sra, sc2, neg2, v0, lacc, pk[0], plo[0]);
           tmem_wait_ld_regs(srb);
-          if (plain) softmax_half<false>(srb, sc2, neg2, 0u, lacc, pk[1]);
-          else softmax_half<true>(srb, sc2, neg2, v1, lacc, pk[1]);
+          if (plain) softmax_half<false, GE::kSplitP>(srb, sc2, neg2, 0u, lacc, pk[1], plo[1]);
+          else softmax_half<true, GE::kSplitP>(srb, sc2, neg2, v1, lacc, pk[1], plo[1]);
         }
         float l0, l1;
         unpack_f2(lacc, l0, l1);
@@ -1112,7 +1156,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
             const float alpha = l_run > 0.f ? ldexpf(1.f, -(int)kf) : 1.f;
             if (it > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
 #pragma unroll 1
-              for (int q4 = 0; q4 < 4; ++q4) {  // O follows (P V of tile it-1 is over)
+              for (int q4 = 0; q4 < HD / 32; ++q4) {  // O follows (P V of tile it-1 is over)
                 uint32_t orr[32];
                 const uint32_t ta = tmem_o + lane_sel + q4 * 32;
                 tmem_ld32(ta, orr);
@@ -1141,14 +1185,18 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
                 p1 = ((vv >> (c + 1)) & 1u) ? p1 : 0.f;
                 l0 += p0;
                 l1 += p1;
-                const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
-                pk[hh][e] = *reinterpret_cast<const uint32_t*>(&pb);
+                if constexpr (GE::kSplitP) pack_p(p0, p1, pk[hh][e], plo[hh][e]);
+                else pack_p(p0, p1, pk[hh][e]);
               }
             }
           }
         }
         tmem_st16(tp, pk[0]);
         tmem_st16(tp + 16, pk[1]);
+        if constexpr (GE::kSplitP) {
+          tmem_st16(tp + 32, plo[0]);
+          tmem_st16(tp + 48, plo[1]);
+        }
         l_run += l0 + l1;
         tmem_wait_st();
         zero_v_tail(it);
@@ -1166,11 +1214,11 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     }
     if (ok && warp_live && ntile > 0) {
       tc_fence_after();
-      if (nsplit > 1) {  // to be merged with other splits: the row normalised by its own sum, in half precision
+      if (HD == 128 && nsplit > 1) {  // to be merged with other splits: the row normalised by its own sum, in half precision
         const float inv_l = l_run > 0.f ? 1.f / l_run : 0.f;
-        __half* sh = reinterpret_cast<__half*>(stage_o) + r * kStageStrideH;
+        __half* sh = reinterpret_cast<__half*>(reinterpret_cast<unsigned char*>(stage_o) + r * kStageStrideP);
 #pragma unroll
-        for (int hh = 0; hh < 4; ++hh) {
+        for (int hh = 0; hh < HD / 32; ++hh) {
           uint32_t orr[32];
           tmem_ld32(tmem_o + lane_sel + hh * 32, orr);
           tmem_wait_ld();
@@ -1186,9 +1234,11 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
             *reinterpret_cast<uint4*>(sh + hh * 32 + c8 * 8) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
         }
-      } else {
+      } else {  // fp32; a partial row normalised as well
+        static_assert(HD == 128 || kStageStride * 4 == kStageStrideP, "fp32 partial rows have the stride of staged rows");
+        const float f = nsplit > 1 && l_run > 0.f ? 1.f / l_run : 1.f;
 #pragma unroll
-        for (int hh = 0; hh < 4; ++hh) {
+        for (int hh = 0; hh < HD / 32; ++hh) {
           uint32_t orr[32];
           tmem_ld32(tmem_o + lane_sel + hh * 32, orr);
           tmem_wait_ld();
@@ -1196,8 +1246,8 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
 #pragma unroll
           for (int c4 = 0; c4 < 8; ++c4)
             *reinterpret_cast<float4*>(so + c4 * 4) =
-                make_float4(__uint_as_float(orr[c4 * 4]), __uint_as_float(orr[c4 * 4 + 1]), __uint_as_float(orr[c4 * 4 + 2]),
-                            __uint_as_float(orr[c4 * 4 + 3]));
+                make_float4(__uint_as_float(orr[c4 * 4]) * f, __uint_as_float(orr[c4 * 4 + 1]) * f,
+                            __uint_as_float(orr[c4 * 4 + 2]) * f, __uint_as_float(orr[c4 * 4 + 3]) * f);
         }
       }
     }
@@ -1215,23 +1265,25 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   if (nsplit == 1) {
     for (int rr = warp; rr < rows_here; rr += kThreadsTC / 32) {
       const int grow = grow0 + rr, tt = grow / G, hh = kvh * G + grow % G;
-      const float4 o4 = *reinterpret_cast<const float4*>(stage_o + rr * kStageStride + lane * 4);
+      constexpr int NC = Part<HD>::NC;
+      float acc[NC];
+#pragma unroll
+      for (int e = 0; e < NC; e += 2) {
+        const float2 o2 = *reinterpret_cast<const float2*>(stage_o + rr * kStageStride + lane * NC + e);
+        acc[e] = o2.x;
+        acc[e + 1] = o2.y;
+      }
       const float l_tot = stage_ml[rr * 2 + 1];
-      const float inv = l_tot > 0.f ? 1.f / l_tot : 0.f;
-      const __nv_bfloat162 a = __floats2bfloat162_rn(o4.x * inv, o4.y * inv), c2 = __floats2bfloat162_rn(o4.z * inv, o4.w * inv);
-      uint2 pk;
-      pk.x = *reinterpret_cast<const uint32_t*>(&a);
-      pk.y = *reinterpret_cast<const uint32_t*>(&c2);
-      *reinterpret_cast<uint2*>(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * kHD + lane * 4) = pk;
+      Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, lane, acc, l_tot > 0.f ? 1.f / l_tot : 0.f);
     }
   } else if (cs == 0) {
     // global-merge mode: partials to the workspace; the last split of this row block to finish merges
-    const __half* sh = reinterpret_cast<const __half*>(stage_o);
+    const unsigned char* sh = reinterpret_cast<const unsigned char*>(stage_o);
     for (int rr = warp; rr < rows_here; rr += kThreadsTC / 32) {
       const int grow = grow0 + rr, tt = grow / G, hh = kvh * G + grow % G;
       const size_t pr = (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max + split;
-      __stcg(reinterpret_cast<uint2*>(p.part_o + pr * kHD + lane * 4),
-             *reinterpret_cast<const uint2*>(sh + rr * kStageStrideH + lane * 4));
+      __stcg(reinterpret_cast<uint2*>(p.part_o + pr * kPartRow + lane * 8),
+             *reinterpret_cast<const uint2*>(sh + rr * kStageStrideP + lane * 8));
       if (lane == 0) {
         __stcg(p.part_ml + pr * 2, stage_ml[rr * 2]);
         __stcg(p.part_ml + pr * 2 + 1, stage_ml[rr * 2 + 1]);
@@ -1249,16 +1301,16 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     }
     __syncthreads();
     if (*last_s) {
-      if (nsplit <= 2) merge_rows_global<4, 2>(p, b, kvh, grow0, rows_here, nsplit);
-      else if (nsplit <= 4) merge_rows_global<4, 4>(p, b, kvh, grow0, rows_here, nsplit);
-      else merge_rows_global<2, kMaxSplit>(p, b, kvh, grow0, rows_here, nsplit);
+      if (nsplit <= 2) merge_rows_global<HD, 4, 2>(p, b, kvh, grow0, rows_here, nsplit);
+      else if (nsplit <= 4) merge_rows_global<HD, 4, 4>(p, b, kvh, grow0, rows_here, nsplit);
+      else merge_rows_global<HD, 2, kMaxSplit>(p, b, kvh, grow0, rows_here, nsplit);
     }
   } else {
     const uint32_t so_s = smem_u32(stage_o), sml_s = smem_u32(stage_ml);
     const int rank0 = crank - split;  // first CTA of this row block's split group
-    if (nsplit <= 2) merge_rows<8, 2>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
-    else if (nsplit <= 4) merge_rows<4, 4>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
-    else merge_rows<2, kMaxSplit>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
+    if (nsplit <= 2) merge_rows<HD, 8, 2>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
+    else if (nsplit <= 4) merge_rows<HD, 4, 4>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
+    else merge_rows<HD, 2, kMaxSplit>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
   }
   if (cs > 1) cluster_sync_all();  // nobody leaves while a peer may still read its shared memory
 }
@@ -1279,11 +1331,11 @@ EncodeTiledFn get_encode() {
 }
 
 // Q [B * Ncap tokens][Hq heads][128 dims]: a box is 128 / G tokens x G heads x 64 dims (one row block, one half)
-bool make_q_map(CUtensorMap* map, const void* base, int B, int Ncap, int Hq, int G) {
+bool make_q_map(CUtensorMap* map, const void* base, int B, int Ncap, int Hq, int G, int D) {
   EncodeTiledFn enc = get_encode();
   if (!enc) return false;
-  const cuuint64_t dims[3] = {kHD, (cuuint64_t)Hq, (cuuint64_t)B * Ncap};
-  const cuuint64_t strides[2] = {kHD * 2, (cuuint64_t)Hq * kHD * 2};
+  const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)Hq, (cuuint64_t)B * Ncap};
+  const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)Hq * D * 2};
   const cuuint32_t box[3] = {64, (cuuint32_t)G, (cuuint32_t)(kBM / G)};
   const cuuint32_t estr[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
@@ -1291,21 +1343,21 @@ bool make_q_map(CUtensorMap* map, const void* base, int B, int Ncap, int Hq, int
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool make_kv_map(CUtensorMap* map, const void* base, int B, int Hkv, int page_size, int seq_capacity, int num_pages) {
+bool make_kv_map(CUtensorMap* map, const void* base, int B, int Hkv, int D, int page_size, int seq_capacity, int num_pages) {
   EncodeTiledFn enc = get_encode();
   if (!enc) return false;
-  const cuuint64_t row_bytes = (cuuint64_t)Hkv * kHD * 2;
+  const cuuint64_t row_bytes = (cuuint64_t)Hkv * D * 2;
   if (page_size == 0) {
-    const cuuint64_t dims[3] = {kHD, (cuuint64_t)Hkv, (cuuint64_t)B * seq_capacity};
-    const cuuint64_t strides[2] = {kHD * 2, row_bytes};
+    const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)Hkv, (cuuint64_t)B * seq_capacity};
+    const cuuint64_t strides[2] = {(cuuint64_t)D * 2, row_bytes};
     const cuuint32_t box[3] = {64, 1, kBN};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   }
-  const cuuint64_t dims[4] = {kHD, (cuuint64_t)Hkv, (cuuint64_t)page_size, (cuuint64_t)num_pages};
-  const cuuint64_t strides[3] = {kHD * 2, row_bytes, row_bytes * page_size};
+  const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)Hkv, (cuuint64_t)page_size, (cuuint64_t)num_pages};
+  const cuuint64_t strides[3] = {(cuuint64_t)D * 2, row_bytes, row_bytes * page_size};
   const cuuint32_t box[4] = {64, 1, (cuuint32_t)page_size, 1};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
@@ -1323,7 +1375,7 @@ struct TcPlan {
 constexpr size_t kTicketBytes = (size_t)CAST_MAX_BATCH * 256 * sizeof(int32_t);
 
 bool tc_shape_ok(int D, int page_size) {
-  if (D != kHD) return false;
+  if (D != 128 && D != 64) return false;
   return page_size == 0 || (page_size >= 8 && page_size <= kBN && (kBN % page_size) == 0 && (page_size % 8) == 0);
 }
 
@@ -1367,7 +1419,7 @@ bool tc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int page_size, int seq_c
       // workspace: a fixed ticket region (B * Hkv * nrb <= 64 * Hq entries), then the partials
       if ((size_t)B * Hkv * nrb * sizeof(int32_t) > kTicketBytes) return false;
       pl->rows = (size_t)B * Hq * Ncap * nsplit_max;
-      pl->ws_bytes = kTicketBytes + pl->rows * (kHD * sizeof(__half) + 2 * sizeof(float));
+      pl->ws_bytes = kTicketBytes + pl->rows * (kPartRow + 2 * sizeof(float));
     }
   }
   return pl->grid <= 0x7fffffffll;
@@ -1404,13 +1456,13 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   TcPlan pl;
   if (!tc_plan(c, B, Hq, Hkv, page_size, seq_capacity, &pl)) return false;
   CUtensorMap map_k, map_v;
-  if (!make_kv_map(&map_k, k, B, Hkv, page_size, seq_capacity, num_pages) ||
-      !make_kv_map(&map_v, v, B, Hkv, page_size, seq_capacity, num_pages))
+  if (!make_kv_map(&map_k, k, B, Hkv, D, page_size, seq_capacity, num_pages) ||
+      !make_kv_map(&map_v, v, B, Hkv, D, page_size, seq_capacity, num_pages))
     return false;
   const int G = Hq / Hkv, Ncap = c->cfg.max_tree;
   const int Nmax = c->cfg.total_token < Ncap ? c->cfg.total_token : Ncap;
   CUtensorMap map_q = map_k;  // (a valid descriptor either way; used only when q_tma is set)
-  const bool q_tma = G <= kBM && (kBM % G) == 0 && make_q_map(&map_q, q, B, Ncap, Hq, G);
+  const bool q_tma = G <= kBM && (kBM % G) == 0 && make_q_map(&map_q, q, B, Ncap, Hq, G, D);
   TcParams p;
   p.q_tma = q_tma ? 1 : 0;
   p.early = (c->attn_early && !c->tree_inputs_fresh && q_tma) ? 1 : 0;
@@ -1434,8 +1486,8 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
       return true;
     }
     p.ticket = reinterpret_cast<int32_t*>(c->attn_tc_ws);
-    p.part_o = reinterpret_cast<__half*>(reinterpret_cast<char*>(c->attn_tc_ws) + kTicketBytes);
-    p.part_ml = reinterpret_cast<float*>(p.part_o + pl.rows * kHD);
+    p.part_o = reinterpret_cast<unsigned char*>(c->attn_tc_ws) + kTicketBytes;
+    p.part_ml = reinterpret_cast<float*>(p.part_o + pl.rows * kPartRow);
   }
   // The work list: under the caller's promise the lengths and tree sizes do not change between the attention
   // calls of a step, so what every CTA would decode for itself is decoded once, by a small kernel launched in
@@ -1459,21 +1511,22 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
     }
     p.worklist = c->attn_worklist;
   }
-  static bool attr_done = false;
-  if (!attr_done) {
-    if (cudaFuncSetAttribute(tree_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
-        cudaSuccess) {
+  auto* const kern = D == 64 ? tree_attn_tc_kernel<64> : tree_attn_tc_kernel<128>;
+  const int smem_bytes = D == 64 ? Geo<64>::kSmemBytes : Geo<128>::kSmemBytes;
+  static bool attr_done[2] = {false, false};
+  if (!attr_done[D == 64]) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess) {
       *status = CAST_ERR_CUDA;
       return true;
     }
     // two CTAs per SM need the largest shared-memory carve-out
-    cudaFuncSetAttribute(tree_attn_tc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    attr_done = true;
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    attr_done[D == 64] = true;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kThreadsTC, 1, 1);
-  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1485,7 +1538,7 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  if (cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel, p, map_k, map_v, map_q) != cudaSuccess) {
+  if (cudaLaunchKernelEx(&cfg, kern, p, map_k, map_v, map_q) != cudaSuccess) {
     cudaGetLastError();
     *status = CAST_ERR_CUDA;
     return true;

@@ -82,3 +82,73 @@ def test_compaction_of_whole_position_rows(binding, Hkv, D, dtype, path):
     assert ctx.cast_poll_status()[0] == 0
     assert torch.equal(k, ref[0]) and torch.equal(v, ref[1])
     assert lens.tolist() == [x + len(path) for x in kv_len]
+
+
+def _attention_reference(q, k, v, page, table, kv_len, anc, n_tree, first=None):
+    """fp64 softmax attention on the device, one sequence at a time (rows outside [first, n_tree) stay NaN)."""
+    B, _, Hq, D = q.shape
+    out = torch.full(q.shape, float("nan"), dtype=torch.float64, device="cuda")
+    for b in range(B):
+        N, L = int(n_tree[b]), int(kv_len[b])
+        pos = torch.arange(L + N, device="cuda")
+        idx = (table[b].long()[pos // page] * page + pos % page) if page else b * k.shape[1] + pos
+        kk, vv = (x.reshape(-1, x.shape[-2], D)[idx].double().repeat_interleave(Hq // x.shape[-2], 1) for x in (k, v))
+        s = torch.einsum("thd,phd->htp", q[b, :N].double(), kk) / D ** 0.5
+        j = torch.arange(N, device="cuda")
+        vis = ((anc[b, :N][:, j // 32] >> (j % 32)[None, :]) & 1).bool()
+        s[:, :, L:] = s[:, :, L:].masked_fill(~vis[None], float("-inf"))
+        f = 0 if first is None else int(first[b])
+        out[b, f:N] = torch.einsum("htp,phd->thd", s.softmax(-1), vv)[f:]
+    return out
+
+
+def _random_trees(rng, B, cap, n_tree):
+    anc = np.zeros((B, cap, (cap + 31) // 32), np.uint32)
+    for b in range(B):
+        for t in range(n_tree[b]):
+            if t:
+                anc[b, t] = anc[b, int(rng.integers(max(0, t - 6), t))]
+            anc[b, t, t // 32] |= np.uint32(1 << (t % 32))
+    return torch.from_numpy(anc.view(np.int32)).cuda()
+
+
+def _attend(binding, rng, B, cap, n_tree, Hq, Hkv, D, page, kv, dtype=torch.bfloat16, gain=1.0, first=None, early=False):
+    """Device output and fp64 reference of one call."""
+    g = torch.Generator(device="cuda").manual_seed(int(rng.integers(1 << 30)))
+    unit = page or 1
+    seq = -(-(max(kv) + cap) // unit)
+    k, v = (torch.randn((B * seq, page, Hkv, D) if page else (B, seq, Hkv, D), generator=g, device="cuda").to(dtype)
+            for _ in range(2))
+    table = torch.randperm(B * seq, generator=g, device="cuda").to(torch.int32).view(B, seq) if page else None
+    q = (torch.randn((B, cap, Hq, D), generator=g, device="cuda") * gain).to(dtype)
+    anc, nt, kv_len = _random_trees(rng, B, cap, n_tree), _ints(n_tree), _ints(kv)
+    ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=cap, max_tree=cap)
+    ctx.cast_reserve_attention(dtype, B, Hq, Hkv, D, page, seq)
+    if early:
+        ctx.cast_set_attention_early_reads(True)
+    out = torch.full_like(q, float("nan"))
+    args = (q, k, v, B, Hq, Hkv, D, page, table, seq, B * seq if page else 0, kv_len, anc, nt)
+    for _ in range(2 if early else 1):
+        if first is None:
+            ctx.cast_tree_attention(*args, 0.0, out)
+        else:
+            ctx.cast_tree_attention_rows(*args, _ints(first), 0.0, out)
+    assert ctx.cast_poll_status()[0] == 0
+    return out, _attention_reference(q, k, v, page, table, kv, anc, n_tree, first)
+
+
+@pytest.mark.parametrize("B,cap,Hq,Hkv,page,kv", [
+    (1, 1, 1, 1, 0, [0]), (1, 33, 8, 8, 0, [63]), (2, 128, 4, 1, 16, [64, 1]), (3, 32, 14, 2, 8, [65, 700, 0]),
+    (1, 60, 32, 8, 16, [2048]), (4, 128, 64, 8, 0, [1500, 1400, 90, 1536]), (40, 12, 32, 8, 64, [37 * i for i in range(40)]),
+    (5, 48, 16, 4, 32, [5000, 10, 3000, 64, 128])])
+def test_attention_of_64_dims_rounds_only_its_output(binding, B, cap, Hq, Hkv, page, kv):
+    """bf16 heads of 64 dims: the probabilities enter the second product with 16 bits, the partials of KV splits are fp32:
+    the result is the exact one rounded to bf16 (2^-9 of the value) but for what the scores' fp32 sums leave."""
+    rng = np.random.default_rng(B * 1000 + cap)
+    n_tree = [int(rng.integers(max(1, cap // 2), cap + 1)) for _ in range(B)]
+    for gain, first in ((1.0, None), (6.0, None), (1.0, [n // 3 for n in n_tree])):
+        got, want = _attend(binding, rng, B, cap, n_tree, Hq, Hkv, 64, page, kv, gain=gain, first=first)
+        keep = ~want.isnan()
+        assert torch.equal(got.isnan(), ~keep)
+        err = (got.double() - want)[keep].abs() - want[keep].abs() * 2.0 ** -8
+        assert float(err.max()) < 2e-5 * gain
