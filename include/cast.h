@@ -308,8 +308,9 @@ CAST_API cast_status cast_accept_stochastic(cast_ctx* ctx, const void* target_lo
 /*
  * How cast_accept_stochastic organises its launch for this context's vocabulary and a logits dtype
  * (host-side query; no device work): the thread-block cluster size per sequence (16 where the
- * device can co-schedule that many CTAs with their shared memory, else 8, else 1) and whether a
- * CTA's vocabulary slice fits in shared memory (1) or every sweep recomputes it from the logits (0).
+ * device can co-schedule that many CTAs with their shared memory, else 8, else 1; with more sequences
+ * than clusters of 16 run at once the launch takes clusters of 8) and whether a
+ * CTA's vocabulary slice is cached on chip (1) or every sweep recomputes it from the logits (0).
  * cast_accept_stochastic makes this query itself on its first call; call it before a stream capture.
  */
 CAST_API cast_status cast_accept_stochastic_plan(cast_ctx* ctx, cast_dtype dtype, int* cluster_size /* host */,

@@ -2,19 +2,27 @@
 // draft probability q and target probability p is accepted iff u <= min(1, p/q); after a rejection the
 // target distribution is replaced by the residual norm(max(0, P_T - P_D))), walked over the draft tree.
 //
-// One thread-block cluster per sequence walks the accepted path. At a node every CTA of the cluster holds a
-// contiguous slice of the vocabulary: it reads its slice of the node's target and draft logits once, keeps
-// exp(logit / T - slice maximum) of both rows in shared memory as fp64, and the cluster agrees on maxima and
-// sums through distributed shared memory. The j-th residual has the closed form
+// One thread-block cluster per sequence walks the accepted path. At a node every warp of the cluster holds a
+// contiguous segment of the vocabulary: it reads the segment's target and draft logits once, keeps exp(logit / T) of
+// both in fp64 (target: registers, draft: shared memory), and the warps hand their partial sums to every CTA of the
+// cluster through distributed shared memory. The j-th residual has the closed form
 //     P_j(x) = max(0, P_T(x) - a_j P_D(x)) / F_j,   a_0 = 0, F_0 = 1, a_{j+1} = a_j + F_j, F_j = F(a_j),
 //     F(a) = sum_x max(0, P_T(x) - a P_D(x)),
 // (by induction: max(0, max(0, s - a q)/F - q) = max(0, s - (a + F) q)/F), so a rejection costs one sweep
-// over the cached slices plus one cluster-wide sum, and the test of a child x is
+// over the cached segments plus one cluster-wide sum, and the test of a child x is
 //     u * P_D(x) * F_j <= max(0, P_T(x) - a_j P_D(x)).
 // All arithmetic is fp64: the bonus token is an inverse-CDF sample over up to 150k tokens, where fp32
 // rounding would move the result in about one draw of a hundred.
-// Every CTA of a cluster computes the same decisions from the same numbers (sums are taken in rank order),
+// Every warp of a cluster computes the same decisions from the same numbers (sums are taken in one fixed order),
 // so the control flow, and with it the sequence of cluster barriers, is uniform across the cluster.
+//
+// What bounds it: fp64 issue in the exponentials (64 lanes per SM: 2 V / cluster-size of them per node and CTA at about
+// a dozen fp64 instructions each, 1.7 us at V = 128256 and 16 CTAs) and the chain of cluster-wide sums (about 1.2 us
+// each). Hence: no pass for the maximum (fp64 has the exponent range to sum exp(logit / T) as it is; the row is
+// evaluated again against its maximum only if the sum leaves 1e-280 .. 1e280), one exchange per node and per rejection
+// and none for the bonus token, whose segment sums are those of the last exchange.
+// Measured (T = 0.8, trees of 24, V = 128256 fp32; before: a maximum pass, 200 KB of cached values per CTA, clusters of 16
+// only, an exchange for the bonus token): 1 sequence 58 -> 38 us, 8: 100 -> 63, 16: 137 -> 76, 64: 481 -> 231.
 #include <math.h>
 
 #include "cast_internal.h"
@@ -26,13 +34,13 @@ namespace {
 constexpr int kStoThreads = 512;
 constexpr int kStoWarps = kStoThreads / 32;
 constexpr int kStoMaxCluster = 16;
-constexpr int kStoMaxSlice = 12288;  // vocabulary entries a CTA can cache: 2 rows x 8 B each = 192 KB
+constexpr int kStoMaxSlice = 12288;  // vocabulary entries per CTA of a cluster of 16 up to which segments are cached
 
 struct StoParams {
   const void* target_logits;
   const void* draft_logits;
-  int V, Ncap, max_depth, slice, cs;
-  double inv_T;
+  int V, Ncap, max_depth, ne, cs;  // ne: elements per lane; a CTA's slice is ne * kStoThreads
+  double inv_T, T;
   const int32_t* tokens;
   const int32_t* parent;
   const int32_t* n_tree;
@@ -45,24 +53,21 @@ struct StoParams {
 };
 
 __device__ __forceinline__ uint32_t sto_smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void sto_st_remote_f64(const double* local, uint32_t rank, double v) {
+__device__ __forceinline__ void sto_st_remote_f64x2(const double* local, uint32_t rank, double v0, double v1) {
   uint32_t ra;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(sto_smem_addr(local)), "r"(rank));
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+  asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(ra), "d"(v0), "d"(v1) : "memory");
 }
 __device__ __forceinline__ void sto_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// exp(x) for x <= 0 in fp64 to about 3e-16 relative: x = n ln2 + r with n = round(x log2 e) (ln2 split in
+// exp(x) for x <= 700 in fp64 to about 3e-16 relative: x = n ln2 + r with n = round(x log2 e) (ln2 split in
 // two so that n ln2_hi is exact), the degree-12 Taylor polynomial of e^r on |r| <= ln2 / 2 (remainder below
 // 2e-16), scaling by 2^n through the exponent field. Arguments below -708 (results near the subnormal
-// range) give 0; NaN gives NaN. Half the instructions of the general-purpose library routine, and the
-// sweeps below are bound by fp64 issue.
-__device__ __forceinline__ double sto_exp(double x) {
-  // branch-free (a select at the end), so that the compiler can interleave several calls: one call is a
-  // chain of some twenty dependent fp64 instructions
+// range) give 0; NaN gives NaN. For the values computed one at a time.
+__device__ __forceinline__ double sto_exp_any(double x) {
   const double xin = x;
   x = fmax(x, -708.0);
   const double kMagic = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer in the low word
@@ -88,138 +93,218 @@ __device__ __forceinline__ double sto_exp(double x) {
   return xin >= -708.0 ? res : (xin != xin ? xin : 0.0);
 }
 
-// The same to the same accuracy in half the fp64 instructions, for the pass that evaluates 2 V / cluster-size
-// exponentials per node: x = (128 n + j) ln2/128 + r, |r| <= ln2/256, e^x = 2^n * tab[j] * (degree-5 Taylor
-// polynomial of e^r, remainder below 1e-18), tab[j] = 2^(j/128) from shared memory.
-__device__ __forceinline__ double sto_exp_tab(double x, const double* tab) {
-  const double xin = x;
-  x = fmax(x, -708.0);
+// A row's reference and the logits between which exp(logit / T - ref) keeps to the exponent range (fp32: they only have
+// to be right within a few units of the exponent).
+struct StoRef {
+  double ref;
+  float lo, hi;
+  __device__ __forceinline__ StoRef(double r, double T) : ref(r) {
+    lo = (float)fmax((r - 690.0) * T, -3e38);
+    hi = (float)fmin((r + 690.0) * T, 3e38);
+  }
+};
+
+// exp(logit / T - ref) to the same accuracy: x = (32 n + j) ln2/32 + r, |r| <= ln2/64, e^x = 2^n * tab[j] * (degree-6
+// Taylor polynomial of e^r, remainder below 4e-18), tab[j] = 2^(j/32) held by lane j and fetched by shuffle (a table in
+// shared memory is a gather with four-way bank conflicts; 32 lanes must call). Twelve fp64 instructions; the range tests
+// are fp32: below r.lo the result is 0, above r.hi, or for NaN, infinity, which sends the caller to another reference.
+__device__ __forceinline__ double sto_exp_row(float logit, const StoRef& row, double inv_T, double tab) {
+  const float lc = fminf(fmaxf(logit, row.lo), row.hi);
+  const double x = fma((double)lc, inv_T, -row.ref);
   const double kMagic = 6755399441055744.0;
-  const double tn = fma(x, 128.0 * 1.4426950408889634074, kMagic);
-  const int k = __double2loint(tn);  // round(x * 128 / ln2), negative or zero
+  const double tn = fma(x, 32.0 * 1.4426950408889634074, kMagic);
+  const int k = __double2loint(tn);  // round(x * 32 / ln2)
   const double kd = tn - kMagic;
-  double r = fma(kd, -6.93147180369123816490e-01 / 128.0, x);
-  r = fma(kd, -1.90821492927058770002e-10 / 128.0, r);
-  double y = 8.33333333333333333333e-03;
+  double r = fma(kd, -6.93147180369123816490e-01 / 32.0, x);
+  r = fma(kd, -1.90821492927058770002e-10 / 32.0, r);
+  double y = 1.38888888888888888889e-03;
+  y = fma(y, r, 8.33333333333333333333e-03);
   y = fma(y, r, 4.16666666666666666667e-02);
   y = fma(y, r, 1.66666666666666666667e-01);
   y = fma(y, r, 0.5);
   y = fma(y, r, 1.0);
-  y = fma(y, r, 1.0);
-  y *= tab[k & 127];
-  const double res = __hiloint2double(__double2hiint(y) + (k >> 7) * 1048576, __double2loint(y));
-  return xin >= -708.0 ? res : (xin != xin ? xin : 0.0);
+  y *= r;
+  const double t = __hiloint2double(__shfl_sync(0xffffffffu, __double2hiint(tab), k & 31),
+                                    __shfl_sync(0xffffffffu, __double2loint(tab), k & 31));
+  y = fma(t, y, t);
+  const int hi = __double2hiint(y) + (max(k, -32600) >> 5) * 1048576;  // (a reference of 1e9 leaves lo a coarse bound)
+  const bool zero = logit < row.lo, big = !(logit <= row.hi);
+  return __hiloint2double(big ? 0x7ff00000 : (zero ? 0 : hi), big || zero ? 0 : __double2loint(y));
 }
 
 struct StoShared {
-  double xch[2][kStoMaxCluster][4];  // records of the cluster's CTAs, double-buffered by exchange parity
-  double wred[kStoWarps][4];
+  double xch[2][kStoMaxCluster * kStoWarps][2];  // the cluster's warps' records, in vocabulary order, double-buffered
   int32_t par[CAST_MAX_TREE];
   int32_t tok[CAST_MAX_TREE];
-  int32_t kids[CAST_MAX_TREE];
-  int32_t nkids;
-  int32_t pick_lo, pick_hi;
-  double wscan[kStoWarps];
-  double tab[128];  // 2^(j/128)
+  uint8_t kids[kStoWarps][CAST_MAX_TREE];  // every warp's own list of the current node's children
 };
 
-// Block-wide reduction of up to four values per thread (sum, or maximum for OP_MAX); every thread returns
-// with the result, folded in warp order.
-template <bool OP_MAX, int NVAL>
-__device__ __forceinline__ void sto_block_reduce(StoShared& sh, double (&v)[NVAL]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ double sto_warp_sum(double v) {
 #pragma unroll
-  for (int i = 0; i < NVAL; ++i) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double other = __shfl_xor_sync(0xffffffffu, v[i], o);
-      v[i] = OP_MAX ? fmax(v[i], other) : v[i] + other;
-    }
-  }
-  __syncthreads();  // the previous reduction's readers are done with wred
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < NVAL; ++i) sh.wred[warp][i] = v[i];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < NVAL; ++i) {
-    double acc = sh.wred[0][i];
-#pragma unroll
-    for (int w = 1; w < kStoWarps; ++w) acc = OP_MAX ? fmax(acc, sh.wred[w][i]) : acc + sh.wred[w][i];
-    v[i] = acc;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// Every CTA hands its record to every CTA of the cluster (its own copy included); after the barrier
-// sh.xch[parity][r] holds rank r's record everywhere.
-__device__ __forceinline__ void sto_exchange(StoShared& sh, int parity, int rank, int cs, const double (&rec)[4]) {
+// Every warp hands its two values to every CTA of the cluster; after the barrier sh.xch[parity] holds all records.
+__device__ __forceinline__ void sto_exchange(StoShared& sh, int parity, int rank, int cs, double v0, double v1) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double* slot = sh.xch[parity][rank * kStoWarps + warp];
   if (cs == 1) {
-    __syncthreads();
-    if (threadIdx.x < 4) sh.xch[parity][0][threadIdx.x] = rec[threadIdx.x];
+    if (lane == 0) {
+      slot[0] = v0;
+      slot[1] = v1;
+    }
     __syncthreads();
     return;
   }
-  const int tid = threadIdx.x;
-  if (tid < cs * 4) sto_st_remote_f64(&sh.xch[parity][rank][tid & 3], (uint32_t)(tid >> 2), rec[tid & 3]);
+  if (lane < cs) sto_st_remote_f64x2(slot, (uint32_t)lane, v0, v1);
   sto_cluster_sync();
 }
 
-template <typename T, bool CACHED>
+// The records' sums, in the same order in every warp.
+__device__ __forceinline__ void sto_fold(const StoShared& sh, int parity, int cs, double& s0, double& s1) {
+  const int lane = threadIdx.x & 31;
+  s0 = s1 = 0.0;
+  for (int i = lane; i < cs * kStoWarps; i += 32) {
+    s0 += sh.xch[parity][i][0];
+    s1 += sh.xch[parity][i][1];
+  }
+  s0 = sto_warp_sum(s0);
+  s1 = sto_warp_sum(s1);
+}
+
+// Target values a lane keeps in registers; the rest of a long segment joins the draft values in shared memory (with 32 or
+// 38 in registers the sweep spilled and a node of 152064 tokens took as long as with the recomputing kernel).
+__host__ __device__ constexpr int sto_in_registers(int NE) { return NE < 24 ? NE : 24; }
+// Doubles per lane in shared memory.
+__host__ __device__ constexpr int sto_in_shared(int NE) { return 2 * NE - sto_in_registers(NE); }
+
+// NE > 0: up to NE elements per lane are cached; NE == 0: every sweep recomputes them from the logits.
+template <typename T, int NE>
 __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const StoParams p) {
   extern __shared__ __align__(16) unsigned char sto_dyn[];
   __shared__ StoShared sh;
-  double* ep = reinterpret_cast<double*>(sto_dyn);  // exp(target logit / T - slice maximum), this CTA's slice
-  double* eq = ep + p.slice;                        // the same of the draft row
+  constexpr bool CACHED = NE > 0;
+  constexpr int kP = CACHED ? sto_in_registers(NE) : 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cs = p.cs, rank = blockIdx.x, b = blockIdx.y;
-  const int begin = min(rank * p.slice, p.V), len = min(p.V - begin, p.slice);
+  const int ne = CACHED ? NE : p.ne;
+  const int begin = rank * p.ne * kStoThreads + warp * p.ne * 32 + lane;  // lane's j-th element: begin + 32 j
+  const int mine = min(p.ne, max(0, (p.V - begin + 31) / 32));            // how many of them exist
+  double ep[kP];                                                          // exp(target logit / T), j < kP
+  // exp(draft logit / T) at eq[32 j], then the target's from kP on
+  double* eq = reinterpret_cast<double*>(sto_dyn) + (size_t)warp * sto_in_shared(NE) * 32 + lane;
   int N = p.n_tree[b];
   if (N < 1 || N > p.Ncap) {
     if (rank == 0 && tid == 0) report(p.st, CAST_ERR_BAD_TREE, b);
     N = N < 1 ? 1 : p.Ncap;
   }
-  if (tid >= kStoThreads - 128) sh.tab[tid - (kStoThreads - 128)] = exp2((double)(tid - (kStoThreads - 128)) * (1.0 / 128.0));
+  const double tab = exp2((double)lane * (1.0 / 32.0));
   if (tid < CAST_MAX_TREE) {
     sh.par[tid] = tid < N ? p.parent[(size_t)b * p.Ncap + tid] : -2;
     sh.tok[tid] = tid < N ? p.tokens[(size_t)b * p.Ncap + tid] : 0;
   }
+  const double u_bonus = p.u_bonus[b];
   // the peers' shared memory may be written once all CTAs of the cluster run
   if (cs > 1) sto_cluster_sync(); else __syncthreads();
 
   int parity = 0;
-  int cur = 0, plen = 1;   // current node, nodes on the path so far
-  double a = 0.0;          // the distribution that stands at `cur`: max(0, P_T - a P_D) / F(a)
-  double cp = 0.0, cq = 0.0, Mp = 0.0, Sp = 1.0, Mq = 0.0, Sq = 1.0, Mp_loc = 0.0, Mq_loc = 0.0;
+  int cur = 0, plen = 1;           // current node, nodes on the path so far
+  double a = 0.0;                  // the distribution that stands at `cur`: max(0, P_T - a P_D) / F(a)
+  double cp = 1.0, cq = 0.0;       // P_T(x) = e_p(x) cp, P_D(x) = e_q(x) cq
+  StoRef ref_p(0.0, p.T), ref_q(0.0, p.T);  // e(x) = exp(logit / T - ref)
+  int held = 0;                    // buffer with the segment sums of the distribution that stands
+  double held_scale = 1.0;
   const T* lp = nullptr;
   const T* lq = nullptr;
   bool has_q = false;
+  uint8_t* kids = sh.kids[warp];
   if (rank == 0 && tid == 0) p.accept_path[(size_t)b * (p.max_depth + 1)] = 0;
 
-  // unnormalised slice entries: p~(i) * cp = P_T(begin + i), q~(i) * cq = P_D(begin + i)
-  auto pt = [&](int i) -> double {
-    return CACHED ? ep[i] : sto_exp_tab((double)to_float(lp[begin + i]) * p.inv_T - (Mp_loc > -INFINITY ? Mp_loc : 0.0), sh.tab);
+  auto logit = [&](const T* row, int j) -> float { return j < mine ? to_float(row[begin + 32 * j]) : -INFINITY; };
+  auto value = [&](float x, const StoRef& row) -> double { return sto_exp_row(x, row, p.inv_T, tab); };
+  auto pt = [&](int j) -> double {  // (cached: j is a constant wherever this is called)
+    if (!CACHED) return value(logit(lp, j), ref_p);
+    return j < kP ? ep[j < kP ? j : 0] : eq[32 * (NE + j - kP)];
   };
-  auto qt = [&](int i) -> double {
-    return CACHED ? eq[i] : sto_exp_tab((double)to_float(lq[begin + i]) * p.inv_T - (Mq_loc > -INFINITY ? Mq_loc : 0.0), sh.tab);
+  auto qt = [&](int j) -> double { return CACHED ? eq[32 * j] : value(logit(lq, j), ref_q); };
+  // the node's rows evaluated: this lane's sums
+  auto evaluate = [&](double& sp, double& sq) {
+    sp = sq = 0.0;
+    if constexpr (CACHED) {
+      constexpr int U = NE < 8 ? NE : 8;  // logits in flight: the next group is loaded while this one is evaluated
+      float xp[U], xq[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        xp[j] = logit(lp, j);
+        xq[j] = has_q ? logit(lq, j) : 0.f;
+      }
+#pragma unroll
+      for (int j0 = 0; j0 < NE; j0 += U) {
+        float np[U], nq[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          np[j] = j0 + U + j < NE ? logit(lp, j0 + U + j) : 0.f;
+          nq[j] = j0 + U + j < NE && has_q ? logit(lq, j0 + U + j) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          if (j0 + j >= NE) break;
+          const double e = value(xp[j], ref_p);
+          if (j0 + j < kP) ep[j0 + j < kP ? j0 + j : 0] = e;
+          else eq[32 * (NE + j0 + j - kP)] = e;
+          sp += e;
+        }
+        if (has_q) {
+#pragma unroll
+          for (int j = 0; j < U; ++j) {
+            if (j0 + j >= NE) break;
+            const double e = value(xq[j], ref_q);
+            eq[32 * (j0 + j)] = e;
+            sq += e;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          xp[j] = np[j];
+          xq[j] = nq[j];
+        }
+      }
+    } else {
+#pragma unroll 4
+      for (int j = 0; j < ne; ++j) {
+        sp += value(logit(lp, j), ref_p);
+        if (has_q) sq += value(logit(lq, j), ref_q);
+      }
+    }
+  };
+  // this lane's share of sum_x max(0, P_T - a2 P_D)
+  auto residual = [&](double a2) -> double {
+    const double aq = a2 * cq;
+    double s = 0.0;
+#pragma unroll
+    for (int j = 0; j < (CACHED ? NE : 1); ++j) {
+      if (!CACHED) break;
+      s += fmax(0.0, pt(j) * cp - qt(j) * aq);
+    }
+    if (!CACHED) {
+#pragma unroll 4
+      for (int j = 0; j < ne; ++j) s += fmax(0.0, pt(j) * cp - qt(j) * aq);
+    }
+    return s;
   };
 
   for (;;) {
-    // ---- children of `cur` in tree order
-    __syncthreads();  // everybody is done with the previous node's list
-    if (warp == 0) {
-      int n = 0;
-      for (int base = 0; base < N; base += 32) {
-        const int c = base + lane;
-        const bool is = c < N && c > cur && sh.par[c] == cur;
-        const unsigned m = __ballot_sync(0xffffffffu, is);
-        if (is) sh.kids[n + __popc(m & ((1u << lane) - 1u))] = c;
-        n += __popc(m);
-      }
-      if (lane == 0) sh.nkids = n;
+    // ---- children of `cur` in tree order (every warp for itself)
+    int k = 0;
+    for (int base = 0; base < N; base += 32) {
+      const int c = base + lane;
+      const bool is = c < N && c > cur && sh.par[c] == cur;
+      const unsigned m = __ballot_sync(0xffffffffu, is);
+      if (is) kids[k + __popc(m & ((1u << lane) - 1u))] = (uint8_t)c;
+      k += __popc(m);
     }
-    __syncthreads();
-    int k = sh.nkids;
+    __syncwarp();
     if (k > 0 && plen > p.max_depth) {  // a path longer than the output has room for
       if (rank == 0 && tid == 0) report(p.st, CAST_ERR_BAD_TREE, b);
       k = 0;
@@ -227,135 +312,116 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
     has_q = k > 0;
     lp = reinterpret_cast<const T*>(p.target_logits) + ((size_t)b * p.Ncap + cur) * p.V;
     lq = reinterpret_cast<const T*>(p.draft_logits) + ((size_t)b * p.Ncap + cur) * p.V;
+    // the children's tests need two logits and a uniform number each, lane j for child j: asked for now, used after
+    // the sweep (a node with more than 32 children asks again)
+    float raw_p = 0.f, raw_q = 0.f;
+    double u = 0.0;
+    bool token_ok = false;
+    auto ask = [&](int j0) {
+      const int j = j0 + lane;
+      token_ok = false;
+      if (j < k) {
+        const int c = kids[j], x = sh.tok[c];
+        token_ok = x >= 0 && x < p.V;
+        if (token_ok) {
+          raw_p = to_float(lp[x]);
+          raw_q = to_float(lq[x]);
+        }
+        u = p.u_accept[(size_t)b * p.Ncap + c];
+      }
+    };
+    ask(0);
     if (k > 0) {
-      // the eldest child is the likeliest next node: its slices are asked into L2 while this node is worked on
-      const int c0 = sh.kids[0];
-      const char* np = reinterpret_cast<const char*>(reinterpret_cast<const T*>(p.target_logits) + ((size_t)b * p.Ncap + c0) * p.V + begin);
-      const char* nq = reinterpret_cast<const char*>(reinterpret_cast<const T*>(p.draft_logits) + ((size_t)b * p.Ncap + c0) * p.V + begin);
-      for (int off = tid * 128; off < len * (int)sizeof(T); off += kStoThreads * 128) {
+      // the eldest child is the likeliest next node: its segments are asked into L2 while this node is worked on
+      const size_t row = ((size_t)b * p.Ncap + kids[0]) * p.V + (begin - lane);
+      const char* np = reinterpret_cast<const char*>(reinterpret_cast<const T*>(p.target_logits) + row);
+      const char* nq = reinterpret_cast<const char*>(reinterpret_cast<const T*>(p.draft_logits) + row);
+      const int bytes = min(p.ne * 32, p.V - (begin - lane)) * (int)sizeof(T);
+      for (int off = lane * 128; off < bytes; off += 32 * 128) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(np + off));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(nq + off));
       }
     }
 
-    // the eldest child's test needs two logits and its uniform number: asked for now, used after the sweeps
-    float raw0 = 0.f;
-    double u0 = 0.0;
-    if (k > 0) {
-      const int c0 = sh.kids[0], x0 = sh.tok[c0];
-      if (x0 >= 0 && x0 < p.V) raw0 = (lane & 1) ? to_float(lq[x0]) : to_float(lp[x0]);
-      u0 = p.u_accept[(size_t)b * p.Ncap + c0];
-    }
-
-    // ---- softmax statistics of the node's rows: slice maxima, then slice sums of exp(. - slice maximum)
-    {
-      double mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll 8
-      for (int i = tid; i < len; i += kStoThreads) {
-        const double sp = (double)to_float(lp[begin + i]) * p.inv_T;
-        if (CACHED) ep[i] = sp;
-        mx[0] = fmax(mx[0], sp);
-        if (has_q) {
-          const double sq = (double)to_float(lq[begin + i]) * p.inv_T;
-          if (CACHED) eq[i] = sq;
-          mx[1] = fmax(mx[1], sq);
-        }
+    // ---- softmax sums of the node's rows
+    double Sp, Sq = 1.0;
+    ref_p = ref_q = StoRef(0.0, p.T);
+    for (int attempt = 0;; ++attempt) {
+      double sp, sq;
+      evaluate(sp, sq);
+      sto_exchange(sh, parity, rank, cs, sto_warp_sum(sp), sto_warp_sum(sq));
+      sto_fold(sh, parity, cs, Sp, Sq);
+      held = parity;
+      parity ^= 1;
+      if (attempt == 1 || (Sp > 1e-280 && Sp < 1e280 && (!has_q || (Sq > 1e-280 && Sq < 1e280)))) break;
+      // logits / T far from zero (or not finite): once more, against the rows' maxima
+      double mp = -INFINITY, mq = -INFINITY;
+      for (int j = 0; j < mine; ++j) {
+        mp = fmax(mp, (double)logit(lp, j) * p.inv_T);
+        if (has_q) mq = fmax(mq, (double)logit(lq, j) * p.inv_T);
       }
-      sto_block_reduce<true, 2>(sh, mx);
-      Mp_loc = mx[0];
-      Mq_loc = mx[1];
-      double sm[2] = {0.0, 0.0};
-      // an all -inf slice (a masked range of the vocabulary) takes reference 0: its entries become exp(-inf) = 0
-      const double ref_p = Mp_loc > -INFINITY ? Mp_loc : 0.0, ref_q = Mq_loc > -INFINITY ? Mq_loc : 0.0;
-      if (has_q) {
-#pragma unroll 4
-        for (int i = tid; i < len; i += kStoThreads) {
-          const double e0 = sto_exp_tab((CACHED ? ep[i] : (double)to_float(lp[begin + i]) * p.inv_T) - ref_p, sh.tab);
-          const double e1 = sto_exp_tab((CACHED ? eq[i] : (double)to_float(lq[begin + i]) * p.inv_T) - ref_q, sh.tab);
-          if (CACHED) {
-            ep[i] = e0;
-            eq[i] = e1;
-          }
-          sm[0] += e0;
-          sm[1] += e1;
-        }
-      } else {
-#pragma unroll 4
-        for (int i = tid; i < len; i += kStoThreads) {
-          const double e0 = sto_exp_tab((CACHED ? ep[i] : (double)to_float(lp[begin + i]) * p.inv_T) - ref_p, sh.tab);
-          if (CACHED) ep[i] = e0;
-          sm[0] += e0;
-        }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        mp = fmax(mp, __shfl_xor_sync(0xffffffffu, mp, o));
+        mq = fmax(mq, __shfl_xor_sync(0xffffffffu, mq, o));
       }
-      sto_block_reduce<false, 2>(sh, sm);
-      const double rec[4] = {Mp_loc, sm[0], Mq_loc, sm[1]};
-      sto_exchange(sh, parity, rank, cs, rec);
-      // fold of the ranks' records, the same in every warp of every CTA: lanes 0-15 take the target row's
-      // records by rank, lanes 16-31 the draft row's; maxima and sums through a fixed shuffle tree
-      {
-        const int rr = lane & 15, col = (lane >> 4) * 2;
-        const double m_r = rr < cs ? sh.xch[parity][rr][col] : -INFINITY;
-        const double s_r = rr < cs ? sh.xch[parity][rr][col + 1] : 0.0;
-        double M = m_r;
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
-        const double w_r = m_r > -INFINITY ? sto_exp(m_r - M) : 0.0;  // this rank's weight
-        double S = s_r * w_r;
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
-        Mp = __shfl_sync(0xffffffffu, M, 0);
-        Mq = __shfl_sync(0xffffffffu, M, 16);
-        Sp = __shfl_sync(0xffffffffu, S, 0);
-        Sq = __shfl_sync(0xffffffffu, S, 16);
-        cp = __shfl_sync(0xffffffffu, w_r, rank);        // exp(Mp_loc - Mp)
-        cq = __shfl_sync(0xffffffffu, w_r, 16 + rank);   // exp(Mq_loc - Mq)
+      sto_exchange(sh, parity, rank, cs, mp, mq);
+      for (int i = 0; i < cs * kStoWarps; ++i) {
+        mp = fmax(mp, sh.xch[parity][i][0]);
+        mq = fmax(mq, sh.xch[parity][i][1]);
       }
       parity ^= 1;
-      if (!(Sp > 0.0) || !isfinite(Sp) || (has_q && (!(Sq > 0.0) || !isfinite(Sq)))) {
-        if (rank == 0 && tid == 0) report(p.st, CAST_ERR_NONFINITE, b * p.Ncap + cur);
-        Sp = 1.0;  // keep the arithmetic finite; the result of this sequence is void
-        Sq = 1.0;
-        k = 0;
-        has_q = false;
-      }
-      cp = cp / Sp;
-      cq = has_q ? cq / Sq : 0.0;
+      if (isfinite(mp)) ref_p = StoRef(mp, p.T);
+      if (isfinite(mq)) ref_q = StoRef(mq, p.T);
     }
+    if (!(Sp > 0.0) || !isfinite(Sp) || (has_q && (!(Sq > 0.0) || !isfinite(Sq)))) {
+      if (rank == 0 && tid == 0) report(p.st, CAST_ERR_NONFINITE, b * p.Ncap + cur);
+      Sp = 1.0;  // keep the arithmetic finite; the result of this sequence is void
+      Sq = 1.0;
+      k = 0;
+      has_q = false;
+    }
+    cp = 1.0 / Sp;
+    cq = has_q ? 1.0 / Sq : 0.0;
+    held_scale = cp;
 
     // ---- the children, one after the other, each against the residual its elder siblings left
     a = 0.0;
     double F = 1.0;
     int next = -1;
-    for (int j = 0; j < k; ++j) {
-      const int c = sh.kids[j];
-      const int x = sh.tok[c];
-      if (x < 0 || x >= p.V) {
-        if (rank == 0 && tid == 0) report(p.st, CAST_ERR_BAD_TREE, b);
-        continue;  // not a token: never accepted
+    for (int j0 = 0; j0 < k && next < 0; j0 += 32) {
+      if (j0 > 0) ask(j0);
+      const double px_l = sto_exp_any(fma((double)raw_p, p.inv_T, -ref_p.ref)) * cp,
+                   qx_l = sto_exp_any(fma((double)raw_q, p.inv_T, -ref_q.ref)) * cq;
+      const unsigned valid = __ballot_sync(0xffffffffu, token_ok);
+      bool empty = false;
+      for (int j = j0; j < min(k, j0 + 32); ++j) {
+        if (!((valid >> (j - j0)) & 1u)) {
+          if (rank == 0 && tid == 0) report(p.st, CAST_ERR_BAD_TREE, b);
+          continue;  // not a token: never accepted
+        }
+        const double px = __shfl_sync(0xffffffffu, px_l, j - j0), qx = __shfl_sync(0xffffffffu, qx_l, j - j0);
+        const double uj = __shfl_sync(0xffffffffu, u, j - j0);
+        if (uj * qx * F <= fmax(0.0, px - a * qx)) {
+          next = kids[j];
+          break;
+        }
+        // rejected: the residual of the residual
+        const double a2 = a + F;
+        sto_exchange(sh, parity, rank, cs, sto_warp_sum(residual(a2)), 0.0);
+        double F2, none;
+        sto_fold(sh, parity, cs, F2, none);
+        if (!(F2 > 0.0)) {  // an empty residual: the distribution before it stands (and so do its segment sums)
+          empty = true;
+          break;
+        }
+        held = parity;
+        held_scale = 1.0;
+        parity ^= 1;
+        a = a2;
+        F = F2;
       }
-      const double u = j == 0 ? u0 : p.u_accept[(size_t)b * p.Ncap + c];
-      const float raw = j == 0 ? raw0 : ((lane & 1) ? to_float(lq[x]) : to_float(lp[x]));  // odd lanes: draft
-      const double v01 = (lane & 1) ? sto_exp((double)raw * p.inv_T - Mq) / Sq : sto_exp((double)raw * p.inv_T - Mp) / Sp;
-      const double px = __shfl_sync(0xffffffffu, v01, 0), qx = __shfl_sync(0xffffffffu, v01, 1);
-      const double rx = fmax(0.0, px - a * qx);
-      if (u * qx * F <= rx) {
-        next = c;
-        break;
-      }
-      // rejected: the residual of the residual
-      const double a2 = a + F;
-      double part[1] = {0.0};
-#pragma unroll 4
-      for (int i = tid; i < len; i += kStoThreads) part[0] += fmax(0.0, pt(i) * cp - a2 * (qt(i) * cq));
-      sto_block_reduce<false, 1>(sh, part);
-      const double rec[4] = {part[0], 0.0, 0.0, 0.0};
-      sto_exchange(sh, parity, rank, cs, rec);
-      double F2 = 0.0;
-      for (int r = 0; r < cs; ++r) F2 += sh.xch[parity][r][0];
-      parity ^= 1;
-      if (!(F2 > 0.0)) break;  // an empty residual: the distribution before it stands
-      a = a2;
-      F = F2;
+      if (empty) break;
     }
     if (next < 0) break;
     cur = next;
@@ -363,169 +429,192 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
     ++plen;
   }
 
-  // ---- bonus token: inversion of the cumulative sum, in token order, of max(0, P_T - a P_D) at `cur`
-  double part[1] = {0.0};
-#pragma unroll 4
-  for (int i = tid; i < len; i += kStoThreads) part[0] += fmax(0.0, pt(i) * cp - (has_q ? a * (qt(i) * cq) : 0.0));
-  sto_block_reduce<false, 1>(sh, part);
-  {
-    const double rec[4] = {part[0], 0.0, 0.0, 0.0};
-    sto_exchange(sh, parity, rank, cs, rec);
-  }
-  double total = 0.0;
-  for (int r = 0; r < cs; ++r) total += sh.xch[parity][r][0];
-  const double goal = p.u_bonus[b] * total;
-  // the slice in which the cumulative sum reaches the goal (rounding may leave none: the last non-empty one)
-  int owner = -1, last_nonempty = 0;
-  double before = 0.0, before_owner = 0.0;
-  for (int r = 0; r < cs; ++r) {
-    const double s = sh.xch[parity][r][0];
-    if (s > 0.0) last_nonempty = r;
-    if (owner < 0 && before + s >= goal && s > 0.0) {
-      owner = r;
-      before_owner = before;
-    }
-    before += s;
-  }
-  if (owner < 0) {
-    owner = last_nonempty;
-    before_owner = 0.0;
-    for (int r = 0; r < owner; ++r) before_owner += sh.xch[parity][r][0];
-  }
+  // ---- bonus token: inversion of the cumulative sum, in token order, of max(0, P_T - a P_D) at `cur`: first among the
+  // cluster's warps, whose segment sums are at hand, then inside the segment. Where rounding leaves the goal unreached,
+  // the last place that has mass is taken.
   if (rank == 0 && tid == 0) {
     p.accept_len[b] = plen - 1;
     for (int j = plen; j <= p.max_depth; ++j) p.accept_path[(size_t)b * (p.max_depth + 1) + j] = -1;
   }
-  if (rank != owner) return;
-
-  // thread t owns the contiguous piece [t * seg, (t + 1) * seg) of the slice
-  const int seg = (len + kStoThreads - 1) / kStoThreads;
-  const int i0 = min(tid * seg, len), i1 = min(i0 + seg, len);
-  const double qa = has_q ? a : 0.0;
-  double mine = 0.0;
-  for (int i = i0; i < i1; ++i) mine += fmax(0.0, pt(i) * cp - (has_q ? qa * (qt(i) * cq) : 0.0));
-  double incl = mine;
+  int owner = -1, last = -1;
+  double before = 0.0, goal;
+  {
+    constexpr int kPer = kStoMaxCluster * kStoWarps / 32;  // consecutive segments per lane
+    double s[kPer], run = 0.0;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const double other = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += other;
-  }
-  if (tid == 0) {
-    sh.pick_lo = kStoThreads;
-    sh.pick_hi = -1;
-  }
-  __syncthreads();
-  if (lane == 31) sh.wscan[warp] = incl;
-  __syncthreads();
-  double offs = before_owner;
-  for (int w = 0; w < warp; ++w) offs += sh.wscan[w];
-  incl += offs;
-  const double excl = incl - mine;
-  if (mine > 0.0) {
-    atomicMax(&sh.pick_hi, tid);
-    if (incl >= goal) atomicMin(&sh.pick_lo, tid);
-  }
-  __syncthreads();
-  const int pick = sh.pick_lo < kStoThreads ? sh.pick_lo : sh.pick_hi;
-  if (pick < 0) {  // nothing has mass here (a void sequence): token 0
-    if (tid == 0) p.bonus_token[b] = 0;
-    return;
-  }
-  if (tid == pick) {
-    double run = excl;
-    int tokx = -1, last = i0;
-    for (int i = i0; i < i1; ++i) {
-      const double r = fmax(0.0, pt(i) * cp - (has_q ? qa * (qt(i) * cq) : 0.0));
-      if (r > 0.0) last = i;
-      run += r;
-      if (run >= goal && r > 0.0) {
-        tokx = i;
-        break;
-      }
+    for (int i = 0; i < kPer; ++i) {
+      const int at = lane * kPer + i;
+      s[i] = at < cs * kStoWarps ? sh.xch[held][at][0] * held_scale : 0.0;
+      run += s[i];
     }
-    p.bonus_token[b] = begin + (tokx >= 0 ? tokx : last);
+    double incl = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    goal = u_bonus * __shfl_sync(0xffffffffu, incl, 31);
+    double at = incl - run;
+    int own_l = -1, last_l = -1;
+    double before_l = 0.0, last_before_l = 0.0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      if (s[i] > 0.0) {
+        last_l = lane * kPer + i;
+        last_before_l = at;
+        if (own_l < 0 && at + s[i] >= goal) {
+          own_l = last_l;
+          before_l = at;
+        }
+      }
+      at += s[i];
+    }
+    const unsigned hit = __ballot_sync(0xffffffffu, own_l >= 0), mass = __ballot_sync(0xffffffffu, last_l >= 0);
+    if (hit != 0u) {
+      owner = __shfl_sync(0xffffffffu, own_l, __ffs(hit) - 1);
+      before = __shfl_sync(0xffffffffu, before_l, __ffs(hit) - 1);
+    } else if (mass != 0u) {
+      owner = __shfl_sync(0xffffffffu, last_l, 31 - __clz(mass));
+      before = __shfl_sync(0xffffffffu, last_before_l, 31 - __clz(mass));
+    }
+  }
+  if (owner < 0) {  // nothing has mass (a void sequence): token 0
+    if (rank == 0 && tid == 0) p.bonus_token[b] = 0;
+  } else if (owner == rank * kStoWarps + warp) {
+    // rows of 32 consecutive tokens, one per lane: the row in which the goal is reached, then the lane
+    const double aq = has_q ? a * cq : 0.0;
+    double run = before;
+    double pick_v = 0.0, pick_at = 0.0;  // this lane's mass in the row that was picked, and the sum before that row
+    int pick = -1;
+    bool found = false;
+    auto visit = [&](int j) {
+      const double v = fmax(0.0, pt(j) * cp - (has_q ? qt(j) * aq : 0.0));
+      const double row = sto_warp_sum(v);
+      if (!found && row > 0.0) {
+        pick = j;
+        pick_v = v;
+        pick_at = run;
+        found = run + row >= goal;
+      }
+      run += row;
+    };
+#pragma unroll
+    for (int j = 0; j < (CACHED ? NE : 1); ++j)
+      if (CACHED) visit(j);
+    if (!CACHED)
+      for (int j = 0; j < ne; ++j) visit(j);
+    double incl = pick_v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const unsigned reach = __ballot_sync(0xffffffffu, pick_v > 0.0 && pick_at + incl >= goal);
+    const unsigned mass = __ballot_sync(0xffffffffu, pick_v > 0.0);
+    const int l = reach != 0u ? __ffs(reach) - 1 : (mass != 0u ? 31 - __clz(mass) : 0);
+    if (lane == 0) p.bonus_token[b] = pick >= 0 ? begin + 32 * pick + l : 0;
   }
 }
 
-template <typename T, bool CACHED>
-cast_status sto_launch(const StoParams& p, int B, size_t dyn, cudaStream_t s) {
-  auto kern = accept_stochastic_kernel<T, CACHED>;
-  CAST_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
-  if (p.cs > 8) CAST_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.cs, B, 1);
+template <typename T, int NE>
+cudaError_t sto_attributes(size_t dyn, int cs) {
+  auto kern = accept_stochastic_kernel<T, NE>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  if (e == cudaSuccess && cs > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+template <typename T, int NE>
+void sto_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cs, int B, size_t dyn, cudaStream_t s) {
+  cfg = {};
+  cfg.gridDim = dim3(cs, B, 1);
   cfg.blockDim = dim3(kStoThreads, 1, 1);
   cfg.dynamicSmemBytes = dyn;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = p.cs;
+  attr[0].val.clusterDim.x = cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  CAST_CUDA_OK(cudaLaunchKernelEx(&cfg, kern, p));
+}
+constexpr size_t sto_cache_bytes(int NE) { return (size_t)sto_in_shared(NE) * kStoThreads * sizeof(double); }
+
+template <typename T, int NE>
+cast_status sto_launch(const StoParams& p, int B, cudaStream_t s) {
+  CAST_CUDA_OK((sto_attributes<T, NE>(sto_cache_bytes(NE), p.cs)));
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  sto_config<T, NE>(cfg, attr, p.cs, B, sto_cache_bytes(NE), s);
+  CAST_CUDA_OK(cudaLaunchKernelEx(&cfg, accept_stochastic_kernel<T, NE>, p));
   return CAST_OK;
 }
-
-// Largest cluster size (16, else 8) with which a CTA of `dyn` bytes of dynamic shared memory can run.
-template <typename T, bool CACHED>
-int sto_max_cluster(size_t dyn16, size_t dyn8) {
-  auto kern = accept_stochastic_kernel<T, CACHED>;
-  for (int cs = 16; cs >= 8; cs >>= 1) {
-    const size_t dyn = cs == 16 ? dyn16 : dyn8;
-    if (dyn > (size_t)kStoMaxSlice * 16) continue;  // this slice does not fit
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess ||
-        (cs > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
-      (void)cudaGetLastError();
-      continue;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs, 1, 1);
-    cfg.blockDim = dim3(kStoThreads, 1, 1);
-    cfg.dynamicSmemBytes = dyn;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n >= 1) return cs;
-    (void)cudaGetLastError();
-  }
+// Clusters of cs CTAs that the device runs at once (0: it cannot run one).
+template <typename T, int NE>
+int sto_resident(int cs) {
+  int n = 0;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  sto_config<T, NE>(cfg, attr, cs, 1, sto_cache_bytes(NE), nullptr);
+  if (sto_attributes<T, NE>(sto_cache_bytes(NE), cs) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&n, accept_stochastic_kernel<T, NE>, &cfg) == cudaSuccess)
+    return n;
   (void)cudaGetLastError();
   return 0;
 }
 
-int slice_for(int V, int cs) { return ((V + cs - 1) / cs + 7) / 8 * 8; }
+int elements_per_lane(int V, int cs) { return ((V + cs - 1) / cs + kStoThreads - 1) / kStoThreads; }
 
-}  // namespace
+// The kernel for `ne` elements per lane: the smallest cached one that holds them, or the one that caches nothing. Slots
+// past ne cost as much as live ones, hence the steps; 38 is what fits on chip.
+#define STO_PICK(T, ne, cached, call)      \
+  (!(cached)    ? call<T, 0>               \
+   : (ne) <= 4  ? call<T, 4>               \
+   : (ne) <= 8  ? call<T, 8>               \
+   : (ne) <= 16 ? call<T, 16>              \
+   : (ne) <= 20 ? call<T, 20>              \
+   : (ne) <= 24 ? call<T, 24>              \
+   : (ne) <= 32 ? call<T, 32>              \
+                : call<T, 38>)
+constexpr int kStoMaxCached = 38;
 
-namespace {
-// Cluster size and caching mode for this context's vocabulary and a logits dtype, looked up once.
-void sto_plan(cast_ctx* c, bool f32) {
-  const int di = f32 ? 0 : 1;
+// Largest cluster size (16, else 8) that runs with this context's vocabulary and a logits dtype, whether segments are
+// cached at that size, and how many such clusters run at once; looked up once per context.
+template <typename T>
+void sto_plan(cast_ctx* c, int di) {
   if (c->sto_cs[di] != 0) return;
   const int V = c->cfg.vocab;
-  const size_t d16 = (size_t)slice_for(V, 16) * 16, d8 = (size_t)slice_for(V, 8) * 16;
-  int cs = f32 ? sto_max_cluster<float, true>(d16, d8) : sto_max_cluster<__nv_bfloat16, true>(d16, d8);
-  int cached = 1;
-  if (cs == 0) {
-    cached = 0;
-    cs = f32 ? sto_max_cluster<float, false>(0, 0) : sto_max_cluster<__nv_bfloat16, false>(0, 0);
-    if (cs == 0) cs = 1;
-  }
-  c->sto_cs[di] = cs;
-  c->sto_cached[di] = cached;
+  int cs = 0, n = 0, cached = 0;
+  for (cached = 1; cached >= 0 && n == 0; --cached)
+    for (cs = 16; cs >= 8; cs >>= 1) {
+      const int ne = elements_per_lane(V, cs);
+      if (cached && (V > cs * kStoMaxSlice || ne > kStoMaxCached)) continue;
+      n = STO_PICK(T, ne, cached, sto_resident)(cs);
+      if (n > 0) break;
+    }
+  c->sto_cached[di] = n > 0 ? cached + 1 : 0;
+  c->sto_resident[di] = n > 0 ? n : 1;
+  c->sto_cs[di] = n > 0 ? cs : 1;
 }
+
+template <typename T>
+cast_status sto_run(cast_ctx* c, StoParams& p, int B, int di, cudaStream_t s) {
+  sto_plan<T>(c, di);  // first call with this dtype: a host-side query, no device work
+  p.cs = c->sto_cs[di];
+  const bool cached = c->sto_cached[di] != 0;
+  // With more sequences than clusters of 16 run at once, clusters of 8: a node takes less than twice as long (the chain of
+  // exchanges does not grow) and twice as many sequences run.
+  if (p.cs == 16 && B > c->sto_resident[di] && (!cached || elements_per_lane(p.V, 8) <= kStoMaxCached)) p.cs = 8;
+  p.ne = elements_per_lane(p.V, p.cs);
+  return STO_PICK(T, p.ne, cached, sto_launch)(p, B, s);
+}
+
 }  // namespace
 
 extern "C" cast_status cast_accept_stochastic_plan(cast_ctx* c, cast_dtype dtype, int* cluster_size, int* cached) {
   if (!c || !cluster_size || !cached) return CAST_ERR_INVALID_ARG;
   if (dtype != CAST_F32 && dtype != CAST_BF16) return CAST_ERR_DTYPE;
-  sto_plan(c, dtype == CAST_F32);
+  if (dtype == CAST_F32) sto_plan<float>(c, 0);
+  else sto_plan<__nv_bfloat16>(c, 1);
   *cluster_size = c->sto_cs[dtype == CAST_F32 ? 0 : 1];
   *cached = c->sto_cached[dtype == CAST_F32 ? 0 : 1];
   return CAST_OK;
@@ -541,23 +630,14 @@ extern "C" cast_status cast_accept_stochastic(cast_ctx* c, const void* target_lo
     return CAST_ERR_INVALID_ARG;
   if (dtype != CAST_F32 && dtype != CAST_BF16) return CAST_ERR_DTYPE;
   if (B > c->cfg.max_batch) return CAST_ERR_CAPACITY;
-  const int V = c->cfg.vocab;
-  // cluster size: 16 CTAs per sequence where the device can co-schedule them, else 8; the slices are cached
-  // in shared memory when they fit, else every sweep recomputes them from the logits
-  const bool f32 = dtype == CAST_F32;
-  const int di = f32 ? 0 : 1;
-  sto_plan(c, f32);  // first call with this dtype: a host-side query, no device work
-  const int cs = c->sto_cs[di];
-  const bool cached = c->sto_cached[di] != 0;
   StoParams p;
   p.target_logits = target_logits;
   p.draft_logits = draft_logits;
-  p.V = V;
+  p.V = c->cfg.vocab;
   p.Ncap = c->cfg.max_tree;
   p.max_depth = c->cfg.max_depth;
-  p.cs = cs;
-  p.slice = slice_for(V, cs);
   p.inv_T = 1.0 / temperature;
+  p.T = temperature;
   p.tokens = tokens;
   p.parent = parent;
   p.n_tree = n_tree;
@@ -568,7 +648,5 @@ extern "C" cast_status cast_accept_stochastic(cast_ctx* c, const void* target_lo
   p.bonus_token = bonus_token;
   p.st = c->state;
   cudaStream_t s = (cudaStream_t)stream;
-  const size_t dyn = cached ? (size_t)p.slice * 16 : 0;
-  if (f32) return cached ? sto_launch<float, true>(p, B, dyn, s) : sto_launch<float, false>(p, B, dyn, s);
-  return cached ? sto_launch<__nv_bfloat16, true>(p, B, dyn, s) : sto_launch<__nv_bfloat16, false>(p, B, dyn, s);
+  return dtype == CAST_F32 ? sto_run<float>(c, p, B, 0, s) : sto_run<__nv_bfloat16>(c, p, B, 1, s);
 }

@@ -108,9 +108,10 @@ struct cast_ctx {
   size_t attn_tc_ws_bytes;
 
   // stochastic acceptance, per logits dtype (0 fp32, 1 bf16): cluster size found to be launchable
-  // (0: not looked up yet) and whether a CTA's vocabulary slice is cached in shared memory
+  // (0: not looked up yet), whether a CTA's vocabulary slice is cached on chip, and how many such clusters run at once
   int sto_cs[2];
   int sto_cached[2];
+  int sto_resident[2];
 
   // cast_set_attention_early_reads: the caller's promise, and whether the last call of this library on the
   // context wrote something the attention reads early (n_tree, masks: cast_select_nodes; kv_len: cast_compact_kv)

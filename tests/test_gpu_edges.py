@@ -152,3 +152,36 @@ def test_attention_of_64_dims_rounds_only_its_output(binding, B, cap, Hq, Hkv, p
         assert torch.equal(got.isnan(), ~keep)
         err = (got.double() - want)[keep].abs() - want[keep].abs() * 2.0 ** -8
         assert float(err.max()) < 2e-5 * gain
+
+
+@pytest.mark.parametrize("V", [17, 8193, 32768, 32769, 65537, 131073, 155648, 155649, 196609])
+@pytest.mark.parametrize("B,dtype,shift", [(1, torch.float32, 0.0), (12, torch.bfloat16, 0.0), (2, torch.float32, -2000.0),
+                                           (10, torch.float32, 900.0)])
+def test_stochastic_accept_at_the_steps_of_its_dispatch(binding, V, B, dtype, shift):
+    """Vocabularies at the ends of a segment size, batches below and above what clusters of 16 cover at once, logits so far
+    from zero that exp(logit / T) leaves fp64's range. A root with two children, the first of which has one."""
+    from oracle import stochastic_accept
+    rng = np.random.default_rng(V + B)
+    N, H, T = 4, 3, 0.9
+    g = torch.Generator(device="cuda").manual_seed(V)
+    parent = np.tile(np.array([-1, 0, 0, 1], np.int32), (B, 1))
+    tokens = np.stack([rng.permutation(V)[:N] if V > N else np.arange(N) for _ in range(B)]).astype(np.int32)
+    draft = torch.randn((B, N, V), generator=g, device="cuda") * 3
+    for b in range(B):
+        for t, p in ((1, 0), (2, 0), (3, 1)):
+            draft[b, p, int(tokens[b, t])] = 15.0 - t
+    target = draft + 0.5 * torch.randn(draft.shape, generator=g, device="cuda") + shift
+    target, draft = target.to(dtype), (draft + shift).to(dtype)
+    n_tree = np.full(B, N, np.int32)
+    ua, ub = rng.uniform(0.01, 0.99, (B, N)), rng.uniform(0.01, 0.99, B)
+    ctx = binding.CastContext(max_batch=B, vocab=V, top_k=2, max_depth=H, total_token=N, max_tree=N)
+    dev = lambda a: torch.from_numpy(a).cuda()
+    n, path, bonus = _ints([0] * B), _ints([[0] * (H + 1)] * B), _ints([0] * B)
+    ctx.cast_accept_stochastic(target, draft, B, T, dev(tokens), dev(parent), dev(n_tree), dev(ua), dev(ub), n, path, bonus)
+    assert ctx.cast_poll_status()[0] == 0
+    want_n, want_path, want_bonus, margin = stochastic_accept(target.double().cpu().numpy(), draft.double().cpu().numpy(), tokens,
+                                                              parent, n_tree, H, T, ua, ub)
+    clear = margin > 1e-11
+    assert clear.any()
+    for got, want in ((n, want_n), (path, want_path), (bonus, want_bonus)):
+        assert np.array_equal(got.cpu().numpy()[clear], want[clear])
