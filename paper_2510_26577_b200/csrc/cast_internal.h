@@ -45,10 +45,7 @@ struct HostTable {
 
 // Limits of the vocabulary sweep.
 constexpr int kSweepThreads = 512;
-constexpr int kSweepEpt = 32;                             // logits per thread per pass
-constexpr int kSweepSub = kSweepThreads * kSweepEpt;      // logits per CTA per pass
 constexpr int kSweepMaxChunks = 8;                        // CTAs per logits row: one thread-block cluster
-constexpr int kCandCap = 4096;                            // 64-bit keys of shared scratch per CTA (warp lists, short list)
 constexpr int kMaxFifo = 64;
 constexpr int kAcceptMaxChunks = 32;
 constexpr int kAttnWorkListCap = 4096;                    // CTAs of an attention launch that a work list can describe

@@ -2,14 +2,13 @@
 //
 // cast_tree_expand is ONE kernel per draft layer, launched as thread-block clusters (the chunks of
 // one logits row form a cluster) with programmatic dependent launch between the layers:
-//   1. vocabulary sweep - one CTA per chunk: streaming 16-byte loads issued before anything else,
-//      online max / sum-exp in base 2, and a list of top-K candidates per warp, filtered against
-//      thresholds the CTA's warps share (the K-th largest of the warps' maxima in the first pass, of
-//      their best logits afterwards: lower bounds on the CTA's K-th largest, so the result is exact
-//      and only a logit or two per warp survives the filter);
-//   2. the chunk's top K, maximum and sum go straight into the shared memory of the cluster's
-//      first CTA, which merges the row after the cluster barrier (log-sum-exp in fp64, lower-bound
-//      merge of the sorted chunk lists) and appends the K children to the node pool;
+//   1. vocabulary sweep - one CTA per chunk: streaming 16-byte loads, two buffers of them in flight, online max / sum-exp
+//      in base 2, and a list of candidates per warp, filtered against a threshold the CTA's warps share (the K-th largest
+//      of the maxima of sixteen parts: a lower bound on the CTA's K-th largest, so the result is exact and only a
+//      logit or two per warp survives the filter);
+//   2. the chunk's candidates, maxima and sums go straight into the shared memory of the cluster's
+//      first CTA, which merges the row after the cluster barrier (log-sum-exp in fp64, the candidates ranked by
+//      counting) and appends the K children to the node pool;
 //   3. the last row-merging CTA of the layer (an atomic ticket; nothing spins) ranks each
 //      sequence's candidates, forms the utility u (Eq. 1) and the cost c (Eq. 2), runs Algorithm 1
 //      (breadth pruning), the depth-pruning test and the FIFO update, and publishes the retained
@@ -57,24 +56,40 @@ struct ExpandParams {
   const int32_t* kv_len;
 };
 
+// Sixteen raw bytes of logits: a thread's sweep buffers hold them as loaded and unpack on use.
 template <typename T> struct Vec;
 template <> struct Vec<float> {
   static constexpr int N = 4;
-  static __device__ __forceinline__ void load(const float* p, float* out) {
-    const float4 a = __ldcs(reinterpret_cast<const float4*>(p));
-    out[0] = a.x; out[1] = a.y; out[2] = a.z; out[3] = a.w;
+  static constexpr uint32_t kMinusInf = 0xff800000u;
+  static __device__ __forceinline__ float max(const uint4& a) {
+    return fmaxf(fmaxf(__uint_as_float(a.x), __uint_as_float(a.y)), fmaxf(__uint_as_float(a.z), __uint_as_float(a.w)));
   }
+  static __device__ __forceinline__ void unpack(const uint4& a, float (&x)[4]) {
+    x[0] = __uint_as_float(a.x); x[1] = __uint_as_float(a.y); x[2] = __uint_as_float(a.z); x[3] = __uint_as_float(a.w);
+  }
+  static __device__ __forceinline__ void put(uint4& a, int e, float x) { (&a.x)[e] = __float_as_uint(x); }
 };
 template <> struct Vec<__nv_bfloat16> {
   static constexpr int N = 8;
-  static __device__ __forceinline__ void load(const __nv_bfloat16* p, float* out) {
-    const uint4 a = __ldcs(reinterpret_cast<const uint4*>(p));
+  static constexpr uint32_t kMinusInf = 0xff80ff80u;
+  static __device__ __forceinline__ float max(const uint4& a) {
+    auto pair = [](uint32_t w) { return *reinterpret_cast<const __nv_bfloat162*>(&w); };
+    const __nv_bfloat162 m = __hmax2(__hmax2(pair(a.x), pair(a.y)), __hmax2(pair(a.z), pair(a.w)));
+    const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
+    return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+  }
+  static __device__ __forceinline__ void unpack(const uint4& a, float (&x)[8]) {
     const uint32_t w[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {  // bf16 -> fp32 is a 16-bit shift
-      out[2 * i] = __uint_as_float(w[i] << 16);
-      out[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+      x[2 * i] = __uint_as_float(w[i] << 16);
+      x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
     }
+  }
+  static __device__ __forceinline__ void put(uint4& a, int e, float x) {
+    uint32_t& w = (&a.x)[e >> 1];
+    const uint32_t h = __float_as_uint(x) >> 16;  // (x came from a bf16)
+    w = (e & 1) ? ((w & 0xffffu) | (h << 16)) : ((w & 0xffff0000u) | h);
   }
 };
 
@@ -136,6 +151,9 @@ __device__ __forceinline__ void st_cluster_u64(uint32_t addr, unsigned long long
 __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 __device__ __forceinline__ void st_cluster_f64(uint32_t addr, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
 }
@@ -175,6 +193,7 @@ __device__ __forceinline__ bool take_ticket(int32_t* counter, int expected, int*
 // sequence ranks that sequence (so the sequences are ranked in parallel) and leaves the first n sorted
 // nodes in global memory, and the last of those CTAs decides.
 
+constexpr int kTailScratch = 28672;  // bytes of shared memory the tail works in
 // Up to this many sequences the one-CTA tail is faster than a second ticket.
 constexpr int kTailSingleMaxB = 4;
 
@@ -197,19 +216,49 @@ __device__ __forceinline__ int tail_width(const ExpandParams& p, int n_prev) {
   return n;
 }
 
+// Ranking by counting. A warp's lanes hold 32 of the items; the items they are compared with are read one (or two) at a time
+// at the same address in all lanes, so that a load is one wavefront; the warps share out the items and the comparisons, and
+// their counts meet in shared memory. (With a lane per share of one item's comparisons every lane read its own address, and
+// shared-memory bandwidth made 126 keys take 1.7 us.) A comparison is a subtraction whose borrow is counted.
+__device__ __forceinline__ void count_less(int& neg, const uint4& a, const uint4& b) {  // neg -= a < b, as 128-bit numbers
+  asm("{\n\t.reg .u32 t;\n\t"
+      "sub.cc.u32 t, %1, %5;\n\tsubc.cc.u32 t, %2, %6;\n\tsubc.cc.u32 t, %3, %7;\n\tsubc.cc.u32 t, %4, %8;\n\t"
+      "subc.u32 %0, %0, 0;\n\t}"
+      : "+r"(neg)
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w));
+}
+__device__ __forceinline__ void count_less64(int& neg, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi) {
+  asm("{\n\t.reg .u32 t;\n\tsub.cc.u32 t, %1, %3;\n\tsubc.cc.u32 t, %2, %4;\n\tsubc.u32 %0, %0, 0;\n\t}"
+      : "+r"(neg)
+      : "r"(alo), "r"(ahi), "r"(blo), "r"(bhi));
+}
+
+// A candidate as one 128-bit number, smaller = earlier in the order (value desc, token asc, creation order): the value's
+// bits mapped so that larger values come first, the token, the place. (Equal siblings are everywhere with half-precision
+// logits: a comparison that looks at the token on equality only took 6 us here.)
+__device__ __forceinline__ uint4 make_cand(double score, int token, int place) {
+  uint64_t b = (uint64_t)__double_as_longlong(score + 0.0);  // (-0 as +0)
+  b = (b >> 63) ? b : ~(b | 0x8000000000000000ull);
+  return make_uint4((uint32_t)place, (uint32_t)token, (uint32_t)b, (uint32_t)(b >> 32));
+}
+__device__ __forceinline__ double cand_score(const uint4& c) {
+  const uint64_t b = ((uint64_t)c.w << 32) | c.z;
+  return __longlong_as_double((long long)((b >> 63) ? b : ~b & 0x7fffffffffffffffull));
+}
+
 // Ranks the layer's candidates of the sequences [b_begin, b_begin + b_count): writes every sequence's sorted
 // list for the rerank (lsort, lscore) and, for rank < n, pool index, token and value to sorted_o, stok_o,
 // vs_o at [b * CAST_MAX_WIDTH + rank] (shared or global memory).
 __device__ __forceinline__ void tail_rank(const ExpandParams& p, int b_begin, int b_count, int n, int n_prev, int base,
                                           unsigned char* scratch, int* sorted_o, int* stok_o, double* vs_o) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int K = p.K, P = p.P;
-  const int Ni = n_prev * K;
-  double* sc = reinterpret_cast<double*>(scratch);              // 1024 scores
-  int* tk = reinterpret_cast<int*>(scratch + 8192);             // 1024 tokens
-  int* rank_s = reinterpret_cast<int*>(scratch + 12288);        // 1024 ranks
+  const int P = p.P;
+  const int Ni = n_prev * p.K;
+  uint4* cand = reinterpret_cast<uint4*>(scratch);            // 1024 candidates
+  int* rank_s = reinterpret_cast<int*>(scratch + 16384);      // 1024 ranks, negated
+  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
   const int group = 1024 / Ni;                                  // sequences ranked per pass
-  const float inv_Ni = 1.f / (float)Ni, inv_K = 1.f / (float)K;
+  const float inv_Ni = 1.f / (float)Ni;
 #pragma unroll 1
   for (int b0 = 0; b0 < b_count; b0 += group) {
     const int nb = (b_count - b0) < group ? (b_count - b0) : group;
@@ -217,103 +266,106 @@ __device__ __forceinline__ void tail_rank(const ExpandParams& p, int b_begin, in
     for (int i = tid; i < tot; i += nt) {
       const int bl = div_small(i, Ni, inv_Ni), ci = i - bl * Ni;
       const size_t o = (size_t)(b_begin + b0 + bl) * P + base + ci;
-      sc[i] = __ldcg(p.pool_score + o);
-      tk[i] = __ldcg(p.pool_token + o);
+      cand[i] = make_cand(__ldcg(p.pool_score + o), __ldcg(p.pool_token + o), ci);
       rank_s[i] = 0;
     }
     __syncthreads();
-    // Rank under the order (value desc, token asc, creation order). Every logits row contributed its K
-    // children already in that order, so the rank of a candidate is, summed over the rows of its sequence,
-    // the number of that row's children that come first: one lower-bound search per (candidate, row) pair (in
-    // its own row it finds its own position). The pairs are spread densely over the threads - what this phase
-    // costs is the warp instructions it issues, so no lane works on a row or a step that does not exist - two
-    // per thread in step so that their shared-memory loads overlap; the counts meet in shared memory.
-    const int pairs = tot * n_prev;
-    const float inv_tot = 1.f / (float)tot;
-    int h0 = 1;
-    while (2 * h0 - 1 < K) h0 <<= 1;  // the search's first stride: positions up to 2 h0 - 1 >= K are reachable
+    // Rank under the order (value desc, token asc, creation order): the number of the sequence's candidates that come
+    // first. Groups of 32 candidates of one sequence; the warps left over split a group's comparisons.
+    const int gps = (Ni + 31) >> 5, groups = nb * gps;
+    const int shares = groups < nw ? nw / groups : 1, len = (Ni + shares - 1) / shares;
 #pragma unroll 1
-    for (int it0 = tid; it0 < pairs; it0 += 2 * nt) {
-      int ii[2], rs[2], rowb[2], r1[2], t2[2], pos[2] = {0, 0};
-      double s2[2];
-      bool act[2];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int it = it0 + q * nt;
-        act[q] = it < pairs;
-        const int itc = act[q] ? it : 0;
-        // (row-major: the lanes of a warp search one row for consecutive candidates, so their shared-memory loads
-        // fall on that row's K entries and their counts go to different words)
-        rs[q] = div_small(itc, tot, inv_tot);    // the row searched
-        ii[q] = itc - rs[q] * tot;               // the candidate (index over the sequences of this pass)
-        const int ci = ii[q] - div_small(ii[q], Ni, inv_Ni) * Ni;
-        r1[q] = div_small(ci, K, inv_K);         // the candidate's own row
-        rowb[q] = ii[q] - ci + rs[q] * K;  // first child of the searched row, same sequence
-        s2[q] = sc[ii[q]];
-        t2[q] = tk[ii[q]];
+    for (int w = warp; w < groups * shares; w += nw) {
+      const int g = w / shares, j0 = (w - g * shares) * len, j1 = min(j0 + len, Ni);
+      const int bl = g / gps, ci = (g - bl * gps) * 32 + lane;
+      const uint4* list = cand + bl * Ni;
+      const uint4 mine = list[ci < Ni ? ci : 0];
+      int neg = 0;
+#pragma unroll 8
+      for (int j = j0; j < j1; ++j) count_less(neg, list[j], mine);
+      if (ci < Ni) {
+        if (shares > 1) atomicAdd(&rank_s[bl * Ni + ci], neg);
+        else rank_s[bl * Ni + ci] = neg;
       }
-#pragma unroll 1
-      for (int half = h0; half >= 1; half >>= 1) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int idx = pos[q] + half - 1;
-          const bool valid = idx < K;
-          const int at = rowb[q] + (valid ? idx : 0);
-          const double sj = sc[at];
-          const int tj = tk[at];
-          const bool first = valid && ((sj > s2[q]) || (sj == s2[q] && (tj < t2[q] || (tj == t2[q] && rs[q] < r1[q]))));
-          pos[q] += first ? half : 0;
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 2; ++q)
-        if (act[q] && pos[q] != 0) atomicAdd(&rank_s[ii[q]], pos[q]);
     }
     __syncthreads();
 #pragma unroll 1
     for (int i = tid; i < tot; i += nt) {
-      const int bl = div_small(i, Ni, inv_Ni), ci = i - bl * Ni, rank = rank_s[i];
-      const int bg = b_begin + b0 + bl;
-      const double s = sc[i];
-      const size_t o = (size_t)bg * P + base + rank;
-      p.lsort[o] = base + ci;  // the layer's sorted list, for the rerank
-      p.lscore[o] = s;
-      if (rank < n) {
-        sorted_o[bg * CAST_MAX_WIDTH + rank] = base + ci;
-        stok_o[bg * CAST_MAX_WIDTH + rank] = tk[i];
-        vs_o[bg * CAST_MAX_WIDTH + rank] = fast_exp_neg(s);
+      const int bl = div_small(i, Ni, inv_Ni), ci = i - bl * Ni, rank = -rank_s[i];
+      const uint4 mine = cand[i];
+      {
+        const int bg = b_begin + b0 + bl;
+        const size_t o = (size_t)bg * P + base + rank;
+        p.lsort[o] = base + ci;  // the layer's sorted list, for the rerank
+        const double s = cand_score(mine);
+        p.lscore[o] = s;
+        if (rank < n) {
+          sorted_o[bg * CAST_MAX_WIDTH + rank] = base + ci;
+          stok_o[bg * CAST_MAX_WIDTH + rank] = (int)mine.y;
+          vs_o[bg * CAST_MAX_WIDTH + rank] = fast_exp_neg(s);
+        }
       }
     }
     __syncthreads();
   }
 }
 
+// What the deciding warp needs from memory, requested as soon as the CTA knows that it ranks (the first warp; per lane).
+struct DecideIn {
+  double c;              // Eq. 2's cost of rank lane + 1
+  double prev[2], cur[2];  // entries lane and lane + 32 of the buffers A_{i-1} (to be pushed to) and A_i (to be averaged)
+  int prev_n, cur_n;
+  int n0;                // layer 1: the longest of two sequences' prefixes
+};
+__device__ __forceinline__ DecideIn decide_load(const ExpandParams& p, const TailState& ts, int B, int n) {
+  DecideIn d;
+  const int lane = threadIdx.x & 31;
+  d.c = 0.0;
+  d.prev[0] = d.prev[1] = d.cur[0] = d.cur[1] = 0.0;
+  d.prev_n = d.cur_n = 0;
+  d.n0 = ts.n0;
+  if (threadIdx.x >= 32) return d;
+  static_assert(CAST_MAX_BATCH <= 64 && kMaxFifo <= 64, "two entries per lane");
+  if (p.layer == 1) d.n0 = max(lane < B ? p.kv_len[lane] : 0, lane + 32 < B ? p.kv_len[lane + 32] : 0);
+  if ((p.enable_bp || p.enable_dp) && lane < n && !(p.layer == 1 && p.ctx_base_mode)) {
+    const int g = select_grid(ts.ctx_sum + (p.ctx_base_mode ? ts.n0 : 0), p.tab.L, p.tab.M);
+    d.c = p.tab.fD[(size_t)(g - 1) * p.tab.Ntab + lane] / p.tab.fT[(size_t)(g - 1) * p.tab.Ntab];
+  }
+  if (p.enable_dp) {
+    if (p.layer >= 2) {
+      const double* A = p.fifo_vals + (size_t)(p.layer - 2) * p.R;
+      if (lane < p.R) d.prev[0] = A[lane];
+      if (lane + 32 < p.R) d.prev[1] = A[lane + 32];
+      d.prev_n = p.fifo_cnt[p.layer - 2];
+    }
+    if (p.layer < p.H) {
+      const double* A = p.fifo_vals + (size_t)(p.layer - 1) * p.R;
+      if (lane < p.R) d.cur[0] = A[lane];
+      if (lane + 32 < p.R) d.cur[1] = A[lane + 32];
+      d.cur_n = p.fifo_cnt[p.layer - 1];
+    }
+  }
+  return d;
+}
+
 // The batch-wide part: Eq. 1 over the sequences' first n sorted values, Eq. 2, Algorithm 1, the depth test,
 // the state for the next layer and the layer's outputs. GLOBAL: the inputs were written to global memory by
-// other CTAs (read past L1).
+// other CTAs (read past L1). One warp decides (n <= CAST_MAX_WIDTH <= 32: a rank per lane, no barriers); the next layer's
+// CTAs wait for this, so it is a chain of shuffles and arithmetic only.
 template <bool GLOBAL>
-__device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailState& ts, int B, int n, int n_prev, int base,
-                                            const int* sorted_i, const int* stok_i, const double* vs_i) {
-  __shared__ double vbar[CAST_MAX_WIDTH], u[CAST_MAX_WIDTH], c[CAST_MAX_WIDTH];
-  __shared__ int s_ni, s_next, s_n0;
-  const int tid = threadIdx.x, nt = blockDim.x;
+__device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailState& ts, const DecideIn& d, int B, int n, int n_prev,
+                                            int base, const int* sorted_i, const int* stok_i, const double* vs_i) {
+  __shared__ double vbar[CAST_MAX_WIDTH];
+  __shared__ int s_ni;
+  constexpr unsigned kAll = 0xffffffffu;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   DevState* st = p.st;
   const int K = p.K, W = p.W, P = p.P;
   const int Ni = n_prev * K;
-  const bool need_cost = p.enable_bp || p.enable_dp;
-  const double u_last = ts.u_last;
-  int n0 = ts.n0;
   if (p.layer == 1) {
     // The first layer of a step also starts the step (cast_step_begin launches nothing): the padded context
     // length n_0 = max_b kv_len[b] and every sequence's root node (value 1, depth 0) at pool index 0.
-    static_assert(CAST_MAX_BATCH <= 64, "two sequences per lane");
-    if (tid < 32) {
-      int m = max(tid < B ? p.kv_len[tid] : 0, tid + 32 < B ? p.kv_len[tid + 32] : 0);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (tid == 0) s_n0 = m;
-    }
-    for (int b = tid; b < B; b += nt) {
+    for (int b = tid - 32; b >= 0 && b < B; b += nt - 32) {
       const size_t o = (size_t)b * P;
       p.pool_score[o] = 0.0;
       p.pool_token[o] = p.root_token[b];
@@ -323,123 +375,121 @@ __device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailSta
       p.lsort[o] = 0;
       p.lscore[o] = 0.0;
     }
-    __syncthreads();
-    n0 = s_n0;
   }
-  // Eq. 1: batch mean of the rank-wise values, then prefix sums; Eq. 2 needs one table row
-  if (tid < n) {
-    double c_mine = 0.0;
-    if (need_cost) {
-      const int ctx = ts.ctx_sum + (p.ctx_base_mode ? n0 : 0);
-      const int g = select_grid(ctx, p.tab.L, p.tab.M);
-      c_mine = p.tab.fD[(size_t)(g - 1) * p.tab.Ntab + tid] / p.tab.fT[(size_t)(g - 1) * p.tab.Ntab];
-    }
-    if (!GLOBAL) {
-      double a = 0.0;
-#pragma unroll 1
-      for (int b = 0; b < B; ++b) a += vs_i[b * CAST_MAX_WIDTH + tid];
-      vbar[tid] = a / (double)B;
-    }
-    c[tid] = c_mine;
-  }
+  // Eq. 1: batch mean of the rank-wise values
   if (GLOBAL) {
-    // many sequences: warp j sums rank j over the sequences, two per lane, then a fixed shuffle tree
-    static_assert(kSweepThreads / 32 >= CAST_MAX_WIDTH && CAST_MAX_BATCH <= 64, "one warp per rank, two sequences per lane");
-    const int j = tid >> 5, lane = tid & 31;
-    if (j < n) {
+    // many sequences: a warp per rank sums over the sequences, two per lane, then a fixed shuffle tree
+    static_assert(CAST_MAX_BATCH <= 64, "two sequences per lane");
+    for (int j = tid >> 5; j < n; j += nt >> 5) {
       double a = (lane < B ? __ldcg(vs_i + lane * CAST_MAX_WIDTH + j) : 0.0) +
                  (lane + 32 < B ? __ldcg(vs_i + (lane + 32) * CAST_MAX_WIDTH + j) : 0.0);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(kAll, a, o);
       if (lane == 0) vbar[j] = a / (double)B;
     }
+    __syncthreads();
   }
-  __syncthreads();
-  if (tid < 32) {  // inclusive scan of at most 16 values
-    double a = tid < n ? vbar[tid] : 0.0;
-#pragma unroll
-    for (int d = 1; d < CAST_MAX_WIDTH; d <<= 1) {
-      const double t = __shfl_up_sync(0xffffffffu, a, d);
-      if (tid >= d) a += t;
-    }
-    if (tid < n) u[tid] = a;
-  }
-  __syncthreads();
-  // Algorithm 1: mark[j] survives iff no earlier i has (u_j - u_i) < C1 (c_j - c_i); n_i = the largest
-  // marked index. n <= CAST_MAX_WIDTH <= 32: one warp, the marks as a ballot.
   if (tid < 32) {
-    int ok = tid < n ? 1 : 0;
-    if (p.enable_bp && tid < n) {
-      const double uj = u[tid], cj = c[tid];
-#pragma unroll 4
-      for (int i = 0; i < tid; ++i)
-        ok &= !((uj - u[i]) < p.C1 * (cj - c[i]));
+    int n0 = d.n0;
+    if (p.layer == 1) n0 = __reduce_max_sync(kAll, n0);
+    double c = d.c;
+    if ((p.enable_bp || p.enable_dp) && p.layer == 1 && p.ctx_base_mode && lane < n) {
+      const int g = select_grid(ts.ctx_sum + n0, p.tab.L, p.tab.M);
+      c = p.tab.fD[(size_t)(g - 1) * p.tab.Ntab + lane] / p.tab.fT[(size_t)(g - 1) * p.tab.Ntab];
     }
-    const unsigned marks = __ballot_sync(0xffffffffu, ok != 0);
-    if (tid == 0) s_ni = marks != 0u ? 32 - __clz(marks) : 1;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const int n_i = s_ni;
+    double u = 0.0;
+    if (lane < n) {
+      if (GLOBAL) {
+        u = vbar[lane];
+      } else {
+#pragma unroll 1
+        for (int b = 0; b < B; ++b) u += vs_i[b * CAST_MAX_WIDTH + lane];
+        u = u / (double)B;
+      }
+    }
+#pragma unroll
+    for (int o = 1; o < CAST_MAX_WIDTH; o <<= 1) {  // prefix sums
+      const double t = __shfl_up_sync(kAll, u, o);
+      if (lane >= o) u += t;
+    }
+    // Algorithm 1: mark[j] survives iff no earlier i has (u_j - u_i) < C1 (c_j - c_i); n_i = the largest marked index
+    bool ok = lane < n;
+    if (p.enable_bp) {
+#pragma unroll 4
+      for (int i = 0; i < n - 1; ++i) {
+        const double ui = __shfl_sync(kAll, u, i), ci = __shfl_sync(kAll, c, i);
+        if (i < lane && (u - ui) < p.C1 * (c - ci)) ok = false;
+      }
+    }
+    const unsigned marks = __ballot_sync(kAll, ok);
+    const int n_i = marks != 0u ? 32 - __clz(marks) : 1;
+    if (lane == 0) s_ni = n_i;
+    const double u_n = __shfl_sync(kAll, u, n_i - 1), c_n = __shfl_sync(kAll, c, n_i - 1);
     bool go = true;
     if (p.enable_dp) {
       if (p.layer >= 2) {  // gain ratio of the previous layer goes into its buffer, FIFO
-        const double phi = u[n_i - 1] / u_last;
+        const double phi = u_n / ts.u_last;
         double* A = p.fifo_vals + (size_t)(p.layer - 2) * p.R;
-        int cnt = p.fifo_cnt[p.layer - 2];
-        if (cnt < p.R) {
-          A[cnt++] = phi;
+        if (d.prev_n < p.R) {
+          if (lane == 0) {
+            A[d.prev_n] = phi;
+            p.fifo_cnt[p.layer - 2] = d.prev_n + 1;
+          }
         } else {
-          for (int k = 1; k < p.R; ++k) A[k - 1] = A[k];
-          A[p.R - 1] = phi;
+          if (lane >= 1 && lane < p.R) A[lane - 1] = d.prev[0];
+          if (lane + 32 < p.R) A[lane + 31] = d.prev[1];
+          if (lane == 0) A[p.R - 1] = phi;
         }
-        p.fifo_cnt[p.layer - 2] = cnt;
       }
       if (p.layer < p.H) {  // generate layer i+1 only if Avg(A_i) * u / c >= C2
-        const double* A = p.fifo_vals + (size_t)(p.layer - 1) * p.R;
-        const int cnt = p.fifo_cnt[p.layer - 1];
         double a = 0.0;
-        for (int k = 0; k < cnt; ++k) a += A[k];
-        const double alpha = a / (double)cnt;
-        go = (alpha * u[n_i - 1] / c[n_i - 1]) >= p.C2;
+        for (int k = 0; k < d.cur_n; ++k) a += __shfl_sync(kAll, k < 32 ? d.cur[0] : d.cur[1], k & 31);
+        const double alpha = a / (double)d.cur_n;
+        go = (alpha * u_n / c_n) >= p.C2;
       }
     }
-    s_next = (p.layer < p.H && go) ? n_i : 0;
+    const int next = (p.layer < p.H && go) ? n_i : 0;
     if (p.layer == 1) {  // per-step state (rows[]: a later layer that is never reached must read 0)
-      st->B = B;
-      st->n0 = n0;
-      st->n_tree = 0;
-      st->n_hist[0] = 1;
-      st->layer_base[0] = 0;
-      st->layer_n[0] = 1;
-      for (int i = 2; i <= CAST_MAX_DEPTH; ++i) {
+      for (int i = lane + 2; i <= CAST_MAX_DEPTH; i += 32) {
         st->n_hist[i] = 0;
         st->layer_base[i] = 0;
         st->layer_n[i] = 0;
       }
-      for (int i = 0; i < CAST_MAX_DEPTH + 2; ++i) st->rows[i] = (i == 1) ? 1 : 0;
+      for (int i = lane; i < CAST_MAX_DEPTH + 2; i += 32)
+        if (i != 2) st->rows[i] = (i == 1) ? 1 : 0;
+      if (lane == 0) {
+        st->B = B;
+        st->n0 = n0;
+        st->n_tree = 0;
+        st->n_hist[0] = 1;
+        st->layer_base[0] = 0;
+        st->layer_n[0] = 1;
+      }
     }
-    st->rows[p.layer + 1] = s_next;
-    st->n_hist[p.layer] = n_i;
-    st->layer_base[p.layer] = base;
-    st->layer_n[p.layer] = Ni;
-    st->ctx_sum = ts.ctx_sum + n_i;
-    st->kept_total = ts.kept_total + n_i;
-    st->u_last = u[n_i - 1];
-    st->pool_size = base + Ni;
-    st->layers_done = p.layer;
-    *p.next_count = s_next;
+    if (lane == 0) {
+      st->rows[p.layer + 1] = next;
+      st->n_hist[p.layer] = n_i;
+      st->layer_base[p.layer] = base;
+      st->layer_n[p.layer] = Ni;
+      st->ctx_sum = ts.ctx_sum + n_i;
+      st->kept_total = ts.kept_total + n_i;
+      st->u_last = u_n;
+      st->pool_size = base + Ni;
+      st->layers_done = p.layer;
+      *p.next_count = next;
+    }
   }
   __syncthreads();
   const int n_i = s_ni;
+  const float inv_W = 1.f / (float)W, inv_K = 1.f / (float)K;
 #pragma unroll 1
   for (int i = tid; i < B * W; i += nt) {
-    const int b = i / W, s = i % W;
+    const int b = div_small(i, W, inv_W), s = i - b * W;
     int tok = -1, prow = -1;
     if (s < n_i) {
       const int idx = GLOBAL ? __ldcg(sorted_i + b * CAST_MAX_WIDTH + s) : sorted_i[b * CAST_MAX_WIDTH + s];
       tok = GLOBAL ? __ldcg(stok_i + b * CAST_MAX_WIDTH + s) : stok_i[b * CAST_MAX_WIDTH + s];
-      prow = (idx - base) / K;
+      prow = div_small(idx - base, K, inv_K);
       p.retained[b * W + s] = idx;
       p.pool_kept[(size_t)b * P + idx] = 1;
     }
@@ -448,76 +498,293 @@ __device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailSta
   }
 }
 
+// ---- vocabulary sweep of one chunk -------------------------------------------------------------------------------
+// A chunk's logits are read in buffers of 64 bytes per thread, two of them in flight: while one is worked on the next is on
+// its way. Per logit the work is a maximum, the exponential and its sum (about five instructions); candidates for the
+// top K are found by one comparison of the buffer's maximum with a threshold, below which almost all buffers lie.
+//
+// Candidates: every warp has a list in shared memory, to which a lane appends what reaches the threshold. The threshold
+// is a lower bound on the CTA's K-th largest logit, shared by its warps: the K-th largest of the sixteen warps' maxima over
+// the first two buffers (K of the chunk's logits are at least that large), raised once more in long chunks. A dozen
+// logits per 16 K pass it, so a list is not put in order until it overflows (a rising row, ties): then the warp ranks
+// it, keeps its K best and raises its own threshold to the K-th; if a single buffer overflows it (constant rows) the K
+// best come from K rounds of a warp-wide maximum. What reaches the threshold is never dropped except for K better
+// ones, and every threshold is at most the K-th largest: the chunk's top K is always among the lists.
+constexpr int kBufVecs = 4;     // 16-byte vectors per thread and buffer
+constexpr int kGroups = 16;     // parts of a CTA whose maxima give the threshold: its warps, or half warps
+constexpr int kListCap = 64;    // keys per warp list
+constexpr int kPushCap = 32;    // keys a warp hands on at most
+static_assert(CAST_MAX_TOP_K <= kGroups, "the K-th largest of the groups' maxima needs K <= groups");
+static_assert(CAST_MAX_TOP_K <= kPushCap, "a warp hands on its K best");
+
+template <typename T, int NT>
+struct Sweep {
+  static constexpr int VEC = Vec<T>::N;
+  static constexpr int kSlots = kBufVecs * VEC;                      // logits of a thread per buffer
+  static constexpr int kBufElems = NT * kSlots;                      // of the CTA
+  uint4 raw[kBufVecs];
+
+  // First element (of the aligned view) of this thread's vector v in the buffer that starts at `base`.
+  static __device__ __forceinline__ int elem(int base, int v) { return base + (v * NT + (int)threadIdx.x) * VEC; }
+
+  // xa: the row from the 16-byte boundary at or below its start; elements [lo, end) of it exist.
+  __device__ __forceinline__ void load(const T* xa, int base, int lo, int end) {
+    if (base >= lo && base + kBufElems <= end) {  // a full buffer: no per-vector checks
+#pragma unroll
+      for (int v = 0; v < kBufVecs; ++v) raw[v] = __ldcs(reinterpret_cast<const uint4*>(xa + elem(base, v)));
+      return;
+    }
+#pragma unroll
+    for (int v = 0; v < kBufVecs; ++v) {
+      const int idx = elem(base, v);
+      if (idx >= lo && idx + VEC <= end) {
+        raw[v] = __ldcs(reinterpret_cast<const uint4*>(xa + idx));
+      } else {
+        raw[v] = make_uint4(Vec<T>::kMinusInf, Vec<T>::kMinusInf, Vec<T>::kMinusInf, Vec<T>::kMinusInf);
+        if (idx < end) {
+#pragma unroll
+          for (int e = 0; e < VEC; ++e)
+            if (idx + e >= lo && idx + e < end) Vec<T>::put(raw[v], e, to_float(xa[idx + e]));
+        }
+      }
+    }
+  }
+  static __device__ __forceinline__ int slot_elem(int base, int i) {
+    return base + ((i / VEC) * NT + (int)threadIdx.x) * VEC + (i % VEC);
+  }
+  // the logit of slot i (not a constant)
+  __device__ __forceinline__ float slot(int i) const {
+    const int w = i * kBufVecs * 4 / kSlots;  // its word of the sixteen
+    const uint4 q = (w & 8) ? ((w & 4) ? raw[3] : raw[2]) : ((w & 4) ? raw[1] : raw[0]);
+    const uint32_t u = (w & 2) ? ((w & 1) ? q.w : q.z) : ((w & 1) ? q.y : q.x);
+    if (VEC == 4) return __uint_as_float(u);
+    return __uint_as_float((i & 1) ? (u & 0xffff0000u) : (u << 16));
+  }
+  __device__ __forceinline__ float max() const {
+    float m = Vec<T>::max(raw[0]);
+#pragma unroll
+    for (int v = 1; v < kBufVecs; ++v) m = fmaxf(m, Vec<T>::max(raw[v]));
+    return m;
+  }
+  // Running maximum M2 (log2 units) and sum of 2^(x log2e - M2) of this thread; m: the buffer's maximum. NaN and +inf
+  // logits poison the sum.
+  __device__ __forceinline__ void sum(float m, float& M2, float& s_run) const {
+    const float t2 = m * kLog2eHi;
+    if (t2 > M2) {
+      s_run *= ex2f(M2 - t2);
+      M2 = t2;
+    }
+    if (!(M2 > -INFINITY)) {  // nothing finite so far: -inf adds nothing, NaN has to be noticed
+      float t = 0.f;
+#pragma unroll
+      for (int v = 0; v < kBufVecs; ++v) {
+        float x[VEC];
+        Vec<T>::unpack(raw[v], x);
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) t += x[i];
+      }
+      if (t != t) s_run = t;
+      return;
+    }
+    // x * log2(e) - M2 with log2(e) in two parts (the product is exact to fp32's last bit and beyond), two logits per
+    // instruction
+    const unsigned long long hi2 = pack2(kLog2eHi, kLog2eHi), lo2 = pack2(kLog2eLo, kLog2eLo), nm2 = pack2(-M2, -M2);
+    unsigned long long acc2 = pack2(0.f, 0.f);
+#pragma unroll
+    for (int v = 0; v < kBufVecs; ++v) {
+      float x[VEC];
+      Vec<T>::unpack(raw[v], x);
+#pragma unroll
+      for (int i = 0; i < VEC; i += 2) {
+        const unsigned long long x2 = pack2(x[i], x[i + 1]);
+        float e0, e1;
+        unpack2(fma2(x2, hi2, fma2(x2, lo2, nm2)), e0, e1);
+        acc2 = add2(acc2, pack2(ex2f(e0), ex2f(e1)));
+      }
+    }
+    float a0, a1;
+    unpack2(acc2, a0, a1);
+    s_run += a0 + a1;
+  }
+  // Appends what reaches `thr` to the warp's list (all 32 lanes call; `thr` is finite, so padding does not pass).
+  // shift: elements of the aligned view before token 0.
+  __device__ __forceinline__ void extract(float m, float& thr, int base, int shift, int K, unsigned long long* list, int* count) const {
+    if (!__any_sync(0xffffffffu, m >= thr)) return;
+    const int lane = threadIdx.x & 31;
+    const int have0 = *count;
+    __syncwarp();
+    // a lane's passing slots as a bit mask, then a loop over its set bits (one round as a rule; unrolled over the slots
+    // the code of the empty ones was most of the sweep's): the slot's logit by selects
+    uint32_t mask = 0u;
+#pragma unroll
+    for (int v = 0; v < kBufVecs; ++v) {
+      float x[VEC];
+      Vec<T>::unpack(raw[v], x);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) mask |= x[e] >= thr ? 1u << (v * VEC + e) : 0u;
+    }
+#pragma unroll 1
+    while (mask != 0u) {
+      const int i = __ffs(mask) - 1;
+      mask &= mask - 1u;
+      const int pos = atomicAdd(count, 1);
+      if (pos < kListCap) list[pos] = make_key(slot(i), slot_elem(base, i) - shift);
+    }
+    __syncwarp();
+    const int n = *count;
+    if (n <= kListCap - 16) return;
+    unsigned long long mine = 0ull;
+    int kept = 0;
+    if (n > kListCap) {
+      // K rounds of "largest key below the last one taken" over the old list and this buffer; lane r keeps the r-th
+      unsigned long long bound = ~0ull;
+#pragma unroll 1
+      for (int round = 0; round < K; ++round) {
+        unsigned long long best = 0ull;
+#pragma unroll
+        for (int v = 0; v < kBufVecs; ++v) {
+          float x[VEC];
+          Vec<T>::unpack(raw[v], x);
+          const int id = elem(base, v) - shift;
+#pragma unroll
+          for (int e = 0; e < VEC; ++e)
+            if (x[e] >= thr) {
+              const unsigned long long k2 = make_key(x[e], id + e);
+              if (k2 < bound && k2 > best) best = k2;
+            }
+        }
+#pragma unroll 1
+        for (int i = lane; i < have0; i += 32)
+          if (list[i] < bound && list[i] > best) best = list[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+          best = other > best ? other : best;
+        }
+        if (best == 0ull) break;
+        if (lane == round) mine = best;
+        bound = best;
+        ++kept;
+      }
+    } else {
+      kept = keep_best(list, n, K, mine);
+    }
+    __syncwarp();
+    if (lane < kept) list[lane] = mine;
+    if (lane == 0) *count = kept;
+    if (kept == K) thr = fmaxf(thr, key_value(__shfl_sync(0xffffffffu, mine, K - 1)));
+    __syncwarp();
+  }
+  // The min(n, K) largest of the list's n <= 64 keys, in order, one per lane.
+  static __device__ __forceinline__ int keep_best(unsigned long long* list, int n, int K, unsigned long long& mine) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long k0 = lane < n ? list[lane] : 0ull, k1 = lane + 32 < n ? list[lane + 32] : 0ull;
+    int r0 = 0, r1 = 0;
+#pragma unroll 1
+    for (int j = 0; j < n; ++j) {
+      const unsigned long long kj = list[j];
+      r0 += (kj > k0);
+      r1 += (kj > k1);
+    }
+    __syncwarp();
+    if (lane < n && r0 < K) list[r0] = k0;
+    if (lane + 32 < n && r1 < K) list[r1] = k1;
+    __syncwarp();
+    const int kept = n < K ? n : K;
+    mine = lane < kept ? list[lane] : 0ull;
+    return kept;
+  }
+};
+
+// The K-th largest of the groups' maxima in shared memory, at least -FLT_MAX (every warp for itself).
+__device__ __forceinline__ float kth_of_groups(const float* v, int K) {
+  const int lane = threadIdx.x & 31;
+  const float mine = v[lane & (kGroups - 1)];
+  int r = 0;
+#pragma unroll
+  for (int j = 0; j < kGroups; ++j) {
+    const float o = v[j];
+    r += (o > mine) || (o == mine && j < lane);  // equal values in lane order: ranks 0..15 are distinct
+  }
+  const unsigned who = __ballot_sync(0xffffffffu, lane < kGroups && r == K - 1);
+  return fmaxf(__shfl_sync(0xffffffffu, mine, who != 0u ? __ffs(who) - 1 : 0), -3.402823466e38f);
+}
+// A thread's share in the groups' maxima; returns the maximum of its group.
+template <int NT>
+__device__ __forceinline__ float group_max(float x, float* v) {
+  constexpr int kLanes = NT / kGroups;
+  static_assert(kLanes == 32 || kLanes == 16, "groups are warps or half warps");
+#pragma unroll
+  for (int o = kLanes / 2; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  if ((threadIdx.x & (kLanes - 1)) == 0) v[threadIdx.x / kLanes] = x;
+  return x;
+}
+__device__ __forceinline__ float warp_max(float x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  return x;
+}
+
 // MINB = 2 compiles the same code for two CTAs per SM (half the registers): for launches with more CTAs than
 // SMs, where a second resident CTA hides the first one's latencies; MINB = 1 is for the short launches.
-template <typename T, int MINB>
-__global__ void __launch_bounds__(kSweepThreads, MINB) expand_kernel(const ExpandParams p) {
-  __shared__ __align__(16) unsigned char scratch[kCandCap * 8];  // the warps' key lists and the short list; later the tail's arrays
+template <typename T, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) {
+  // filled in the first CTA of the row's cluster by all CTAs of the cluster: chunk c's candidate keys, and per warp of
+  // chunk c its maximum (log2 units) and sum of 2^(. - maximum); later the tail's arrays
+  constexpr int kWarps = NT / 32, kChunkCap = kWarps * kPushCap;
+  __shared__ __align__(16) unsigned char scratch[kSweepMaxChunks * kChunkCap * 8 > kTailScratch ? kSweepMaxChunks * kChunkCap * 8 : kTailScratch];
+  __shared__ float row_max[kSweepMaxChunks * kWarps];
+  __shared__ double row_sum[kSweepMaxChunks * kWarps];
+  __shared__ int row_n[kSweepMaxChunks];
+  __shared__ float row_bound[kSweepMaxChunks];  // the chunks' thresholds: lower bounds on the row's K-th largest logit
+  constexpr int kListMax = kWarps * kListCap;
+  __shared__ int rank_s[kListMax], list_n;
+  __shared__ __align__(16) unsigned long long wlist[kWarps * kListCap];
   __shared__ unsigned long long topk[CAST_MAX_TOP_K];
-  __shared__ float red_f[kSweepThreads / 32];
-  __shared__ double red_d[kSweepThreads / 32];
+  __shared__ int wcount[kWarps];
+  __shared__ float gmax[2][kGroups];
   __shared__ int sorted[kTailSingleMaxB * CAST_MAX_WIDTH];  // small batches: pool indices of the first sorted candidates
-  __shared__ int s_flag, short_n;
-  __shared__ float pass_heads[2][kSweepThreads / 32];  // the warps' largest logits after a pass (see cta_bound)
-  __shared__ float pass_wmax[kSweepThreads / 32];                   // the warps' maxima of the first pass
-  static_assert(CAST_MAX_TOP_K <= kSweepThreads / 32, "the K-th largest of the warps' maxima needs K <= warps");
-  // filled in the first CTA of the row's cluster by all CTAs of the cluster: chunk c's top-K keys
-  // (descending), maximum (log2 units) and sum of 2^(. - maximum)
-  __shared__ unsigned long long row_keys[kSweepMaxChunks * CAST_MAX_TOP_K];
-  __shared__ float row_max[kSweepMaxChunks];
-  __shared__ double row_sum[kSweepMaxChunks];
-  unsigned long long* cand = reinterpret_cast<unsigned long long*>(scratch);
+  __shared__ int s_flag, push_n;
+  __shared__ double s_lse;
+  unsigned long long* row_keys = reinterpret_cast<unsigned long long*>(scratch);
 
   const int chunk = blockIdx.x, r = blockIdx.y, b = blockIdx.z, B = gridDim.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   DevState* st = p.st;
   const int K = p.K;
   const int row = b * p.W + r;
+  using S = Sweep<T, NT>;
+  constexpr int E = S::kBufElems;
+  // the row from the 16-byte boundary at or below its start: its tokens are elements [shift, V + shift) of that view
   const T* x = reinterpret_cast<const T*>(p.logits) + (size_t)row * p.V;
+  const int shift = (int)((reinterpret_cast<uintptr_t>(x) & 15) / sizeof(T));
+  const T* xa = x - shift;
   const int begin = chunk * p.chunk_elems;
-  const int end = min(begin + p.chunk_elems, p.V);
-  constexpr int VEC = Vec<T>::N;
-  constexpr int NV = kSweepEpt / VEC;
-  const bool aligned = (reinterpret_cast<uintptr_t>(x) & 15) == 0;  // chunk starts are multiples of 8 logits
-
-  // the first pass of logits is requested before the state is read (every row r < W exists in memory):
-  // one memory round trip for both
-  float xv[kSweepEpt];
-  auto load_pass = [&](int sub) {
-    if (aligned && sub + kSweepSub <= end) {  // a full pass: no per-vector checks
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Vec<T>::load(x + sub + (v * kSweepThreads + tid) * VEC, xv + v * VEC);
-      return;
-    }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const int idx = sub + (v * kSweepThreads + tid) * VEC;
-      if (aligned && idx + VEC <= end) {
-        Vec<T>::load(x + idx, xv + v * VEC);
-      } else {
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) xv[v * VEC + e] = (idx + e < end) ? to_float(x[idx + e]) : -INFINITY;
-      }
-    }
-  };
+  const int end = min(begin + p.chunk_elems, p.V + shift);
+  if (p.nchunks > 1) cluster_arrive_release();  // (waited for before the first store to another CTA: all of them run by then)
+  if (tid < kWarps) wcount[tid] = 0;
+  if (tid == 0) push_n = list_n = 0;
   // Programmatic dependent launch: this grid may have become resident while the previous kernel of the
   // stream was still finishing. Nothing that kernel may have written is read above this line - not the
   // logits either: in a serving loop the previous kernel is the draft model's, and it writes them. What a
   // CTA may do is ask the L2 cache for its chunk: a prefetch returns no value, and a line that the previous
   // kernel writes afterwards is written in that same cache, so the loads below see it. When the previous kernel
-  // is not the one that writes the logits (layers queued back to back) the first pass then costs a round trip
+  // is not the one that writes the logits (layers queued back to back) the first loads then cost a round trip
   // to L2 instead of one to HBM; rows that turn out not to exist are fetched for nothing, hence only for small
   // layers.
   if (p.prefetch) {
-    const char* cb = reinterpret_cast<const char*>(x + begin);
-    const int bytes = (end - begin) * (int)sizeof(T);
+    const char* cb = reinterpret_cast<const char*>(chunk == 0 ? x : xa + begin);
+    const int bytes = (int)(reinterpret_cast<const char*>(xa + end) - cb);
 #pragma unroll 1
-    for (int off = tid * 128; off < bytes; off += kSweepThreads * 128)
+    for (int off = tid * 128; off < bytes; off += NT * 128)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(cb + off));
   }
   grid_dependency_wait();
   grid_launch_dependents();  // the next grid may now take the SMs this one leaves idle
-  load_pass(begin);
+  // the first logits are requested before the state is read (every row r < W exists in memory): one memory round trip
+  S q0, q1;
+  q0.load(xa, begin, shift, end);
+  q1.load(xa, begin + E, shift, end);
   // what the layer tail needs of the state is read now, together with the row count: one round trip.
   // (Layer 1 starts the step: one row per sequence, the root at pool index 0 with value 1.)
   int n_prev = 1, base = 1;
@@ -539,7 +806,7 @@ __global__ void __launch_bounds__(kSweepThreads, MINB) expand_kernel(const Expan
     return;
   }
   if (r >= n_prev) return;
-  // the parent of this row's children and its log-value (only the row's last CTA uses them: fetched now,
+  // the parent of this row's children and its log-value (only the row's first CTA uses them: fetched now,
   // off the critical path)
   int parent = 0;
   double parent_score = 0.0;
@@ -548,387 +815,196 @@ __global__ void __launch_bounds__(kSweepThreads, MINB) expand_kernel(const Expan
     parent_score = p.pool_score[(size_t)b * p.P + parent];
   }
 
-  float M2 = -INFINITY, s_run = 0.f;  // running maximum (log2 units) and sum of 2^(x log2e - M2)
-  // Every warp keeps the exact top K of the logits it has seen, as a descending list in shared memory;
-  // the warps never meet during the sweep. `have` (warp-uniform) is the list's length, thr_key its K-th
-  // key (0 while it is shorter than K).
-  constexpr int kWarpCap = 64;
-  constexpr int kWarps = kSweepThreads / 32;
-  unsigned long long* wlist = cand + warp * kWarpCap;
-  int have = 0;
-  unsigned long long thr_key = 0ull;
-  // A lower bound on the CTA's K-th largest logit that all warps share from the second pass on: the K-th
-  // largest of the warps' best logits so far (K of the CTA's logits are at least that large). A warp's own K-th
-  // key only knows the warp's sixteenth of the data; against this bound few logits of a later pass reach any
-  // list at all, so the exact tests, the appends and the re-ranking below mostly do not run. (A logit of the
-  // CTA's final top K is >= every such bound, and a warp drops it only for K better ones: the chunk result is
-  // exact. The bound is a value, not a key: logits equal to it pass, which only lengthens a list.)
-  float cta_bound = -INFINITY;
-  int pass = 0;
-  const int npass = (end - begin + kSweepSub - 1) / kSweepSub;
-
-  for (int sub = begin; sub < end; sub += kSweepSub, ++pass) {
-    if (sub != begin) load_pass(sub);
-    // The bound is refreshed where it still moves: before the second pass (from the first pass's threshold to the
-    // K-th largest of sixteen warps' best it rises a great deal) and, in long chunks, before the third. Later it
-    // hardly rises, the warps' own K-th keys have caught up, and the refresh - a CTA barrier and a rank of 16 heads
-    // in every warp, about a third of a pass's instructions - costs more than the few extractions it saves
-    // (batch 64, eight passes: 302 -> 278 us per tree build; batch 16, four passes: 171 -> 166).
-    if (pass == 1 || (pass == 2 && npass >= 6)) {
-      float* hd = pass_heads[pass & 1];
-      if (lane == 0) hd[warp] = have > 0 ? key_value(wlist[0]) : -INFINITY;
-      __syncthreads();
-      const float head = lane < kWarps ? hd[lane] : -INFINITY;
-      int rh = 0;
-#pragma unroll
-      for (int j = 0; j < kWarps; ++j) {
-        const float o = __shfl_sync(0xffffffffu, head, j);
-        rh += (o > head) || (o == head && j < lane);  // equal heads in lane order: ranks 0..15 are distinct
-      }
-      const unsigned who = __ballot_sync(0xffffffffu, lane < kWarps && rh == K - 1);
-      const float bnd = __shfl_sync(0xffffffffu, head, who != 0u ? __ffs(who) - 1 : 0);
-      cta_bound = fmaxf(cta_bound, bnd);
-    }
-    // (the maxima of the four groups of eight slots on the way: the extraction below looks only into the groups
-    // that hold a passer)
-    float gmax[4];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      gmax[g] = xv[8 * g];
-#pragma unroll
-      for (int j = 1; j < 8; ++j) gmax[g] = fmaxf(gmax[g], xv[8 * g + j]);
-    }
-    const float tmax = fmaxf(fmaxf(gmax[0], gmax[1]), fmaxf(gmax[2], gmax[3]));
-    const float t2 = tmax * kLog2eHi;
-    if (t2 > M2) {
-      s_run *= ex2f(M2 - t2);
-      M2 = t2;
-    }
-    if (M2 > -INFINITY) {
-      // x * log2(e) - M2 with log2(e) in two parts (the product is exact to fp32's last bit and beyond), two
-      // logits per instruction; NaN and +inf logits poison the sum
-      const unsigned long long hi2 = pack2(kLog2eHi, kLog2eHi), lo2 = pack2(kLog2eLo, kLog2eLo), nm2 = pack2(-M2, -M2);
-      unsigned long long acc2 = pack2(0.f, 0.f);
-#pragma unroll
-      for (int i = 0; i < kSweepEpt; i += 2) {
-        const unsigned long long x2 = pack2(xv[i], xv[i + 1]);
-        float e0, e1;
-        unpack2(fma2(x2, hi2, fma2(x2, lo2, nm2)), e0, e1);
-        acc2 = add2(acc2, pack2(ex2f(e0), ex2f(e1)));
-      }
-      float a0, a1;
-      unpack2(acc2, a0, a1);
-      s_run += a0 + a1;
-    }
-    // filter threshold: the warp's exact K-th key once it has K, else the K-th largest of the lanes'
-    // maxima of this pass (at least K of the warp's logits are >= it)
-    float thr_val;
-    const unsigned long long gate = thr_key;  // keys at or below the warp's own K-th cannot matter
-    if (pass == 0) {
-      // nothing is known yet: the K-th largest of the 16 warps' maxima (K <= 16 of the CTA's logits are at
-      // least that large). Against it one or two logits per warp pass; against the K-th largest of a warp's
-      // own lane maxima, which needs no barrier but a 15-stage sorting network, K to 2K per warp did.
-      float wm = tmax;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, o));
-      float* wmax = pass_wmax;
-      if (lane == 0) wmax[warp] = wm;
-      __syncthreads();
-      const float mine = lane < kWarps ? wmax[lane] : -INFINITY;
-      int rh = 0;
-#pragma unroll
-      for (int j = 0; j < kWarps; ++j) {
-        const float o = __shfl_sync(0xffffffffu, mine, j);
-        rh += (o > mine) || (o == mine && j < lane);  // equal maxima in lane order: ranks 0..15 are distinct
-      }
-      const unsigned who = __ballot_sync(0xffffffffu, lane < kWarps && rh == K - 1);
-      thr_val = __shfl_sync(0xffffffffu, mine, who != 0u ? __ffs(who) - 1 : 0);
-    } else if (gate == 0ull && !(cta_bound > -INFINITY)) {
-      float kx = tmax;
-#pragma unroll
-      for (int k = 2; k <= 32; k <<= 1)
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-          const float o = __shfl_xor_sync(0xffffffffu, kx, j);
-          const bool desc = ((lane & k) == 0), low = ((lane & j) == 0);
-          kx = (desc == low) ? fmaxf(kx, o) : fminf(kx, o);
-        }
-      thr_val = __shfl_sync(0xffffffffu, kx, K - 1);
-    } else {
-      thr_val = gate != 0ull ? fmaxf(key_value(gate), cta_bound) : cta_bound;
-    }
-    // Few logits pass, and against the shared thresholds most passes of a warp have none: one vote on the
-    // lanes' maxima settles that. Otherwise the same vote per group of eight slots, and in a group with a passer
-    // every lane marks its passing slots in a bit mask, the warp takes the union with one reduction and walks its
-    // set bits (a loop over the set bits only: unrolled over all slots, the tests and reconvergence points of the
-    // empty ones were most of the sweep's time); a slot's logit is picked out of the group's registers by three
-    // rounds of warp-uniform selects, takes the exact test on the full key and is appended to the warp's list.
-    // (The order of the appends does not matter: the list is ranked afterwards.)
-    const int have0 = have;
-    if (__any_sync(0xffffffffu, tmax >= thr_val)) {
-      static_assert(kSweepEpt == 32, "four groups of eight slots");
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        if (!__any_sync(0xffffffffu, gmax[g] >= thr_val)) continue;
-        unsigned mine_mask = 0u;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) mine_mask |= (xv[8 * g + j] >= thr_val) ? (1u << j) : 0u;
-        unsigned any_mask = __reduce_or_sync(0xffffffffu, mine_mask);
+  // ---- sweep
+  unsigned long long* list = wlist + warp * kListCap;
+  float m_run = -INFINITY, M2 = -INFINITY, s_run = 0.f, thr = 0.f;
+  auto work = [&](S& q, float m, int at) {
+    q.extract(m, thr, at, shift, K, list, &wcount[warp]);
+    if (at + 2 * E < end) q.load(xa, at + 2 * E, shift, end);
+  };
+  auto threshold = [&](float m, float* g) {
+    group_max<NT>(m, g);
+    __syncthreads();
+    return kth_of_groups(g, K);
+  };
 #pragma unroll 1
-        while (any_mask != 0u) {
-          const int j = __ffs(any_mask) - 1;
-          any_mask &= any_mask - 1u;
-          const bool b0 = (j & 1) != 0, b1 = (j & 2) != 0, b2 = (j & 4) != 0;
-          float s4[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) s4[q] = b0 ? xv[8 * g + 2 * q + 1] : xv[8 * g + 2 * q];
-          const float s2a = b1 ? s4[1] : s4[0], s2b = b1 ? s4[3] : s4[2];
-          const float xi = b2 ? s2b : s2a;
-          const int i = 8 * g + j;
-          const int id = sub + ((i / VEC) * kSweepThreads + tid) * VEC + (i % VEC);
-          const unsigned long long key = make_key(xi, id);
-          const bool ok = xi >= thr_val && id < end && key > gate;
-          const unsigned m = __ballot_sync(0xffffffffu, ok);
-          const int pos = have + __popc(m & ((1u << lane) - 1u));
-          if (ok && pos < kWarpCap) wlist[pos] = key;
-          have += __popc(m);
-        }
-      }
-    }
-    __syncwarp();
-    if (have > kWarpCap) {
-      // flood (a mass of ties at the threshold): K rounds of "largest key below the last one taken" over
-      // the old list and this pass's logits; lane r keeps the r-th result
-      unsigned long long bound = ~0ull, mine = 0ull;
-      int n = 0;
-#pragma unroll 1
-      for (int round = 0; round < K; ++round) {
-        unsigned long long best = 0ull;
-#pragma unroll
-        for (int i = 0; i < kSweepEpt; ++i) {
-          const int id = sub + ((i / VEC) * kSweepThreads + tid) * VEC + (i % VEC);
-          if (id < end && xv[i] == xv[i]) {
-            const unsigned long long k2 = make_key(xv[i], id);
-            if (k2 < bound && k2 > best) best = k2;
-          }
-        }
-        if (lane < have0) {
-          const unsigned long long k2 = wlist[lane];
-          if (k2 < bound && k2 > best) best = k2;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-          best = other > best ? other : best;
-        }
-        if (best == 0ull) break;
-        if (lane == round) mine = best;
-        ++n;
-        bound = best;
-      }
-      __syncwarp();
-      if (lane < n) wlist[lane] = mine;
-      have = n;
-      __syncwarp();
-    } else if (have == have0 + 1) {
-      // one newcomer (the usual case): the old entries are in order, so it is an insertion - the newcomer's rank is
-      // the number of larger keys (one vote), the smaller ones move down one place, the K-th of K falls off
-      const unsigned long long nk = wlist[have0];
-      const unsigned long long mine = lane < have0 ? wlist[lane] : 0ull;
-      const int rnk = __popc(__ballot_sync(0xffffffffu, lane < have0 && mine > nk));
-      __syncwarp();
-      if (lane < have0 && lane >= rnk && lane + 1 < K) wlist[lane + 1] = mine;
-      if (lane == 0 && rnk < K) wlist[rnk] = nk;
-      have = have < K ? have : K;
-      __syncwarp();
-    } else if (have > have0) {
-      // exact order of the list (old entries and newcomers, at most 64): rank by counting, keys are distinct
-      const int n = have;
-      const unsigned long long k0 = lane < n ? wlist[lane] : 0ull;
-      const unsigned long long k1 = lane + 32 < n ? wlist[lane + 32] : 0ull;
-      int r0 = 0, r1 = 0;
-#pragma unroll 4
-      for (int j = 0; j < n; ++j) {
-        const unsigned long long kj = wlist[j];
-        r0 += (kj > k0);
-        r1 += (kj > k1);
-      }
-      __syncwarp();
-      if (lane < n && r0 < K) wlist[r0] = k0;
-      if (lane + 32 < n && r1 < K) wlist[r1] = k1;
-      have = n < K ? n : K;
-      __syncwarp();
-    }
-    thr_key = have == K ? wlist[K - 1] : 0ull;
+  for (int at = begin; at < end; at += 2 * E) {  // (two copies of the work: a buffer that is moved is waited for)
+    const float m0 = q0.max();
+    m_run = fmaxf(m_run, m0);
+    q0.sum(m0, M2, s_run);
+    // the threshold from the first two buffers, and once more when four of seven buffers or more are done
+    if (at == begin) thr = threshold(fmaxf(m0, q1.max()), gmax[0]);
+    else if (at == begin + 4 * E && end - at > 2 * E) thr = fmaxf(thr, threshold(m_run, gmax[1]));
+    work(q0, m0, at);
+    if (at + E >= end) break;
+    const float m1 = q1.max();
+    m_run = fmaxf(m_run, m1);
+    q1.sum(m1, M2, s_run);
+    work(q1, m1, at + E);
   }
 
-  // chunk result: the top K of the warps' lists (each in descending order; the rank of a key is the
-  // number of larger keys, list by list: a lower-bound search each, two lanes per key slot), the
-  // maximum and the sum of 2^(. - maximum) in fp64. It goes straight into the shared memory of the
-  // cluster's first CTA, which merges the row.
+  // ---- chunk result: what is left of the warps' lists above the threshold, and every warp's maximum and sum, straight
+  // into the shared memory of the cluster's first CTA, which merges the row
   {
-    if (lane >= have && lane < CAST_MAX_TOP_K) wlist[lane] = 0ull;  // short lists end in "no entry"
-    float Mw = M2;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) Mw = fmaxf(Mw, __shfl_xor_sync(0xffffffffu, Mw, o));
-    double sd = (M2 > -INFINITY) ? (double)s_run * (double)ex2f(M2 - Mw) : 0.0;
+    const float Mw = warp_max(M2);
+    double sd = (M2 > -INFINITY) ? (double)s_run * (double)ex2f(M2 - Mw) : (double)s_run;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sd += __shfl_xor_sync(0xffffffffu, sd, o);
-    if (lane == 0) {
-      red_f[warp] = Mw;
-      red_d[warp] = sd;
+    const int n = wcount[warp];
+    unsigned long long k0 = lane < n ? list[lane] : 0ull, k1 = lane + 32 < n ? list[lane + 32] : 0ull;
+    if (k0 != 0ull && key_value(k0) < thr) k0 = 0ull;  // (appended before the threshold was raised)
+    if (k1 != 0ull && key_value(k1) < thr) k1 = 0ull;
+    unsigned m0 = __ballot_sync(0xffffffffu, k0 != 0ull), m1 = __ballot_sync(0xffffffffu, k1 != 0ull);
+    if (__popc(m0) + __popc(m1) > kPushCap) {  // (warp-uniform) its K best
+      __syncwarp();
+      S::keep_best(list, n, K, k0);
+      k1 = 0ull;
+      m0 = __ballot_sync(0xffffffffu, k0 != 0ull);
+      m1 = 0u;
     }
-    if (tid < K) topk[tid] = 0ull;
-    if (tid == 0) short_n = 0;  // length of the CTA's short list
-    __syncthreads();
-    // The K-th largest of the warps' list heads bounds the CTA's top K from below (every list is in
-    // descending order), so only keys at or above it can belong: a dozen or so. Every warp finds that
-    // bound by itself (16 heads, one per lane), appends its survivors to a short list with one atomic,
-    // and the first warp ranks the short list by counting.
-    unsigned long long bound;
-    {
-      const unsigned long long head = lane < kWarps ? cand[lane * kWarpCap] : 0ull;
-      int rh = 0;
-#pragma unroll
-      for (int j = 0; j < kWarps; ++j) rh += (__shfl_sync(0xffffffffu, head, j) > head);
-      bound = (rh == K - 1) ? head : 0ull;  // heads are distinct unless 0 ("no entry")
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, bound, o);
-        bound = other > bound ? other : bound;
-      }
-    }
-    unsigned long long* shortlist = cand + kWarps * kWarpCap;  // at most kWarps * K keys
-    {
-      const unsigned long long key = lane < have ? wlist[lane] : 0ull;
-      const bool keep = key != 0ull && key >= bound;
-      const unsigned m = __ballot_sync(0xffffffffu, keep);
-      int basepos = 0;
-      if (lane == 0 && m != 0u) basepos = atomicAdd(&short_n, __popc(m));
-      basepos = __shfl_sync(0xffffffffu, basepos, 0);
-      if (keep) shortlist[basepos + __popc(m & ((1u << lane) - 1u))] = key;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      const int n = short_n;  // <= kWarps * K = 256: up to 8 keys per lane
-#pragma unroll 1
-      for (int i0 = 0; i0 < n; i0 += 32) {
-        const int i = i0 + lane;
-        const unsigned long long key = i < n ? shortlist[i] : ~0ull;
-        int rk2 = 0;
-#pragma unroll 4
-        for (int j = 0; j < n; ++j) rk2 += (shortlist[j] > key);
-        if (i < n && rk2 < K) topk[rk2] = key;
-      }
-    }
-    // meanwhile the last warp folds the warps' (maximum, sum) pairs
-    float M = -INFINITY;
-    double S = 0.0;
-    if (warp == kWarps - 1) {
-      const float Ml = lane < kWarps ? red_f[lane] : -INFINITY;
-      const double Sl = lane < kWarps ? red_d[lane] : 0.0;
-      M = Ml;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-      S = Ml > -INFINITY ? Sl * (double)ex2f(Ml - M) : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
-    }
-    __syncthreads();
+    const int total = __popc(m0) + __popc(m1);
+    int pos = 0;
+    if (lane == 0 && total > 0) pos = atomicAdd(&push_n, total);
+    pos = chunk * kChunkCap + __shfl_sync(0xffffffffu, pos, 0);
+    const unsigned below = (1u << lane) - 1u;
+    const int p0 = pos + __popc(m0 & below), p1 = pos + __popc(m0) + __popc(m1 & below);
     if (p.nchunks == 1) {
-      if (tid < K) row_keys[tid] = topk[tid];
-      if (tid == kSweepThreads - 32) {
-        row_max[0] = M;
-        row_sum[0] = S;
+      if (k0 != 0ull) row_keys[p0] = k0;
+      if (k1 != 0ull) row_keys[p1] = k1;
+      if (lane == 0) {
+        row_max[warp] = Mw;
+        row_sum[warp] = sd;
       }
+      __syncthreads();
+      if (tid == 0) {
+        row_n[0] = push_n;
+        row_bound[0] = thr;
+      }
+      __syncthreads();
     } else {
-      if (tid < K) st_cluster_u64(map_to_rank(smem_addr(&row_keys[chunk * CAST_MAX_TOP_K + tid]), 0u), topk[tid]);
-      if (tid == kSweepThreads - 32) {
-        st_cluster_f32(map_to_rank(smem_addr(&row_max[chunk]), 0u), M);
-        st_cluster_f64(map_to_rank(smem_addr(&row_sum[chunk]), 0u), S);
+      cluster_wait_acquire();
+      if (k0 != 0ull) st_cluster_u64(map_to_rank(smem_addr(&row_keys[p0]), 0u), k0);
+      if (k1 != 0ull) st_cluster_u64(map_to_rank(smem_addr(&row_keys[p1]), 0u), k1);
+      if (lane == 0) {
+        st_cluster_f32(map_to_rank(smem_addr(&row_max[chunk * kWarps + warp]), 0u), Mw);
+        st_cluster_f64(map_to_rank(smem_addr(&row_sum[chunk * kWarps + warp]), 0u), sd);
       }
+      __syncthreads();
+      if (tid == 0) {
+        st_cluster_u32(map_to_rank(smem_addr(&row_n[chunk]), 0u), (uint32_t)push_n);
+        st_cluster_f32(map_to_rank(smem_addr(&row_bound[chunk]), 0u), thr);
+      }
+      cluster_arrive_release();
+      if (chunk != 0) return;  // the results are on their way; the first CTA waits for them
+      cluster_wait_acquire();
     }
   }
 
-  // ---- row merge by the first CTA of the row's cluster
-  if (p.nchunks > 1) {
-    cluster_arrive_release();
-    if (chunk != 0) return;  // the results are on their way; the first CTA waits for them
-    cluster_wait_acquire();
-  } else {
-    __syncthreads();
-  }
-  // the row's top K out of the chunks' lists (each in descending order): the rank of a key is its
-  // position in its own list plus, for every other list, the number of larger keys there (a binary
-  // search each; in its own list it finds its own position). Neighbouring lanes share a key slot.
-  if (p.nchunks > 1) {  // (a row of one chunk has its top K in `topk` already)
+  // ---- row merge by the first CTA of the row's cluster: the candidates (a dozen or two per chunk) that reach the largest
+  // of the chunks' thresholds go side by side, then the last warp forms the log-sum-exp while the others rank them
+  const float row_thr = [&] {
+    float t = row_bound[0];
+#pragma unroll
+    for (int c = 1; c < kSweepMaxChunks; ++c) t = c < p.nchunks ? fmaxf(t, row_bound[c]) : t;
+    return t;
+  }();
   if (tid < K) topk[tid] = 0ull;
-  __syncthreads();
   {
-    constexpr int kLps = kSweepThreads / (kSweepMaxChunks * CAST_MAX_TOP_K);  // lanes per key slot: one pass
-    constexpr int kLpl = kSweepMaxChunks / kLps;                              // lists per lane
-    static_assert(kLps >= 1 && kLps <= 8 && kLps * kLpl == kSweepMaxChunks, "lanes of a slot cover the lists");
-    const int slot = tid / kLps, sub = tid % kLps;
-    const int c1 = slot >> 4, t = slot & 15;  // slot = list * CAST_MAX_TOP_K + position
-    const bool act = c1 < p.nchunks && t < K;
-    const unsigned long long key = act ? row_keys[slot] : 0ull;
-    int pos[kLpl];
-#pragma unroll
-    for (int q = 0; q < kLpl; ++q) pos[q] = 0;
-#pragma unroll
-    for (int half = 16; half >= 1; half >>= 1) {
-#pragma unroll
-      for (int q = 0; q < kLpl; ++q) {
-        const int c2 = sub + kLps * q;
-        const int idx = pos[q] + half - 1;
-        const bool valid = act && c2 < p.nchunks && idx < K;
-        const unsigned long long other = row_keys[valid ? c2 * CAST_MAX_TOP_K + idx : 0];
-        pos[q] += (valid && other > key) ? half : 0;
+    constexpr int kLanes = NT / kSweepMaxChunks;  // threads per chunk: whole warps
+    static_assert(kLanes % 32 == 0, "a warp looks at one chunk");
+    const int c = tid / kLanes, nc = c < p.nchunks ? row_n[c] : 0;
+#pragma unroll 1
+    for (int i0 = (tid % kLanes) - lane; i0 < nc; i0 += kLanes) {
+      const int i = i0 + lane;
+      const unsigned long long key = i < nc ? row_keys[c * kChunkCap + i] : 0ull;
+      const bool keep = key != 0ull && key_value(key) >= row_thr;
+      const unsigned m = __ballot_sync(0xffffffffu, keep);
+      int pos = 0;
+      if (lane == 0 && m != 0u) pos = atomicAdd(&list_n, __popc(m));
+      pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
+      if (keep && pos < kListMax) {
+        wlist[pos] = key;
+        rank_s[pos] = 0;
       }
     }
-    int cnt = 0;
-#pragma unroll
-    for (int q = 0; q < kLpl; ++q) cnt += pos[q];
-#pragma unroll
-    for (int o = kLps >> 1; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if (act && sub == 0 && cnt < K) topk[cnt] = key;
   }
   __syncthreads();
-  }
-  if (warp == 0) {
-    float M0 = -INFINITY, M1 = -INFINITY;
-    double S0 = 0.0, S1 = 0.0;
-    if (lane < p.nchunks) {
-      M0 = row_max[lane];
-      S0 = row_sum[lane];
-    }
-    // (d) log-sum-exp over the chunk partials: weights by the fp32 unit, sums in fp64
-    float Mr = fmaxf(M0, M1);
+  const int total = list_n;
+  const bool packed = total <= kListMax;  // (else: ties without number, ranked where they are)
+  if (warp == kWarps - 1) {
+    constexpr int kPer = kSweepMaxChunks * kWarps / 32;
+    float Mv[kPer], Mr = -INFINITY;
+    double Sv[kPer], term = 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) Mr = fmaxf(Mr, __shfl_xor_sync(0xffffffffu, Mr, o));
-    double term = (M0 > -INFINITY ? S0 * (double)ex2f(M0 - Mr) : 0.0) + (M1 > -INFINITY ? S1 * (double)ex2f(M1 - Mr) : 0.0);
+    for (int i = 0; i < kPer; ++i) {
+      const int at = lane + 32 * i;
+      const bool in = at < p.nchunks * kWarps;
+      Mv[i] = in ? row_max[at] : -INFINITY;
+      Sv[i] = in ? row_sum[at] : 0.0;
+      Mr = fmaxf(Mr, Mv[i]);
+    }
+    Mr = warp_max(Mr);
+    // weights by the fp32 unit, sums in fp64 (a warp without a finite maximum adds 0, or the NaN it met)
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) term += Mv[i] > -INFINITY ? Sv[i] * (double)ex2f(Mv[i] - Mr) : Sv[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) term += __shfl_xor_sync(0xffffffffu, term, o);
     const double lse = ((double)Mr + fast_log2(term)) * 0.69314718055994530942;
-    if (lane == 0 && !(term > 0.0 && isfinite(lse))) report(st, CAST_ERR_NONFINITE, row);
-    __syncwarp();
-    // (e) the K children join the pool
-    if (lane < K) {
-      const unsigned long long key = topk[lane];
-      const float val = key_value(key);
-      int tok = key_token(key);
-      if (key == 0ull || !(val > -INFINITY) || tok < 0 || tok >= p.V) {  // fewer than K finite logits
-        report(st, CAST_ERR_NONFINITE, row);
-        tok = 0;
-      }
-      const size_t o = (size_t)b * p.P;
-      const int idx = base + r * K + lane;
-      p.pool_score[o + idx] = parent_score + ((double)val - lse);
-      p.pool_token[o + idx] = tok;
-      p.pool_parent[o + idx] = parent;
-      p.pool_depth[o + idx] = p.layer;
-      p.pool_kept[o + idx] = 0;
+    if (lane == 0) {
+      if (!(term > 0.0 && isfinite(lse))) report(st, CAST_ERR_NONFINITE, row);
+      s_lse = lse;
     }
+  } else if (packed) {
+    const int groups = (total + 31) >> 5, nw = kWarps - 1;
+    const int shares = groups < nw ? nw / groups : 1, len = (total + shares - 1) / shares;
+#pragma unroll 1
+    for (int w = warp; w < groups * shares; w += nw) {
+      const int g = w / shares, j0 = (w - g * shares) * len, j1 = min(j0 + len, total), i = g * 32 + lane;
+      const unsigned long long key = wlist[i < total ? i : 0];
+      const uint32_t lo = (uint32_t)key, hi = (uint32_t)(key >> 32);
+      int neg = 0;
+#pragma unroll 8
+      for (int j = j0; j < j1; ++j) {
+        const uint2 o = *reinterpret_cast<const uint2*>(wlist + j);
+        count_less64(neg, lo, hi, o.x, o.y);
+      }
+      if (i < total) atomicAdd(&rank_s[i], neg);
+    }
+  } else {
+#pragma unroll 1
+    for (int c1 = 0; c1 < p.nchunks; ++c1)
+#pragma unroll 1
+      for (int i = tid; i < row_n[c1]; i += NT - 32) {
+        const unsigned long long key = row_keys[c1 * kChunkCap + i];
+        int cnt = 0;
+#pragma unroll 1
+        for (int c = 0; c < p.nchunks; ++c)
+#pragma unroll 4
+          for (int j = 0; j < row_n[c]; ++j) cnt += row_keys[c * kChunkCap + j] > key;
+        if (cnt < K) topk[cnt] = key;
+      }
+  }
+  __syncthreads();
+  if (packed) {
+    for (int i = tid; i < total; i += NT)
+      if (-rank_s[i] < K) topk[-rank_s[i]] = wlist[i];
+    __syncthreads();
+  }
+  if (tid < K) {  // the K children join the pool
+    const unsigned long long key = topk[tid];
+    const float val = key_value(key);
+    int tok = key_token(key);
+    if (key == 0ull || !(val > -INFINITY) || tok < 0 || tok >= p.V) {  // fewer than K finite logits
+      report(st, CAST_ERR_NONFINITE, row);
+      tok = 0;
+    }
+    const size_t o = (size_t)b * p.P;
+    const int idx = base + r * K + tid;
+    p.pool_score[o + idx] = parent_score + ((double)val - s_lse);
+    p.pool_token[o + idx] = tok;
+    p.pool_parent[o + idx] = parent;
+    p.pool_depth[o + idx] = p.layer;
+    p.pool_kept[o + idx] = 0;
   }
 
   // ---- layer tail
@@ -936,16 +1012,18 @@ __global__ void __launch_bounds__(kSweepThreads, MINB) expand_kernel(const Expan
   const int n_tail = tail_width(p, n_prev);
   if (B <= kTailSingleMaxB) {  // the last CTA of the layer ranks and decides, everything in shared memory
     if (!take_ticket(p.layer_ticket, B * n_prev, &s_flag)) return;
-    double* vs = reinterpret_cast<double*>(scratch + 16384);  // [B][CAST_MAX_WIDTH] sorted values
+    double* vs = reinterpret_cast<double*>(scratch + 20480);  // [B][CAST_MAX_WIDTH] sorted values
     int* stok = reinterpret_cast<int*>(scratch + 24576);      // [B][CAST_MAX_WIDTH] tokens of the sorted nodes
+    const DecideIn d = decide_load(p, ts, B, n_tail);
     tail_rank(p, 0, B, n_tail, n_prev, base, scratch, sorted, stok, vs);
-    tail_decide<false>(p, ts, B, n_tail, n_prev, base, sorted, stok, vs);
+    tail_decide<false>(p, ts, d, B, n_tail, n_prev, base, sorted, stok, vs);
   } else {  // the last CTA of every sequence ranks that sequence; the last of those decides for the batch
     if (!take_ticket(p.seq_ticket + b, n_prev, &s_flag)) return;
     tail_rank(p, b, 1, n_tail, n_prev, base, scratch, p.tail_sorted, p.tail_tok, p.tail_vs);
     // (tail_rank ends with a CTA barrier: the ticket below releases what all threads wrote)
+    const DecideIn d = decide_load(p, ts, B, n_tail);
     if (!take_ticket(p.layer_ticket, B, &s_flag)) return;
-    tail_decide<true>(p, ts, B, n_tail, n_prev, base, p.tail_sorted, p.tail_tok, p.tail_vs);
+    tail_decide<true>(p, ts, d, B, n_tail, n_prev, base, p.tail_sorted, p.tail_tok, p.tail_vs);
   }
 }
 
@@ -1234,15 +1312,18 @@ extern "C" cast_status cast_tree_expand(cast_ctx* c, int layer, const void* draf
   // up (figures fitted to the measured layer times of the benchmark shapes). The chunk count with the smallest estimate wins: few rows get many one-pass chunks (latency), many
   // rows get few chunks of several full passes (throughput).
   const int rows = B * rows_per_seq;
-  int nchunks = 1, chunk_elems = (V + 7) / 8 * 8;
+  // (a row's aligned view starts up to one vector before the row; V % 8 == 0 keeps every row as aligned as the first)
+  const int room = V + (V % 8 != 0 || ((uintptr_t)draft_logits & 15) != 0 ? 7 : 0);
+  const int buf_elems = kSweepThreads * 64 / (dtype == CAST_F32 ? 4 : 2);
+  int nchunks = 1, chunk_elems = (room + 7) / 8 * 8;
   {
     double best = 1e30;
     for (int n = 1; n <= kSweepMaxChunks; ++n) {
-      int ce = ((V + n - 1) / n + 7) / 8 * 8;
+      int ce = ((room + n - 1) / n + 7) / 8 * 8;
       if (n > 1 && ce < 2048) break;  // below this a chunk is all overhead
-      const int ne = (V + ce - 1) / ce;
-      const int passes = (ce + kSweepSub - 1) / kSweepSub;
-      const double per_cta = (ne == 1 ? 2.0 : 2.5) + 4.0 * passes;
+      const int ne = (room + ce - 1) / ce;
+      const int bufs = (ce + buf_elems - 1) / buf_elems;
+      const double per_cta = (ne == 1 ? 2.0 : 2.5) + 2.0 * bufs;
       // (a launch a little larger than the machine costs a good part of a second round: the few CTAs left over
       // run while the other SMs idle)
       const double queue = (double)rows * ne / c->num_sms;
@@ -1276,6 +1357,7 @@ extern "C" cast_status cast_tree_expand(cast_ctx* c, int layer, const void* draf
   p.root_token = c->step_root; p.kv_len = c->step_kv_len;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nchunks, rows_per_seq, B);
+  const bool queued = (long long)rows * nchunks > c->num_sms;
   cfg.blockDim = dim3(kSweepThreads, 1, 1);
   cfg.dynamicSmemBytes = 0;
   cfg.stream = (cudaStream_t)stream;
@@ -1289,13 +1371,12 @@ extern "C" cast_status cast_tree_expand(cast_ctx* c, int layer, const void* draf
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const bool queued = (long long)rows * nchunks > c->num_sms;
   cudaError_t e;
   if (dtype == CAST_F32)
-    e = queued ? cudaLaunchKernelEx(&cfg, expand_kernel<float, 2>, p) : cudaLaunchKernelEx(&cfg, expand_kernel<float, 1>, p);
+    e = queued ? cudaLaunchKernelEx(&cfg, expand_kernel<float, 512, 2>, p) : cudaLaunchKernelEx(&cfg, expand_kernel<float, 512, 1>, p);
   else
-    e = queued ? cudaLaunchKernelEx(&cfg, expand_kernel<__nv_bfloat16, 2>, p)
-               : cudaLaunchKernelEx(&cfg, expand_kernel<__nv_bfloat16, 1>, p);
+    e = queued ? cudaLaunchKernelEx(&cfg, expand_kernel<__nv_bfloat16, 512, 2>, p)
+               : cudaLaunchKernelEx(&cfg, expand_kernel<__nv_bfloat16, 512, 1>, p);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return CAST_ERR_CUDA;

@@ -185,3 +185,34 @@ def test_stochastic_accept_at_the_steps_of_its_dispatch(binding, V, B, dtype, sh
     assert clear.any()
     for got, want in ((n, want_n), (path, want_path), (bonus, want_bonus)):
         assert np.array_equal(got.cpu().numpy()[clear], want[clear])
+
+
+@pytest.mark.parametrize("logits", ["f32", "bf16"])
+@pytest.mark.parametrize("V", [33, 8191, 16385, 32769, 65529, 131073, 262147])
+@pytest.mark.parametrize("kind", ["random", "rising", "constant", "one_block", "few_finite"])
+def test_tree_layer_at_the_edges_of_the_sweep(binding, logits, V, kind):
+    """Vocabularies around the buffers' sizes (unaligned rows), values that overflow the candidate lists: a row that rises with
+    the token, equal logits everywhere, all large logits in one thread's reach, hardly more finite ones than K."""
+    from helpers import assert_tree_equal, gpu_tree, oracle_tree
+    B, K, H = 2, 16, 2
+    g = torch.Generator().manual_seed(V)
+    dt = torch.bfloat16 if logits == "bf16" else torch.float32
+    layers = []
+    for _ in range(H):
+        x = torch.randn((B, K, V), generator=g) * 3
+        if kind == "rising":
+            x = x.sort(-1).values
+        elif kind == "constant":
+            x = torch.full_like(x, -1.5)
+        elif kind == "one_block":
+            x[..., V // 2:V // 2 + 16] += torch.arange(16) * 0.5 + 40.0
+        elif kind == "few_finite":
+            keep = torch.zeros(V, dtype=torch.bool)
+            keep[torch.randperm(V, generator=g)[:K + 1]] = True
+            x[..., ~keep] = float("-inf")
+        layers.append(x.to(dt))
+    kw = dict(vocab=V, top_k=K, max_depth=H, total_token=40, max_tree=40)
+    root, kv = torch.tensor([1, 2], dtype=torch.int32), torch.tensor([5, 6], dtype=torch.int32)
+    want = oracle_tree(kw, None, root, kv, layers)
+    ctx = binding.CastContext(max_batch=B, **kw)
+    assert_tree_equal(gpu_tree(ctx, root.cuda(), kv.cuda(), [x.cuda() for x in layers]), want)
