@@ -197,7 +197,7 @@ constexpr int kTailScratch = 28672;  // bytes of shared memory the tail works in
 // Up to this many sequences the one-CTA tail is faster than a second ticket.
 constexpr int kTailSingleMaxB = 4;
 
-// a / b for 0 <= a < 2^20 and 1 <= b <= 2^10 through the fp32 reciprocal (inv_b = 1.f / b) with one correction step:
+// a / b for 0 <= a < 2^20 and 1 <= b <= 2^10 through the fp32 reciprocal (inv_b, to a few ulp) with one correction step:
 // the integer division by a run-time divisor is some twenty instructions, and the ranking below does several per
 // thread in a phase whose time is what its instructions take to issue.
 __device__ __forceinline__ int div_small(int a, int b, float inv_b) {
@@ -216,26 +216,26 @@ __device__ __forceinline__ int tail_width(const ExpandParams& p, int n_prev) {
   return n;
 }
 
-// Ranking by counting. A warp's lanes hold 32 of the items; the items they are compared with are read one (or two) at a time
-// at the same address in all lanes, so that a load is one wavefront; the warps share out the items and the comparisons, and
-// their counts meet in shared memory. (With a lane per share of one item's comparisons every lane read its own address, and
-// shared-memory bandwidth made 126 keys take 1.7 us.) A comparison is a subtraction whose borrow is counted.
-__device__ __forceinline__ void count_less(int& neg, const uint4& a, const uint4& b) {  // neg -= a < b, as 128-bit numbers
-  asm("{\n\t.reg .u32 t;\n\t"
-      "sub.cc.u32 t, %1, %5;\n\tsubc.cc.u32 t, %2, %6;\n\tsubc.cc.u32 t, %3, %7;\n\tsubc.cc.u32 t, %4, %8;\n\t"
-      "subc.u32 %0, %0, 0;\n\t}"
-      : "+r"(neg)
-      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w));
-}
+// Ranking by counting. A warp's lanes hold 32 of the items; the items they are compared with are read one at a
+// time, the same in all lanes; the warps share out the comparisons and their counts meet in shared memory. (With a lane
+// per share of one item's comparisons the shared-memory reads made 126 keys take 1.7 us.) A comparison of 64-bit keys is a
+// subtraction whose borrow is counted.
 __device__ __forceinline__ void count_less64(int& neg, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi) {
   asm("{\n\t.reg .u32 t;\n\tsub.cc.u32 t, %1, %3;\n\tsubc.cc.u32 t, %2, %4;\n\tsubc.u32 %0, %0, 0;\n\t}"
       : "+r"(neg)
       : "r"(alo), "r"(ahi), "r"(blo), "r"(bhi));
 }
 
+// log2 of the warps per group when `nw` warps share `groups` groups (an integer division is a chain of some 130 cycles)
+__device__ __forceinline__ int share_log(int groups, int nw) {
+  int l = 0;
+  while (groups << (l + 1) <= nw) ++l;
+  return l;
+}
+
 // A candidate as one 128-bit number, smaller = earlier in the order (value desc, token asc, creation order): the value's
 // bits mapped so that larger values come first, the token, the place. (Equal siblings are everywhere with half-precision
-// logits: a comparison that looks at the token on equality only took 6 us here.)
+// logits: comparisons that look at the token on equality only took 4 us for 144 candidates, these 1.2.)
 __device__ __forceinline__ uint4 make_cand(double score, int token, int place) {
   uint64_t b = (uint64_t)__double_as_longlong(score + 0.0);  // (-0 as +0)
   b = (b >> 63) ? b : ~(b | 0x8000000000000000ull);
@@ -244,6 +244,38 @@ __device__ __forceinline__ uint4 make_cand(double score, int token, int place) {
 __device__ __forceinline__ double cand_score(const uint4& c) {
   const uint64_t b = ((uint64_t)c.w << 32) | c.z;
   return __longlong_as_double((long long)((b >> 63) ? b : ~b & 0x7fffffffffffffffull));
+}
+__device__ __forceinline__ void count_less(int& neg, const uint4& a, const uint4& b) {  // neg -= a < b
+  asm("{\n\t.reg .u32 t;\n\t"
+      "sub.cc.u32 t, %1, %5;\n\tsubc.cc.u32 t, %2, %6;\n\tsubc.cc.u32 t, %3, %7;\n\tsubc.cc.u32 t, %4, %8;\n\t"
+      "subc.u32 %0, %0, 0;\n\t}"
+      : "+r"(neg)
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w));
+}
+
+// rank_s[i] -= the number of candidates of i's sequence that come before it; nb sequences of Ni candidates, one after the
+// other. Groups of 32 candidates of one sequence, one per lane; the warps left over split a group's comparisons. Bound by
+// the ALU: more candidates per lane only add padding.
+__device__ __forceinline__ void rank_candidates(const uint4* cand, int* rank_s, int nb, int Ni) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int gps = (Ni + 31) >> 5, groups = nb * gps;
+  int shares = 1;
+  while ((shares + 1) * groups <= nw) ++shares;
+  const int len = div_small(Ni + shares - 1, shares, __fdividef(1.f, (float)shares));
+#pragma unroll 1
+  for (int w = threadIdx.x >> 5; w < groups * shares; w += nw) {
+    const int wg = div_small(w, shares, __fdividef(1.f, (float)shares));
+    const int j0 = (w - wg * shares) * len, j1 = min(j0 + len, Ni);
+    int bl = 0, g = wg;
+    for (; g >= gps; g -= gps) ++bl;
+    const uint4* list = cand + bl * Ni;
+    const int ci = g * 32 + lane;
+    const uint4 mine = list[ci < Ni ? ci : 0];
+    int neg = 0;
+#pragma unroll 8
+    for (int j = j0; j < j1; ++j) count_less(neg, list[j], mine);
+    if (ci < Ni) atomicAdd(&rank_s[bl * Ni + ci], neg);
+  }
 }
 
 // Ranks the layer's candidates of the sequences [b_begin, b_begin + b_count): writes every sequence's sorted
@@ -256,9 +288,8 @@ __device__ __forceinline__ void tail_rank(const ExpandParams& p, int b_begin, in
   const int Ni = n_prev * p.K;
   uint4* cand = reinterpret_cast<uint4*>(scratch);            // 1024 candidates
   int* rank_s = reinterpret_cast<int*>(scratch + 16384);      // 1024 ranks, negated
-  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-  const int group = 1024 / Ni;                                  // sequences ranked per pass
-  const float inv_Ni = 1.f / (float)Ni;
+  const float inv_Ni = __fdividef(1.f, (float)Ni);
+  const int group = div_small(1024, Ni, inv_Ni);              // sequences ranked per pass
 #pragma unroll 1
   for (int b0 = 0; b0 < b_count; b0 += group) {
     const int nb = (b_count - b0) < group ? (b_count - b0) : group;
@@ -270,24 +301,8 @@ __device__ __forceinline__ void tail_rank(const ExpandParams& p, int b_begin, in
       rank_s[i] = 0;
     }
     __syncthreads();
-    // Rank under the order (value desc, token asc, creation order): the number of the sequence's candidates that come
-    // first. Groups of 32 candidates of one sequence; the warps left over split a group's comparisons.
-    const int gps = (Ni + 31) >> 5, groups = nb * gps;
-    const int shares = groups < nw ? nw / groups : 1, len = (Ni + shares - 1) / shares;
-#pragma unroll 1
-    for (int w = warp; w < groups * shares; w += nw) {
-      const int g = w / shares, j0 = (w - g * shares) * len, j1 = min(j0 + len, Ni);
-      const int bl = g / gps, ci = (g - bl * gps) * 32 + lane;
-      const uint4* list = cand + bl * Ni;
-      const uint4 mine = list[ci < Ni ? ci : 0];
-      int neg = 0;
-#pragma unroll 8
-      for (int j = j0; j < j1; ++j) count_less(neg, list[j], mine);
-      if (ci < Ni) {
-        if (shares > 1) atomicAdd(&rank_s[bl * Ni + ci], neg);
-        else rank_s[bl * Ni + ci] = neg;
-      }
-    }
+    // Rank under the order (value desc, token asc, creation order): the number of the sequence's candidates that come first.
+    rank_candidates(cand, rank_s, nb, Ni);
     __syncthreads();
 #pragma unroll 1
     for (int i = tid; i < tot; i += nt) {
@@ -348,6 +363,12 @@ __device__ __forceinline__ DecideIn decide_load(const ExpandParams& p, const Tai
   return d;
 }
 
+// a / B; for a power of two by an exact product (a division in fp64 is a chain of some 200 cycles)
+__device__ __forceinline__ double mean_of(double a, int B) {
+  if ((B & (B - 1)) == 0) return a * __longlong_as_double((long long)(1023 - (31 - __clz(B))) << 52);
+  return a / (double)B;
+}
+
 // The batch-wide part: Eq. 1 over the sequences' first n sorted values, Eq. 2, Algorithm 1, the depth test,
 // the state for the next layer and the layer's outputs. GLOBAL: the inputs were written to global memory by
 // other CTAs (read past L1). One warp decides (n <= CAST_MAX_WIDTH <= 32: a rank per lane, no barriers); the next layer's
@@ -385,7 +406,7 @@ __device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailSta
                  (lane + 32 < B ? __ldcg(vs_i + (lane + 32) * CAST_MAX_WIDTH + j) : 0.0);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(kAll, a, o);
-      if (lane == 0) vbar[j] = a / (double)B;
+      if (lane == 0) vbar[j] = mean_of(a, B);
     }
     __syncthreads();
   }
@@ -404,7 +425,7 @@ __device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailSta
       } else {
 #pragma unroll 1
         for (int b = 0; b < B; ++b) u += vs_i[b * CAST_MAX_WIDTH + lane];
-        u = u / (double)B;
+        u = mean_of(u, B);
       }
     }
 #pragma unroll
@@ -481,7 +502,7 @@ __device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailSta
   }
   __syncthreads();
   const int n_i = s_ni;
-  const float inv_W = 1.f / (float)W, inv_K = 1.f / (float)K;
+  const float inv_W = __fdividef(1.f, (float)W), inv_K = __fdividef(1.f, (float)K);
 #pragma unroll 1
   for (int i = tid; i < B * W; i += nt) {
     const int b = div_small(i, W, inv_W), s = i - b * W;
@@ -956,17 +977,16 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
     }
   } else if (packed) {
     const int groups = (total + 31) >> 5, nw = kWarps - 1;
-    const int shares = groups < nw ? nw / groups : 1, len = (total + shares - 1) / shares;
+    const int sl = share_log(groups, nw), shares = 1 << sl, len = (total + shares - 1) >> sl;
 #pragma unroll 1
-    for (int w = warp; w < groups * shares; w += nw) {
-      const int g = w / shares, j0 = (w - g * shares) * len, j1 = min(j0 + len, total), i = g * 32 + lane;
+    for (int w = warp; w < groups << sl; w += nw) {
+      const int j0 = (w & (shares - 1)) * len, j1 = min(j0 + len, total), i = (w >> sl) * 32 + lane;
       const unsigned long long key = wlist[i < total ? i : 0];
-      const uint32_t lo = (uint32_t)key, hi = (uint32_t)(key >> 32);
       int neg = 0;
 #pragma unroll 8
       for (int j = j0; j < j1; ++j) {
         const uint2 o = *reinterpret_cast<const uint2*>(wlist + j);
-        count_less64(neg, lo, hi, o.x, o.y);
+        count_less64(neg, (uint32_t)key, (uint32_t)(key >> 32), o.x, o.y);
       }
       if (i < total) atomicAdd(&rank_s[i], neg);
     }
