@@ -1057,6 +1057,7 @@ struct SelectParams {
   const double* lscore;
   DevState* st;
   int P, Ncap, words, m, pool_mode, enable_dr, per_row;
+  int list_cap;  // entries of the lists in shared memory: (H + 1) m, rounded up
   double C3;
   DevTable tab;
   double* sel_score;
@@ -1075,55 +1076,80 @@ struct SelectParams {
 // publish the best min(pool, m) nodes with their values. The pool is the root plus one sorted list
 // per layer (written by the layer tails in exactly that order restricted to the layer), so the rank
 // of the k-th node of a list is k plus, for every other list, the number of its nodes that come
-// first: a binary search each. Lists are cut to their first m nodes (later ones cannot rank < m).
-__device__ __noinline__ void select_rank_phase(const SelectParams& p, int b, unsigned char* smem) {
+// first: a binary search each. Lists are cut to their first m nodes (later ones cannot rank < m), and a node below
+// the m-th of any list is passed over. The searches of a node are shared by as many threads as the CTA has to spare.
+__device__ __forceinline__ void select_rank_phase(const SelectParams& p, int b, unsigned char* smem) {
   __shared__ int lbase[CAST_MAX_DEPTH + 1], llen[CAST_MAX_DEPTH + 1], loff[CAST_MAX_DEPTH + 2];
-  double* ls = reinterpret_cast<double*>(smem);  // the lists' values, list l at loff[l]
   const int tid = threadIdx.x, nt = blockDim.x;
   const size_t o = (size_t)b * p.P;
   const int nl = p.st->layers_done + 1;  // lists: depth 0 (the root) .. layers_done
-  if (tid < nl) {  // one memory round trip for all lists
-    int len = p.pool_mode == 0 ? p.st->layer_n[tid] : p.st->n_hist[tid];
-    llen[tid] = len > p.m ? p.m : len;
-    lbase[tid] = p.st->layer_base[tid];
+  if (tid < 32) {  // one memory round trip for all lists
+    static_assert(CAST_MAX_DEPTH + 1 <= 32, "a list per lane");
+    int len = 0, at = 0;
+    if (tid < nl) {
+      len = p.pool_mode == 0 ? p.st->layer_n[tid] : p.st->n_hist[tid];
+      at = p.st->layer_base[tid];
+    }
+    len = len > p.m ? p.m : len;
+    int incl = len;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, d);
+      if (tid >= d) incl += t;
+    }
+    if (tid < nl) {
+      llen[tid] = len;
+      lbase[tid] = at;
+      loff[tid + 1] = incl;
+    }
+    if (tid == 0) loff[0] = 0;
   }
   const int peff = p.pool_mode == 0 ? p.st->pool_size : p.st->kept_total;  // (needed further down)
   __syncthreads();
-  if (tid == 0) {
-    int acc = 0;
-    for (int l = 0; l < nl; ++l) {
-      loff[l] = acc;
-      acc += llen[l];
-    }
-    loff[nl] = acc;
-  }
-  __syncthreads();
   const int total = loff[nl];
+  double* ls = reinterpret_cast<double*>(smem);                  // the lists' values, list l at loff[l]
+  int* rank_s = reinterpret_cast<int*>(ls + p.list_cap);         // ranks
+  unsigned char* lst = reinterpret_cast<unsigned char*>(rank_s + p.list_cap);  // which list
 #pragma unroll 1
   for (int i = tid; i < total; i += nt) {
     int l = 0;
     while (i >= loff[l + 1]) ++l;
     ls[i] = p.lscore[o + lbase[l] + (i - loff[l])];
+    rank_s[i] = i - loff[l];
+    lst[i] = (unsigned char)l;
   }
   __syncthreads();
   const int n_out = min(min(peff, p.m), p.Ncap);
+  double bound = -INFINITY;
+#pragma unroll 4
+  for (int l = 0; l < nl; ++l)
+    if (llen[l] >= p.m) bound = fmax(bound, ls[loff[l] + p.m - 1]);
+  int parts = 1;  // threads per node, a multiple of four lists each at a time
+  while ((parts + 1) * total <= nt && parts < nl) ++parts;
   int half0 = 1;  // first stride of the searches: positions up to 2 half0 - 1 >= the longest list are reachable
   while (2 * half0 - 1 < p.m && half0 < CAST_MAX_TREE) half0 <<= 1;
+  int part = 0, i = tid;
+  while (i >= total && part < parts) {
+    i -= total;
+    ++part;
+  }
 #pragma unroll 1
-  for (int i = tid; i < total; i += nt) {
-    int l = 0;
-    while (i >= loff[l + 1]) ++l;
-    const int k = i - loff[l];
+  for (; part < parts && i < total; i += nt) {  // (more nodes than threads: parts is 1)
+    const int l = lst[i];
     const double s = ls[i];
-    int rank = k;
+    if (s < bound) {
+      if (part == 0) rank_s[i] = 0x40000000;
+      continue;
+    }
+    int before = 0;
     // nodes of another list l2 that come first: value > s, or value == s when their depth is smaller.
     // Lower-bound searches, four lists in lockstep and branch-free so that their loads overlap.
 #pragma unroll 1
-    for (int l0 = 0; l0 < nl; l0 += 4) {
+    for (int l0 = part; l0 < nl; l0 += 4 * parts) {
       int pos[4] = {0, 0, 0, 0}, len4[4], off4[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const int l2 = l0 + q;
+        const int l2 = l0 + q * parts;
         const bool valid = l2 < nl && l2 != l;
         len4[q] = valid ? llen[l2] : 0;
         off4[q] = valid ? loff[l2] : 0;
@@ -1135,129 +1161,138 @@ __device__ __noinline__ void select_rank_phase(const SelectParams& p, int b, uns
           const int idx = pos[q] + half - 1;
           const bool inb = idx < len4[q];
           const double a = ls[off4[q] + (inb ? idx : 0)];
-          const bool first = inb && ((l0 + q < l) ? (a >= s) : (a > s));
+          const bool first = inb && ((l0 + q * parts < l) ? (a >= s) : (a > s));
           pos[q] += first ? half : 0;
         }
       }
-      rank += pos[0] + pos[1] + pos[2] + pos[3];
+      before += pos[0] + pos[1] + pos[2] + pos[3];
     }
+    if (before != 0) atomicAdd(&rank_s[i], before);
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int j = tid; j < total; j += nt) {
+    const int rank = rank_s[j];
     if (rank < n_out) {
+      const int l = lst[j];
+      const double s = ls[j];
       p.sel_score[(size_t)b * p.Ncap + rank] = s;
       p.sel_value[(size_t)b * p.Ncap + rank] = fast_exp_neg(s);
-      p.sel_idx[(size_t)b * p.Ncap + rank] = p.lsort[o + lbase[l] + k];
+      p.sel_idx[(size_t)b * p.Ncap + rank] = p.lsort[o + lbase[l] + (j - loff[l])];
     }
   }
 }
 
-// Phase 2: batch-mean utility, target-cost ratio, Algorithm 1 -> N; then sequence b's tree.
-__device__ __noinline__ void select_finalize_phase(const SelectParams& p, int b, int B) {
+// Phase 2: batch-mean utility, target-cost ratio, Algorithm 1 -> N; then sequence b's tree. Four threads per rank in the
+// phases that loop over the ranks (512 threads): with one, those loops were most of this phase.
+constexpr int kSelThreads = 512, kSelShares = kSelThreads / CAST_MAX_TREE;
+static_assert(kSelShares == 4, "four lanes of a warp share a rank");
+__device__ __forceinline__ void select_finalize_phase(const SelectParams& p, int b, int B) {
   __shared__ double u[CAST_MAX_TREE], c[CAST_MAX_TREE];
   __shared__ int kept[CAST_MAX_TREE], lin_parent[CAST_MAX_TREE];
   __shared__ short lin_of[1 + CAST_MAX_TOP_K + (CAST_MAX_DEPTH - 1) * CAST_MAX_WIDTH * CAST_MAX_TOP_K];
   __shared__ int s_N;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int rk = tid >> 2, sub = tid & 3;  // this thread's rank (or node) and share
   const size_t o = (size_t)b * p.P;
   const int pool = p.st->pool_size;
   const int peff = p.pool_mode == 0 ? pool : p.st->kept_total;
   int n = min(min(peff, p.m), p.Ncap);
   if (p.enable_dr && p.tab.Ntab < n) n = p.tab.Ntab;
   if (tid == 0) s_N = 1;
-  // u_k = sum_{s<=k} v(s), v(s) = batch mean of the rank-s values (Eq. 1), or this sequence's own
-  // rank-s value when every sequence sizes its tree by itself. The means first, a thread per rank with
-  // several loads in flight (u doubles as their buffer), then the prefix sums in one warp.
-#pragma unroll 1
-  for (int s = tid; s < n; s += nt) {
-    double a = 0.0;
-    if (p.per_row) {
-      a = p.sel_value[(size_t)b * p.Ncap + s];
-    } else {
-#pragma unroll 8
-      for (int bb = 0; bb < B; ++bb) a += p.sel_value[(size_t)bb * p.Ncap + s];
-      a /= (double)B;
-    }
-    u[s] = a;
-  }
-  __syncthreads();
-  if (tid < 32) {
-    double v[4], run = 0.0;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int s = lane * 4 + e;
-      run += s < n ? u[s] : 0.0;
-      v[e] = run;
-    }
-    double incl = run;  // inclusive scan of the lane totals
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const double t = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += t;
-    }
-    const double excl = incl - run;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int s = lane * 4 + e;
-      if (s < n) u[s] = excl + v[e];
-    }
-  }
   if (p.enable_dr) {
     const int g0 = select_grid(p.st->n0, p.tab.L, p.tab.M);
     const double* f = p.tab.fT + (size_t)(g0 - 1) * p.tab.Ntab;
-#pragma unroll 1
-    for (int k = tid; k < n; k += nt) c[k] = f[k] / f[0];
+    if (tid < n) c[tid] = f[tid] / f[0];
   }
-  __syncthreads();
-  int N = n;
+  // u_k = sum_{s<=k} v(s), v(s) = batch mean of the rank-s values (Eq. 1), or this sequence's own
+  // rank-s value when every sequence sizes its tree by itself. The means first (u doubles as their buffer), then the
+  // prefix sums in one warp. (Without the dynamic rerank nothing of this is used.)
   if (p.enable_dr) {
-#pragma unroll 1
-    for (int j = tid; j < n; j += nt) {
-      bool ok = true;
-#pragma unroll 1
-      for (int i = 0; i < j; ++i)
-        if ((u[j] - u[i]) < p.C3 * (c[j] - c[i])) ok = false;
-      if (ok) atomicMax(&s_N, j + 1);
+    double a = 0.0;
+    if (rk < n) {
+      if (p.per_row) {
+        a = sub == 0 ? p.sel_value[(size_t)b * p.Ncap + rk] : 0.0;
+      } else {
+#pragma unroll 16
+        for (int bb = sub; bb < B; bb += kSelShares) a += p.sel_value[(size_t)bb * p.Ncap + rk];
+      }
+    }
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    if (sub == 0 && rk < n) u[rk] = p.per_row ? a : a / (double)B;
+    __syncthreads();
+    if (tid < 32) {
+      double v[4], run = 0.0;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int s = lane * 4 + e;
+        run += s < n ? u[s] : 0.0;
+        v[e] = run;
+      }
+      double incl = run;  // inclusive scan of the lane totals
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const double t = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += t;
+      }
+      const double excl = incl - run;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int s = lane * 4 + e;
+        if (s < n) u[s] = excl + v[e];
+      }
     }
     __syncthreads();
-    N = s_N;
+    bool ok = rk < n;
+    const double uj = ok ? u[rk] : 0.0, cj = ok ? c[rk] : 0.0;
+#pragma unroll 4
+    for (int i = sub; i < rk && i < n; i += kSelShares)
+      if ((uj - u[i]) < p.C3 * (cj - c[i])) ok = false;
+    const unsigned good = __ballot_sync(0xffffffffu, ok);
+    if (sub == 0 && ((good >> (lane & ~3)) & 15u) == 15u) atomicMax(&s_N, rk + 1);
+    __syncthreads();
   }
+  const int N = p.enable_dr ? s_N : n;
   // linearise: kept nodes in creation order (ascending pool index)
-#pragma unroll 1
-  for (int s = tid; s < N; s += nt) kept[s] = p.sel_idx[(size_t)b * p.Ncap + s];
+  if (tid < N) kept[tid] = p.sel_idx[(size_t)b * p.Ncap + tid];
   __syncthreads();
-#pragma unroll 1
-  for (int s = tid; s < N; s += nt) {
-    const int mine = kept[s];
-    int t0 = 0, t1 = 0, j = 0;
-    for (; j + 2 <= N; j += 2) {
-      t0 += (kept[j] < mine);
-      t1 += (kept[j + 1] < mine);
-    }
-    for (; j < N; ++j) t0 += (kept[j] < mine);
-    lin_of[mine] = (short)(t0 + t1);
+  const int pi = rk < N ? kept[rk] : 0;
+  int tok = 0, par = -1, dep = 0;
+  double score = 0.0;
+  if (rk < N && sub == 0) {  // requested now, used once the order is known
+    tok = p.pool_token[o + pi];
+    par = p.pool_parent[o + pi];
+    dep = p.pool_depth[o + pi];
+    score = p.pool_score[o + pi];
   }
+  int t = 0;
+#pragma unroll 4
+  for (int j = sub; j < N; j += kSelShares) t += kept[j] < pi;
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  if (rk < N && sub == 0) lin_of[pi] = (short)t;
   __syncthreads();
-#pragma unroll 1
-  for (int s = tid; s < N; s += nt) {
-    const int pi = kept[s];
-    const int t = lin_of[pi];
-    const int pp = p.pool_parent[o + pi];
-    const int lp = pp >= 0 ? (int)lin_of[pp] : -1;
+  if (rk < N && sub == 0) {
+    const int lp = par >= 0 ? (int)lin_of[par] : -1;
     lin_parent[t] = lp;
     const size_t q = (size_t)b * p.Ncap + t;
-    p.tokens[q] = p.pool_token[o + pi];
+    p.tokens[q] = tok;
     p.parent[q] = lp;
-    p.depth[q] = p.pool_depth[o + pi];
+    p.depth[q] = dep;
     p.pool_idx[q] = pi;
-    if (p.scores) p.scores[q] = p.pool_score[o + pi];
+    if (p.scores) p.scores[q] = score;
   }
   __syncthreads();
-#pragma unroll 1
-  for (int t = tid; t < p.Ncap; t += nt) {
+  if (tid < p.Ncap) {
     uint32_t w[CAST_MAX_TREE / 32] = {0u, 0u, 0u, 0u};
-    const size_t q = (size_t)b * p.Ncap + t;
-    if (t < N) {
-      int a = t, guard = 0;
+    const size_t q = (size_t)b * p.Ncap + tid;
+    if (tid < N) {
+      int a = tid, guard = 0;
       while (a >= 0 && a < N && guard++ <= CAST_MAX_DEPTH + 1) {  // walk to the root, one bit per ancestor
-        w[a >> 5] |= 1u << (a & 31);
+        const uint32_t bit = 1u << (a & 31);
+#pragma unroll
+        for (int k = 0; k < CAST_MAX_TREE / 32; ++k) w[k] |= (a >> 5) == k ? bit : 0u;
         a = lin_parent[a];
       }
     } else {
@@ -1267,7 +1302,9 @@ __device__ __noinline__ void select_finalize_phase(const SelectParams& p, int b,
       p.pool_idx[q] = -1;
       if (p.scores) p.scores[q] = 0.0;
     }
-    for (int k = 0; k < p.words; ++k) p.anc[q * p.words + k] = w[k];
+#pragma unroll
+    for (int k = 0; k < CAST_MAX_TREE / 32; ++k)
+      if (k < p.words) p.anc[q * p.words + k] = w[k];
   }
   if (tid == 0) {
     p.n_tree[b] = N;
@@ -1275,15 +1312,17 @@ __device__ __noinline__ void select_finalize_phase(const SelectParams& p, int b,
   }
 }
 
-__global__ void __launch_bounds__(512) select_rank_kernel(const SelectParams p) {
+__global__ void __launch_bounds__(kSelThreads) select_rank_kernel(const SelectParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   grid_dependency_wait();
+  grid_launch_dependents();
   select_rank_phase(p, blockIdx.x, smem);
 }
-__global__ void __launch_bounds__(512) select_finalize_kernel(const SelectParams p) {
+__global__ void __launch_bounds__(kSelThreads) select_finalize_kernel(const SelectParams p) {
+  grid_dependency_wait();
   select_finalize_phase(p, blockIdx.x, gridDim.x);
 }
-__global__ void __launch_bounds__(512) select_fused_kernel(const SelectParams p) {  // batch 1: one launch
+__global__ void __launch_bounds__(kSelThreads) select_fused_kernel(const SelectParams p) {  // batch 1: one launch
   extern __shared__ __align__(16) unsigned char smem[];
   grid_dependency_wait();
   select_rank_phase(p, 0, smem);
@@ -1421,32 +1460,30 @@ extern "C" cast_status cast_select_nodes(cast_ctx* c, int32_t* tokens, int32_t* 
   p.sel_score = c->sel_score; p.sel_value = c->sel_value; p.sel_idx = c->sel_idx;
   p.tokens = tokens; p.parent = parent; p.depth = depth; p.anc = anc_mask; p.pool_idx = pool_idx;
   p.scores = scores; p.n_tree = n_tree;
-  // the lists' values: (H + 1) lists of at most m nodes
-  const size_t smem = (size_t)(c->cfg.max_depth + 1) * c->cfg.total_token * sizeof(double);
-  cudaStream_t s = (cudaStream_t)stream;
-  int threads = ((c->cfg.max_depth + 1) * c->cfg.total_token + 31) / 32 * 32;
-  threads = threads > 512 ? 512 : (threads < 128 ? 128 : threads);
+  // (H + 1) lists of at most m nodes: value, rank, list
+  p.list_cap = ((c->cfg.max_depth + 1) * c->cfg.total_token + 15) / 16 * 16;
+  const size_t smem = (size_t)p.list_cap * (sizeof(double) + sizeof(int32_t) + 1);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(c->cur_B, 1, 1);
-  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.blockDim = dim3(kSelThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
+  cfg.stream = (cudaStream_t)stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see cast_tree_expand
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  cudaError_t e;
   if (c->cur_B == 1) {
-    if (cudaLaunchKernelEx(&cfg, select_fused_kernel, p) != cudaSuccess) {
-      cudaGetLastError();
-      return CAST_ERR_CUDA;
-    }
+    e = cudaLaunchKernelEx(&cfg, select_fused_kernel, p);
   } else {
-    if (cudaLaunchKernelEx(&cfg, select_rank_kernel, p) != cudaSuccess) {
-      cudaGetLastError();
-      return CAST_ERR_CUDA;
-    }
-    select_finalize_kernel<<<c->cur_B, 128, 0, s>>>(p);
+    e = cudaLaunchKernelEx(&cfg, select_rank_kernel, p);
+    cfg.dynamicSmemBytes = 0;
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, select_finalize_kernel, p);
   }
-  return launch_status();
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return CAST_ERR_CUDA;
+  }
+  return CAST_OK;
 }
