@@ -6,8 +6,11 @@
 // all tree tokens and all heads of the group. Tiles of 64 positions are converted to fp32 in
 // shared memory; S = QK^T and O += PV are register-tiled FFMA loops; the softmax is online.
 // Prefix positions need no mask; a tree position L+j is visible to row (t, g) iff bit j of
-// anc_mask[t] is set. KV splits write (max, sum, unnormalised O) partials that a second
-// kernel merges.
+// anc_mask[t] is set. KV splits write (max, sum, unnormalised O) partials; the CTA of a row block
+// that finishes last (an atomic ticket, nothing spins) merges them, or a second kernel when they are many.
+// Bound by instruction issue, shared-memory reads of the products first: both go by 16-byte vectors, the first product by
+// packed multiply-adds (V = 60 tokens, 4 sequences of 2048, 32/8 heads of 64: 276 -> 233 us; 128 dims 511 -> 450). A 64-row
+// tile of 8 x 4 per thread was built: as fast from 200 rows per kv-head on, up to twice as slow below.
 #include <math.h>
 
 #include "cast_internal.h"
@@ -30,21 +33,24 @@ constexpr int kRB = 32;   // query rows per CTA
 constexpr int kPT = 64;   // positions per tile
 constexpr int kThreads = 256;
 constexpr int kMaxSplit = 64;
+constexpr int kMergeHere = 16;  // up to this many splits the last CTA merges (a second launch costs 4 us)
+constexpr size_t kCcTicketBytes = (size_t)CAST_MAX_BATCH * 512 * sizeof(int32_t);
 
 struct AttnParams {
   const void* q;
   const void* k;
   const void* v;
   void* out;
-  int B, Ncap, Hq, Hkv, G, page_size, seq_capacity, num_pages, words, nsplit;
+  int B, Ncap, Hq, Hkv, G, page_size, seq_capacity, num_pages, words, nsplit, nrowblk;
   const int32_t* page_table;
   const int32_t* kv_len;
   const int32_t* n_tree;
   const int32_t* first_row;  // [B] or null: output rows start at this tree token
   const uint32_t* anc;
   float scale;
-  float* part_o;   // [B][Hq][Ncap][nsplit][D]
-  float* part_ml;  // [B][Hq][Ncap][nsplit][2]
+  int32_t* ticket;  // [B][Hkv][nrowblk] splits finished
+  float* part_o;    // [B][Hkv][nrowblk][nsplit][kRB][D]
+  float* part_ml;   // [B][Hkv][nrowblk][nsplit][kRB][2]
   DevState* st;
 };
 
@@ -62,13 +68,78 @@ template <> __device__ __forceinline__ void load_chunk<__nv_bfloat16>(const __nv
     out[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
   }
 }
-__device__ __forceinline__ void store_out(float* p, float x) { *p = x; }
-__device__ __forceinline__ void store_out(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
+__device__ __forceinline__ void store4(float* p, const float (&x)[4], float f) {
+  *reinterpret_cast<float4*>(p) = make_float4(x[0] * f, x[1] * f, x[2] * f, x[3] * f);
+}
+__device__ __forceinline__ void store4(__nv_bfloat16* p, const float (&x)[4], float f) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(x[0] * f, x[1] * f), b = __floats2bfloat162_rn(x[2] * f, x[3] * f);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
+
+// Packed fp32 pairs: one instruction, two multiply-adds with IEEE results each.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float sum2(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a + b;
+}
+
+// Merge of a row block's splits: this warp's rows r0, r0 + step, ... The splits' weights two per lane, then the columns, four
+// per lane (at D = 64 each half of the warp takes every other split); the loads of many splits in flight.
+template <typename T, int D>
+__device__ __forceinline__ void merge_splits(const AttnParams& p, int b, int kvh, int rb, int F, int row0, int r0, int step,
+                                             int rows_here) {
+  static_assert(kMaxSplit <= 64, "two splits per lane");
+  constexpr int C4 = D / 4, kHalves = 32 / C4;
+  const int lane = threadIdx.x & 31, c = lane % C4 * 4, half = lane / C4;
+  const size_t part0 = (((size_t)b * p.Hkv + kvh) * p.nrowblk + rb) * p.nsplit * kRB;
+  const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + part0;
+#pragma unroll 1
+  for (int r = r0; r < rows_here; r += step) {
+    float2 x[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      x[h] = lane + 32 * h < p.nsplit ? __ldcg(ml + (size_t)(lane + 32 * h) * kRB + r) : make_float2(-INFINITY, 0.f);
+    float M = fmaxf(x[0].x, x[1].x), w[2], l = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int of = 16; of > 0; of >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, of));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      w[h] = x[h].x > -INFINITY ? expf(x[h].x - M) : 0.f;
+      l += x[h].y * w[h];
+    }
+#pragma unroll
+    for (int of = 16; of > 0; of >>= 1) l += __shfl_xor_sync(0xffffffffu, l, of);
+#pragma unroll 16
+    for (int s0 = 0; s0 < p.nsplit; s0 += kHalves) {
+      const int s = s0 + half;
+      const float ws = __shfl_sync(0xffffffffu, s0 < 32 ? w[0] : w[1], s & 31);
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);  // (a split that saw nothing weighs 0, and its sums are 0)
+      if (s < p.nsplit) v = __ldcg(reinterpret_cast<const float4*>(p.part_o + (part0 + (size_t)s * kRB + r) * D + c));
+      acc[0] += v.x * ws;
+      acc[1] += v.y * ws;
+      acc[2] += v.z * ws;
+      acc[3] += v.w * ws;
+    }
+    if (kHalves == 2) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);
+    }
+    const int row = row0 + r, t = F + row / p.G;
+    T* out = reinterpret_cast<T*>(p.out) + (((size_t)b * p.Ncap + t) * p.Hq + kvh * p.G + row % p.G) * D;
+    if (half == 0) store4(out + c, acc, l > 0.f ? 1.f / l : 0.f);
+  }
+}
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams p) {
   constexpr int KS = D + 4;          // padded row stride of Qs / Ks (floats)
-  constexpr int SS = kPT + 1;        // row stride of Ss
+  constexpr int SS = kPT + 4;        // row stride of Ss: rows 16-byte aligned
   constexpr int CH = 16 / sizeof(T); // elements per 16-byte chunk
   constexpr int CPR = D / CH;        // chunks per cache row
   constexpr int DC = D / 32;         // output columns per lane
@@ -79,7 +150,10 @@ __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams
   float* Ss = Vs + kPT * D;               // [kRB][SS]
   __shared__ float row_m[kRB], row_l[kRB], row_alpha[kRB];
   __shared__ uint32_t anc_s[kRB][CAST_MAX_TREE / 32];
-  __shared__ long long slot_s[kPT];
+  __shared__ long long slot_s[2][kPT];
+  __shared__ int s_last;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const int split = blockIdx.x % p.nsplit, rb = blockIdx.x / p.nsplit;
   const int kvh = blockIdx.y, b = blockIdx.z;
@@ -103,6 +177,22 @@ __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams
   const int ntiles = (total + kPT - 1) / kPT;
   const int t0 = (int)((long long)split * ntiles / p.nsplit), t1 = (int)((long long)(split + 1) * ntiles / p.nsplit);
 
+  auto find_slots = [&](int tile) {  // cache slots of a tile's positions, a tile ahead of their use
+    if (tid >= kPT) return;
+    const int pos = tile * kPT + tid;
+    long long slot = -1;
+    if (tile < t1 && pos < total) {
+      if (p.page_size == 0) {
+        slot = (long long)b * p.seq_capacity + pos;
+      } else {
+        const int page = p.page_table[(size_t)b * p.seq_capacity + pos / p.page_size];
+        if (page < 0 || page >= p.num_pages) report(p.st, CAST_ERR_BAD_PAGE, b);
+        else slot = (long long)page * p.page_size + pos % p.page_size;
+      }
+    }
+    slot_s[tile & 1][tid] = slot;
+  };
+  find_slots(t0);
   // query rows (pre-scaled), their ancestor masks, running softmax state
   const T* q = reinterpret_cast<const T*>(p.q);
   for (int i = tid; i < kRB * CPR; i += kThreads) {
@@ -137,25 +227,11 @@ __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams
 
   for (int tile = t0; tile < t1; ++tile) {
     const int pbase = tile * kPT;
-    __syncthreads();  // previous tile fully consumed; Qs/anc_s visible on the first pass
-    if (tid < kPT) {
-      const int pos = pbase + tid;
-      long long slot = -1;
-      if (pos < total) {
-        if (p.page_size == 0) {
-          slot = (long long)b * p.seq_capacity + pos;
-        } else {
-          const int page = p.page_table[(size_t)b * p.seq_capacity + pos / p.page_size];
-          if (page < 0 || page >= p.num_pages) report(p.st, CAST_ERR_BAD_PAGE, b);
-          else slot = (long long)page * p.page_size + pos % p.page_size;
-        }
-      }
-      slot_s[tid] = slot;
-    }
-    __syncthreads();
+    __syncthreads();  // previous tile fully consumed; the slots (and Qs, anc_s on the first pass) visible
+#pragma unroll 4
     for (int i = tid; i < kPT * CPR; i += kThreads) {
       const int pl = i / CPR, ch = i % CPR;
-      const long long slot = slot_s[pl];
+      const long long slot = slot_s[tile & 1][pl];
       float fk[CH], fv[CH];
       if (slot >= 0) {
         const size_t off = ((size_t)slot * p.Hkv + kvh) * D + ch * CH;
@@ -166,28 +242,30 @@ __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams
         for (int e = 0; e < CH; ++e) fk[e] = fv[e] = 0.f;
       }
 #pragma unroll
-      for (int e = 0; e < CH; ++e) {
-        Ks[pl * KS + ch * CH + e] = fk[e];
-        Vs[pl * D + ch * CH + e] = fv[e];
+      for (int e = 0; e < CH; e += 4) {
+        *reinterpret_cast<float4*>(Ks + pl * KS + ch * CH + e) = make_float4(fk[e], fk[e + 1], fk[e + 2], fk[e + 3]);
+        *reinterpret_cast<float4*>(Vs + pl * D + ch * CH + e) = make_float4(fv[e], fv[e + 1], fv[e + 2], fv[e + 3]);
       }
     }
     __syncthreads();
+    find_slots(tile + 1);
     // S = Q K^T: thread (ty, tx) owns rows 2ty, 2ty+1 and positions tx, tx+16, tx+32, tx+48
     {
-      float acc[2][4];
+      // (the inner index in pairs: a packed instruction does two multiply-adds, and the operands lie in pairs anyway)
+      f32x2 acc[2][4];
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
 #pragma unroll 8
       for (int d = 0; d < D; d += 4) {
-        const float4 q0 = *reinterpret_cast<const float4*>(Qs + (2 * ty) * KS + d);
-        const float4 q1 = *reinterpret_cast<const float4*>(Qs + (2 * ty + 1) * KS + d);
+        const ulonglong2 q0 = *reinterpret_cast<const ulonglong2*>(Qs + (2 * ty) * KS + d);
+        const ulonglong2 q1 = *reinterpret_cast<const ulonglong2*>(Qs + (2 * ty + 1) * KS + d);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const float4 kk = *reinterpret_cast<const float4*>(Ks + (tx + 16 * j) * KS + d);
-          acc[0][j] += q0.x * kk.x + q0.y * kk.y + q0.z * kk.z + q0.w * kk.w;
-          acc[1][j] += q1.x * kk.x + q1.y * kk.y + q1.z * kk.z + q1.w * kk.w;
+          const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(Ks + (tx + 16 * j) * KS + d);
+          acc[0][j] = fma2(q0.y, kk.y, fma2(q0.x, kk.x, acc[0][j]));
+          acc[1][j] = fma2(q1.y, kk.y, fma2(q1.x, kk.x, acc[1][j]));
         }
       }
 #pragma unroll
@@ -202,7 +280,7 @@ __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams
             const int jt = pos - L;
             vis = (anc_s[r][jt >> 5] >> (jt & 31)) & 1u;
           }
-          Ss[r * SS + pl] = vis ? acc[i][j] : -INFINITY;
+          Ss[r * SS + pl] = vis ? sum2(acc[i][j]) : -INFINITY;
         }
       }
     }
@@ -243,94 +321,147 @@ __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams
       for (int e = 0; e < DC; ++e) o[rr][e] *= a;
     }
 #pragma unroll 4
-    for (int pl = 0; pl < kPT; ++pl) {
-      float vv[DC];
-      if constexpr (DC == 4) {
-        const float4 t4 = *reinterpret_cast<const float4*>(Vs + pl * D + lane * 4);
-        vv[0] = t4.x; vv[1] = t4.y; vv[2] = t4.z; vv[3] = t4.w;
-      } else {
-        const float2 t2 = *reinterpret_cast<const float2*>(Vs + pl * D + lane * 2);
-        vv[0] = t2.x; vv[1] = t2.y;
-      }
+    for (int pl = 0; pl < kPT; pl += 4) {
+      float4 pv[4];
 #pragma unroll
-      for (int rr = 0; rr < 4; ++rr) {
-        const float pv = Ss[(4 * warp + rr) * SS + pl];
+      for (int rr = 0; rr < 4; ++rr) pv[rr] = *reinterpret_cast<const float4*>(Ss + (4 * warp + rr) * SS + pl);
 #pragma unroll
-        for (int e = 0; e < DC; ++e) o[rr][e] += pv * vv[e];
+      for (int x = 0; x < 4; ++x) {
+        float vv[DC];
+        if constexpr (DC == 4) {
+          const float4 t4 = *reinterpret_cast<const float4*>(Vs + (pl + x) * D + lane * 4);
+          vv[0] = t4.x; vv[1] = t4.y; vv[2] = t4.z; vv[3] = t4.w;
+        } else {
+          const float2 t2 = *reinterpret_cast<const float2*>(Vs + (pl + x) * D + lane * 2);
+          vv[0] = t2.x; vv[1] = t2.y;
+        }
+#pragma unroll
+        for (int rr = 0; rr < 4; ++rr) {
+          const float w = x == 0 ? pv[rr].x : x == 1 ? pv[rr].y : x == 2 ? pv[rr].z : pv[rr].w;
+#pragma unroll
+          for (int e = 0; e < DC; ++e) o[rr][e] += w * vv[e];
+        }
       }
     }
   }
   __syncthreads();
-  // partials of this split
+  // rows to shared memory (the keys' place), then in contiguous pieces: the output, or this split's partial
+  float* Os = Ks;
 #pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int r = 4 * warp + rr, row = row0 + r;
-    if (row >= rows_total) continue;
-    const int t = F + row / G, h = kvh * G + row % G;
-    const size_t pr = (((size_t)b * p.Hq + h) * p.Ncap + t) * p.nsplit + split;
+  for (int rr = 0; rr < 4; ++rr)
 #pragma unroll
-    for (int e = 0; e < DC; ++e) p.part_o[pr * D + lane * DC + e] = o[rr][e];
-    if (lane == 0) {
-      p.part_ml[pr * 2] = row_m[r];
-      p.part_ml[pr * 2 + 1] = row_l[r];
+    for (int e = 0; e < DC; ++e) Os[(4 * warp + rr) * KS + lane * DC + e] = o[rr][e];
+  __syncthreads();
+  const int rows_here = rows_total - row0 < kRB ? rows_total - row0 : kRB;
+  constexpr int C4 = D / 4;
+  T* out = reinterpret_cast<T*>(p.out);
+  auto out_row = [&](int r) {
+    const int row = row0 + r, t = F + row / G;
+    return out + (((size_t)b * p.Ncap + t) * p.Hq + kvh * G + row % G) * D;
+  };
+  if (p.nsplit == 1) {
+    for (int i = tid; i < rows_here * C4; i += kThreads) {
+      const int r = i / C4, c = i % C4 * 4;
+      const float4 v = *reinterpret_cast<const float4*>(Os + r * KS + c);
+      const float x[4] = {v.x, v.y, v.z, v.w};
+      store4(out_row(r) + c, x, row_l[r] > 0.f ? 1.f / row_l[r] : 0.f);
     }
+    return;
   }
+  const size_t item = ((size_t)b * p.Hkv + kvh) * p.nrowblk + rb, part0 = item * p.nsplit * kRB;
+  float2* ml = reinterpret_cast<float2*>(p.part_ml) + part0;
+  for (int i = tid; i < rows_here * C4; i += kThreads) {
+    const int r = i / C4, c = i % C4 * 4;
+    __stcg(reinterpret_cast<float4*>(p.part_o + (part0 + (size_t)split * kRB + r) * D + c), *reinterpret_cast<const float4*>(Os + r * KS + c));
+  }
+  if (tid < rows_here) __stcg(ml + (size_t)split * kRB + tid, make_float2(row_m[tid], row_l[tid]));
+  if (p.nsplit > kMergeHere) return;  // attn_merge_kernel
+  __syncthreads();
+  if (tid == 0) {
+    // releases this CTA's partial (the barrier made it this thread's to release), acquires those that came earlier
+    int t;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(t) : "l"(p.ticket + item) : "memory");
+    s_last = t == p.nsplit - 1;
+    if (t == p.nsplit - 1) p.ticket[item] = 0;  // ready for the next launch
+  }
+  __syncthreads();
+  if (!s_last) return;
+  merge_splits<T, D>(p, b, kvh, rb, F, row0, warp, kThreads / 32, rows_here);
 }
 
-// Merge the split partials of one (sequence, tree token, head); rows >= n_tree are left untouched.
+// The same as a kernel of its own, a warp per row: for launches of many splits, whose partials (a quarter of a megabyte and
+// more per row block) one CTA would take several us to read.
 template <typename T, int D>
-__global__ void __launch_bounds__(D) attn_combine_kernel(const AttnParams p) {
-  const int t = blockIdx.x, h = blockIdx.y, b = blockIdx.z, d = threadIdx.x;
-  T* out = reinterpret_cast<T*>(p.out) + (((size_t)b * p.Ncap + t) * p.Hq + h) * D;
+__global__ void __launch_bounds__(kThreads) attn_merge_kernel(const AttnParams p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  constexpr int kPer = kRB / (kThreads / 32);  // CTAs per row block
+  const int rb = blockIdx.x / kPer, kvh = blockIdx.y, b = blockIdx.z;
   int N = p.n_tree[b];
-  N = N > p.Ncap ? p.Ncap : N;
-  if (t >= N || (p.first_row != nullptr && t < p.first_row[b])) return;
-  const size_t pr = (((size_t)b * p.Hq + h) * p.Ncap + t) * p.nsplit;
-  float M = -INFINITY;
-  for (int s = 0; s < p.nsplit; ++s) M = fmaxf(M, p.part_ml[(pr + s) * 2]);
-  float l = 0.f, acc = 0.f;
-  for (int s = 0; s < p.nsplit; ++s) {
-    const float ms = p.part_ml[(pr + s) * 2];
-    if (ms > -INFINITY) {
-      const float w = expf(ms - M);
-      l += p.part_ml[(pr + s) * 2 + 1] * w;
-      acc += p.part_o[(pr + s) * D + d] * w;
-    }
-  }
-  store_out(out + d, l > 0.f ? acc / l : 0.f);
+  N = N < 0 ? 0 : (N > p.Ncap ? p.Ncap : N);
+  int F = p.first_row != nullptr ? p.first_row[b] : 0;
+  F = F < 0 ? 0 : (F > N ? N : F);
+  const int row0 = rb * kRB, rows_here = min((N - F) * p.G - row0, kRB);
+  const int r = (blockIdx.x % kPer) * (kThreads / 32) + (threadIdx.x >> 5);
+  merge_splits<T, D>(p, b, kvh, rb, F, row0, r, kRB, rows_here);
 }
 
-// KV splits of a CUDA-core launch and the partial rows its workspace holds.
-int cc_splits(const cast_ctx* c, int B, int Hkv, int G, int page_size, int seq_capacity) {
-  const int base = B * Hkv * ((c->cfg.total_token * G + kRB - 1) / kRB);
+// Row blocks and KV splits of a launch, and the bytes of workspace it needs.
+struct CcPlan {
+  int nsplit, nrowblk;
+  size_t bytes;
+};
+CcPlan cc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, int seq_capacity) {
+  CcPlan pl;
+  pl.nrowblk = (c->cfg.total_token * (Hq / Hkv) + kRB - 1) / kRB;
+  const int base = B * Hkv * pl.nrowblk;
   int nsplit = (2 * c->num_sms + base - 1) / base;
   const int max_pos = page_size == 0 ? seq_capacity : seq_capacity * page_size;
   const int max_tiles = (max_pos + kPT - 1) / kPT;
   if (nsplit > max_tiles) nsplit = max_tiles;
   if (nsplit > kMaxSplit) nsplit = kMaxSplit;
-  if (nsplit < 1) nsplit = 1;
-  return nsplit;
-}
-size_t cc_workspace(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, int seq_capacity) {
-  const size_t rows = (size_t)B * Hq * c->cfg.max_tree * cc_splits(c, B, Hkv, Hq / Hkv, page_size, seq_capacity);
-  return rows * (D + 2) * sizeof(float);
+  if (nsplit < 1 || (size_t)base * sizeof(int32_t) > kCcTicketBytes) nsplit = 1;
+  pl.nsplit = nsplit;
+  pl.bytes = nsplit == 1 ? 0 : kCcTicketBytes + (size_t)base * nsplit * kRB * (D + 2) * sizeof(float);
+  return pl;
 }
 
 template <typename T, int D>
 cast_status launch_cc(cast_ctx* c, AttnParams& p, cudaStream_t s) {
-  const int nrowblk = (p.Ncap * p.G + kRB - 1) / kRB;
-  const int nsplit = cc_splits(c, p.B, p.Hkv, p.G, p.page_size, p.seq_capacity);
-  p.nsplit = nsplit;
-  const size_t rows = (size_t)p.B * p.Hq * p.Ncap * nsplit;
+  const CcPlan pl = cc_plan(c, p.B, p.Hq, p.Hkv, D, p.page_size, p.seq_capacity);
   // compute calls never allocate: the workspace comes from cast_reserve_attention
-  if (rows * (D + 2) * sizeof(float) > c->attn_ws_bytes) return CAST_ERR_CAPACITY;
-  p.part_o = reinterpret_cast<float*>(c->attn_ws);
-  p.part_ml = p.part_o + rows * D;
-  const size_t smem = (size_t)(kRB * (D + 4) + kPT * (D + 4) + kPT * D + kRB * (kPT + 1)) * sizeof(float);
-  CAST_CUDA_OK(cudaFuncSetAttribute(tree_attn_cc_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  tree_attn_cc_kernel<T, D><<<dim3(nsplit * nrowblk, p.Hkv, p.B), kThreads, smem, s>>>(p);
-  attn_combine_kernel<T, D><<<dim3(p.Ncap, p.Hq, p.B), D, 0, s>>>(p);
-  return launch_status();
+  if (pl.bytes > c->attn_ws_bytes) return CAST_ERR_CAPACITY;
+  p.nsplit = pl.nsplit;
+  p.nrowblk = pl.nrowblk;
+  if (pl.nsplit > 1) {
+    p.ticket = reinterpret_cast<int32_t*>(c->attn_ws);
+    p.part_o = reinterpret_cast<float*>(reinterpret_cast<char*>(c->attn_ws) + kCcTicketBytes);
+    p.part_ml = p.part_o + (size_t)p.B * p.Hkv * pl.nrowblk * pl.nsplit * kRB * D;
+  }
+  const size_t smem = (size_t)(kRB * (D + 4) + kPT * (D + 4) + kPT * D + kRB * (kPT + 4)) * sizeof(float);
+  auto kern = tree_attn_cc_kernel<T, D>;
+  CAST_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(pl.nsplit * pl.nrowblk, p.Hkv, p.B);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // launched while its predecessor drains; waits for it
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
+  if (e == cudaSuccess && pl.nsplit > kMergeHere) {
+    cfg.gridDim = dim3(pl.nrowblk * (kRB / (kThreads / 32)), p.Hkv, p.B);
+    cfg.dynamicSmemBytes = 0;
+    e = cudaLaunchKernelEx(&cfg, attn_merge_kernel<T, D>, p);
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return CAST_ERR_CUDA;
+  }
+  return CAST_OK;
 }
 
 }  // namespace
@@ -354,13 +485,15 @@ extern "C" cast_status cast_reserve_attention(cast_ctx* c, cast_dtype dtype, int
     const cast_status st = tree_attention_tc_reserve(c, tree_attention_tc_workspace(c, B, Hq, Hkv, D, page_size, seq_capacity));
     if (st != CAST_OK) return st;
   }
-  const size_t need = cc_workspace(c, B, Hq, Hkv, D, page_size, seq_capacity);
+  const size_t need = cc_plan(c, B, Hq, Hkv, D, page_size, seq_capacity).bytes;
   if (need > c->attn_ws_bytes) {
     CAST_CUDA_OK(cudaDeviceSynchronize());
     if (c->attn_ws) cudaFree(c->attn_ws);
     c->attn_ws = nullptr;
     c->attn_ws_bytes = 0;
     CAST_CUDA_OK(cudaMalloc(&c->attn_ws, need));
+    // tickets start at zero; every merge leaves its ticket at zero again
+    CAST_CUDA_OK(cudaMemset(c->attn_ws, 0, kCcTicketBytes));
     c->attn_ws_bytes = need;
   }
   return CAST_OK;
@@ -394,9 +527,8 @@ extern "C" cast_status cast_tree_attention_rows(cast_ctx* c, const void* q, cons
   p.q = q; p.k = k_cache; p.v = v_cache; p.out = out;
   p.B = B; p.Ncap = c->cfg.max_tree; p.Hq = Hq; p.Hkv = Hkv; p.G = Hq / Hkv;
   p.page_size = page_size; p.seq_capacity = seq_capacity; p.num_pages = num_pages; p.words = c->words;
-  p.nsplit = 1;
   p.page_table = page_table; p.kv_len = kv_len; p.n_tree = n_tree; p.first_row = first_row; p.anc = anc_mask;
-  p.scale = scale; p.part_o = nullptr; p.part_ml = nullptr; p.st = c->state;
+  p.scale = scale; p.ticket = nullptr; p.part_o = nullptr; p.part_ml = nullptr; p.st = c->state;
   if (dtype == CAST_F32) return D == 64 ? launch_cc<float, 64>(c, p, s) : launch_cc<float, 128>(c, p, s);
   return D == 64 ? launch_cc<__nv_bfloat16, 64>(c, p, s) : launch_cc<__nv_bfloat16, 128>(c, p, s);
 }

@@ -216,3 +216,18 @@ def test_tree_layer_at_the_edges_of_the_sweep(binding, logits, V, kind):
     want = oracle_tree(kw, None, root, kv, layers)
     ctx = binding.CastContext(max_batch=B, **kw)
     assert_tree_equal(gpu_tree(ctx, root.cuda(), kv.cuda(), [x.cuda() for x in layers]), want)
+
+
+@pytest.mark.parametrize("dtype,D,page", [(torch.float32, 64, 16), (torch.float32, 128, 0), (torch.bfloat16, 128, 128)])
+@pytest.mark.parametrize("B,cap,Hq,Hkv,kv", [(1, 1, 1, 1, [0]), (1, 32, 4, 1, [6000]), (2, 33, 6, 2, [1000, 3]), (3, 9, 8, 8, [64, 63, 500]),
+                                             (64, 5, 8, 8, [(i * 29) % 300 for i in range(64)])])
+def test_cuda_core_attention_merges(binding, dtype, D, page, B, cap, Hq, Hkv, kv):
+    """One split, up to sixteen (merged by the last CTA), more (a kernel of its own), splits without tiles; windows."""
+    rng = np.random.default_rng(B * 100 + cap)
+    n_tree = [int(rng.integers(max(1, cap // 2), cap + 1)) for _ in range(B)]
+    for first in (None, [n // 2 for n in n_tree]):
+        got, want = _attend(binding, rng, B, cap, n_tree, Hq, Hkv, D, page, kv, dtype=dtype, first=first)
+        keep = ~want.isnan()
+        assert torch.equal(got.isnan(), ~keep)
+        tol = 1e-5 if dtype == torch.float32 else 1e-5 + want[keep].abs() * 2.0 ** -8
+        assert bool(((got.double() - want)[keep].abs() <= tol).all())
