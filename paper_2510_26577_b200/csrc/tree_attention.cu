@@ -415,12 +415,21 @@ CcPlan cc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, 
   CcPlan pl;
   pl.nrowblk = (c->cfg.total_token * (Hq / Hkv) + kRB - 1) / kRB;
   const int base = B * Hkv * pl.nrowblk;
-  int nsplit = (2 * c->num_sms + base - 1) / base;
   const int max_pos = page_size == 0 ? seq_capacity : seq_capacity * page_size;
   const int max_tiles = (max_pos + kPT - 1) / kPT;
-  if (nsplit > max_tiles) nsplit = max_tiles;
-  if (nsplit > kMaxSplit) nsplit = kMaxSplit;
-  if (nsplit < 1 || (size_t)base * sizeof(int32_t) > kCcTicketBytes) nsplit = 1;
+  // The count for which rounds of resident CTAs (three per SM at D = 64, two at 128) x tiles per CTA is smallest, a CTA's
+  // prologue and partial counted as two tiles: 512 CTAs on 444 places would run as two rounds.
+  const int slots = (D == 64 ? 3 : 2) * c->num_sms;
+  int nsplit = 1;
+  long long best = -1;
+  for (int n = 1; n <= kMaxSplit && n <= max_tiles; ++n) {
+    const long long cost = (long long)(((long long)base * n + slots - 1) / slots) * ((max_tiles + n - 1) / n + 2);
+    if (best < 0 || cost < best) {
+      best = cost;
+      nsplit = n;
+    }
+  }
+  if ((size_t)base * sizeof(int32_t) > kCcTicketBytes) nsplit = 1;
   pl.nsplit = nsplit;
   pl.bytes = nsplit == 1 ? 0 : kCcTicketBytes + (size_t)base * nsplit * kRB * (D + 2) * sizeof(float);
   return pl;
