@@ -189,13 +189,13 @@ __device__ __forceinline__ bool take_ticket(int32_t* counter, int expected, int*
 
 // Layer tail (Eq. 1, Eq. 2, Algorithm 1, depth pruning) in two parts. tail_rank orders the candidates of
 // some sequences and is what costs time with many sequences; tail_decide is the batch-wide rest. With up to
-// four sequences the last CTA of the layer runs both from shared memory; with more, the last CTA of every
+// four sequences (eight, of few candidates) the last CTA of the layer runs both from shared memory; with more, the last CTA of every
 // sequence ranks that sequence (so the sequences are ranked in parallel) and leaves the first n sorted
 // nodes in global memory, and the last of those CTAs decides.
 
 constexpr int kTailScratch = 28672;  // bytes of shared memory the tail works in
-// Up to this many sequences the one-CTA tail is faster than a second ticket.
-constexpr int kTailSingleMaxB = 4;
+// Up to this many sequences, or candidates, the one-CTA tail is faster than a second ticket (V = 32000, 8 sequences: 92 -> 89 us).
+constexpr int kTailSingleMaxB = 8, kTailAlwaysSingleB = 4, kTailSingleCands = 512;
 
 // a / b for 0 <= a < 2^20 and 1 <= b <= 2^10 through the fp32 reciprocal (inv_b, to a few ulp) with one correction step:
 // the integer division by a run-time divisor is some twenty instructions, and the ranking below does several per
@@ -397,6 +397,21 @@ __device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailSta
       p.lscore[o] = 0.0;
     }
   }
+  const float inv_W = __fdividef(1.f, (float)W), inv_K = __fdividef(1.f, (float)K);
+  // the nodes that may be retained, requested together with their values
+  constexpr int kOut = CAST_MAX_BATCH * CAST_MAX_WIDTH / kSweepThreads;
+  int idx_k[kOut], tok_k[kOut];
+  if (GLOBAL) {
+#pragma unroll
+    for (int k = 0; k < kOut; ++k) {
+      const int i = tid + k * nt, b = div_small(i, W, inv_W), s = i - b * W;
+      idx_k[k] = tok_k[k] = 0;
+      if (i < B * W && s < n) {
+        idx_k[k] = __ldcg(sorted_i + b * CAST_MAX_WIDTH + s);
+        tok_k[k] = __ldcg(stok_i + b * CAST_MAX_WIDTH + s);
+      }
+    }
+  }
   // Eq. 1: batch mean of the rank-wise values
   if (GLOBAL) {
     // many sequences: a warp per rank sums over the sequences, two per lane, then a fixed shuffle tree
@@ -502,14 +517,15 @@ __device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailSta
   }
   __syncthreads();
   const int n_i = s_ni;
-  const float inv_W = __fdividef(1.f, (float)W), inv_K = __fdividef(1.f, (float)K);
-#pragma unroll 1
-  for (int i = tid; i < B * W; i += nt) {
+#pragma unroll
+  for (int k = 0; k < kOut; ++k) {
+    const int i = tid + k * nt;
+    if (i >= B * W) break;
     const int b = div_small(i, W, inv_W), s = i - b * W;
     int tok = -1, prow = -1;
     if (s < n_i) {
-      const int idx = GLOBAL ? __ldcg(sorted_i + b * CAST_MAX_WIDTH + s) : sorted_i[b * CAST_MAX_WIDTH + s];
-      tok = GLOBAL ? __ldcg(stok_i + b * CAST_MAX_WIDTH + s) : stok_i[b * CAST_MAX_WIDTH + s];
+      const int idx = GLOBAL ? idx_k[k] : sorted_i[b * CAST_MAX_WIDTH + s];
+      tok = GLOBAL ? tok_k[k] : stok_i[b * CAST_MAX_WIDTH + s];
       prow = div_small(idx - base, K, inv_K);
       p.retained[b * W + s] = idx;
       p.pool_kept[(size_t)b * P + idx] = 1;
@@ -1030,7 +1046,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
   // ---- layer tail
   __syncthreads();
   const int n_tail = tail_width(p, n_prev);
-  if (B <= kTailSingleMaxB) {  // the last CTA of the layer ranks and decides, everything in shared memory
+  if (B <= kTailAlwaysSingleB || (B <= kTailSingleMaxB && B * n_prev * K <= kTailSingleCands)) {  // the last CTA of the layer ranks and decides, everything in shared memory
     if (!take_ticket(p.layer_ticket, B * n_prev, &s_flag)) return;
     double* vs = reinterpret_cast<double*>(scratch + 20480);  // [B][CAST_MAX_WIDTH] sorted values
     int* stok = reinterpret_cast<int*>(scratch + 24576);      // [B][CAST_MAX_WIDTH] tokens of the sorted nodes
