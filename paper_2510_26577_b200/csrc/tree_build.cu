@@ -554,7 +554,10 @@ constexpr int kPushCap = 32;    // keys a warp hands on at most
 static_assert(CAST_MAX_TOP_K <= kGroups, "the K-th largest of the groups' maxima needs K <= groups");
 static_assert(CAST_MAX_TOP_K <= kPushCap, "a warp hands on its K best");
 
-template <typename T, int NT>
+// OUT: the overflow handling is a function of its own. Inlined twice it is half of the sweep's code, and in the short launches,
+// which run everything once, the warps wait for instructions (1-2 us per tree); in the 64-register launches the call costs
+// more registers than there are (batch 64 307 -> 329 us).
+template <typename T, int NT, bool OUT>
 struct Sweep {
   static constexpr int VEC = Vec<T>::N;
   static constexpr int kSlots = kBufVecs * VEC;                      // logits of a thread per buffer
@@ -564,13 +567,14 @@ struct Sweep {
   // First element (of the aligned view) of this thread's vector v in the buffer that starts at `base`.
   static __device__ __forceinline__ int elem(int base, int v) { return base + (v * NT + (int)threadIdx.x) * VEC; }
 
-  // xa: the row from the 16-byte boundary at or below its start; elements [lo, end) of it exist.
-  __device__ __forceinline__ void load(const T* xa, int base, int lo, int end) {
-    if (base >= lo && base + kBufElems <= end) {  // a full buffer: no per-vector checks
+  // A whole buffer; `at`: this thread's first vector of it. (One address per buffer, the rest are immediate offsets.)
+  __device__ __forceinline__ void load(const uint4* at) {
 #pragma unroll
-      for (int v = 0; v < kBufVecs; ++v) raw[v] = __ldcs(reinterpret_cast<const uint4*>(xa + elem(base, v)));
-      return;
-    }
+    for (int v = 0; v < kBufVecs; ++v) raw[v] = __ldcs(at + v * NT);
+  }
+  // A buffer that is not all there. xa: the row from the 16-byte boundary at or below its start; elements [lo, end) of it
+  // exist.
+  __device__ __forceinline__ void load_part(const T* xa, int base, int lo, int end) {
 #pragma unroll
     for (int v = 0; v < kBufVecs; ++v) {
       const int idx = elem(base, v);
@@ -669,7 +673,21 @@ struct Sweep {
     }
     __syncwarp();
     const int n = *count;
-    if (n <= kListCap - 16) return;
+    if (n > kListCap - 16) {
+      uint4 copy[kBufVecs];
+#pragma unroll
+      for (int v = 0; v < kBufVecs; ++v) copy[v] = raw[v];
+      thr = OUT ? overflow_call(copy, thr, base, shift, K, list, count, have0, n) : overflow(copy, thr, base, shift, K, list, count, have0, n);
+    }
+  }
+  static __device__ __noinline__ float overflow_call(const uint4 (&buf)[kBufVecs], float thr, int base, int shift, int K,
+                                                     unsigned long long* list, int* count, int have0, int n) {
+    return overflow(buf, thr, base, shift, K, list, count, have0, n);
+  }
+  // The list has run over, or will soon: its K best stay, in order; returns the threshold (the K-th, once there are K).
+  static __device__ __forceinline__ float overflow(const uint4 (&buf)[kBufVecs], float thr, int base, int shift, int K,
+                                                unsigned long long* list, int* count, int have0, int n) {
+    const int lane = threadIdx.x & 31;
     unsigned long long mine = 0ull;
     int kept = 0;
     if (n > kListCap) {
@@ -681,7 +699,7 @@ struct Sweep {
 #pragma unroll
         for (int v = 0; v < kBufVecs; ++v) {
           float x[VEC];
-          Vec<T>::unpack(raw[v], x);
+          Vec<T>::unpack(buf[v], x);
           const int id = elem(base, v) - shift;
 #pragma unroll
           for (int e = 0; e < VEC; ++e)
@@ -711,6 +729,7 @@ struct Sweep {
     if (lane == 0) *count = kept;
     if (kept == K) thr = fmaxf(thr, key_value(__shfl_sync(0xffffffffu, mine, K - 1)));
     __syncwarp();
+    return thr;
   }
   // The min(n, K) largest of the list's n <= 64 keys, in order, one per lane.
   static __device__ __forceinline__ int keep_best(unsigned long long* list, int n, int K, unsigned long long& mine) {
@@ -733,28 +752,28 @@ struct Sweep {
   }
 };
 
-// The K-th largest of the groups' maxima in shared memory, at least -FLT_MAX (every warp for itself).
-__device__ __forceinline__ float kth_of_groups(const float* v, int K) {
-  const int lane = threadIdx.x & 31;
-  const float mine = v[lane & (kGroups - 1)];
-  int r = 0;
-#pragma unroll
-  for (int j = 0; j < kGroups; ++j) {
-    const float o = v[j];
-    r += (o > mine) || (o == mine && j < lane);  // equal values in lane order: ranks 0..15 are distinct
-  }
-  const unsigned who = __ballot_sync(0xffffffffu, lane < kGroups && r == K - 1);
-  return fmaxf(__shfl_sync(0xffffffffu, mine, who != 0u ? __ffs(who) - 1 : 0), -3.402823466e38f);
-}
-// A thread's share in the groups' maxima; returns the maximum of its group.
+// A thread's share in the groups' maxima, which go to shared memory as integers: the value's ordered bits, the last four
+// replaced by the group's number, so that they are distinct and one comparison orders two of them.
 template <int NT>
-__device__ __forceinline__ float group_max(float x, float* v) {
+__device__ __forceinline__ void group_max(float x, uint32_t* v) {
   constexpr int kLanes = NT / kGroups;
   static_assert(kLanes == 32 || kLanes == 16, "groups are warps or half warps");
 #pragma unroll
   for (int o = kLanes / 2; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-  if ((threadIdx.x & (kLanes - 1)) == 0) v[threadIdx.x / kLanes] = x;
-  return x;
+  if ((threadIdx.x & (kLanes - 1)) == 0) v[threadIdx.x / kLanes] = (ordered_bits(x) & ~15u) | (threadIdx.x / kLanes);
+}
+// The K-th largest of the groups' maxima, rounded down in its last bits: still a lower bound on the K-th largest of the
+// logits. At least -FLT_MAX. (Every warp for itself.)
+__device__ __forceinline__ float kth_of_groups(const uint32_t* v, int K) {
+  const uint32_t mine = v[threadIdx.x & (kGroups - 1)];
+  int r = 0;
+#pragma unroll
+  for (int j = 0; j < kGroups; j += 4) {
+    const uint4 o = *reinterpret_cast<const uint4*>(v + j);
+    r += (o.x > mine) + (o.y > mine) + (o.z > mine) + (o.w > mine);
+  }
+  const unsigned who = __ballot_sync(0xffffffffu, r == K - 1);
+  return fmaxf(from_ordered_bits(__shfl_sync(0xffffffffu, mine, __ffs(who) - 1) & ~15u), -3.402823466e38f);
 }
 __device__ __forceinline__ float warp_max(float x) {
 #pragma unroll
@@ -779,10 +798,12 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
   __shared__ __align__(16) unsigned long long wlist[kWarps * kListCap];
   __shared__ unsigned long long topk[CAST_MAX_TOP_K];
   __shared__ int wcount[kWarps];
-  __shared__ float gmax[2][kGroups];
+  __shared__ __align__(16) uint32_t gmax[2][kGroups];
   __shared__ int sorted[kTailSingleMaxB * CAST_MAX_WIDTH];  // small batches: pool indices of the first sorted candidates
   __shared__ int s_flag, push_n;
-  __shared__ double s_lse;
+  __shared__ double s_lse, s_parent_score;
+  __shared__ TailState s_ts;
+  __shared__ int s_base, s_n_prev, s_parent;
   unsigned long long* row_keys = reinterpret_cast<unsigned long long*>(scratch);
 
   const int chunk = blockIdx.x, r = blockIdx.y, b = blockIdx.z, B = gridDim.z;
@@ -790,7 +811,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
   DevState* st = p.st;
   const int K = p.K;
   const int row = b * p.W + r;
-  using S = Sweep<T, NT>;
+  using S = Sweep<T, NT, MINB == 1>;
   constexpr int E = S::kBufElems;
   // the row from the 16-byte boundary at or below its start: its tokens are elements [shift, V + shift) of that view
   const T* x = reinterpret_cast<const T*>(p.logits) + (size_t)row * p.V;
@@ -820,64 +841,76 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
   grid_launch_dependents();  // the next grid may now take the SMs this one leaves idle
   // the first logits are requested before the state is read (every row r < W exists in memory): one memory round trip
   S q0, q1;
-  q0.load(xa, begin, shift, end);
-  q1.load(xa, begin + E, shift, end);
-  // what the layer tail needs of the state is read now, together with the row count: one round trip.
-  // (Layer 1 starts the step: one row per sequence, the root at pool index 0 with value 1.)
-  int n_prev = 1, base = 1;
-  TailState ts;
-  ts.ctx_sum = 0;
-  ts.n0 = 0;  // layer 1: the deciding CTA works it out from kv_len
-  ts.kept_total = 1;
-  ts.u_last = 1.0;
-  if (p.layer > 1) {
-    n_prev = st->rows[p.layer];
-    ts.ctx_sum = st->ctx_sum;
-    ts.n0 = st->n0;
-    ts.kept_total = st->kept_total;
-    ts.u_last = st->u_last;
-    base = st->pool_size;
+  const uint4* at_mine = reinterpret_cast<const uint4*>(xa + begin) + tid;  // this thread's place in buffer `at`
+  constexpr int kStep = kBufVecs * NT;                                       // vectors per buffer
+  if (begin >= shift && begin + 2 * E <= end) {
+    q0.load(at_mine);
+    q1.load(at_mine + kStep);
+  } else {
+    q0.load_part(xa, begin, shift, end);
+    q1.load_part(xa, begin + E, shift, end);
   }
-  if (n_prev == 0) {
-    if (chunk == 0 && r == 0 && b == 0 && tid == 0) *p.next_count = 0;
-    return;
-  }
-  if (r >= n_prev) return;
-  // the parent of this row's children and its log-value (only the row's first CTA uses them: fetched now,
-  // off the critical path)
-  int parent = 0;
-  double parent_score = 0.0;
-  if (p.layer > 1) {
-    parent = p.retained[b * p.W + r];
-    parent_score = p.pool_score[(size_t)b * p.P + parent];
+  // what the layer tail needs of the state is read now, together with the row count: one round trip; it waits in shared
+  // memory, out of the sweep's registers. (Layer 1 starts the step: one row per sequence, the root at pool index 0 with
+  // value 1.)
+  {
+    int n_prev = 1;
+    if (p.layer > 1) n_prev = st->rows[p.layer];
+    if (tid == 0) {
+      s_ts.ctx_sum = 0;
+      s_ts.n0 = 0;  // layer 1: the deciding CTA works it out from kv_len
+      s_ts.kept_total = 1;
+      s_ts.u_last = 1.0;
+      s_base = 1;
+      if (p.layer > 1) {
+        s_ts.ctx_sum = st->ctx_sum;
+        s_ts.n0 = st->n0;
+        s_ts.kept_total = st->kept_total;
+        s_ts.u_last = st->u_last;
+        s_base = st->pool_size;
+      }
+      s_n_prev = n_prev;
+    }
+    if (n_prev == 0) {
+      if (chunk == 0 && r == 0 && b == 0 && tid == 0) *p.next_count = 0;
+      return;
+    }
+    if (r >= n_prev) return;
+    // the parent of this row's children and its log-value
+    if (tid == 32 && chunk == 0) {
+      const int parent = p.layer > 1 ? p.retained[b * p.W + r] : 0;
+      s_parent = parent;
+      s_parent_score = p.layer > 1 ? p.pool_score[(size_t)b * p.P + parent] : 0.0;
+    }
   }
 
   // ---- sweep
   unsigned long long* list = wlist + warp * kListCap;
   float m_run = -INFINITY, M2 = -INFINITY, s_run = 0.f, thr = 0.f;
-  auto work = [&](S& q, float m, int at) {
+  auto work = [&](S& q, float m, int at, const uint4* mine) {
     q.extract(m, thr, at, shift, K, list, &wcount[warp]);
-    if (at + 2 * E < end) q.load(xa, at + 2 * E, shift, end);
+    if (at + 3 * E <= end) q.load(mine + 2 * kStep);
+    else if (at + 2 * E < end) q.load_part(xa, at + 2 * E, shift, end);
   };
-  auto threshold = [&](float m, float* g) {
+  auto threshold = [&](float m, uint32_t* g) {
     group_max<NT>(m, g);
     __syncthreads();
     return kth_of_groups(g, K);
   };
 #pragma unroll 1
-  for (int at = begin; at < end; at += 2 * E) {  // (two copies of the work: a buffer that is moved is waited for)
+  for (int at = begin; at < end; at += 2 * E, at_mine += 2 * kStep) {  // (two copies of the work: a buffer that is moved is waited for)
     const float m0 = q0.max();
     m_run = fmaxf(m_run, m0);
     q0.sum(m0, M2, s_run);
     // the threshold from the first two buffers, and once more when four of seven buffers or more are done
     if (at == begin) thr = threshold(fmaxf(m0, q1.max()), gmax[0]);
     else if (at == begin + 4 * E && end - at > 2 * E) thr = fmaxf(thr, threshold(m_run, gmax[1]));
-    work(q0, m0, at);
+    work(q0, m0, at, at_mine);
     if (at + E >= end) break;
     const float m1 = q1.max();
     m_run = fmaxf(m_run, m1);
     q1.sum(m1, M2, s_run);
-    work(q1, m1, at + E);
+    work(q1, m1, at + E, at_mine + kStep);
   }
 
   // ---- chunk result: what is left of the warps' lists above the threshold, and every warp's maximum and sum, straight
@@ -1026,6 +1059,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
       if (-rank_s[i] < K) topk[-rank_s[i]] = wlist[i];
     __syncthreads();
   }
+  const int base = s_base;
   if (tid < K) {  // the K children join the pool
     const unsigned long long key = topk[tid];
     const float val = key_value(key);
@@ -1036,16 +1070,17 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
     }
     const size_t o = (size_t)b * p.P;
     const int idx = base + r * K + tid;
-    p.pool_score[o + idx] = parent_score + ((double)val - s_lse);
+    p.pool_score[o + idx] = s_parent_score + ((double)val - s_lse);
     p.pool_token[o + idx] = tok;
-    p.pool_parent[o + idx] = parent;
+    p.pool_parent[o + idx] = s_parent;
     p.pool_depth[o + idx] = p.layer;
     p.pool_kept[o + idx] = 0;
   }
 
   // ---- layer tail
   __syncthreads();
-  const int n_tail = tail_width(p, n_prev);
+  const int n_prev = s_n_prev, n_tail = tail_width(p, n_prev);
+  const TailState ts = s_ts;
   if (B <= kTailAlwaysSingleB || (B <= kTailSingleMaxB && B * n_prev * K <= kTailSingleCands)) {  // the last CTA of the layer ranks and decides, everything in shared memory
     if (!take_ticket(p.layer_ticket, B * n_prev, &s_flag)) return;
     double* vs = reinterpret_cast<double*>(scratch + 20480);  // [B][CAST_MAX_WIDTH] sorted values
