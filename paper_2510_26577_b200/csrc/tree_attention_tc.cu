@@ -67,6 +67,7 @@ struct Geo {
   static constexpr int kSmemV = kSmemK + kStagesK * kTileKV;    // kStagesV tiles
   static constexpr int kSmemBar = kSmemV + kStagesV * kTileKV;  // mbarriers and two words
   static constexpr int kBars = 2 * kStagesK + 2 * kStagesV + 5;
+  static constexpr int kSmemTmem = kSmemBar + kBars * 8; // the TMEM address, then the ticket's verdict
   static constexpr int kSmemBytes = kSmemBar + 256;      // 112 KB at 128 dims: two CTAs per SM
   static constexpr int kStageStride = HD + 4;            // floats per staged output row: 16-byte accesses stay conflict-free
   static_assert(kBM * kStageStride * 4 <= (kStagesK + kStagesV) * kTileKV, "staged rows fit in the rings");
@@ -744,6 +745,23 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_v)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_q)) : "memory");
   }
+  // TMEM (two S buffers and O) before anything else: an SM starts its second CTA only after the first one has given up
+  // the right to allocate. Behind the dependency wait and the work decode, where this stood before, the second CTAs came
+  // 2.4-3.7 us after the first and a third round of clusters 5 us after (draft rows of 4 sequences of 512: 14.2 -> 11.4 us).
+  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + GE::kSmemTmem);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_s)),
+                 "n"(kTmemCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  // an early exit returns it
+  auto tmem_return = [&] {
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_base_s), "n"(kTmemCols));
+  };
   // Programmatic dependent launch: this grid may become resident while the previous kernel of the
   // stream drains; nothing written by earlier kernels is read before this point. (No-ops for a plain launch.)
   // In the default mode nothing is read before the wait. In "early" mode (a promise of the caller, see
@@ -762,7 +780,10 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
                       : cs == 0            ? decode_work_chunked(p, (int)blockIdx.x, (int)gridDim.x)
                                            : decode_work(p, (int)blockIdx.x / cs, crank);
   if (blockIdx.x < p.B && tid == 0 && p.n_tree[blockIdx.x] > p.Nmax) report(p.st, CAST_ERR_BAD_TREE, blockIdx.x);
-  if (!wk.valid) return;  // the whole cluster leaves (a CTA that exits counts as having released its dependents)
+  if (!wk.valid) {
+    tmem_return();
+    return;  // the whole cluster leaves (a CTA that exits counts as having released its dependents)
+  }
   const int b = wk.b, kvh = wk.kvh, rb = wk.rb, split = wk.split, N = wk.N, L = wk.L;
   const int nsplit = wk.nsplit;
   const int G = p.G, F = wk.F, rows_total = (N - F) * G, row0 = rb * kBM;
@@ -785,6 +806,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
       stage_ml[tid * 2] = -INFINITY;
       stage_ml[tid * 2 + 1] = 0.f;
     }
+    tmem_return();
     if (cs > 1) {
       cluster_sync_all();
       cluster_sync_all();
@@ -805,8 +827,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   uint64_t* bar_s = bar_freev + kStagesV;                                  // [2]
   uint64_t* bar_p = bar_s + 2;                                             // [2]: tile it uses bar_p[it & 1], phase it >> 1
   uint64_t* bar_q = bar_p + 2;                                             // the Q row block has landed (TMA)
-  uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(bar_q + 1);
-  int* last_s = reinterpret_cast<int*>(bar_q + 1) + 1;
+  int* last_s = reinterpret_cast<int*>(tmem_base_s) + 1;
 
   // ---- producer helper (warp 4; all 32 lanes call it): which = 0: K tile j, which = 1: V tile j
   // Paged caches: a producer warp reads the page table 32 entries at a time (one coalesced load, lane l keeps
@@ -919,11 +940,6 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     // the first K tiles need no stage wait: the ring fills while Q is on its way
     for (; k_issued < kStagesK && k_issued < ntile; ++k_issued) issue_tile(k_issued, 0);
   } else if (warp < 4) {
-    if (warp == 0) {  // TMEM: two S buffers and O
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_s)),
-                   "n"(kTmemCols));
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
     // ancestor mask -> registers; without TMA for Q: the Q row -> swizzled shared memory (rows past the tree zero)
     if (row_ok) {
 #pragma unroll
