@@ -402,9 +402,11 @@ __device__ __forceinline__ WorkItem decode_work(const TcParams& p, int cid, int 
 
 // ---- cluster primitives
 __device__ __forceinline__ uint32_t cluster_ctarank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 __device__ __forceinline__ uint32_t map_to_rank(uint32_t saddr, uint32_t rank) {
   uint32_t r;
@@ -457,62 +459,90 @@ __device__ __forceinline__ uint2 ld_cluster_u2(uint32_t addr) {
   return v;
 }
 
+// a / b for 0 <= a < 2^22, inv_b = 1 / b: an integer division by a run-time divisor is a chain of well over 100 cycles
+__device__ __forceinline__ int div_small(int a, int b, float inv_b) {
+  int q = (int)((float)a * inv_b);
+  const int r = a - q * b;
+  return q + (r >= b ? 1 : 0) - (r < 0 ? 1 : 0);
+}
+
+// The merge of a row's splits: split s weighs sum_s * e^(max_s - max). A warp merges ROWS rows of at most SPL splits at a
+// time; lane u * SPL + s holds row u's split s, so one load and two short butterflies give the weights of all the rows
+// (a butterfly over the whole warp for each row, and a branch on each weight, made the merge of two rows a chain of
+// 2.8 us in a launch of 13: 128 CTAs, 8 splits; now 1.3). Returns the weight over the row's sum of weights.
+template <int SPL>
+__device__ __forceinline__ float split_weight(float mx, float sum) {
+  float M = mx;
+#pragma unroll
+  for (int o = SPL / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+  const float w = mx > -INFINITY ? sum * expf(mx - M) : 0.f;
+  float tot = w;
+#pragma unroll
+  for (int o = SPL / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  return tot > 0.f ? w * (1.f / tot) : 0.f;
+}
+template <int HD, int SPL>
+__device__ __forceinline__ void add_splits(float (&acc)[Part<HD>::NC], const uint2 (&v)[SPL], float wgt, int u) {
+#pragma unroll
+  for (int s2 = 0; s2 < SPL; ++s2) {
+    const float w = __shfl_sync(0xffffffffu, wgt, u * SPL + s2);
+    // a split without visible positions staged nothing: its buffer may hold anything
+    Part<HD>::add(acc, w > 0.f ? v[s2] : make_uint2(0u, 0u), w);
+  }
+}
+
 // Merge of the splits of a row block through distributed shared memory. Every CTA of the split
 // group has staged its partial output rows, normalised by their own sum and rounded to half precision
 // (the merge moves half the bytes that way; the rounding, 2^-11 relative, is a quarter of the bf16
 // output's), and (max, sum) per row in its own shared memory. This CTA owns the rows rr with
-// rr % nsplit == split and reads them from all peers: split s weighs sum_s * e^(max_s - max).
-// Warp w takes owned rows w, w+8, ...; a lane owns 4 output columns; ROWS x SPL loads in flight.
+// rr % nsplit == split and reads them from all peers.
+// Warp w takes owned rows w, w+8, ...; a lane owns 8 bytes of a row; ROWS x SPL loads in flight. A warp arrives at the
+// cluster's last barrier with its last loads, not after its stores: the arrival would wait for them (0.9 us).
 template <int HD, int ROWS, int SPL>
 __device__ __forceinline__ void merge_rows(const TcParams& p, uint32_t stage_o_s, uint32_t stage_ml_s, int rank0,
                                            int b, int kvh, int row0, int rows_here, int nsplit, int split) {
   const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5, G = p.G;
-  const int owned = rows_here > split ? (rows_here - split + nsplit - 1) / nsplit : 0;
+  const float inv_G = 1.f / (float)G;
+  const int owned = rows_here > split ? div_small(rows_here - split + nsplit - 1, nsplit, 1.f / (float)nsplit) : 0;
+  const int mu = lane / SPL, msp = lane % SPL;  // whose (max, sum) this lane reads
+  bool arrived = false;
   for (int i0 = wv; i0 < owned; i0 += 8 * ROWS) {
     uint2 v[ROWS][SPL];
-    float wgt[ROWS], inv[ROWS];
-    size_t orow[ROWS];
+    float mx = -INFINITY, sum = 0.f;
+    if (mu < ROWS && msp < nsplit) {
+      const int im = i0 + 8 * mu;
+      const float2 ml = ld_cluster_f2(map_to_rank(stage_ml_s + (uint32_t)(split + nsplit * (im < owned ? im : i0)) * 8u,
+                                                  (uint32_t)(rank0 + msp)));
+      mx = ml.x;
+      sum = ml.y;
+    }
 #pragma unroll
-    for (int u = 0; u < ROWS; ++u) {
-      const int i2 = i0 + 8 * u;
-      const int rr = split + nsplit * (i2 < owned ? i2 : i0);
-      const int grow = row0 + rr, tt = grow / G, hh = kvh * G + grow % G;
-      orow[u] = (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD;
-      float ms = -INFINITY, ls = 0.f;  // lane s holds split s's (max, sum)
-      if (lane < nsplit) {
-        const float2 ml = ld_cluster_f2(map_to_rank(stage_ml_s + (uint32_t)rr * 8u, (uint32_t)(rank0 + lane)));
-        ms = ml.x;
-        ls = ml.y;
+    for (int s2 = 0; s2 < SPL; ++s2) {
+      const uint32_t base = map_to_rank(stage_o_s + (uint32_t)(lane * 8), (uint32_t)(rank0 + (s2 < nsplit ? s2 : 0)));
+#pragma unroll
+      for (int u = 0; u < ROWS; ++u) {
+        const int i2 = i0 + 8 * u;
+        const int rr = split + nsplit * (i2 < owned ? i2 : i0);
+        v[u][s2] = s2 < nsplit ? ld_cluster_u2(base + (uint32_t)(rr * kStageStrideP)) : make_uint2(0u, 0u);
       }
-#pragma unroll
-      for (int s2 = 0; s2 < SPL; ++s2)
-        v[u][s2] = s2 < nsplit ? ld_cluster_u2(map_to_rank(stage_o_s + (uint32_t)(rr * kStageStrideP + lane * 8),
-                                                           (uint32_t)(rank0 + s2)))
-                               : make_uint2(0u, 0u);
-      float M = ms;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-      wgt[u] = ms > -INFINITY ? ls * expf(ms - M) : 0.f;
-      float lsum = wgt[u];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-      inv[u] = lsum > 0.f ? 1.f / lsum : 0.f;
+    }
+    const float wgt = split_weight<SPL>(mx, sum);
+    if (i0 + 8 * ROWS >= owned) {
+      cluster_arrive();
+      arrived = true;
     }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
       float acc[Part<HD>::NC] = {};
-#pragma unroll
-      for (int s2 = 0; s2 < SPL; ++s2) {
-        const float w = __shfl_sync(0xffffffffu, wgt[u], s2);
-        if (w > 0.f) {  // a split without visible positions staged nothing: its buffer may hold anything
-          Part<HD>::add(acc, v[u][s2], w);
-        }
-      }
-      if (i0 + 8 * u < owned) {
-        Part<HD>::store(p.out + orow[u], lane, acc, inv[u]);
+      add_splits<HD, SPL>(acc, v[u], wgt, u);
+      const int i2 = i0 + 8 * u;
+      if (i2 < owned) {
+        const int grow = row0 + split + nsplit * i2, tt = div_small(grow, G, inv_G), hh = kvh * G + grow - tt * G;
+        Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, lane, acc, 1.f);
       }
     }
   }
+  if (!arrived) cluster_arrive();
 }
 
 // ---- global-merge mode -------------------------------------------------------------------------
@@ -644,59 +674,45 @@ __device__ __forceinline__ WorkItem decode_work_chunked(const TcParams& p, int i
 }
 
 // Merge of the split partials of a row block, run by all 8 warps of the last CTA to finish it.
-// Warp w takes rows w, w+8, ...; a lane owns 4 output columns. ROWS rows x SPL splits = 16 loads are
+// Warp w takes rows w, w+8, ...; a lane owns 8 bytes of a row. ROWS rows x SPL splits loads are
 // in flight per lane: the merge is bound by L2 latency, not by bytes.
 template <int HD, int ROWS, int SPL>
 __device__ __forceinline__ void merge_rows_global(const TcParams& p, int b, int kvh, int row0, int rows_here, int nsplit) {
   const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5, G = p.G;
+  const float inv_G = 1.f / (float)G;
+  const int mu = lane / SPL, msp = lane % SPL;  // whose (max, sum) this lane reads
+  auto token_head = [&](int rr, int& tt, int& hh) {
+    const int grow = row0 + rr;
+    tt = div_small(grow, G, inv_G);
+    hh = kvh * G + grow - tt * G;
+  };
   for (int rr = wv; rr < rows_here; rr += 8 * ROWS) {
     uint2 v[ROWS][SPL];
-    float wgt[ROWS], inv[ROWS], msv[ROWS], lsv[ROWS];
-    size_t orow[ROWS];
-    // every load of every row first, then the reductions (a reduction waits for its row's loads; with the next
-    // row's loads issued behind it the rows cost one round trip to L2 each, 6-7 us for eight)
+    float mx = -INFINITY, sum = 0.f;
+    int tt, hh;
+    if (mu < ROWS && msp < nsplit) {
+      token_head(rr + 8 * mu < rows_here ? rr + 8 * mu : rr, tt, hh);
+      const size_t pr = (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max + msp;
+      const float2 ml = __ldcg(reinterpret_cast<const float2*>(p.part_ml + pr * 2));
+      mx = ml.x;
+      sum = ml.y;
+    }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
-      const int r2 = rr + 8 * u;
-      const int grow = row0 + (r2 < rows_here ? r2 : rr), tt = grow / G, hh = kvh * G + grow % G;
-      const size_t pr = (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max;
-      orow[u] = (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD;
-      msv[u] = -INFINITY;  // lane s holds split s's (max, sum)
-      lsv[u] = 0.f;
-      if (lane < nsplit) {
-        const float2 ml = __ldcg(reinterpret_cast<const float2*>(p.part_ml + (pr + lane) * 2));
-        msv[u] = ml.x;
-        lsv[u] = ml.y;
-      }
+      token_head(rr + 8 * u < rows_here ? rr + 8 * u : rr, tt, hh);
+      const unsigned char* src = p.part_o + (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max * kPartRow + lane * 8;
 #pragma unroll
       for (int s2 = 0; s2 < SPL; ++s2)
-        v[u][s2] = s2 < nsplit ? __ldcg(reinterpret_cast<const uint2*>(p.part_o + (pr + s2) * kPartRow + lane * 8))
-                               : make_uint2(0u, 0u);
+        v[u][s2] = s2 < nsplit ? __ldcg(reinterpret_cast<const uint2*>(src + s2 * kPartRow)) : make_uint2(0u, 0u);
     }
-#pragma unroll
-    for (int u = 0; u < ROWS; ++u) {
-      const float ms = msv[u], ls = lsv[u];
-      float M = ms;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-      wgt[u] = ms > -INFINITY ? ls * expf(ms - M) : 0.f;  // split s weighs sum_s * e^(max_s - max)
-      float lsum = wgt[u];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-      inv[u] = lsum > 0.f ? 1.f / lsum : 0.f;
-    }
+    const float wgt = split_weight<SPL>(mx, sum);
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
       float acc[Part<HD>::NC] = {};
-#pragma unroll
-      for (int s2 = 0; s2 < SPL; ++s2) {
-        const float w = __shfl_sync(0xffffffffu, wgt[u], s2);
-        if (w > 0.f) {  // a split without visible positions wrote zeros at best
-          Part<HD>::add(acc, v[u][s2], w);
-        }
-      }
+      add_splits<HD, SPL>(acc, v[u], wgt, u);
       if (rr + 8 * u < rows_here) {
-        Part<HD>::store(p.out + orow[u], lane, acc, inv[u]);
+        token_head(rr + 8 * u, tt, hh);
+        Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, lane, acc, 1.f);
       }
     }
   }
@@ -813,7 +829,8 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     }
     return;
   }
-  const int t0 = (int)((long long)split * ntiles / nsplit), t1 = (int)((long long)(split + 1) * ntiles / nsplit);
+  // (rounded up: the last split, whose last tiles are masked and cost more, is never the one with a tile more)
+  const int t0 = (int)(((long long)split * ntiles + nsplit - 1) / nsplit), t1 = (int)(((long long)(split + 1) * ntiles + nsplit - 1) / nsplit);
   const int ntile = t1 - t0;
   const int r = tid & (kBM - 1);  // softmax role: the query row of this thread
   const int row = row0 + r;
@@ -1271,16 +1288,18 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     stage_ml[r * 2 + 1] = l_run;
   }
   tc_fence_before();
-  __syncthreads();
+  if (cs > 1) cluster_sync_all();  // every CTA of the cluster has staged its rows
+  else __syncthreads();
   if (warp == 0) {  // every TMEM access of this CTA is over
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols));
   }
-  if (cs > 1) cluster_sync_all();  // every CTA of the cluster has staged its rows
   const int rows_here = rows_total - row0 < kBM ? rows_total - row0 : kBM;
+  const float inv_G = 1.f / (float)G;
   if (nsplit == 1) {
+#pragma unroll 4
     for (int rr = warp; rr < rows_here; rr += kThreadsTC / 32) {
-      const int grow = grow0 + rr, tt = grow / G, hh = kvh * G + grow % G;
+      const int grow = grow0 + rr, tt = div_small(grow, G, inv_G), hh = kvh * G + grow - tt * G;
       constexpr int NC = Part<HD>::NC;
       float acc[NC];
 #pragma unroll
@@ -1295,14 +1314,14 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   } else if (cs == 0) {
     // global-merge mode: partials to the workspace; the last split of this row block to finish merges
     const unsigned char* sh = reinterpret_cast<const unsigned char*>(stage_o);
+#pragma unroll 4
     for (int rr = warp; rr < rows_here; rr += kThreadsTC / 32) {
-      const int grow = grow0 + rr, tt = grow / G, hh = kvh * G + grow % G;
+      const int grow = grow0 + rr, tt = div_small(grow, G, inv_G), hh = kvh * G + grow - tt * G;
       const size_t pr = (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max + split;
       __stcg(reinterpret_cast<uint2*>(p.part_o + pr * kPartRow + lane * 8),
              *reinterpret_cast<const uint2*>(sh + rr * kStageStrideP + lane * 8));
       if (lane == 0) {
-        __stcg(p.part_ml + pr * 2, stage_ml[rr * 2]);
-        __stcg(p.part_ml + pr * 2 + 1, stage_ml[rr * 2 + 1]);
+        __stcg(reinterpret_cast<float2*>(p.part_ml + pr * 2), *reinterpret_cast<const float2*>(stage_ml + rr * 2));
       }
     }
     __syncthreads();
@@ -1328,7 +1347,10 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     else if (nsplit <= 4) merge_rows<HD, 4, 4>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
     else merge_rows<HD, 2, kMaxSplit>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
   }
-  if (cs > 1) cluster_sync_all();  // nobody leaves while a peer may still read its shared memory
+  if (cs > 1) {  // nobody leaves while a peer may still read its shared memory
+    if (nsplit == 1) cluster_arrive();
+    cluster_wait();
+  }
 }
 
 
