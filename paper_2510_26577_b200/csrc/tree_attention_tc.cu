@@ -402,10 +402,9 @@ __device__ __forceinline__ WorkItem decode_work(const TcParams& p, int cid, int 
 
 // ---- cluster primitives
 __device__ __forceinline__ uint32_t cluster_ctarank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
-  cluster_arrive();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   cluster_wait();
 }
 __device__ __forceinline__ uint32_t map_to_rank(uint32_t saddr, uint32_t rank) {
@@ -421,41 +420,49 @@ __device__ __forceinline__ float2 ld_cluster_f2(uint32_t addr) {
 
 constexpr int kStageStrideP = kPartRow + 16;  // bytes per staged partial row (272)
 
-// Partial rows: 256 bytes, a lane owns 8 of them. 128 dims: halves (their rounding, 2^-11 relative, is a quarter of the
-// bf16 output's; half the bytes to move), four columns per lane. 64 dims: floats, two columns per lane.
+// Partial rows: 256 bytes, read by half a warp, 16 bytes a lane. 128 dims: halves (their rounding, 2^-11 relative, is a
+// quarter of the bf16 output's; half the bytes to move), eight columns per lane. 64 dims: floats, four columns per lane.
 template <int HD> struct Part;
 template <> struct Part<128> {
-  static constexpr int NC = 4;
-  static __device__ __forceinline__ void add(float (&acc)[4], uint2 v, float w) {
-    const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&v.x));
-    const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&v.y));
-    acc[0] += lo.x * w;
-    acc[1] += lo.y * w;
-    acc[2] += hi.x * w;
-    acc[3] += hi.y * w;
+  static constexpr int NC = 8;
+  static __device__ __forceinline__ void add(float (&acc)[8], uint4 v, float w) {
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&u[e]));
+      acc[2 * e] += f.x * w;
+      acc[2 * e + 1] += f.y * w;
+    }
   }
-  static __device__ __forceinline__ void store(__nv_bfloat16* row, int lane, const float (&acc)[4], float inv) {
+  static __device__ __forceinline__ void store(__nv_bfloat16* row, int l16, const float (&acc)[8], float inv) {
+    uint32_t u[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const __nv_bfloat162 a = __floats2bfloat162_rn(acc[2 * e] * inv, acc[2 * e + 1] * inv);
+      u[e] = *reinterpret_cast<const uint32_t*>(&a);
+    }
+    *reinterpret_cast<uint4*>(row + l16 * 8) = make_uint4(u[0], u[1], u[2], u[3]);
+  }
+};
+template <> struct Part<64> {
+  static constexpr int NC = 4;
+  static __device__ __forceinline__ void add(float (&acc)[4], uint4 v, float w) {
+    acc[0] += __uint_as_float(v.x) * w;
+    acc[1] += __uint_as_float(v.y) * w;
+    acc[2] += __uint_as_float(v.z) * w;
+    acc[3] += __uint_as_float(v.w) * w;
+  }
+  static __device__ __forceinline__ void store(__nv_bfloat16* row, int l16, const float (&acc)[4], float inv) {
     const __nv_bfloat162 a = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv), c = __floats2bfloat162_rn(acc[2] * inv, acc[3] * inv);
     uint2 pk;
     pk.x = *reinterpret_cast<const uint32_t*>(&a);
     pk.y = *reinterpret_cast<const uint32_t*>(&c);
-    *reinterpret_cast<uint2*>(row + lane * 4) = pk;
+    *reinterpret_cast<uint2*>(row + l16 * 4) = pk;
   }
 };
-template <> struct Part<64> {
-  static constexpr int NC = 2;
-  static __device__ __forceinline__ void add(float (&acc)[2], uint2 v, float w) {
-    acc[0] += __uint_as_float(v.x) * w;
-    acc[1] += __uint_as_float(v.y) * w;
-  }
-  static __device__ __forceinline__ void store(__nv_bfloat16* row, int lane, const float (&acc)[2], float inv) {
-    const __nv_bfloat162 a = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv);
-    *reinterpret_cast<uint32_t*>(row + lane * 2) = *reinterpret_cast<const uint32_t*>(&a);
-  }
-};
-__device__ __forceinline__ uint2 ld_cluster_u2(uint32_t addr) {
-  uint2 v;
-  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
+__device__ __forceinline__ uint4 ld_cluster_u4(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
   return v;
 }
 
@@ -466,10 +473,10 @@ __device__ __forceinline__ int div_small(int a, int b, float inv_b) {
   return q + (r >= b ? 1 : 0) - (r < 0 ? 1 : 0);
 }
 
-// The merge of a row's splits: split s weighs sum_s * e^(max_s - max). A warp merges ROWS rows of at most SPL splits at a
-// time; lane u * SPL + s holds row u's split s, so one load and two short butterflies give the weights of all the rows
-// (a butterfly over the whole warp for each row, and a branch on each weight, made the merge of two rows a chain of
-// 2.8 us in a launch of 13: 128 CTAs, 8 splits; now 1.3). Returns the weight over the row's sum of weights.
+// The merge of a row's splits: split s weighs sum_s * e^(max_s - max). Half a warp merges ROWS rows of at most SPL splits
+// (ROWS * SPL <= 16) at a time; its lane u * SPL + s holds row u's split s, so one load and two short butterflies give the
+// weights of all the rows (a butterfly over the whole warp for each row, and a branch on each weight, made the merge of two
+// rows a chain of 2.8 us in a launch of 13: 128 CTAs, 8 splits). Returns the weight over the row's sum of weights.
 template <int SPL>
 __device__ __forceinline__ float split_weight(float mx, float sum) {
   float M = mx;
@@ -482,12 +489,13 @@ __device__ __forceinline__ float split_weight(float mx, float sum) {
   return tot > 0.f ? w * (1.f / tot) : 0.f;
 }
 template <int HD, int SPL>
-__device__ __forceinline__ void add_splits(float (&acc)[Part<HD>::NC], const uint2 (&v)[SPL], float wgt, int u) {
+__device__ __forceinline__ void add_splits(float (&acc)[Part<HD>::NC], const uint4 (&v)[SPL], float wgt, int u) {
 #pragma unroll
   for (int s2 = 0; s2 < SPL; ++s2) {
-    const float w = __shfl_sync(0xffffffffu, wgt, u * SPL + s2);
+    const float w = __shfl_sync(0xffffffffu, wgt, (threadIdx.x & 16) + u * SPL + s2);
     // a split without visible positions staged nothing: its buffer may hold anything
-    Part<HD>::add(acc, w > 0.f ? v[s2] : make_uint2(0u, 0u), w);
+    const uint32_t m = w > 0.f ? 0xffffffffu : 0u;
+    Part<HD>::add(acc, make_uint4(v[s2].x & m, v[s2].y & m, v[s2].z & m, v[s2].w & m), w);
   }
 }
 
@@ -496,53 +504,44 @@ __device__ __forceinline__ void add_splits(float (&acc)[Part<HD>::NC], const uin
 // (the merge moves half the bytes that way; the rounding, 2^-11 relative, is a quarter of the bf16
 // output's), and (max, sum) per row in its own shared memory. This CTA owns the rows rr with
 // rr % nsplit == split and reads them from all peers.
-// Warp w takes owned rows w, w+8, ...; a lane owns 8 bytes of a row; ROWS x SPL loads in flight. A warp arrives at the
-// cluster's last barrier with its last loads, not after its stores: the arrival would wait for them (0.9 us).
+// Half warp w takes owned rows w, w+16, ...; ROWS x SPL loads of 16 bytes in flight per lane.
 template <int HD, int ROWS, int SPL>
 __device__ __forceinline__ void merge_rows(const TcParams& p, uint32_t stage_o_s, uint32_t stage_ml_s, int rank0,
                                            int b, int kvh, int row0, int rows_here, int nsplit, int split) {
-  const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5, G = p.G;
+  const int l16 = threadIdx.x & 15, hw = threadIdx.x >> 4, G = p.G;
   const float inv_G = 1.f / (float)G;
   const int owned = rows_here > split ? div_small(rows_here - split + nsplit - 1, nsplit, 1.f / (float)nsplit) : 0;
-  const int mu = lane / SPL, msp = lane % SPL;  // whose (max, sum) this lane reads
-  bool arrived = false;
-  for (int i0 = wv; i0 < owned; i0 += 8 * ROWS) {
-    uint2 v[ROWS][SPL];
+  const int mu = l16 / SPL, msp = l16 % SPL;  // whose (max, sum) this lane reads
+  for (int i0 = hw; (i0 & ~1) < owned; i0 += 16 * ROWS) {  // (the same trips for both halves of a warp)
+    uint4 v[ROWS][SPL];
     float mx = -INFINITY, sum = 0.f;
-    if (mu < ROWS && msp < nsplit) {
-      const int im = i0 + 8 * mu;
-      const float2 ml = ld_cluster_f2(map_to_rank(stage_ml_s + (uint32_t)(split + nsplit * (im < owned ? im : i0)) * 8u,
+    if (mu < ROWS && msp < nsplit && i0 + 16 * mu < owned) {
+      const float2 ml = ld_cluster_f2(map_to_rank(stage_ml_s + (uint32_t)(split + nsplit * (i0 + 16 * mu)) * 8u,
                                                   (uint32_t)(rank0 + msp)));
       mx = ml.x;
       sum = ml.y;
     }
 #pragma unroll
     for (int s2 = 0; s2 < SPL; ++s2) {
-      const uint32_t base = map_to_rank(stage_o_s + (uint32_t)(lane * 8), (uint32_t)(rank0 + (s2 < nsplit ? s2 : 0)));
+      const uint32_t base = map_to_rank(stage_o_s + (uint32_t)(l16 * 16), (uint32_t)(rank0 + (s2 < nsplit ? s2 : 0)));
 #pragma unroll
-      for (int u = 0; u < ROWS; ++u) {
-        const int i2 = i0 + 8 * u;
-        const int rr = split + nsplit * (i2 < owned ? i2 : i0);
-        v[u][s2] = s2 < nsplit ? ld_cluster_u2(base + (uint32_t)(rr * kStageStrideP)) : make_uint2(0u, 0u);
-      }
+      for (int u = 0; u < ROWS; ++u)
+        v[u][s2] = s2 < nsplit && i0 + 16 * u < owned
+                       ? ld_cluster_u4(base + (uint32_t)((split + nsplit * (i0 + 16 * u)) * kStageStrideP))
+                       : make_uint4(0u, 0u, 0u, 0u);
     }
     const float wgt = split_weight<SPL>(mx, sum);
-    if (i0 + 8 * ROWS >= owned) {
-      cluster_arrive();
-      arrived = true;
-    }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
       float acc[Part<HD>::NC] = {};
       add_splits<HD, SPL>(acc, v[u], wgt, u);
-      const int i2 = i0 + 8 * u;
+      const int i2 = i0 + 16 * u;
       if (i2 < owned) {
         const int grow = row0 + split + nsplit * i2, tt = div_small(grow, G, inv_G), hh = kvh * G + grow - tt * G;
-        Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, lane, acc, 1.f);
+        Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, l16, acc, 1.f);
       }
     }
   }
-  if (!arrived) cluster_arrive();
 }
 
 // ---- global-merge mode -------------------------------------------------------------------------
@@ -674,24 +673,24 @@ __device__ __forceinline__ WorkItem decode_work_chunked(const TcParams& p, int i
 }
 
 // Merge of the split partials of a row block, run by all 8 warps of the last CTA to finish it.
-// Warp w takes rows w, w+8, ...; a lane owns 8 bytes of a row. ROWS rows x SPL splits loads are
-// in flight per lane: the merge is bound by L2 latency, not by bytes.
+// Half warp w takes rows w, w+16, ...; ROWS rows x SPL splits loads of 16 bytes are in flight per lane: the merge is
+// bound by L2 latency, not by bytes.
 template <int HD, int ROWS, int SPL>
 __device__ __forceinline__ void merge_rows_global(const TcParams& p, int b, int kvh, int row0, int rows_here, int nsplit) {
-  const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5, G = p.G;
+  const int l16 = threadIdx.x & 15, hw = threadIdx.x >> 4, G = p.G;
   const float inv_G = 1.f / (float)G;
-  const int mu = lane / SPL, msp = lane % SPL;  // whose (max, sum) this lane reads
+  const int mu = l16 / SPL, msp = l16 % SPL;  // whose (max, sum) this lane reads
   auto token_head = [&](int rr, int& tt, int& hh) {
     const int grow = row0 + rr;
     tt = div_small(grow, G, inv_G);
     hh = kvh * G + grow - tt * G;
   };
-  for (int rr = wv; rr < rows_here; rr += 8 * ROWS) {
-    uint2 v[ROWS][SPL];
+  for (int r0 = hw; (r0 & ~1) < rows_here; r0 += 16 * ROWS) {  // (the same trips for both halves of a warp)
+    uint4 v[ROWS][SPL];
     float mx = -INFINITY, sum = 0.f;
     int tt, hh;
-    if (mu < ROWS && msp < nsplit) {
-      token_head(rr + 8 * mu < rows_here ? rr + 8 * mu : rr, tt, hh);
+    if (mu < ROWS && msp < nsplit && r0 + 16 * mu < rows_here) {
+      token_head(r0 + 16 * mu, tt, hh);
       const size_t pr = (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max + msp;
       const float2 ml = __ldcg(reinterpret_cast<const float2*>(p.part_ml + pr * 2));
       mx = ml.x;
@@ -699,20 +698,21 @@ __device__ __forceinline__ void merge_rows_global(const TcParams& p, int b, int 
     }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
-      token_head(rr + 8 * u < rows_here ? rr + 8 * u : rr, tt, hh);
-      const unsigned char* src = p.part_o + (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max * kPartRow + lane * 8;
+      const bool have = r0 + 16 * u < rows_here;
+      token_head(have ? r0 + 16 * u : 0, tt, hh);
+      const unsigned char* src = p.part_o + (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max * kPartRow + l16 * 16;
 #pragma unroll
       for (int s2 = 0; s2 < SPL; ++s2)
-        v[u][s2] = s2 < nsplit ? __ldcg(reinterpret_cast<const uint2*>(src + s2 * kPartRow)) : make_uint2(0u, 0u);
+        v[u][s2] = have && s2 < nsplit ? __ldcg(reinterpret_cast<const uint4*>(src + s2 * kPartRow)) : make_uint4(0u, 0u, 0u, 0u);
     }
     const float wgt = split_weight<SPL>(mx, sum);
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
       float acc[Part<HD>::NC] = {};
       add_splits<HD, SPL>(acc, v[u], wgt, u);
-      if (rr + 8 * u < rows_here) {
-        token_head(rr + 8 * u, tt, hh);
-        Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, lane, acc, 1.f);
+      if (r0 + 16 * u < rows_here) {
+        token_head(r0 + 16 * u, tt, hh);
+        Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, l16, acc, 1.f);
       }
     }
   }
@@ -1296,31 +1296,34 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   }
   const int rows_here = rows_total - row0 < kBM ? rows_total - row0 : kBM;
   const float inv_G = 1.f / (float)G;
+  const int l16 = lane & 15, hw = tid >> 4;
   if (nsplit == 1) {
 #pragma unroll 4
-    for (int rr = warp; rr < rows_here; rr += kThreadsTC / 32) {
+    for (int rr = hw; rr < rows_here; rr += kThreadsTC / 16) {
       const int grow = grow0 + rr, tt = div_small(grow, G, inv_G), hh = kvh * G + grow - tt * G;
       constexpr int NC = Part<HD>::NC;
       float acc[NC];
 #pragma unroll
-      for (int e = 0; e < NC; e += 2) {
-        const float2 o2 = *reinterpret_cast<const float2*>(stage_o + rr * kStageStride + lane * NC + e);
-        acc[e] = o2.x;
-        acc[e + 1] = o2.y;
+      for (int e = 0; e < NC; e += 4) {
+        const float4 o4 = *reinterpret_cast<const float4*>(stage_o + rr * kStageStride + l16 * NC + e);
+        acc[e] = o4.x;
+        acc[e + 1] = o4.y;
+        acc[e + 2] = o4.z;
+        acc[e + 3] = o4.w;
       }
       const float l_tot = stage_ml[rr * 2 + 1];
-      Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, lane, acc, l_tot > 0.f ? 1.f / l_tot : 0.f);
+      Part<HD>::store(p.out + (((size_t)b * p.Ncap + tt) * p.Hq + hh) * HD, l16, acc, l_tot > 0.f ? 1.f / l_tot : 0.f);
     }
   } else if (cs == 0) {
     // global-merge mode: partials to the workspace; the last split of this row block to finish merges
     const unsigned char* sh = reinterpret_cast<const unsigned char*>(stage_o);
 #pragma unroll 4
-    for (int rr = warp; rr < rows_here; rr += kThreadsTC / 32) {
+    for (int rr = hw; rr < rows_here; rr += kThreadsTC / 16) {
       const int grow = grow0 + rr, tt = div_small(grow, G, inv_G), hh = kvh * G + grow - tt * G;
       const size_t pr = (((size_t)b * p.Hq + hh) * p.Ncap + tt) * p.nsplit_max + split;
-      __stcg(reinterpret_cast<uint2*>(p.part_o + pr * kPartRow + lane * 8),
-             *reinterpret_cast<const uint2*>(sh + rr * kStageStrideP + lane * 8));
-      if (lane == 0) {
+      __stcg(reinterpret_cast<uint4*>(p.part_o + pr * kPartRow + l16 * 16),
+             *reinterpret_cast<const uint4*>(sh + rr * kStageStrideP + l16 * 16));
+      if (l16 == 0) {
         __stcg(reinterpret_cast<float2*>(p.part_ml + pr * 2), *reinterpret_cast<const float2*>(stage_ml + rr * 2));
       }
     }
@@ -1337,18 +1340,20 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     __syncthreads();
     if (*last_s) {
       if (nsplit <= 2) merge_rows_global<HD, 4, 2>(p, b, kvh, grow0, rows_here, nsplit);
-      else if (nsplit <= 4) merge_rows_global<HD, 4, 4>(p, b, kvh, grow0, rows_here, nsplit);
-      else merge_rows_global<HD, 2, kMaxSplit>(p, b, kvh, grow0, rows_here, nsplit);
+      else if (nsplit <= 4) merge_rows_global<HD, 2, 4>(p, b, kvh, grow0, rows_here, nsplit);
+      else merge_rows_global<HD, 1, kMaxSplit>(p, b, kvh, grow0, rows_here, nsplit);
     }
   } else {
     const uint32_t so_s = smem_u32(stage_o), sml_s = smem_u32(stage_ml);
     const int rank0 = crank - split;  // first CTA of this row block's split group
-    if (nsplit <= 2) merge_rows<HD, 8, 2>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
-    else if (nsplit <= 4) merge_rows<HD, 4, 4>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
-    else merge_rows<HD, 2, kMaxSplit>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
+    if (nsplit <= 2) merge_rows<HD, 4, 2>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
+    else if (nsplit <= 4) merge_rows<HD, 2, 4>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
+    else merge_rows<HD, 1, kMaxSplit>(p, so_s, sml_s, rank0, b, kvh, grow0, rows_here, nsplit, split);
   }
-  if (cs > 1) {  // nobody leaves while a peer may still read its shared memory
-    if (nsplit == 1) cluster_arrive();
+  // Nobody leaves while a peer may still read its shared memory. The rows that were read have been stored, so the reads are
+  // over; releasing the stores as well would have every warp wait for them (0.9 us of a launch of 13).
+  if (cs > 1) {
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     cluster_wait();
   }
 }
