@@ -1339,9 +1339,9 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     }
     __syncthreads();
     if (*last_s) {
-      if (nsplit <= 2) merge_rows_global<HD, 4, 2>(p, b, kvh, grow0, rows_here, nsplit);
-      else if (nsplit <= 4) merge_rows_global<HD, 2, 4>(p, b, kvh, grow0, rows_here, nsplit);
-      else merge_rows_global<HD, 1, kMaxSplit>(p, b, kvh, grow0, rows_here, nsplit);
+      if (nsplit <= 2) merge_rows_global<HD, 8, 2>(p, b, kvh, grow0, rows_here, nsplit);
+      else if (nsplit <= 4) merge_rows_global<HD, 4, 4>(p, b, kvh, grow0, rows_here, nsplit);
+      else merge_rows_global<HD, 2, kMaxSplit>(p, b, kvh, grow0, rows_here, nsplit);
     }
   } else {
     const uint32_t so_s = smem_u32(stage_o), sml_s = smem_u32(stage_ml);
