@@ -89,50 +89,83 @@ __device__ __forceinline__ float sum2(f32x2 v) {
   return a + b;
 }
 
-// Merge of a row block's splits: this warp's rows r0, r0 + step, ... The splits' weights two per lane, then the columns, four
-// per lane (at D = 64 each half of the warp takes every other split); the loads of many splits in flight.
-template <typename T, int D>
+// Merge of a row block's splits: this warp's rows r0, r0 + step, ... (ROWS of them). The splits' weights H per lane, then the
+// columns, four per lane (at D = 64 each half of the warp takes every other split). The rows advance together and their first
+// loads go out ahead of the weights: row after row, each with two round trips to L2, four rows were 6 us of a launch of 14.
+template <typename T, int D, int ROWS, int H>
 __device__ __forceinline__ void merge_splits(const AttnParams& p, int b, int kvh, int rb, int F, int row0, int r0, int step,
                                              int rows_here) {
-  static_assert(kMaxSplit <= 64, "two splits per lane");
-  constexpr int C4 = D / 4, kHalves = 32 / C4;
+  static_assert(kMaxSplit <= 64 && kMergeHere <= 32, "H splits per lane");
+  constexpr int C4 = D / 4, kHalves = 32 / C4, UN = ROWS > 1 ? 2 : 8;
   const int lane = threadIdx.x & 31, c = lane % C4 * 4, half = lane / C4;
   const size_t part0 = (((size_t)b * p.Hkv + kvh) * p.nrowblk + rb) * p.nsplit * kRB;
   const float2* ml = reinterpret_cast<const float2*>(p.part_ml) + part0;
-#pragma unroll 1
-  for (int r = r0; r < rows_here; r += step) {
-    float2 x[2];
+  float2 x[ROWS][H];
+  float4 v[ROWS][UN];
+  auto load = [&](int s0) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-      x[h] = lane + 32 * h < p.nsplit ? __ldcg(ml + (size_t)(lane + 32 * h) * kRB + r) : make_float2(-INFINITY, 0.f);
-    float M = fmaxf(x[0].x, x[1].x), w[2], l = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int u = 0; u < ROWS; ++u)
+#pragma unroll
+      for (int k = 0; k < UN; ++k) {
+        const int s = s0 + k * kHalves + half, r = r0 + u * step;
+        v[u][k] = s < p.nsplit && r < rows_here
+                      ? __ldcg(reinterpret_cast<const float4*>(p.part_o + (part0 + (size_t)s * kRB + r) * D + c))
+                      : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+  };
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u)
+#pragma unroll
+    for (int h = 0; h < H; ++h)
+      x[u][h] = lane + 32 * h < p.nsplit && r0 + u * step < rows_here ? __ldcg(ml + (size_t)(lane + 32 * h) * kRB + r0 + u * step)
+                                                                      : make_float2(-INFINITY, 0.f);
+  load(0);
+  float w[ROWS][H], l[ROWS], acc[ROWS][4];
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {
+    float M = x[u][0].x;
+    if (H == 2) M = fmaxf(M, x[u][H - 1].x);
+    l[u] = 0.f;
 #pragma unroll
     for (int of = 16; of > 0; of >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, of));
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      w[h] = x[h].x > -INFINITY ? expf(x[h].x - M) : 0.f;
-      l += x[h].y * w[h];
+    for (int h = 0; h < H; ++h) {
+      w[u][h] = x[u][h].x > -INFINITY ? expf(x[u][h].x - M) : 0.f;
+      l[u] += x[u][h].y * w[u][h];
     }
 #pragma unroll
-    for (int of = 16; of > 0; of >>= 1) l += __shfl_xor_sync(0xffffffffu, l, of);
-#pragma unroll 16
-    for (int s0 = 0; s0 < p.nsplit; s0 += kHalves) {
-      const int s = s0 + half;
-      const float ws = __shfl_sync(0xffffffffu, s0 < 32 ? w[0] : w[1], s & 31);
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);  // (a split that saw nothing weighs 0, and its sums are 0)
-      if (s < p.nsplit) v = __ldcg(reinterpret_cast<const float4*>(p.part_o + (part0 + (size_t)s * kRB + r) * D + c));
-      acc[0] += v.x * ws;
-      acc[1] += v.y * ws;
-      acc[2] += v.z * ws;
-      acc[3] += v.w * ws;
+    for (int of = 16; of > 0; of >>= 1) l[u] += __shfl_xor_sync(0xffffffffu, l[u], of);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[u][e] = 0.f;
+  }
+#pragma unroll 1
+  for (int s0 = 0;;) {
+#pragma unroll
+    for (int k = 0; k < UN; ++k) {
+      const int s = s0 + k * kHalves + half;
+#pragma unroll
+      for (int u = 0; u < ROWS; ++u) {
+        // (a split that saw nothing weighs 0, and its sums are 0)
+        const float ws = __shfl_sync(0xffffffffu, H == 1 || s0 + k * kHalves < 32 ? w[u][0] : w[u][H - 1], s & 31);
+        acc[u][0] += v[u][k].x * ws;
+        acc[u][1] += v[u][k].y * ws;
+        acc[u][2] += v[u][k].z * ws;
+        acc[u][3] += v[u][k].w * ws;
+      }
     }
+    s0 += UN * kHalves;
+    if (s0 >= p.nsplit) break;
+    load(s0);
+  }
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {
     if (kHalves == 2) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], 16);
+      for (int e = 0; e < 4; ++e) acc[u][e] += __shfl_xor_sync(0xffffffffu, acc[u][e], 16);
     }
-    const int row = row0 + r, t = F + row / p.G;
+    const int r = r0 + u * step, row = row0 + r, t = F + row / p.G;
     T* out = reinterpret_cast<T*>(p.out) + (((size_t)b * p.Ncap + t) * p.Hq + kvh * p.G + row % p.G) * D;
-    if (half == 0) store4(out + c, acc, l > 0.f ? 1.f / l : 0.f);
+    if (half == 0 && r < rows_here) store4(out + c, acc[u], l[u] > 0.f ? 1.f / l[u] : 0.f);
   }
 }
 
@@ -386,7 +419,7 @@ __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams
   }
   __syncthreads();
   if (!s_last) return;
-  merge_splits<T, D>(p, b, kvh, rb, F, row0, warp, kThreads / 32, rows_here);
+  merge_splits<T, D, kRB / (kThreads / 32), 1>(p, b, kvh, rb, F, row0, warp, kThreads / 32, rows_here);
 }
 
 // The same as a kernel of its own, a warp per row: for launches of many splits, whose partials (a quarter of a megabyte and
@@ -403,7 +436,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(const AttnParams p
   F = F < 0 ? 0 : (F > N ? N : F);
   const int row0 = rb * kRB, rows_here = min((N - F) * p.G - row0, kRB);
   const int r = (blockIdx.x % kPer) * (kThreads / 32) + (threadIdx.x >> 5);
-  merge_splits<T, D>(p, b, kvh, rb, F, row0, r, kRB, rows_here);
+  merge_splits<T, D, 1, 2>(p, b, kvh, rb, F, row0, r, kRB, rows_here);
 }
 
 // Row blocks and KV splits of a launch, and the bytes of workspace it needs.
