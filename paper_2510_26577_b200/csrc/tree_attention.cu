@@ -450,14 +450,16 @@ CcPlan cc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, 
   const int base = B * Hkv * pl.nrowblk;
   const int max_pos = page_size == 0 ? seq_capacity : seq_capacity * page_size;
   const int max_tiles = (max_pos + kPT - 1) / kPT;
-  // The count for which rounds of resident CTAs (three per SM at D = 64, two at 128) x tiles per CTA is smallest, a CTA's
-  // prologue and partial counted as two tiles: 512 CTAs on 444 places would run as two rounds.
-  const int slots = (D == 64 ? 3 : 2) * c->num_sms;
+  // The count for which a machine evenly loaded with all tiles, half a tile added per CTA for its prologue and partial, and
+  // one CTA left running alone at its end (1.3 times as slow a tile) take least; past kMergeHere splits a second launch, as
+  // long as a tile. Sequences differ in length, so more and shorter CTAs than the machine holds at once are no loss:
+  // 8 sequences of 300-2000, 128 rows, 3 splits (one round of resident CTAs) 98 us, 8 splits 62.
   int nsplit = 1;
-  long long best = -1;
+  float best = 0.f;
   for (int n = 1; n <= kMaxSplit && n <= max_tiles; ++n) {
-    const long long cost = (long long)(((long long)base * n + slots - 1) / slots) * ((max_tiles + n - 1) / n + 2);
-    if (best < 0 || cost < best) {
+    const float cost = (float)base * ((float)max_tiles + 0.5f * (float)n) / (float)c->num_sms +
+                       1.3f * ((float)((max_tiles + n - 1) / n) + 0.5f) + (n > kMergeHere ? 1.f : 0.f);
+    if (n == 1 || cost < best) {
       best = cost;
       nsplit = n;
     }
