@@ -52,6 +52,8 @@ constexpr int kArgUnroll = 8;
 // the element in it at the end. With a compare and two selects per unpacked logit the bf16 sweep ran at 2.6 TB/s.
 // A row whose start is not 16-byte aligned (an odd vocabulary) is swept from the boundary below it: element v of the
 // aligned view is token v - shift, and only the vectors at the row's two ends are assembled element by element.
+// (Those apart from the rest, and whole rounds without tests: with the assembly inside the unrolled loop the fp32 sweep took
+// 102 registers, two CTAs per SM instead of four, and 1.2 GB of logits 223 us instead of 170.)
 template <typename T>
 __global__ void __launch_bounds__(kArgThreads) argmax_sweep_kernel(const T* __restrict__ logits, int V, int Ncap,
                                                                    int chunk_elems, const int32_t* __restrict__ n_tree,
@@ -75,26 +77,39 @@ __global__ void __launch_bounds__(kArgThreads) argmax_sweep_kernel(const T* __re
   uint4 braw = make_uint4(none, none, none, none);
   for (int base = begin; base < end; base += kArgThreads * VEC * kArgUnroll) {
     uint4 raw[kArgUnroll];
+    if (base >= shift && base + kArgThreads * VEC * kArgUnroll <= end) {  // a whole round: nothing to test per vector
 #pragma unroll
-    for (int v = 0; v < kArgUnroll; ++v) {
-      const int idx = base + (v * kArgThreads + tid) * VEC;
-      if (idx >= shift && idx + VEC <= end) {
-        raw[v] = __ldcs(reinterpret_cast<const uint4*>(xa + idx));
-      } else {
+      for (int v = 0; v < kArgUnroll; ++v) raw[v] = __ldcs(reinterpret_cast<const uint4*>(xa + base + (v * kArgThreads + tid) * VEC));
+    } else {
+#pragma unroll
+      for (int v = 0; v < kArgUnroll; ++v) {
+        const int idx = base + (v * kArgThreads + tid) * VEC;
         raw[v] = make_uint4(none, none, none, none);
-        if (idx < end) {
+        if (idx >= shift && idx + VEC <= end) raw[v] = __ldcs(reinterpret_cast<const uint4*>(xa + idx));
+      }
+#pragma unroll 1
+      for (int v = 0; v < kArgUnroll; ++v) {  // at most one vector at each end of the row
+        const int idx = base + (v * kArgThreads + tid) * VEC;
+        if (idx >= end || (idx >= shift && idx + VEC <= end)) continue;
+        uint4 a = make_uint4(none, none, none, none);
 #pragma unroll
-          for (int e = 0; e < VEC; ++e)
-            if (idx + e >= shift && idx + e < end) Vec<T>::put(raw[v], e, to_float(xa[idx + e]));
+        for (int e = 0; e < VEC; ++e)
+          if (idx + e >= shift && idx + e < end) Vec<T>::put(a, e, to_float(xa[idx + e]));
+        const float m = Vec<T>::max(a);
+        if (m > best || (m == best && idx < bvec)) {
+          best = m;
+          bvec = idx;
+          braw = a;
         }
       }
     }
 #pragma unroll
     for (int v = 0; v < kArgUnroll; ++v) {
       const float m = Vec<T>::max(raw[v]);
-      if (m > best) {  // elements ascend within a thread: the first maximum has the lowest id
+      const int idx = base + (v * kArgThreads + tid) * VEC;
+      if (m > best || (m == best && idx < bvec)) {  // (bvec is past idx where an end's vector came first)
         best = m;
-        bvec = base + (v * kArgThreads + tid) * VEC;
+        bvec = idx;
         braw = raw[v];
       }
     }

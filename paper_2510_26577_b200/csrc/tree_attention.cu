@@ -453,10 +453,11 @@ CcPlan cc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, 
   // The count for which a machine evenly loaded with all tiles, half a tile added per CTA for its prologue and partial, and
   // one CTA left running alone at its end (1.3 times as slow a tile) take least; past kMergeHere splits a second launch, as
   // long as a tile. Sequences differ in length, so more and shorter CTAs than the machine holds at once are no loss:
-  // 8 sequences of 300-2000, 128 rows, 3 splits (one round of resident CTAs) 98 us, 8 splits 62.
+  // 8 sequences of 300-2000, 128 rows, 3 splits (one round of resident CTAs) 98 us, 8 splits 62. No more than 16 CTAs per
+  // SM (that bounds the workspace to 40 MB).
   int nsplit = 1;
   float best = 0.f;
-  for (int n = 1; n <= kMaxSplit && n <= max_tiles; ++n) {
+  for (int n = 1; n <= kMaxSplit && n <= max_tiles && (n == 1 || (long long)base * n <= 16ll * c->num_sms); ++n) {
     const float cost = (float)base * ((float)max_tiles + 0.5f * (float)n) / (float)c->num_sms +
                        1.3f * ((float)((max_tiles + n - 1) / n) + 0.5f) + (n > kMergeHere ? 1.f : 0.f);
     if (n == 1 || cost < best) {
