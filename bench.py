@@ -435,7 +435,7 @@ def measure(args, w, rep, full):
     attn_flops = int(sum(4 * D * int(n_tree[b]) * G * Hkv * (int(kvl[b]) + int(n_tree[b])) for b in range(B)))
     hbm_peak, tensor_peak, which = peaks()
     attn_us = ms_attn * 1e3 / nl
-    tensor_path = w.kv_dtype == "bf16" and D == 128
+    tensor_path = w.kv_dtype == "bf16" and D in (64, 128)
     ridge = tensor_peak * 1e12 / (hbm_peak * 1e9)
     gbs = attn_bytes / (attn_us * 1e-6) / 1e9
     tfs = attn_flops / (attn_us * 1e-6) / 1e12
@@ -463,7 +463,7 @@ def measure(args, w, rep, full):
                    "logit_copies_rotated": n_tsets},
     }
     sel_launches = 1 if B == 1 else 2
-    attn_launches = 1 if tensor_path else 2  # CUDA-core path: main + combine
+    attn_launches = 1  # the splits are merged in the kernel (on the CUDA cores up to 16 of them; c1_tiny has 5)
     # H expand + select + attention layers (+ the work-list kernel in front of the first one) + sweep, walk + compaction
     launches_per_step = H + sel_launches + attn_launches * nl + (1 if tensor_path else 0) + 2 + 1
     res = {
