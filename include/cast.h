@@ -220,7 +220,8 @@ CAST_API cast_status cast_set_attention_early_reads(cast_ctx* ctx, int promise);
  * out[b,t,h] = softmax over {prefix positions 0..kv_len[b]-1} U {tree positions
  * kv_len[b]+j : bit j of anc_mask[b,t]} of (q . k) * scale, times v, for
  * t < n_tree[b]; rows t >= n_tree[b] of `out` are left untouched.
- * n_tree[b] must not exceed the context's total_token (device error BAD_TREE).
+ * n_tree[b] must not exceed the context's total_token (device error BAD_TREE; the rows t < total_token are computed all
+ * the same, those past it are left untouched).
  *   q, out        [B, Ncap, Hq, D], dtype `dtype`; rows t >= n_tree[b] of q may hold anything (NaN and
  *                 inf included): they may be loaded with their neighbours but reach no output
  *   k_cache, v_cache  paged: [num_pages, page_size, Hkv, D]; the cache rows of
@@ -231,7 +232,7 @@ CAST_API cast_status cast_set_attention_early_reads(cast_ctx* ctx, int promise);
  *   scale         0 selects 1/sqrt(D)
  * Accumulation is fp32. Needs Hq % Hkv == 0, D in {64, 128}, 16-byte aligned
  * pointers, and a workspace reserved for this shape (cast_reserve_attention; else CAST_ERR_CAPACITY).
- * Device errors: BAD_PAGE.
+ * Device errors: BAD_TREE, BAD_PAGE.
  */
 CAST_API cast_status cast_tree_attention(cast_ctx* ctx, const void* q, const void* k_cache, const void* v_cache,
                                 cast_dtype dtype, int B, int Hq, int Hkv, int D, int page_size,

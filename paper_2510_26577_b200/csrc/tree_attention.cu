@@ -41,7 +41,7 @@ struct AttnParams {
   const void* k;
   const void* v;
   void* out;
-  int B, Ncap, Hq, Hkv, G, page_size, seq_capacity, num_pages, words, nsplit, nrowblk;
+  int B, Ncap, Nmax, Hq, Hkv, G, page_size, seq_capacity, num_pages, words, nsplit, nrowblk;  // Nmax: most tokens of a tree
   const int32_t* page_table;
   const int32_t* kv_len;
   const int32_t* n_tree;
@@ -192,7 +192,11 @@ __global__ void __launch_bounds__(kThreads) tree_attn_cc_kernel(const AttnParams
   const int kvh = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int N = p.n_tree[b];
-  N = N < 0 ? 0 : (N > p.Ncap ? p.Ncap : N);
+  if (N > p.Nmax) {  // row blocks are launched for Nmax tokens: the rows past it stay untouched, and the caller is told
+    if (blockIdx.x == 0 && kvh == 0 && tid == 0) report(p.st, CAST_ERR_BAD_TREE, b);
+    N = p.Nmax;
+  }
+  N = N < 0 ? 0 : N;
   int L = p.kv_len[b];
   if (L < 0) L = 0;
   const int G = p.G;
@@ -431,7 +435,7 @@ __global__ void __launch_bounds__(kThreads) attn_merge_kernel(const AttnParams p
   constexpr int kPer = kRB / (kThreads / 32);  // CTAs per row block
   const int rb = blockIdx.x / kPer, kvh = blockIdx.y, b = blockIdx.z;
   int N = p.n_tree[b];
-  N = N < 0 ? 0 : (N > p.Ncap ? p.Ncap : N);
+  N = N < 0 ? 0 : (N > p.Nmax ? p.Nmax : N);
   int F = p.first_row != nullptr ? p.first_row[b] : 0;
   F = F < 0 ? 0 : (F > N ? N : F);
   const int row0 = rb * kRB, rows_here = min((N - F) * p.G - row0, kRB);
@@ -570,7 +574,7 @@ extern "C" cast_status cast_tree_attention_rows(cast_ctx* c, const void* q, cons
   }
   AttnParams p;
   p.q = q; p.k = k_cache; p.v = v_cache; p.out = out;
-  p.B = B; p.Ncap = c->cfg.max_tree; p.Hq = Hq; p.Hkv = Hkv; p.G = Hq / Hkv;
+  p.B = B; p.Ncap = c->cfg.max_tree; p.Nmax = c->cfg.total_token; p.Hq = Hq; p.Hkv = Hkv; p.G = Hq / Hkv;
   p.page_size = page_size; p.seq_capacity = seq_capacity; p.num_pages = num_pages; p.words = c->words;
   p.page_table = page_table; p.kv_len = kv_len; p.n_tree = n_tree; p.first_row = first_row; p.anc = anc_mask;
   p.scale = scale; p.ticket = nullptr; p.part_o = nullptr; p.part_ml = nullptr; p.st = c->state;

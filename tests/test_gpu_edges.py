@@ -231,3 +231,34 @@ def test_cuda_core_attention_merges(binding, dtype, D, page, B, cap, Hq, Hkv, kv
         assert torch.equal(got.isnan(), ~keep)
         tol = 1e-5 if dtype == torch.float32 else 1e-5 + want[keep].abs() * 2.0 ** -8
         assert bool(((got.double() - want)[keep].abs() <= tol).all())
+
+
+@pytest.mark.parametrize("dtype,page", [(torch.float32, 16), (torch.float32, 0), (torch.bfloat16, 128), (torch.bfloat16, 16)])
+@pytest.mark.parametrize("Hq,kv", [(4, 70), (4, 2000), (1, 9)])
+def test_attention_reports_a_tree_beyond_total_token(binding, dtype, page, Hq, kv):
+    """n_tree of total_token, one more and max_tree, on the CUDA cores (splits merged by the last CTA or by a kernel of its
+    own) and the tensor cores: BAD_TREE names the sequence, the rows of the first total_token tokens come, the rest stay."""
+    B, cap, total, D = 3, 64, 40, 64
+    rng = np.random.default_rng(kv)
+    g = torch.Generator(device="cuda").manual_seed(kv)
+    seq = -(-(kv + cap) // page) if page else kv + cap
+    k, v = (torch.randn((B * seq, page, 1, D) if page else (B, seq, 1, D), generator=g, device="cuda").to(dtype) for _ in range(2))
+    table = torch.arange(B * seq, device="cuda", dtype=torch.int32).view(B, seq) if page else None
+    q = torch.randn((B, cap, Hq, D), generator=g, device="cuda").to(dtype)
+    anc = _random_trees(rng, B, cap, [cap] * B)
+    ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=total, max_tree=cap)
+    ctx.cast_reserve_attention(dtype, B, Hq, 1, D, page, seq)
+    want = _attention_reference(q, k, v, page, table, [kv] * B, anc, [total] * B)
+    for n_tree, status in (([total] * 3, (0, None)), ([total, total + 1, total], (6, 1)), ([total, 5, cap], (6, 2))):
+        out = torch.full_like(q, float("nan"))
+        ctx.cast_tree_attention(q, k, v, B, Hq, 1, D, page, table, seq, B * seq if page else 0, _ints([kv] * B), anc,
+                                _ints(n_tree), 0.0, out)
+        st, detail = ctx.cast_poll_status()
+        assert st == status[0] and (st == 0 or detail == status[1])
+        for b in range(B):
+            n = min(n_tree[b], total)
+            assert out[b, n:].isnan().all()
+            # (a token sees its ancestors, all of them before it: the rows of a cut tree are those of the whole one)
+            # (tolerances as above: fp32 sums, the output's rounding, two bf16 terms of P on the tensor cores)
+            tol = 1e-5 if dtype == torch.float32 else 2e-5 + want[b, :n].abs() * 2.0 ** -8
+            assert bool(((out[b, :n].double() - want[b, :n]).abs() <= tol).all())
