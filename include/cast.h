@@ -34,7 +34,8 @@
  *  - cast_tree_expand, cast_select_nodes and cast_tree_attention are launched with programmatic
  *    dependent launch: their thread blocks may become resident while the previous kernel of the
  *    stream is still finishing, but they read no input (logits, Q, K/V, tree arrays, lengths) before
- *    that kernel has completed, so stream order keeps its usual meaning for the caller.
+ *    that kernel has completed, so stream order keeps its usual meaning for the caller. They hold no tensor memory
+ *    meanwhile either (unless cast_set_attention_early_reads was called, which states what it needs for that).
  *  - Precision of the tree-sizing decisions: node values, u, c and every comparison are fp64, but a row's
  *    log-sum-exp is accumulated in fp32 (about 3e-7 absolute per layer). The retained sets, n_i, go/stop
  *    and N equal those of an exact evaluation whenever no two neighbouring values across a kept/dropped

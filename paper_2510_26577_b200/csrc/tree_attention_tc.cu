@@ -88,6 +88,7 @@ struct TcParams {
   int q_tma;  // Q row blocks are fetched by TMA (the group size divides 128)
   const int32_t* worklist;  // one decoded work item per CTA (8 ints each), or null: every CTA decodes for itself
   int early;  // the tree arrays, lengths, page table and prefix rows may be read before the dependency wait
+  int tmem_first;  // tensor memory may be taken before the dependency wait (see the kernel)
   int cs;   // CTAs per cluster (1..8); 0: no clusters, splits sized on the device and merged through global memory
   int rpc;  // cluster mode: row blocks a cluster covers at most (cs is a multiple of it)
   int nsplit_max, num_sms, nrb;  // global-merge mode
@@ -761,21 +762,22 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_v)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_q)) : "memory");
   }
-  // TMEM (two S buffers and O) before anything else: an SM starts its second CTA only after the first one has given up
-  // the right to allocate. Behind the dependency wait and the work decode, where this stood before, the second CTAs came
-  // 2.4-3.7 us after the first and a third round of clusters 5 us after (draft rows of 4 sequences of 512: 14.2 -> 11.4 us).
+  // TMEM: two S buffers and O
   uint32_t* tmem_base_s = reinterpret_cast<uint32_t*>(smem + GE::kSmemTmem);
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_s)),
-                 "n"(kTmemCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
+  auto tmem_take = [&] {
+    if (warp == 4) {
+      __syncwarp();
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_s)),
+                   "n"(kTmemCols));
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+  };
   // an early exit returns it
   auto tmem_return = [&] {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0)
+    if (warp == 4)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_base_s), "n"(kTmemCols));
   };
   // Programmatic dependent launch: this grid may become resident while the previous kernel of the
@@ -787,10 +789,18 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   // that depends on it (the Q load, a tile that reaches the tree rows, the output rows). The dependents are
   // released only after this CTA's own wait, so "everything before my predecessor is complete" keeps holding
   // down the chain.
+  // Tensor memory is taken before the work decode: an SM starts its second CTA only after the first one has given up the
+  // right to allocate, and behind the decode the second CTAs came 2.4-3.7 us late and a third round of clusters 5 us. In
+  // the default mode it is taken behind the wait: a predecessor that releases its dependents first and allocates later
+  // would wait on its SM for what this CTA holds, and this CTA for the predecessor. Before the wait (tmem_first) only where
+  // there is no such predecessor: by the promise of the early mode, or behind this call's own work list. The warp that
+  // allocates releases the dependents, after it has, so that it is no such predecessor itself.
   const bool early = p.early != 0;
+  if (p.tmem_first) tmem_take();
   if (!early) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!p.tmem_first) tmem_take();
+    if (warp == 4) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
   const WorkItem wk = p.worklist != nullptr ? load_item(p.worklist + (size_t)blockIdx.x * 8)
                       : cs == 0            ? decode_work_chunked(p, (int)blockIdx.x, (int)gridDim.x)
@@ -1290,7 +1300,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   tc_fence_before();
   if (cs > 1) cluster_sync_all();  // every CTA of the cluster has staged its rows
   else __syncthreads();
-  if (warp == 0) {  // every TMEM access of this CTA is over
+  if (warp == 4) {  // every TMEM access of this CTA is over
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols));
   }
@@ -1509,6 +1519,7 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   TcParams p;
   p.q_tma = q_tma ? 1 : 0;
   p.early = (c->attn_early && !c->tree_inputs_fresh && q_tma) ? 1 : 0;
+  p.tmem_first = p.early;
   p.q = (const __nv_bfloat16*)q; p.out = (__nv_bfloat16*)out;
   p.B = B; p.Ncap = Ncap; p.Nmax = Nmax; p.Hq = Hq; p.Hkv = Hkv; p.G = G; p.page_size = page_size;
   p.seq_capacity = seq_capacity; p.num_pages = num_pages; p.words = c->words;
@@ -1551,6 +1562,7 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
       for (int i = 0; i < 8; ++i) c->wl_key[i] = key[i];
       c->wl_valid = 1;
       p.early = 0;  // the list is the previous kernel's: read it after the wait
+      p.tmem_first = 1;  // (that kernel has no tensor memory, and as a plain launch it ran after all that was before it)
     }
     p.worklist = c->attn_worklist;
   }

@@ -1,0 +1,57 @@
+"""What must not be tried on a GPU, because getting it wrong is a wait without end: the order of the tensor-memory
+allocation, the dependency wait and the release of the dependents in the tensor-core attention, read from its source.
+
+A block that holds tensor memory while it waits for its predecessor is waited for by a predecessor on the same SM that
+released its dependents before it allocated. So the default mode allocates behind the wait, an allocation ahead of it
+needs a reason the host gives, and the kernel itself releases its dependents behind its own allocation."""
+import os
+import re
+
+SRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2510_26577_b200", "csrc",
+                   "tree_attention_tc.cu")
+
+
+def _source():
+    text = re.sub(r"/\*.*?\*/", "", open(SRC).read(), flags=re.S)
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def _body(text, head):
+    """The braces that follow `head`."""
+    start = text.index("{", text.index(head))
+    depth = 0
+    for i in range(start, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[start:i + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def test_tensor_memory_is_taken_behind_the_wait():
+    kernel = _body(_source(), "tree_attn_tc_kernel(const TcParams p")
+    assert kernel.count("tcgen05.alloc") == 1
+    take = _body(kernel, "auto tmem_take = [&]")
+    assert "tcgen05.alloc" in take and take.index("tcgen05.alloc") < take.index("tcgen05.relinquish_alloc_permit")
+    calls = [m.start() for m in re.finditer(r"\btmem_take\(\)", kernel)]
+    guards = [re.search(r"if \((!?p\.tmem_first)\) $", kernel[:c]).group(1) for c in calls]
+    assert guards == ["p.tmem_first", "!p.tmem_first"]
+    default = _body(kernel, "if (!early)")
+    order = [default.index(x) for x in ("griddepcontrol.wait", "tmem_take()", "griddepcontrol.launch_dependents")]
+    assert order == sorted(order)
+
+
+def test_dependents_are_released_by_the_warp_that_allocates():
+    kernel = _body(_source(), "tree_attn_tc_kernel(const TcParams p")
+    warp = re.search(r"if \(warp == (\d)\)", _body(kernel, "auto tmem_take = [&]")).group(1)
+    released = [m.start() for m in re.finditer("griddepcontrol.launch_dependents", kernel)]
+    assert len(released) == 2
+    assert re.search(r"if \(warp == %s\) asm volatile\(\"$" % warp, kernel[:released[0]])
+    early = kernel.rindex("if (warp == %s) {" % warp, 0, released[1])  # the producer's branch, which holds `if (early)`
+    assert "griddepcontrol.wait" in kernel[early:released[1]] and released[1] < early + len(_body(kernel[early:], "if ("))
+
+
+def test_who_may_take_it_ahead_of_the_wait():
+    """The early mode (the caller's promise), and the call that has just launched its own work list."""
+    launch = _body(_source(), "bool tree_attention_tc_launch(")
+    assert re.findall(r"p\.tmem_first = ([^;]*);", launch) == ["p.early", "1"]
+    assert re.search(r"attn_worklist_kernel<<<.*?p\.early = 0;\s*p\.tmem_first = 1;", launch, flags=re.S)
