@@ -563,6 +563,7 @@ extern "C" cast_status cast_tree_attention_rows(cast_ctx* c, const void* q, cons
   if (scale == 0.f) scale = 1.0f / sqrtf((float)D);
   cudaStream_t s = (cudaStream_t)stream;
   const int fresh = c->tree_inputs_fresh;
+  if (fresh) c->wl_valid = 0;  // also where this call takes no list itself: a later one must not find the old one
   c->tree_inputs_fresh = 0;  // whatever is launched below waits for its predecessor before it releases its own dependents
   if (dtype == CAST_BF16) {
     cast_status st = CAST_OK;

@@ -1554,7 +1554,7 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
                                        ((unsigned long long)seq_capacity << 32) | (unsigned)grid,
                                        ((unsigned long long)(unsigned)p.cs << 32) | ((unsigned)p.rpc << 16) | (unsigned)p.nsplit_max,
                                        (unsigned long long)Nmax, (unsigned long long)c->num_sms};
-    bool same = c->wl_valid && !c->tree_inputs_fresh;
+    bool same = c->wl_valid != 0;  // (the caller of this function has discarded it where the tree or the lengths are new)
     for (int i = 0; i < 8 && same; ++i) same = c->wl_key[i] == key[i];
     if (!same) {
       attn_worklist_kernel<<<(unsigned)((grid + 7) / 8), 256, 0, stream>>>(p, (int)grid, c->attn_worklist);

@@ -262,3 +262,57 @@ def test_attention_reports_a_tree_beyond_total_token(binding, dtype, page, Hq, k
             # (tolerances as above: fp32 sums, the output's rounding, two bf16 terms of P on the tensor cores)
             tol = 1e-5 if dtype == torch.float32 else 2e-5 + want[b, :n].abs() * 2.0 ** -8
             assert bool(((out[b, :n].double() - want[b, :n]).abs() <= tol).all())
+
+
+def _early_setup(binding, B, cap, Hq, Hkv, D, page, kv, dtype=torch.bfloat16):
+    """A context with the early-read promise and one layer's inputs: its attention call, and the state the call reads."""
+    rng = np.random.default_rng(Hq * D)
+    g = torch.Generator(device="cuda").manual_seed(Hq * D)
+    seq = -(-(max(kv) + 2 * cap) // page)
+    k, v = (torch.randn((B * seq, page, Hkv, D), generator=g, device="cuda").to(dtype) for _ in range(2))
+    table = torch.randperm(B * seq, generator=g, device="cuda").to(torch.int32).view(B, seq)
+    q = torch.randn((B, cap, Hq, D), generator=g, device="cuda").to(dtype)
+    anc = _random_trees(rng, B, cap, [cap] * B)
+    ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=cap, max_tree=cap)
+    ctx.cast_reserve_attention(dtype, B, Hq, Hkv, D, page, seq)
+    ctx.cast_set_attention_early_reads(True)
+    kv_len, n_tree = _ints(kv), _ints([cap] * B)
+
+    def call(first=None):
+        out = torch.full_like(q, float("nan"))
+        a = (q, k, v, B, Hq, Hkv, D, page, table, seq, B * seq, kv_len, anc, n_tree)
+        ctx.cast_tree_attention(*a, 0.0, out) if first is None else ctx.cast_tree_attention_rows(*a, _ints(first), 0.0, out)
+        return out
+
+    def check(out):
+        want = _attention_reference(q, k, v, page, table, kv_len.tolist(), anc, n_tree.tolist())
+        live = ~want.isnan()
+        assert torch.equal(out.isnan(), ~live)
+        # P in bf16 (a term of the sum off by 2^-9 of itself, all of them by no more than that of max |v|), then the output
+        assert float((out.double() - want)[live].abs().max()) <= 2.0 ** -9 * float(v.abs().max()) + 2.0 ** -8 * float(want[live].abs().max())
+        assert ctx.cast_poll_status()[0] == 0
+
+    def compact(path):
+        full = path + [-1] * (5 - len(path))
+        ctx.cast_compact_kv(k, v, B, 1, k.numel() * k.element_size(), Hkv, D, page, table, seq, B * seq, _ints([full] * B),
+                            _ints([len(path) - 1] * B), kv_len)
+    return ctx, call, check, compact, kv_len, n_tree
+
+
+@pytest.mark.parametrize("between", ["window", "f32"])
+def test_a_call_between_does_not_keep_an_old_work_list(binding, between):
+    """Under the early-read promise: attention, a compaction (which moves the lengths), a call that takes no work list
+    - a draft's window, a 32-bit layer - and the first attention again: it must see the new lengths."""
+    ctx, call, check, compact, kv_len, n_tree = _early_setup(binding, 2, 8, 8, 2, 128, 16, [40, 700])
+    check(call())
+    check(call())
+    compact([0, 2, 3])
+    assert kv_len.tolist() == [43, 703]
+    if between == "window":
+        call(first=[3, 4])
+    else:
+        x = torch.zeros((2, 8, 4, 64), device="cuda")
+        ctx.cast_reserve_attention(torch.float32, 2, 4, 1, 64, 0, 16)
+        c = torch.zeros((2, 16, 1, 64), device="cuda")
+        ctx.cast_tree_attention(x, c, c, 2, 4, 1, 64, 0, None, 16, 0, _ints([1, 2]), _ints([[[1]] * 8] * 2), n_tree, 0.0, x.clone())
+    check(call())
