@@ -1518,7 +1518,9 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   const bool q_tma = G <= kBM && (kBM % G) == 0 && make_q_map(&map_q, q, B, Ncap, Hq, G, D);
   TcParams p;
   p.q_tma = q_tma ? 1 : 0;
-  p.early = (c->attn_early && !c->tree_inputs_fresh && q_tma) ? 1 : 0;
+  // the shapes the header names: a caller of others may have set the promise without keeping it
+  const bool promised = c->attn_early && D == 128 && q_tma;
+  p.early = (promised && !c->tree_inputs_fresh) ? 1 : 0;
   p.tmem_first = p.early;
   p.q = (const __nv_bfloat16*)q; p.out = (__nv_bfloat16*)out;
   p.B = B; p.Ncap = Ncap; p.Nmax = Nmax; p.Hq = Hq; p.Hkv = Hkv; p.G = G; p.page_size = page_size;
@@ -1547,7 +1549,7 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   // calls of a step, so what every CTA would decode for itself is decoded once, by a small kernel launched in
   // front of the first such call (or when the call's shape changes), and the calls after it read one item each.
   p.worklist = nullptr;
-  if (c->attn_early && first_row == nullptr && grid <= kAttnWorkListCap) {  // (a window call names new sizes every time)
+  if (promised && first_row == nullptr && grid <= kAttnWorkListCap) {  // (a window call names new sizes every time)
     const unsigned long long key[8] = {(unsigned long long)(uintptr_t)n_tree, (unsigned long long)(uintptr_t)kv_len,
                                        (unsigned long long)(uintptr_t)first_row,
                                        ((unsigned long long)B << 48) | ((unsigned long long)Hq << 32) | ((unsigned long long)Hkv << 16) | (unsigned)page_size,

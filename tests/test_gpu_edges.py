@@ -316,3 +316,19 @@ def test_a_call_between_does_not_keep_an_old_work_list(binding, between):
         c = torch.zeros((2, 16, 1, 64), device="cuda")
         ctx.cast_tree_attention(x, c, c, 2, 4, 1, 64, 0, None, 16, 0, _ints([1, 2]), _ints([[[1]] * 8] * 2), n_tree, 0.0, x.clone())
     check(call())
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(8, 2, 64), (14, 2, 128), (8, 2, 128)])
+def test_shapes_outside_the_early_reads_ignore_the_promise(binding, Hq, Hkv, D):
+    """The header's shapes (128 dims, a group size that divides 128) take a reused work list, and a caller that changes the
+    lengths by itself says so; the other shapes see such a change without being told."""
+    ctx, call, check, _, kv_len, n_tree = _early_setup(binding, 2, 8, Hq, Hkv, D, 16, [40, 700])
+    check(call())
+    for lengths, sizes in (([9, 64], [8, 5]), ([500, 7], [1, 8])):
+        kv_len.copy_(_ints(lengths))
+        n_tree.copy_(_ints(sizes))
+        if D == 128 and 128 % (Hq // Hkv) == 0:
+            ctx.cast_set_attention_early_reads(True)
+        torch.cuda.synchronize()
+        check(call())
+        check(call())
