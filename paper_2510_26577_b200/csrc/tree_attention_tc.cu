@@ -808,6 +808,8 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   if (blockIdx.x < p.B && tid == 0 && p.n_tree[blockIdx.x] > p.Nmax) report(p.st, CAST_ERR_BAD_TREE, blockIdx.x);
   if (!wk.valid) {
     tmem_return();
+    // (a launch without any work must not be over before its predecessor either: its successor waits for this grid alone)
+    if (early && blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
     return;  // the whole cluster leaves (a CTA that exits counts as having released its dependents)
   }
   const int b = wk.b, kvh = wk.kvh, rb = wk.rb, split = wk.split, N = wk.N, L = wk.L;

@@ -50,6 +50,15 @@ def test_dependents_are_released_by_the_warp_that_allocates():
     assert "griddepcontrol.wait" in kernel[early:released[1]] and released[1] < early + len(_body(kernel[early:], "if ("))
 
 
+def test_a_launch_without_work_waits_for_its_predecessor():
+    """What follows a launch waits for that launch alone: one that ended ahead of its predecessor would break the order of
+    the stream. In the early mode a block without work leaves at once, so the first one waits on behalf of all."""
+    kernel = _body(_source(), "tree_attn_tc_kernel(const TcParams p")
+    idle = _body(kernel, "if (!wk.valid)")
+    assert re.search(r"if \(early && blockIdx\.x == 0\) asm volatile\(\"griddepcontrol\.wait;", idle)
+    assert idle.index("tmem_return()") < idle.index("griddepcontrol.wait") < idle.index("return;", idle.index("griddepcontrol"))
+
+
 def test_who_may_take_it_ahead_of_the_wait():
     """The early mode (the caller's promise), and the call that has just launched its own work list."""
     launch = _body(_source(), "bool tree_attention_tc_launch(")
