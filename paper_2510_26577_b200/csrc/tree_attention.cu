@@ -23,6 +23,7 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
                               int page_size, const int32_t* page_table, int seq_capacity, int num_pages,
                               const int32_t* kv_len, const uint32_t* anc, const int32_t* n_tree, const int32_t* first_row,
                               float scale, void* out, cudaStream_t stream, cast_status* status);
+bool tree_attention_tc_takes(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, int seq_capacity);
 size_t tree_attention_tc_workspace(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, int seq_capacity);
 cast_status tree_attention_tc_reserve(cast_ctx* c, size_t bytes);
 }
@@ -448,7 +449,10 @@ struct CcPlan {
   int nsplit, nrowblk;
   size_t bytes;
 };
-CcPlan cc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, int seq_capacity) {
+// per_sm: CTAs per SM at most, which bounds the workspace: kOwn (40 MB) for the shapes this path is for, kFallback (5 MB) for
+// those that come here only when a pointer is not aligned for the tensor path, whose callers reserve both workspaces.
+constexpr int kOwn = 16, kFallback = 2;
+CcPlan cc_plan(const cast_ctx* c, int per_sm, int B, int Hq, int Hkv, int D, int page_size, int seq_capacity) {
   CcPlan pl;
   pl.nrowblk = (c->cfg.total_token * (Hq / Hkv) + kRB - 1) / kRB;
   const int base = B * Hkv * pl.nrowblk;
@@ -457,11 +461,10 @@ CcPlan cc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, 
   // The count for which a machine evenly loaded with all tiles, half a tile added per CTA for its prologue and partial, and
   // one CTA left running alone at its end (1.3 times as slow a tile) take least; past kMergeHere splits a second launch, as
   // long as a tile. Sequences differ in length, so more and shorter CTAs than the machine holds at once are no loss:
-  // 8 sequences of 300-2000, 128 rows, 3 splits (one round of resident CTAs) 98 us, 8 splits 62. No more than 16 CTAs per
-  // SM (that bounds the workspace to 40 MB).
+  // 8 sequences of 300-2000, 128 rows, 3 splits (one round of resident CTAs) 98 us, 8 splits 62.
   int nsplit = 1;
   float best = 0.f;
-  for (int n = 1; n <= kMaxSplit && n <= max_tiles && (n == 1 || (long long)base * n <= 16ll * c->num_sms); ++n) {
+  for (int n = 1; n <= kMaxSplit && n <= max_tiles && (n == 1 || (long long)base * n <= (long long)per_sm * c->num_sms); ++n) {
     const float cost = (float)base * ((float)max_tiles + 0.5f * (float)n) / (float)c->num_sms +
                        1.3f * ((float)((max_tiles + n - 1) / n) + 0.5f) + (n > kMergeHere ? 1.f : 0.f);
     if (n == 1 || cost < best) {
@@ -476,8 +479,8 @@ CcPlan cc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, 
 }
 
 template <typename T, int D>
-cast_status launch_cc(cast_ctx* c, AttnParams& p, cudaStream_t s) {
-  const CcPlan pl = cc_plan(c, p.B, p.Hq, p.Hkv, D, p.page_size, p.seq_capacity);
+cast_status launch_cc(cast_ctx* c, AttnParams& p, int per_sm, cudaStream_t s) {
+  const CcPlan pl = cc_plan(c, per_sm, p.B, p.Hq, p.Hkv, D, p.page_size, p.seq_capacity);
   // compute calls never allocate: the workspace comes from cast_reserve_attention
   if (pl.bytes > c->attn_ws_bytes) return CAST_ERR_CAPACITY;
   p.nsplit = pl.nsplit;
@@ -530,11 +533,13 @@ extern "C" cast_status cast_reserve_attention(cast_ctx* c, cast_dtype dtype, int
   if (Hq % Hkv != 0 || (D != 64 && D != 128)) return CAST_ERR_SHAPE;
   // a bf16 call takes the tensor-core path when shape and pointer alignment allow and the CUDA-core path
   // otherwise: both workspaces are sized, so the choice at call time never needs memory
+  bool own = true;
   if (dtype == CAST_BF16) {
+    own = !tree_attention_tc_takes(c, B, Hq, Hkv, D, page_size, seq_capacity);
     const cast_status st = tree_attention_tc_reserve(c, tree_attention_tc_workspace(c, B, Hq, Hkv, D, page_size, seq_capacity));
     if (st != CAST_OK) return st;
   }
-  const size_t need = cc_plan(c, B, Hq, Hkv, D, page_size, seq_capacity).bytes;
+  const size_t need = cc_plan(c, own ? kOwn : kFallback, B, Hq, Hkv, D, page_size, seq_capacity).bytes;
   if (need > c->attn_ws_bytes) {
     CAST_CUDA_OK(cudaDeviceSynchronize());
     if (c->attn_ws) cudaFree(c->attn_ws);
@@ -579,8 +584,9 @@ extern "C" cast_status cast_tree_attention_rows(cast_ctx* c, const void* q, cons
   p.page_size = page_size; p.seq_capacity = seq_capacity; p.num_pages = num_pages; p.words = c->words;
   p.page_table = page_table; p.kv_len = kv_len; p.n_tree = n_tree; p.first_row = first_row; p.anc = anc_mask;
   p.scale = scale; p.ticket = nullptr; p.part_o = nullptr; p.part_ml = nullptr; p.st = c->state;
-  if (dtype == CAST_F32) return D == 64 ? launch_cc<float, 64>(c, p, s) : launch_cc<float, 128>(c, p, s);
-  return D == 64 ? launch_cc<__nv_bfloat16, 64>(c, p, s) : launch_cc<__nv_bfloat16, 128>(c, p, s);
+  if (dtype == CAST_F32) return D == 64 ? launch_cc<float, 64>(c, p, kOwn, s) : launch_cc<float, 128>(c, p, kOwn, s);
+  const int per_sm = tree_attention_tc_takes(c, B, Hq, Hkv, D, page_size, seq_capacity) ? kFallback : kOwn;
+  return D == 64 ? launch_cc<__nv_bfloat16, 64>(c, p, per_sm, s) : launch_cc<__nv_bfloat16, 128>(c, p, per_sm, s);
 }
 
 extern "C" cast_status cast_tree_attention(cast_ctx* c, const void* q, const void* k_cache, const void* v_cache,

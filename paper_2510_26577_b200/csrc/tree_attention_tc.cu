@@ -1482,6 +1482,11 @@ bool tc_plan(const cast_ctx* c, int B, int Hq, int Hkv, int page_size, int seq_c
 
 }  // namespace
 
+// Whether calls of this shape come here when their pointers are aligned for it.
+bool tree_attention_tc_takes(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, int seq_capacity) {
+  TcPlan pl;
+  return tc_shape_ok(D, page_size) && tc_plan(c, B, Hq, Hkv, page_size, seq_capacity, &pl);
+}
 // Workspace bytes a tensor-core launch of this shape needs (0: none, or the shape is not the tensor path's).
 size_t tree_attention_tc_workspace(const cast_ctx* c, int B, int Hq, int Hkv, int D, int page_size, int seq_capacity) {
   TcPlan pl;

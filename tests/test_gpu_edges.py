@@ -332,3 +332,36 @@ def test_shapes_outside_the_early_reads_ignore_the_promise(binding, Hq, Hkv, D):
         torch.cuda.synchronize()
         check(call())
         check(call())
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,D,page,positions", [(1, 32, 8, 128, 16, 4096), (8, 32, 8, 128, 0, 4096), (2, 16, 4, 64, 16, 1024)])
+def test_the_fallback_of_a_tensor_core_shape_stays_small(binding, B, Hq, Hkv, D, page, positions):
+    """bf16 keys and values on 16-byte boundaries that are not the tensor path's 128 go to the CUDA cores: the workspace
+    reserved for that is a few megabytes (two CTAs per SM of 17 KB partials, whole 2 MB pages), and the call runs with it."""
+    cap = 60
+    rng = np.random.default_rng(B)
+    unit = page or 1
+    seq = positions // unit
+    g = torch.Generator(device="cuda").manual_seed(B)
+    shape = (B * seq, page, Hkv, D) if page else (B, seq, Hkv, D)
+    n = int(np.prod(shape))
+    k, v = (torch.randn(n + 8, generator=g, device="cuda").to(torch.bfloat16)[8:].view(shape) for _ in range(2))
+    assert k.data_ptr() % 128 == 16
+    table = torch.randperm(B * seq, generator=g, device="cuda").to(torch.int32).view(B, seq) if page else None
+    q = torch.randn((B, cap, Hq, D), generator=g, device="cuda").to(torch.bfloat16)
+    n_tree = [cap - 7 * (b % 3) for b in range(B)]
+    kv = [int(x) for x in rng.integers(1, positions - cap, B)]
+    anc = _random_trees(rng, B, cap, n_tree)
+    ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=cap, max_tree=cap)
+    out = torch.full_like(q, float("nan"))
+    args = (B, Hq, Hkv, D, page)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    ctx.cast_reserve_attention(q.dtype, *args, seq)
+    assert before - torch.cuda.mem_get_info()[0] <= 8 << 20
+    ctx.cast_tree_attention(q, k, v, *args, table, seq, B * seq if page else 0, _ints(kv), anc, _ints(n_tree), 0.0, out)
+    assert ctx.cast_poll_status()[0] == 0
+    want = _attention_reference(q, k, v, page, table, kv, anc, n_tree)
+    live = ~want.isnan()
+    assert torch.equal(out.isnan(), ~live)
+    assert bool(((out.double() - want)[live].abs() <= 1e-5 + want[live].abs() * 2.0 ** -8).all())
