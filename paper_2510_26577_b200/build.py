@@ -35,12 +35,23 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _built_against(torch_dir: str) -> str:
+    """What the extension module is good for: this torch (its classes are linked to by mangled name) and this Python."""
+    with open(os.path.join(torch_dir, "version.py")) as f:
+        return (sysconfig.get_config_var("SOABI") or sys.version) + "\n" + torch_dir + "\n" + f.read()
+
+
 def _build_calls() -> None:
     """The extension module the binding calls through (host code against torch's headers; links the CUDA library)."""
     src = os.path.join(CSRC, "binding_calls.cpp")
-    if not _stale(CALLS, [src, os.path.join(ROOT, "include", "cast.h")]):
-        return
     torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)
+    stamp, against = os.path.join(OBJ, "binding_calls.against"), _built_against(torch_dir)
+    same = False
+    if os.path.exists(stamp):
+        with open(stamp) as f:
+            same = f.read() == against
+    if same and not _stale(CALLS, [src, os.path.join(ROOT, "include", "cast.h"), os.path.abspath(__file__)]):
+        return
     inc, lib = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
     cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
     cmd = ["g++", "-shared", "-fPIC", "-O2", "-std=c++17", "-fvisibility=hidden", "-I", os.path.join(ROOT, "include"),
@@ -51,6 +62,8 @@ def _build_calls() -> None:
     if r.returncode != 0:
         sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
         raise RuntimeError("g++ failed for binding_calls.cpp")
+    with open(stamp, "w") as f:
+        f.write(against)
 
 
 def build(verbose: bool = False, force: bool = False) -> str:
