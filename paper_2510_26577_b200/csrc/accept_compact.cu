@@ -7,40 +7,6 @@ using namespace cast;
 
 namespace {
 
-// One 16-byte vector of logits: its largest element, and the place of the first element equal to a value.
-// (NaN is dropped by the maxima, as by a comparison; -0 and +0 compare equal.)
-template <typename T> struct Vec;
-template <> struct Vec<float> {
-  static constexpr int N = 4;
-  static __device__ __forceinline__ float max(const uint4& a) {
-    return fmaxf(fmaxf(__uint_as_float(a.x), __uint_as_float(a.y)), fmaxf(__uint_as_float(a.z), __uint_as_float(a.w)));
-  }
-  static __device__ __forceinline__ float get(const uint4& a, int e) {
-    return __uint_as_float(e == 0 ? a.x : e == 1 ? a.y : e == 2 ? a.z : a.w);
-  }
-  static __device__ __forceinline__ uint32_t minus_inf() { return 0xff800000u; }
-  static __device__ __forceinline__ void put(uint4& a, int e, float x) { (&a.x)[e] = __float_as_uint(x); }
-};
-template <> struct Vec<__nv_bfloat16> {
-  static constexpr int N = 8;
-  static __device__ __forceinline__ float max(const uint4& a) {
-    auto pair = [](uint32_t w) { return *reinterpret_cast<const __nv_bfloat162*>(&w); };
-    const __nv_bfloat162 m = __hmax2(__hmax2(pair(a.x), pair(a.y)), __hmax2(pair(a.z), pair(a.w)));
-    const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
-    return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-  }
-  static __device__ __forceinline__ float get(const uint4& a, int e) {
-    const uint32_t w = (e >> 1) == 0 ? a.x : (e >> 1) == 1 ? a.y : (e >> 1) == 2 ? a.z : a.w;
-    return __uint_as_float((e & 1) ? (w & 0xffff0000u) : (w << 16));
-  }
-  static __device__ __forceinline__ uint32_t minus_inf() { return 0xff80ff80u; }
-  static __device__ __forceinline__ void put(uint4& a, int e, float x) {
-    uint32_t& w = (&a.x)[e >> 1];
-    const uint32_t h = __float_as_uint(x) >> 16;  // (x came from a bf16)
-    w = (e & 1) ? ((w & 0xffffu) | (h << 16)) : ((w & 0xffff0000u) | h);
-  }
-};
-
 constexpr int kArgThreads = 256;
 constexpr int kArgUnroll = 8;
 
@@ -71,7 +37,7 @@ __global__ void __launch_bounds__(kArgThreads) argmax_sweep_kernel(const T* __re
   const T* xa = x - shift;  // 16-byte aligned; token id = element - shift
   const int begin = chunk * chunk_elems;
   const int end = min(begin + chunk_elems, V + shift);
-  const uint32_t none = Vec<T>::minus_inf();
+  const uint32_t none = Vec<T>::kMinusInf;
   float best = -INFINITY;
   int bvec = -1;  // first element of the best vector
   uint4 braw = make_uint4(none, none, none, none);

@@ -169,4 +169,58 @@ __device__ __forceinline__ int select_grid(int c, int L, int M) {
 __device__ __forceinline__ float to_float(float x) { return x; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
 
+// Sixteen raw bytes of logits, kept as loaded and unpacked on use. (NaN is dropped by the maxima, as by a comparison; -0 and
+// +0 compare equal.)
+template <typename T> struct Vec;
+template <> struct Vec<float> {
+  static constexpr int N = 4;
+  static constexpr uint32_t kMinusInf = 0xff800000u;
+  static __device__ __forceinline__ float max(const uint4& a) {
+    return fmaxf(fmaxf(__uint_as_float(a.x), __uint_as_float(a.y)), fmaxf(__uint_as_float(a.z), __uint_as_float(a.w)));
+  }
+  static __device__ __forceinline__ void unpack(const uint4& a, float (&x)[4]) {
+    x[0] = __uint_as_float(a.x); x[1] = __uint_as_float(a.y); x[2] = __uint_as_float(a.z); x[3] = __uint_as_float(a.w);
+  }
+  static __device__ __forceinline__ float get(const uint4& a, int e) {
+    return __uint_as_float(e == 0 ? a.x : e == 1 ? a.y : e == 2 ? a.z : a.w);
+  }
+  static __device__ __forceinline__ void put(uint4& a, int e, float x) { (&a.x)[e] = __float_as_uint(x); }
+};
+template <> struct Vec<__nv_bfloat16> {
+  static constexpr int N = 8;
+  static constexpr uint32_t kMinusInf = 0xff80ff80u;
+  static __device__ __forceinline__ float max(const uint4& a) {
+    auto pair = [](uint32_t w) { return *reinterpret_cast<const __nv_bfloat162*>(&w); };
+    const __nv_bfloat162 m = __hmax2(__hmax2(pair(a.x), pair(a.y)), __hmax2(pair(a.z), pair(a.w)));
+    const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
+    return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+  }
+  static __device__ __forceinline__ void unpack(const uint4& a, float (&x)[8]) {
+    const uint32_t w[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {  // bf16 -> fp32 is a 16-bit shift
+      x[2 * i] = __uint_as_float(w[i] << 16);
+      x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+  }
+  static __device__ __forceinline__ float get(const uint4& a, int e) {
+    const uint32_t w = (e >> 1) == 0 ? a.x : (e >> 1) == 1 ? a.y : (e >> 1) == 2 ? a.z : a.w;
+    return __uint_as_float((e & 1) ? (w & 0xffff0000u) : (w << 16));
+  }
+  static __device__ __forceinline__ void put(uint4& a, int e, float x) {
+    uint32_t& w = (&a.x)[e >> 1];
+    const uint32_t h = __float_as_uint(x) >> 16;  // (x came from a bf16)
+    w = (e & 1) ? ((w & 0xffffu) | (h << 16)) : ((w & 0xffff0000u) | h);
+  }
+};
+
+// a / b for a >= 0 and b >= 1 through the fp32 reciprocal with one correction step: an integer division by a run-time divisor
+// is a chain of well over 100 cycles. Right for a < 2^22 with inv_b = 1 / b, and for a < 2^20 with a reciprocal that is good
+// to a few ulp (__fdividef): the quotient is then off by less than one.
+__device__ __forceinline__ int div_small(int a, int b, float inv_b) {
+  const int q = (int)((float)a * inv_b);
+  const int r = a - q * b;
+  return q + (r >= b ? 1 : 0) - (r < 0 ? 1 : 0);
+}
+
 }  // namespace cast

@@ -35,7 +35,8 @@ constexpr int kPT = 64;   // positions per tile
 constexpr int kThreads = 256;
 constexpr int kMaxSplit = 64;
 constexpr int kMergeHere = 16;  // up to this many splits the last CTA merges (a second launch costs 4 us)
-constexpr size_t kCcTicketBytes = (size_t)CAST_MAX_BATCH * 512 * sizeof(int32_t);
+// A ticket per row block of a split launch, of which there are at most kOwn / 2 per SM: room for 4096 SMs.
+constexpr size_t kCcTicketBytes = (size_t)32768 * sizeof(int32_t);
 
 struct AttnParams {
   const void* q;
@@ -472,7 +473,6 @@ CcPlan cc_plan(const cast_ctx* c, int per_sm, int B, int Hq, int Hkv, int D, int
       nsplit = n;
     }
   }
-  if ((size_t)base * sizeof(int32_t) > kCcTicketBytes) nsplit = 1;
   pl.nsplit = nsplit;
   pl.bytes = nsplit == 1 ? 0 : kCcTicketBytes + (size_t)base * nsplit * kRB * (D + 2) * sizeof(float);
   return pl;

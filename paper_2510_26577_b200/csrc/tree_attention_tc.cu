@@ -467,13 +467,6 @@ __device__ __forceinline__ uint4 ld_cluster_u4(uint32_t addr) {
   return v;
 }
 
-// a / b for 0 <= a < 2^22, inv_b = 1 / b: an integer division by a run-time divisor is a chain of well over 100 cycles
-__device__ __forceinline__ int div_small(int a, int b, float inv_b) {
-  int q = (int)((float)a * inv_b);
-  const int r = a - q * b;
-  return q + (r >= b ? 1 : 0) - (r < 0 ? 1 : 0);
-}
-
 // The merge of a row's splits: split s weighs sum_s * e^(max_s - max). Half a warp merges ROWS rows of at most SPL splits
 // (ROWS * SPL <= 16) at a time; its lane u * SPL + s holds row u's split s, so one load and two short butterflies give the
 // weights of all the rows (a butterfly over the whole warp for each row, and a branch on each weight, made the merge of two

@@ -56,43 +56,6 @@ struct ExpandParams {
   const int32_t* kv_len;
 };
 
-// Sixteen raw bytes of logits: a thread's sweep buffers hold them as loaded and unpack on use.
-template <typename T> struct Vec;
-template <> struct Vec<float> {
-  static constexpr int N = 4;
-  static constexpr uint32_t kMinusInf = 0xff800000u;
-  static __device__ __forceinline__ float max(const uint4& a) {
-    return fmaxf(fmaxf(__uint_as_float(a.x), __uint_as_float(a.y)), fmaxf(__uint_as_float(a.z), __uint_as_float(a.w)));
-  }
-  static __device__ __forceinline__ void unpack(const uint4& a, float (&x)[4]) {
-    x[0] = __uint_as_float(a.x); x[1] = __uint_as_float(a.y); x[2] = __uint_as_float(a.z); x[3] = __uint_as_float(a.w);
-  }
-  static __device__ __forceinline__ void put(uint4& a, int e, float x) { (&a.x)[e] = __float_as_uint(x); }
-};
-template <> struct Vec<__nv_bfloat16> {
-  static constexpr int N = 8;
-  static constexpr uint32_t kMinusInf = 0xff80ff80u;
-  static __device__ __forceinline__ float max(const uint4& a) {
-    auto pair = [](uint32_t w) { return *reinterpret_cast<const __nv_bfloat162*>(&w); };
-    const __nv_bfloat162 m = __hmax2(__hmax2(pair(a.x), pair(a.y)), __hmax2(pair(a.z), pair(a.w)));
-    const uint32_t w = *reinterpret_cast<const uint32_t*>(&m);
-    return fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-  }
-  static __device__ __forceinline__ void unpack(const uint4& a, float (&x)[8]) {
-    const uint32_t w[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {  // bf16 -> fp32 is a 16-bit shift
-      x[2 * i] = __uint_as_float(w[i] << 16);
-      x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-    }
-  }
-  static __device__ __forceinline__ void put(uint4& a, int e, float x) {
-    uint32_t& w = (&a.x)[e >> 1];
-    const uint32_t h = __float_as_uint(x) >> 16;  // (x came from a bf16)
-    w = (e & 1) ? ((w & 0xffffu) | (h << 16)) : ((w & 0xffff0000u) | h);
-  }
-};
-
 __device__ __forceinline__ float ex2f(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -196,17 +159,6 @@ __device__ __forceinline__ bool take_ticket(int32_t* counter, int expected, int*
 constexpr int kTailScratch = 28672;  // bytes of shared memory the tail works in
 // Up to this many sequences, or candidates, the one-CTA tail is faster than a second ticket (V = 32000, 8 sequences: 92 -> 89 us).
 constexpr int kTailSingleMaxB = 8, kTailAlwaysSingleB = 4, kTailSingleCands = 512;
-
-// a / b for 0 <= a < 2^20 and 1 <= b <= 2^10 through the fp32 reciprocal (inv_b, to a few ulp) with one correction step:
-// the integer division by a run-time divisor is some twenty instructions, and the ranking below does several per
-// thread in a phase whose time is what its instructions take to issue.
-__device__ __forceinline__ int div_small(int a, int b, float inv_b) {
-  int q = (int)((float)a * inv_b);
-  const int r = a - q * b;
-  q += (r >= b) ? 1 : 0;
-  q -= (r < 0) ? 1 : 0;
-  return q;
-}
 
 // Candidates Algorithm 1 looks at: the first n of the sorted list.
 __device__ __forceinline__ int tail_width(const ExpandParams& p, int n_prev) {
@@ -548,29 +500,30 @@ __device__ __forceinline__ void tail_decide(const ExpandParams& p, const TailSta
 // best come from K rounds of a warp-wide maximum. What reaches the threshold is never dropped except for K better
 // ones, and every threshold is at most the K-th largest: the chunk's top K is always among the lists.
 constexpr int kBufVecs = 4;     // 16-byte vectors per thread and buffer
-constexpr int kGroups = 16;     // parts of a CTA whose maxima give the threshold: its warps, or half warps
+constexpr int kGroups = kSweepThreads / 32;  // parts of a CTA whose maxima give the threshold: its warps
 constexpr int kListCap = 64;    // keys per warp list
 constexpr int kPushCap = 32;    // keys a warp hands on at most
+static_assert(kGroups == 16, "a group's number takes the last four bits of its maximum");
 static_assert(CAST_MAX_TOP_K <= kGroups, "the K-th largest of the groups' maxima needs K <= groups");
 static_assert(CAST_MAX_TOP_K <= kPushCap, "a warp hands on its K best");
 
 // OUT: the overflow handling is a function of its own. Inlined twice it is half of the sweep's code, and in the short launches,
 // which run everything once, the warps wait for instructions (1-2 us per tree); in the 64-register launches the call costs
 // more registers than there are (batch 64 307 -> 329 us).
-template <typename T, int NT, bool OUT>
+template <typename T, bool OUT>
 struct Sweep {
   static constexpr int VEC = Vec<T>::N;
   static constexpr int kSlots = kBufVecs * VEC;                      // logits of a thread per buffer
-  static constexpr int kBufElems = NT * kSlots;                      // of the CTA
+  static constexpr int kBufElems = kSweepThreads * kSlots;                      // of the CTA
   uint4 raw[kBufVecs];
 
   // First element (of the aligned view) of this thread's vector v in the buffer that starts at `base`.
-  static __device__ __forceinline__ int elem(int base, int v) { return base + (v * NT + (int)threadIdx.x) * VEC; }
+  static __device__ __forceinline__ int elem(int base, int v) { return base + (v * kSweepThreads + (int)threadIdx.x) * VEC; }
 
   // A whole buffer; `at`: this thread's first vector of it. (One address per buffer, the rest are immediate offsets.)
   __device__ __forceinline__ void load(const uint4* at) {
 #pragma unroll
-    for (int v = 0; v < kBufVecs; ++v) raw[v] = __ldcs(at + v * NT);
+    for (int v = 0; v < kBufVecs; ++v) raw[v] = __ldcs(at + v * kSweepThreads);
   }
   // A buffer that is not all there. xa: the row from the 16-byte boundary at or below its start; elements [lo, end) of it
   // exist.
@@ -591,7 +544,7 @@ struct Sweep {
     }
   }
   static __device__ __forceinline__ int slot_elem(int base, int i) {
-    return base + ((i / VEC) * NT + (int)threadIdx.x) * VEC + (i % VEC);
+    return base + ((i / VEC) * kSweepThreads + (int)threadIdx.x) * VEC + (i % VEC);
   }
   // the logit of slot i (not a constant)
   __device__ __forceinline__ float slot(int i) const {
@@ -752,15 +705,16 @@ struct Sweep {
   }
 };
 
+__device__ __forceinline__ float warp_max(float x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  return x;
+}
 // A thread's share in the groups' maxima, which go to shared memory as integers: the value's ordered bits, the last four
 // replaced by the group's number, so that they are distinct and one comparison orders two of them.
-template <int NT>
 __device__ __forceinline__ void group_max(float x, uint32_t* v) {
-  constexpr int kLanes = NT / kGroups;
-  static_assert(kLanes == 32 || kLanes == 16, "groups are warps or half warps");
-#pragma unroll
-  for (int o = kLanes / 2; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-  if ((threadIdx.x & (kLanes - 1)) == 0) v[threadIdx.x / kLanes] = (ordered_bits(x) & ~15u) | (threadIdx.x / kLanes);
+  x = warp_max(x);
+  if ((threadIdx.x & 31) == 0) v[threadIdx.x >> 5] = (ordered_bits(x) & ~15u) | (threadIdx.x >> 5);
 }
 // The K-th largest of the groups' maxima, rounded down in its last bits: still a lower bound on the K-th largest of the
 // logits. At least -FLT_MAX. (Every warp for itself.)
@@ -775,19 +729,14 @@ __device__ __forceinline__ float kth_of_groups(const uint32_t* v, int K) {
   const unsigned who = __ballot_sync(0xffffffffu, r == K - 1);
   return fmaxf(from_ordered_bits(__shfl_sync(0xffffffffu, mine, __ffs(who) - 1) & ~15u), -3.402823466e38f);
 }
-__device__ __forceinline__ float warp_max(float x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
-}
 
 // MINB = 2 compiles the same code for two CTAs per SM (half the registers): for launches with more CTAs than
 // SMs, where a second resident CTA hides the first one's latencies; MINB = 1 is for the short launches.
-template <typename T, int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) {
+template <typename T, int MINB>
+__global__ void __launch_bounds__(kSweepThreads, MINB) expand_kernel(const ExpandParams p) {
   // filled in the first CTA of the row's cluster by all CTAs of the cluster: chunk c's candidate keys, and per warp of
   // chunk c its maximum (log2 units) and sum of 2^(. - maximum); later the tail's arrays
-  constexpr int kWarps = NT / 32, kChunkCap = kWarps * kPushCap;
+  constexpr int kWarps = kSweepThreads / 32, kChunkCap = kWarps * kPushCap;
   __shared__ __align__(16) unsigned char scratch[kSweepMaxChunks * kChunkCap * 8 > kTailScratch ? kSweepMaxChunks * kChunkCap * 8 : kTailScratch];
   __shared__ float row_max[kSweepMaxChunks * kWarps];
   __shared__ double row_sum[kSweepMaxChunks * kWarps];
@@ -811,7 +760,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
   DevState* st = p.st;
   const int K = p.K;
   const int row = b * p.W + r;
-  using S = Sweep<T, NT, MINB == 1>;
+  using S = Sweep<T, MINB == 1>;
   constexpr int E = S::kBufElems;
   // the row from the 16-byte boundary at or below its start: its tokens are elements [shift, V + shift) of that view
   const T* x = reinterpret_cast<const T*>(p.logits) + (size_t)row * p.V;
@@ -834,7 +783,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
     const char* cb = reinterpret_cast<const char*>(chunk == 0 ? x : xa + begin);
     const int bytes = (int)(reinterpret_cast<const char*>(xa + end) - cb);
 #pragma unroll 1
-    for (int off = tid * 128; off < bytes; off += NT * 128)
+    for (int off = tid * 128; off < bytes; off += kSweepThreads * 128)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(cb + off));
   }
   grid_dependency_wait();
@@ -842,7 +791,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
   // the first logits are requested before the state is read (every row r < W exists in memory): one memory round trip
   S q0, q1;
   const uint4* at_mine = reinterpret_cast<const uint4*>(xa + begin) + tid;  // this thread's place in buffer `at`
-  constexpr int kStep = kBufVecs * NT;                                       // vectors per buffer
+  constexpr int kStep = kBufVecs * kSweepThreads;                                       // vectors per buffer
   if (begin >= shift && begin + 2 * E <= end) {
     q0.load(at_mine);
     q1.load(at_mine + kStep);
@@ -893,7 +842,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
     else if (at + 2 * E < end) q.load_part(xa, at + 2 * E, shift, end);
   };
   auto threshold = [&](float m, uint32_t* g) {
-    group_max<NT>(m, g);
+    group_max(m, g);
     __syncthreads();
     return kth_of_groups(g, K);
   };
@@ -980,7 +929,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
   }();
   if (tid < K) topk[tid] = 0ull;
   {
-    constexpr int kLanes = NT / kSweepMaxChunks;  // threads per chunk: whole warps
+    constexpr int kLanes = kSweepThreads / kSweepMaxChunks;  // threads per chunk: whole warps
     static_assert(kLanes % 32 == 0, "a warp looks at one chunk");
     const int c = tid / kLanes, nc = c < p.nchunks ? row_n[c] : 0;
 #pragma unroll 1
@@ -1043,7 +992,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
 #pragma unroll 1
     for (int c1 = 0; c1 < p.nchunks; ++c1)
 #pragma unroll 1
-      for (int i = tid; i < row_n[c1]; i += NT - 32) {
+      for (int i = tid; i < row_n[c1]; i += kSweepThreads - 32) {
         const unsigned long long key = row_keys[c1 * kChunkCap + i];
         int cnt = 0;
 #pragma unroll 1
@@ -1055,7 +1004,7 @@ __global__ void __launch_bounds__(NT, MINB) expand_kernel(const ExpandParams p) 
   }
   __syncthreads();
   if (packed) {
-    for (int i = tid; i < total; i += NT)
+    for (int i = tid; i < total; i += kSweepThreads)
       if (-rank_s[i] < K) topk[-rank_s[i]] = wlist[i];
     __syncthreads();
   }
@@ -1483,10 +1432,10 @@ extern "C" cast_status cast_tree_expand(cast_ctx* c, int layer, const void* draf
   cfg.numAttrs = 2;
   cudaError_t e;
   if (dtype == CAST_F32)
-    e = queued ? cudaLaunchKernelEx(&cfg, expand_kernel<float, 512, 2>, p) : cudaLaunchKernelEx(&cfg, expand_kernel<float, 512, 1>, p);
+    e = queued ? cudaLaunchKernelEx(&cfg, expand_kernel<float, 2>, p) : cudaLaunchKernelEx(&cfg, expand_kernel<float, 1>, p);
   else
-    e = queued ? cudaLaunchKernelEx(&cfg, expand_kernel<__nv_bfloat16, 512, 2>, p)
-               : cudaLaunchKernelEx(&cfg, expand_kernel<__nv_bfloat16, 512, 1>, p);
+    e = queued ? cudaLaunchKernelEx(&cfg, expand_kernel<__nv_bfloat16, 2>, p)
+               : cudaLaunchKernelEx(&cfg, expand_kernel<__nv_bfloat16, 1>, p);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return CAST_ERR_CUDA;
