@@ -102,7 +102,7 @@ extern "C" cast_status cast_create(const cast_config* cfg, cast_ctx** out) {
   if (e == cudaSuccess) e = dev_alloc(&c->lsort, BP);
   if (e == cudaSuccess) e = dev_alloc(&c->lscore, BP);
   if (e == cudaSuccess) e = dev_alloc(&c->state, 1);
-  if (e == cudaSuccess) e = dev_alloc(&c->attn_worklist, (size_t)kAttnWorkListCap * 8);
+  if (e == cudaSuccess) e = dev_alloc(&c->attn_worklist, (size_t)kAttnWorkListCap * 8 + 2 * CAST_MAX_BATCH);
   if (e == cudaSuccess) e = dev_alloc(&c->layer_ticket, 1);
   if (e == cudaSuccess) e = dev_alloc(&c->seq_ticket, cfg->max_batch);
   if (e == cudaSuccess) e = dev_alloc(&c->tail_vs, (size_t)cfg->max_batch * CAST_MAX_WIDTH);

@@ -117,7 +117,7 @@ struct cast_ctx {
   // work list of the tensor-core attention (one decoded item per CTA), written by a small kernel at the first
   // attention call after the tree or the lengths changed and reused by the calls that follow while the promise
   // above holds and the call's shape is the same (wl_key)
-  int32_t* attn_worklist;          // [kAttnWorkListCap][8]
+  int32_t* attn_worklist;          // [kAttnWorkListCap][8], then the [2][CAST_MAX_BATCH] n_tree and kv_len it was decoded from
   int wl_valid;
   unsigned long long wl_key[8];
 

@@ -87,6 +87,7 @@ struct TcParams {
   int B, Ncap, Nmax, Hq, Hkv, G, page_size, seq_capacity, num_pages, words;
   int q_tma;  // Q row blocks are fetched by TMA (the group size divides 128)
   const int32_t* worklist;  // one decoded work item per CTA (8 ints each), or null: every CTA decodes for itself
+  const int32_t* wl_sizes;  // [2][CAST_MAX_BATCH] the n_tree and kv_len that the list was decoded from, or null: it holds
   int early;  // the tree arrays, lengths, page table and prefix rows may be read before the dependency wait
   int tmem_first;  // tensor memory may be taken before the dependency wait (see the kernel)
   int cs;   // CTAs per cluster (1..8); 0: no clusters, splits sized on the device and merged through global memory
@@ -730,8 +731,31 @@ __device__ __forceinline__ WorkItem load_item(const int32_t* src) {
   w.N = a.z; w.L = a.w; w.F = f;
   return w;
 }
+// Whether the list was decoded from the sizes that stand now (the whole warp calls; the same answer everywhere). One round
+// trip to memory, at the time of the item's own.
+__device__ __forceinline__ bool list_holds(const TcParams& p) {
+  constexpr int KB = CAST_MAX_BATCH / 32;
+  int32_t now[KB][2], then[KB][2];
+#pragma unroll
+  for (int k = 0; k < KB; ++k) {
+    const int b = k * 32 + (threadIdx.x & 31);
+    const bool in = b < p.B;
+    now[k][0] = in ? p.n_tree[b] : 0;
+    now[k][1] = in ? p.kv_len[b] : 0;
+    then[k][0] = in ? p.wl_sizes[b] : 0;
+    then[k][1] = in ? p.wl_sizes[CAST_MAX_BATCH + b] : 0;
+  }
+  int32_t off = 0;
+#pragma unroll
+  for (int k = 0; k < KB; ++k) off |= (now[k][0] ^ then[k][0]) | (now[k][1] ^ then[k][1]);
+  return __all_sync(0xffffffffu, off == 0);
+}
 // The work decode of every CTA of a launch, done once: warp i decodes what CTA i would decode for itself.
-__global__ void __launch_bounds__(256) attn_worklist_kernel(const TcParams p, int grid, int32_t* list) {
+__global__ void __launch_bounds__(256) attn_worklist_kernel(const TcParams p, int grid, int32_t* list, int32_t* sizes) {
+  if (blockIdx.x == 0 && (int)threadIdx.x < p.B) {
+    sizes[threadIdx.x] = p.n_tree[threadIdx.x];
+    sizes[CAST_MAX_BATCH + threadIdx.x] = p.kv_len[threadIdx.x];
+  }
   const int idx = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5);
   if (idx >= grid) return;
   const WorkItem w = p.cs == 0 ? decode_work_chunked(p, idx, grid) : decode_work(p, idx / p.cs, idx % p.cs);
@@ -795,9 +819,13 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     if (!p.tmem_first) tmem_take();
     if (warp == 4) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
-  const WorkItem wk = p.worklist != nullptr ? load_item(p.worklist + (size_t)blockIdx.x * 8)
-                      : cs == 0            ? decode_work_chunked(p, (int)blockIdx.x, (int)gridDim.x)
-                                           : decode_work(p, (int)blockIdx.x / cs, crank);
+  WorkItem wk;
+  bool listed = false;
+  if (p.worklist != nullptr) {
+    wk = load_item(p.worklist + (size_t)blockIdx.x * 8);
+    listed = p.wl_sizes == nullptr || list_holds(p);
+  }
+  if (!listed) wk = cs == 0 ? decode_work_chunked(p, (int)blockIdx.x, (int)gridDim.x) : decode_work(p, (int)blockIdx.x / cs, crank);
   if (blockIdx.x < p.B && tid == 0 && p.n_tree[blockIdx.x] > p.Nmax) report(p.st, CAST_ERR_BAD_TREE, blockIdx.x);
   if (!wk.valid) {
     tmem_return();
@@ -1546,10 +1574,10 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
     p.part_ml = reinterpret_cast<float*>(p.part_o + pl.rows * kPartRow);
   }
   // The work list: under the caller's promise the lengths and tree sizes do not change between the attention
-  // calls of a step, so what every CTA would decode for itself is decoded once, by a small kernel launched in
+  // calls of a step (outside it they hardly ever do), so what every CTA would decode for itself is decoded once, by a small kernel launched in
   // front of the first such call (or when the call's shape changes), and the calls after it read one item each.
-  p.worklist = nullptr;
-  if (promised && first_row == nullptr && grid <= kAttnWorkListCap) {  // (a window call names new sizes every time)
+  p.worklist = p.wl_sizes = nullptr;
+  if (c->attn_early && first_row == nullptr && grid <= kAttnWorkListCap) {  // (a window call names new sizes every time)
     const unsigned long long key[8] = {(unsigned long long)(uintptr_t)n_tree, (unsigned long long)(uintptr_t)kv_len,
                                        (unsigned long long)(uintptr_t)first_row,
                                        ((unsigned long long)B << 48) | ((unsigned long long)Hq << 32) | ((unsigned long long)Hkv << 16) | (unsigned)page_size,
@@ -1559,7 +1587,7 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
     bool same = c->wl_valid != 0;  // (the caller of this function has discarded it where the tree or the lengths are new)
     for (int i = 0; i < 8 && same; ++i) same = c->wl_key[i] == key[i];
     if (!same) {
-      attn_worklist_kernel<<<(unsigned)((grid + 7) / 8), 256, 0, stream>>>(p, (int)grid, c->attn_worklist);
+      attn_worklist_kernel<<<(unsigned)((grid + 7) / 8), 256, 0, stream>>>(p, (int)grid, c->attn_worklist, c->attn_worklist + (size_t)kAttnWorkListCap * 8);
       if (cudaGetLastError() != cudaSuccess) { *status = CAST_ERR_CUDA; return true; }
       for (int i = 0; i < 8; ++i) c->wl_key[i] = key[i];
       c->wl_valid = 1;
@@ -1567,6 +1595,10 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
       p.tmem_first = 1;  // (that kernel has no tensor memory, and as a plain launch it ran after all that was before it)
     }
     p.worklist = c->attn_worklist;
+    // It holds when this call has just launched it, or by the promise. For the shapes outside the promise every CTA compares
+    // the sizes and decodes for itself where they differ (64 dims, us per layer, decoding always / comparing / trusting:
+    // one sequence of 1024 9.4 / 8.8 / 8.6, 64 of 512-1024 41.0 / 34.0 / 33.3; in early mode comparing would cost 0.3 of 11.9).
+    p.wl_sizes = p.tmem_first ? nullptr : c->attn_worklist + (size_t)kAttnWorkListCap * 8;
   }
   auto* const kern = D == 64 ? tree_attn_tc_kernel<64> : tree_attn_tc_kernel<128>;
   const int smem_bytes = D == 64 ? Geo<64>::kSmemBytes : Geo<128>::kSmemBytes;
