@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(CAST_MAX_TREE) accept_walk_kernel(
       bonus[b] = 0;
       for (int j = 0; j <= H; ++j) accept_path[b * (H + 1) + j] = -1;
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // (the launch must not be over before the sweep is)
     return;
   }
   // the tree arrays were written before the sweep was launched; the sweep's winners are read after the wait

@@ -1,5 +1,5 @@
-"""What must not be tried on a GPU, because getting it wrong is a wait without end: the order of the tensor-memory
-allocation, the dependency wait and the release of the dependents in the tensor-core attention, read from its source.
+"""What must not be tried on a GPU, because getting it wrong is a wait without end or a race: the order of the tensor-memory
+allocation, the dependency wait and the release of the dependents, read from the kernels' source.
 
 A block that holds tensor memory while it waits for its predecessor is waited for by a predecessor on the same SM that
 released its dependents before it allocated. So the default mode allocates behind the wait, an allocation ahead of it
@@ -7,12 +7,11 @@ needs a reason the host gives, and the kernel itself releases its dependents beh
 import os
 import re
 
-SRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2510_26577_b200", "csrc",
-                   "tree_attention_tc.cu")
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2510_26577_b200", "csrc")
 
 
-def _source():
-    text = re.sub(r"/\*.*?\*/", "", open(SRC).read(), flags=re.S)
+def _source(name="tree_attention_tc.cu"):
+    text = re.sub(r"/\*.*?\*/", "", open(os.path.join(CSRC, name)).read(), flags=re.S)
     return re.sub(r"//[^\n]*", "", text)
 
 
@@ -57,6 +56,12 @@ def test_a_launch_without_work_waits_for_its_predecessor():
     idle = _body(kernel, "if (!wk.valid)")
     assert re.search(r"if \(early && blockIdx\.x == 0\) asm volatile\(\"griddepcontrol\.wait;", idle)
     assert idle.index("tmem_return()") < idle.index("griddepcontrol.wait") < idle.index("return;", idle.index("griddepcontrol"))
+
+
+def test_the_acceptance_walk_waits_for_the_sweep_in_refused_sequences_too():
+    walk = _body(_source("accept_compact.cu"), "accept_walk_kernel(")
+    refused = _body(walk, "if (N < 1)")
+    assert 0 < refused.index("griddepcontrol.wait") < refused.rindex("return;")
 
 
 def test_who_may_take_it_ahead_of_the_wait():
