@@ -1602,15 +1602,14 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   }
   auto* const kern = D == 64 ? tree_attn_tc_kernel<64> : tree_attn_tc_kernel<128>;
   const int smem_bytes = D == 64 ? Geo<64>::kSmemBytes : Geo<128>::kSmemBytes;
-  static bool attr_done[2] = {false, false};
-  if (!attr_done[D == 64]) {
+  if (!c->attn_attr_set[D == 64]) {  // (a function's attributes belong to the device, as the context does)
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess) {
       *status = CAST_ERR_CUDA;
       return true;
     }
     // two CTAs per SM need the largest shared-memory carve-out
     cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    attr_done[D == 64] = true;
+    c->attn_attr_set[D == 64] = 1;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);

@@ -1,4 +1,4 @@
-"""What must not be tried on a GPU, because getting it wrong is a wait without end or a race: the order of the tensor-memory
+"""What cannot be tried on one GPU, or must not be, because getting it wrong is a wait without end or a race: the order of the tensor-memory
 allocation, the dependency wait and the release of the dependents, read from the kernels' source.
 
 A block that holds tensor memory while it waits for its predecessor is waited for by a predecessor on the same SM that
@@ -69,3 +69,9 @@ def test_who_may_take_it_ahead_of_the_wait():
     launch = _body(_source(), "bool tree_attention_tc_launch(")
     assert re.findall(r"p\.tmem_first = ([^;]*);", launch) == ["p.early", "1"]
     assert re.search(r"attn_worklist_kernel<<<.*?p\.early = 0;\s*p\.tmem_first = 1;", launch, flags=re.S)
+
+
+def test_kernel_attributes_are_remembered_per_context():
+    """They hold for one device: a process that drives two has a context on each."""
+    launch = _body(_source(), "bool tree_attention_tc_launch(")
+    assert "cudaFuncSetAttribute" in launch and not re.search(r"\bstatic\b", launch)
