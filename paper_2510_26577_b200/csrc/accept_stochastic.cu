@@ -21,8 +21,7 @@
 // each). Hence: no pass for the maximum (fp64 has the exponent range to sum exp(logit / T) as it is; the row is
 // evaluated again against its maximum only if the sum leaves 1e-280 .. 1e280), one exchange per node and per rejection
 // and none for the bonus token, whose segment sums are those of the last exchange.
-// Measured (T = 0.8, trees of 24, V = 128256 fp32; before: a maximum pass, 200 KB of cached values per CTA, clusters of 16
-// only, an exchange for the bonus token): 1 sequence 58 -> 38 us, 8: 100 -> 63, 16: 137 -> 76, 64: 481 -> 231.
+// Measured (T = 0.8, trees of 24, V = 128256 fp32): 1 sequence 38 us, 8 63, 16 76, 64 231.
 #include <math.h>
 
 #include "cast_internal.h"
@@ -34,7 +33,10 @@ namespace {
 constexpr int kStoThreads = 512;
 constexpr int kStoWarps = kStoThreads / 32;
 constexpr int kStoMaxCluster = 16;
-constexpr int kStoMaxSlice = 12288;  // vocabulary entries per CTA of a cluster of 16 up to which segments are cached
+// Vocabulary entries per CTA up to which the plan caches segments (196 608 tokens in clusters of 16): the rule that
+// cast_accept_stochastic_plan has always answered by, set when a slice of both rows filled shared memory. The kernels hold
+// up to 38 x 512 entries now, so the times do not cross here: V = 262144, one sequence, 76 us recomputing and 41 cached.
+constexpr int kStoMaxSlice = 12288;
 
 struct StoParams {
   const void* target_logits;
@@ -64,7 +66,7 @@ __device__ __forceinline__ void sto_cluster_sync() {
 }
 
 // exp(x) for x <= 700 in fp64 to about 3e-16 relative: x = n ln2 + r with n = round(x log2 e) (ln2 split in
-// two so that n ln2_hi is exact), the degree-12 Taylor polynomial of e^r on |r| <= ln2 / 2 (remainder below
+// two so that n ln2_hi is exact: the split of fdlibm's e_exp.c), the degree-12 Taylor polynomial of e^r on |r| <= ln2 / 2 (remainder below
 // 2e-16), scaling by 2^n through the exponent field. Arguments below -708 (results near the subnormal
 // range) give 0; NaN gives NaN. For the values computed one at a time.
 __device__ __forceinline__ double sto_exp_any(double x) {
@@ -565,7 +567,8 @@ int sto_resident(int cs) {
 int elements_per_lane(int V, int cs) { return ((V + cs - 1) / cs + kStoThreads - 1) / kStoThreads; }
 
 // The kernel for `ne` elements per lane: the smallest cached one that holds them, or the one that caches nothing. Slots
-// past ne cost as much as live ones, hence the steps; 38 is what fits on chip.
+// past ne cost as much as live ones, hence the steps. 38 is what fits on chip: 76 doubles per lane, 24 of them in registers
+// and 52 in shared memory (213 KB of 227). Clusters of 16 use the steps up to 24 (kStoMaxSlice), clusters of 8 all of them.
 #define STO_PICK(T, ne, cached, call)      \
   (!(cached)    ? call<T, 0>               \
    : (ne) <= 4  ? call<T, 4>               \
@@ -602,7 +605,8 @@ cast_status sto_run(cast_ctx* c, StoParams& p, int B, int di, cudaStream_t s) {
   p.cs = c->sto_cs[di];
   const bool cached = c->sto_cached[di] != 0;
   // With more sequences than clusters of 16 run at once, clusters of 8: a node takes less than twice as long (the chain of
-  // exchanges does not grow) and twice as many sequences run.
+  // exchanges does not grow) and twice as many sequences run. Only where those hold the segments as well (155 648 tokens):
+  // 16 sequences of V = 190000 take 82 us in clusters of 16 one after the other, 207 recomputing in clusters of 8.
   if (p.cs == 16 && B > c->sto_resident[di] && (!cached || elements_per_lane(p.V, 8) <= kStoMaxCached)) p.cs = 8;
   p.ne = elements_per_lane(p.V, p.cs);
   return STO_PICK(T, p.ne, cached, sto_launch)(p, B, s);

@@ -1,7 +1,7 @@
 // cast_tree_attention: tree-masked verification attention.
 //
-// CUDA-core path (fp32 inputs, and bf16 caches the tensor-core path does not take: pages below 8 or above 64 positions): a
-// flash-style kernel. One CTA owns (sequence, kv-head, block of 32 query rows, KV split); a
+// CUDA-core path (fp32 inputs, and bf16 caches the tensor-core path does not take: pages other than 8, 16, 32 and 64
+// positions, pointers not aligned for it): a flash-style kernel. One CTA owns (sequence, kv-head, block of 32 query rows, KV split); a
 // query row is a (tree token, head of the GQA group) pair, so a K/V tile fetched once serves
 // all tree tokens and all heads of the group. Tiles of 64 positions are converted to fp32 in
 // shared memory; S = QK^T and O += PV are register-tiled FFMA loops; the softmax is online.
@@ -9,8 +9,8 @@
 // anc_mask[t] is set. KV splits write (max, sum, unnormalised O) partials; the CTA of a row block
 // that finishes last (an atomic ticket, nothing spins) merges them, or a second kernel when they are many.
 // Bound by instruction issue, shared-memory reads of the products first: both go by 16-byte vectors, the first product by
-// packed multiply-adds (V = 60 tokens, 4 sequences of 2048, 32/8 heads of 64: 276 -> 233 us; 128 dims 511 -> 450). A 64-row
-// tile of 8 x 4 per thread was built: as fast from 200 rows per kv-head on, up to twice as slow below.
+// packed multiply-adds (60 tokens, 4 sequences of 2048, 32/8 heads of 64: 233 us, 276 without the packing; 128 dims 450 and
+// 511). A 64-row tile of 8 x 4 per thread is as fast from 200 rows per kv-head on and up to twice as slow below.
 #include <math.h>
 
 #include "cast_internal.h"

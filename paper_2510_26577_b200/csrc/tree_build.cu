@@ -152,8 +152,8 @@ __device__ __forceinline__ bool take_ticket(int32_t* counter, int expected, int*
 
 // Layer tail (Eq. 1, Eq. 2, Algorithm 1, depth pruning) in two parts. tail_rank orders the candidates of
 // some sequences and is what costs time with many sequences; tail_decide is the batch-wide rest. With up to
-// four sequences (eight, of few candidates) the last CTA of the layer runs both from shared memory; with more, the last CTA of every
-// sequence ranks that sequence (so the sequences are ranked in parallel) and leaves the first n sorted
+// four sequences (eight, of few candidates) the last CTA of the layer runs both from shared memory; with more, the last CTA
+// of every sequence ranks that sequence (so the sequences are ranked in parallel) and leaves the first n sorted
 // nodes in global memory, and the last of those CTAs decides.
 
 constexpr int kTailScratch = 28672;  // bytes of shared memory the tail works in
@@ -1365,11 +1365,11 @@ extern "C" cast_status cast_tree_expand(cast_ctx* c, int layer, const void* draf
   c->next_layer = layer + 1;
   const int B = c->cur_B, V = c->cfg.vocab;
   const int rows_per_seq = layer == 1 ? 1 : c->W;
-  // A logits row is swept by one cluster of 1 to 8 CTAs. A CTA pays for its fixed phases (prologue, chunk
-  // result, cluster barrier and row merge when there is more than one chunk: about 2.5 us, 2 without) and
-  // about 4 us per pass of kSweepSub logits, whether the pass is full or not; CTAs beyond one per SM queue
-  // up (figures fitted to the measured layer times of the benchmark shapes). The chunk count with the smallest estimate wins: few rows get many one-pass chunks (latency), many
-  // rows get few chunks of several full passes (throughput).
+  // A logits row is swept by one cluster of 1 to 8 CTAs. A CTA pays for its fixed phases (prologue, chunk result, cluster
+  // barrier and row merge when there is more than one chunk: about 2.5 us, 2 without) and about 2 us per buffer of 64 bytes a
+  // thread, whether the buffer is full or not; CTAs beyond one per SM queue up (figures fitted to the measured layer times of
+  // the benchmark shapes). The chunk count with the smallest estimate wins: few rows get many short chunks (latency), many
+  // rows get few chunks of several full buffers (throughput).
   const int rows = B * rows_per_seq;
   // (a row's aligned view starts up to one vector before the row; V % 8 == 0 keeps every row as aligned as the first)
   const int room = V + (V % 8 != 0 || ((uintptr_t)draft_logits & 15) != 0 ? 7 : 0);

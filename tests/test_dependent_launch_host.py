@@ -1,5 +1,5 @@
-"""What cannot be tried on one GPU, or must not be, because getting it wrong is a wait without end or a race: the order of the tensor-memory
-allocation, the dependency wait and the release of the dependents, read from the kernels' source.
+"""What cannot be tried on one GPU, or must not be, because getting it wrong is a wait without end or a race: the order of
+the tensor-memory allocation, the dependency wait and the release of the dependents, read from the kernels' source.
 
 A block that holds tensor memory while it waits for its predecessor is waited for by a predecessor on the same SM that
 released its dependents before it allocated. So the default mode allocates behind the wait, an allocation ahead of it
