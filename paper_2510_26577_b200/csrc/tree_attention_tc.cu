@@ -1579,7 +1579,7 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   p.worklist = p.wl_sizes = nullptr;
   if (c->attn_early && first_row == nullptr && grid <= kAttnWorkListCap) {  // (a window call names new sizes every time)
     const unsigned long long key[8] = {(unsigned long long)(uintptr_t)n_tree, (unsigned long long)(uintptr_t)kv_len,
-                                       (unsigned long long)(uintptr_t)first_row,
+                                       promised ? 1ull : 0ull,  // (a caller need not announce what it changes between other calls)
                                        ((unsigned long long)B << 48) | ((unsigned long long)Hq << 32) | ((unsigned long long)Hkv << 16) | (unsigned)page_size,
                                        ((unsigned long long)seq_capacity << 32) | (unsigned)grid,
                                        ((unsigned long long)(unsigned)p.cs << 32) | ((unsigned)p.rpc << 16) | (unsigned)p.nsplit_max,

@@ -264,8 +264,9 @@ def test_attention_reports_a_tree_beyond_total_token(binding, dtype, page, Hq, k
             assert bool(((out[b, :n].double() - want[b, :n]).abs() <= tol).all())
 
 
-def _early_setup(binding, B, cap, Hq, Hkv, D, page, kv, dtype=torch.bfloat16):
-    """A context with the early-read promise and one layer's inputs: its attention call, and the state the call reads."""
+def _early_setup(binding, B, cap, Hq, Hkv, D, page, kv, dtype=torch.bfloat16, share=None):
+    """A context with the early-read promise and one layer's inputs: its attention call, and the state the call reads.
+    share: another such context, its lengths and its tree sizes, to be used here too."""
     rng = np.random.default_rng(Hq * D)
     g = torch.Generator(device="cuda").manual_seed(Hq * D)
     seq = -(-(max(kv) + 2 * cap) // page)
@@ -273,10 +274,13 @@ def _early_setup(binding, B, cap, Hq, Hkv, D, page, kv, dtype=torch.bfloat16):
     table = torch.randperm(B * seq, generator=g, device="cuda").to(torch.int32).view(B, seq)
     q = torch.randn((B, cap, Hq, D), generator=g, device="cuda").to(dtype)
     anc = _random_trees(rng, B, cap, [cap] * B)
-    ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=cap, max_tree=cap)
+    if share is None:
+        ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=cap, max_tree=cap)
+        ctx.cast_set_attention_early_reads(True)
+        kv_len, n_tree = _ints(kv), _ints([cap] * B)
+    else:
+        ctx, kv_len, n_tree = share
     ctx.cast_reserve_attention(dtype, B, Hq, Hkv, D, page, seq)
-    ctx.cast_set_attention_early_reads(True)
-    kv_len, n_tree = _ints(kv), _ints([cap] * B)
 
     def call(first=None):
         out = torch.full_like(q, float("nan"))
@@ -365,3 +369,16 @@ def test_the_fallback_of_a_tensor_core_shape_stays_small(binding, B, Hq, Hkv, D,
     live = ~want.isnan()
     assert torch.equal(out.isnan(), ~live)
     assert bool(((out.double() - want)[live].abs() <= 1e-5 + want[live].abs() * 2.0 ** -8).all())
+
+
+def test_a_list_of_a_shape_outside_the_promise_is_not_trusted_inside(binding):
+    """64-dim heads, a change of the lengths that need not be announced there, and a layer of 128-dim heads of the same
+    call shape: it decodes its own list."""
+    ctx, call64, check64, _, kv_len, n_tree = _early_setup(binding, 2, 8, 8, 2, 64, 16, [40, 700])
+    _, call128, check128, _, _, _ = _early_setup(binding, 2, 8, 8, 2, 128, 16, [40, 700], share=(ctx, kv_len, n_tree))
+    check64(call64())
+    kv_len.copy_(_ints([333, 12]))
+    n_tree.copy_(_ints([4, 8]))
+    torch.cuda.synchronize()
+    check128(call128())
+    check64(call64())
