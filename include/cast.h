@@ -31,7 +31,7 @@
  *    Errors only the device can see (non-finite logits, a malformed tree, a
  *    page index out of range) are written to a device status word; read it with
  *    cast_poll_status, which synchronises `stream`.
- *  - cast_tree_expand, cast_select_nodes and cast_tree_attention are launched with programmatic
+ *  - cast_tree_expand, cast_select_nodes, cast_tree_attention and cast_compact_kv are launched with programmatic
  *    dependent launch: their thread blocks may become resident while the previous kernel of the
  *    stream is still finishing, but they read no input (logits, Q, K/V, tree arrays, lengths) before
  *    that kernel has completed, so stream order keeps its usual meaning for the caller. They hold no tensor memory
@@ -318,7 +318,8 @@ CAST_API cast_status cast_accept_stochastic(cast_ctx* ctx, const void* target_lo
  * How cast_accept_stochastic organises its launch for this context's vocabulary and a logits dtype
  * (host-side query; no device work): the thread-block cluster size per sequence (16 where the
  * device can co-schedule that many CTAs with their shared memory, else 8, else 1; with more sequences
- * than clusters of 16 run at once the launch takes clusters of 8) and whether a
+ * than clusters of 16 run at once the launch takes clusters of 8, unless only clusters of 16 hold the
+ * vocabulary on chip) and whether a
  * CTA's vocabulary slice is cached on chip (1) or every sweep recomputes it from the logits (0).
  * cast_accept_stochastic makes this query itself on its first call; call it before a stream capture.
  */
