@@ -85,7 +85,9 @@ struct TcParams {
   const __nv_bfloat16* q;
   __nv_bfloat16* out;
   int B, Ncap, Nmax, Hq, Hkv, G, page_size, seq_capacity, num_pages, words;
-  int q_tma;  // Q row blocks are fetched by TMA (the group size divides 128)
+  int q_tma;   // Q row blocks are fetched by TMA (the group size divides 128)
+  int q_box;   // rows of such a copy: the block's 128, or whole tokens, at least 8 rows (a power of two, as G is then)
+  int g_log2;  // log2 of the group size, where it divides 128
   const int32_t* worklist;  // one decoded work item per CTA (8 ints each), or null: every CTA decodes for itself
   const int32_t* wl_sizes;  // [2][CAST_MAX_BATCH] the n_tree and kv_len that the list was decoded from, or null: it holds
   int early;  // the tree arrays, lengths, page table and prefix rows may be read before the dependency wait
@@ -869,6 +871,8 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   const int row = row0 + r;
   const bool row_ok = warp < 4 && row < rows_total;
   const int t_tok = row_ok ? F + row / G : 0, h_q = kvh * G + (row_ok ? row % G : 0);
+  // Rows of Q that come by TMA: the boxes that hold live rows. The rest are zeros.
+  const int q_live = (min(rows_total - row0, kBM) + p.q_box - 1) & -p.q_box;
 
   uint64_t* bar_fullk = reinterpret_cast<uint64_t*>(smem + GE::kSmemBar);  // [kStagesK]
   uint64_t* bar_fullv = bar_fullk + kStagesK;                              // [kStagesV]
@@ -974,18 +978,19 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     __threadfence_block();
     asm volatile("bar.arrive 2, %0;" ::"n"(kThreadsTC) : "memory");
     // The Q row block: rows are (tree token, head of the group) pairs, so a block is 128 / G consecutive
-    // tokens x the group's G heads x 128 dims: one 3-D box per 64-dim half, 128-byte swizzled like K. (Rows
-    // past the tree hold whatever the caller's buffer holds: their P is masked to exact zeros.)
+    // tokens x the group's G heads x 128 dims: one 3-D box per 64-dim half, 128-byte swizzled like K, or (see the host) boxes of
+    // eight rows. (A box's rows past the tree hold whatever the caller's buffer holds: their P is masked to exact zeros.)
     if (early) {  // prefix tiles first, then the wait, then Q (the previous kernel may have written it)
       for (; k_issued < kStagesK && k_issued < ntile && (t0 + k_issued + 1) * kBN <= L; ++k_issued) issue_tile(k_issued, 0);
       asm volatile("griddepcontrol.wait;" ::: "memory");
       asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
     if (p.q_tma && ntile > 0) {  // (a split without tiles stages its empty partial in this region right away)
-      if (lane == 0) mbar_expect_tx(bar_q, kReg * kRegionQ);
+      if (lane == 0) mbar_expect_tx(bar_q, (uint32_t)(kReg * 128 * q_live));
       __syncwarp();
-      if (lane < kReg)
-        tma_load_3d(&map_q, smem + kSmemQ + lane * kRegionQ, bar_q, lane * 64, kvh * G, b * p.Ncap + F + row0 / G);
+      const int first = lane / kReg * p.q_box, reg = lane % kReg;  // one (box, half of the dims) per lane: at most 16 boxes
+      if (first < q_live)
+        tma_load_3d(&map_q, smem + kSmemQ + reg * kRegionQ + first * 128, bar_q, reg * 64, kvh * G, b * p.Ncap + F + ((row0 + first) >> p.g_log2));
     }
     // the first K tiles need no stage wait: the ring fills while Q is on its way
     for (; k_issued < kStagesK && k_issued < ntile; ++k_issued) issue_tile(k_issued, 0);
@@ -995,6 +1000,12 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
 #pragma unroll
       for (int w = 0; w < 4; ++w)
         if (w < p.words) aw[w] = p.anc[((size_t)b * p.Ncap + t_tok) * p.words + w];
+    }
+    if (p.q_tma && r >= q_live && ntile > 0) {
+#pragma unroll
+      for (int c = 0; c < HD / 8; ++c)
+        *reinterpret_cast<uint4*>(smem + kSmemQ + (c >> 3) * kRegionQ + r * 128 + (c & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+      fence_proxy_async();
     }
     if (!p.q_tma) {
       const __nv_bfloat16* qrow = p.q + (((size_t)b * p.Ncap + t_tok) * p.Hq + h_q) * HD;
@@ -1406,13 +1417,13 @@ EncodeTiledFn get_encode() {
   return fn;
 }
 
-// Q [B * Ncap tokens][Hq heads][128 dims]: a box is 128 / G tokens x G heads x 64 dims (one row block, one half)
-bool make_q_map(CUtensorMap* map, const void* base, int B, int Ncap, int Hq, int G, int D) {
+// Q [B * Ncap tokens][Hq heads][128 dims]: a box is `tokens` tokens x G heads x 64 dims (128 / G: one row block, one half)
+bool make_q_map(CUtensorMap* map, const void* base, int B, int Ncap, int Hq, int G, int D, int tokens) {
   EncodeTiledFn enc = get_encode();
   if (!enc) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)Hq, (cuuint64_t)B * Ncap};
   const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)Hq * D * 2};
-  const cuuint32_t box[3] = {64, (cuuint32_t)G, (cuuint32_t)(kBM / G)};
+  const cuuint32_t box[3] = {64, (cuuint32_t)G, (cuuint32_t)tokens};
   const cuuint32_t estr[3] = {1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1542,10 +1553,20 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
     return false;
   const int G = Hq / Hkv, Ncap = c->cfg.max_tree;
   const int Nmax = c->cfg.total_token < Ncap ? c->cfg.total_token : Ncap;
+  // Q comes in one copy per row block and half of the dims, or in copies of eight rows (a period of the swizzle's pattern), only
+  // those with live rows, zeros for the others: products with dead rows are computed all the same, and on other sequences'
+  // queries they cost power, which is what bounds a loaded machine (64 sequences of 512-4096, 12 tokens, two layers back to
+  // back: 235 -> 223 us at 1.3 GHz and above, 197 -> 195 from rest). Not where CTAs are short: the copies are on the chain of a
+  // split (six draft windows on 4 sequences 85 -> 90 us) and of sequences under some 1000 positions (48 of 64-512, 17.6 -> 19.1).
+  const int max_pos = page_size == 0 ? seq_capacity : seq_capacity * page_size;
+  const bool fine = G < kBM && !(pl.cluster_mode && pl.cs > 1) && max_pos >= 1024;
+  const int q_tokens = G > kBM ? 0 : !fine ? kBM / G : G < 8 ? 8 / G : 1;  // (G divides 128 where this is used: a power of two)
   CUtensorMap map_q = map_k;  // (a valid descriptor either way; used only when q_tma is set)
-  const bool q_tma = G <= kBM && (kBM % G) == 0 && make_q_map(&map_q, q, B, Ncap, Hq, G, D);
+  const bool q_tma = G <= kBM && (kBM % G) == 0 && make_q_map(&map_q, q, B, Ncap, Hq, G, D, q_tokens);
   TcParams p;
   p.q_tma = q_tma ? 1 : 0;
+  p.q_box = q_tma ? q_tokens * G : kBM;
+  p.g_log2 = q_tma ? __builtin_ctz((unsigned)G) : 0;
   // the shapes the header names: a caller of others may have set the promise without keeping it
   const bool promised = c->attn_early && D == 128 && q_tma;
   p.early = (promised && !c->tree_inputs_fresh) ? 1 : 0;

@@ -112,8 +112,9 @@ def _random_trees(rng, B, cap, n_tree):
     return torch.from_numpy(anc.view(np.int32)).cuda()
 
 
-def _attend(binding, rng, B, cap, n_tree, Hq, Hkv, D, page, kv, dtype=torch.bfloat16, gain=1.0, first=None, early=False):
-    """Device output and fp64 reference of one call."""
+def _attend(binding, rng, B, cap, n_tree, Hq, Hkv, D, page, kv, dtype=torch.bfloat16, gain=1.0, first=None, early=False,
+            beyond=None):
+    """Device output and fp64 reference of one call. `beyond`: what the query rows past a tree hold."""
     g = torch.Generator(device="cuda").manual_seed(int(rng.integers(1 << 30)))
     unit = page or 1
     seq = -(-(max(kv) + cap) // unit)
@@ -121,6 +122,9 @@ def _attend(binding, rng, B, cap, n_tree, Hq, Hkv, D, page, kv, dtype=torch.bflo
             for _ in range(2))
     table = torch.randperm(B * seq, generator=g, device="cuda").to(torch.int32).view(B, seq) if page else None
     q = (torch.randn((B, cap, Hq, D), generator=g, device="cuda") * gain).to(dtype)
+    if beyond is not None:
+        for b, n in enumerate(n_tree):
+            q[b, n:] = beyond
     anc, nt, kv_len = _random_trees(rng, B, cap, n_tree), _ints(n_tree), _ints(kv)
     ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=cap, max_tree=cap)
     ctx.cast_reserve_attention(dtype, B, Hq, Hkv, D, page, seq)
@@ -382,3 +386,21 @@ def test_a_list_of_a_shape_outside_the_promise_is_not_trusted_inside(binding):
     torch.cuda.synchronize()
     check128(call128())
     check64(call64())
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("B,Hkv,G,cap,longest", [
+    (38, 8, 1, 24, 1100), (40, 8, 2, 17, 1000), (38, 8, 4, 33, 1024), (64, 8, 8, 19, 1030), (64, 5, 16, 9, 1200),
+    (38, 8, 64, 4, 1100), (38, 8, 128, 2, 1100), (3, 2, 4, 40, 9000), (38, 8, 4, 33, 300)])
+def test_query_rows_past_the_tree_are_left_out(binding, D, B, Hkv, G, cap, longest):
+    """Many sequences, or pieces of long ones: a row block's queries come eight rows at a time, those with live rows only. The
+    tree sizes run over the edges of the copies; what lies past the trees is NaN. (The last two: pieces of long sequences, and
+    sequences too short for it.) Two bf16 roundings, of the probabilities and of the output: 2^-9 of |v|'s maximum each."""
+    rng = np.random.default_rng(B + G)
+    n_tree = [1 + i % cap for i in range(B)]
+    kv = [longest] + [int(x) for x in rng.integers(0, 200, B - 1)]
+    for first in (None, [n // 2 for n in n_tree]):
+        got, want = _attend(binding, rng, B, cap, n_tree, Hkv * G, Hkv, D, 16, kv, first=first, beyond=float("nan"))
+        keep = ~want.isnan()
+        assert torch.equal(got.isnan(), ~keep)
+        assert float((got.double() - want)[keep].abs().max()) < 2.0 ** -8 * 6
