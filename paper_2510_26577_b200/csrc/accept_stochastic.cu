@@ -17,11 +17,12 @@
 // so the control flow, and with it the sequence of cluster barriers, is uniform across the cluster.
 //
 // What bounds it: fp64 issue in the exponentials (64 lanes per SM: 2 V / cluster-size of them per node and CTA at about
-// a dozen fp64 instructions each, 1.7 us at V = 128256 and 16 CTAs) and the chain of cluster-wide sums (about 1.2 us
-// each). Hence: no pass for the maximum (fp64 has the exponent range to sum exp(logit / T) as it is; the row is
+// a dozen fp64 instructions each; with the rest of an exponential 3.1 us a node at V = 128256 and 16 CTAs, 6.4 with 8) and
+// the chain of cluster-wide sums (about 1.2 us each). Hence: no pass for the maximum (fp64 has the exponent range to sum exp(logit / T) as it is; the row is
 // evaluated again against its maximum only if the sum leaves 1e-280 .. 1e280), one exchange per node and per rejection
 // and none for the bonus token, whose segment sums are those of the last exchange.
-// Measured (T = 0.8, trees of 24, V = 128256 fp32): 1 sequence 38 us, 8 63, 16 76, 64 231.
+// Measured with the compaction behind it (T = 0.8, trees of 24, fp32): V = 128256 1 sequence 46 -> 40 us, 16 87 -> 80 by
+// taking the exponentials side by side; V = 32000 64 sequences 110 -> 104.
 #include <math.h>
 
 #include "cast_internal.h"
@@ -33,6 +34,7 @@ namespace {
 constexpr int kStoThreads = 512;
 constexpr int kStoWarps = kStoThreads / 32;
 constexpr int kStoMaxCluster = 16;
+constexpr int kStoInFlight = 8;  // exponentials of a lane that are worked on side by side, at most
 // Vocabulary entries per CTA up to which the plan caches segments (196 608 tokens in clusters of 16): the rule that
 // cast_accept_stochastic_plan has always answered by, set when a slice of both rows filled shared memory. The kernels hold
 // up to 38 x 512 entries now, so the times do not cross here: V = 262144, one sequence, 76 us recomputing and 41 cached.
@@ -43,6 +45,7 @@ struct StoParams {
   const void* draft_logits;
   int V, Ncap, max_depth, ne, cs;  // ne: elements per lane; a CTA's slice is ne * kStoThreads
   double inv_T, T;
+  double c_hi, c_lo;  // 32 / (T ln2) in two parts
   const int32_t* tokens;
   const int32_t* parent;
   const int32_t* n_tree;
@@ -134,6 +137,56 @@ __device__ __forceinline__ double sto_exp_row(float logit, const StoRef& row, do
   return __hiloint2double(big ? 0x7ff00000 : (zero ? 0 : hi), big || zero ? 0 : __double2loint(y));
 }
 
+// The same for a group of logits, a reference of 0 and logits within the limits on either side (the caller has looked), as
+// almost all are. Step by step for M of them side by side: each is a chain of a dozen dependent fp64 instructions, and taken
+// one after the other they left the pipe half idle (cycles of a warp per exponential, V = 128256: 56 before, 48 now, of which
+// the fp64 instructions take 29 and the two shuffles and the conversion, which other pipes run, 8 each). No range tests, and
+// the argument is reduced from the logit itself, t = logit * 32 / (T ln2) = k + f, |f| <= 1/2, by a factor in two parts (f is
+// right to 2^-54 of its own size; through x = logit / T it carried x's rounding). The polynomial of e^r is taken in f.
+// (The conversion by integer instructions: 80.9 -> 83.5 us for the 16 sequences below; M = 2 or 4: 86.1, 82.9.)
+template <int U>
+__device__ __forceinline__ void sto_exp_plain(const float (&logit)[U], double c_hi, double c_lo, double tab, double (&e)[U]) {
+  constexpr double kL = 6.93147180559945309417e-01 / 32.0;
+  constexpr int M = U < kStoInFlight ? U : kStoInFlight;
+  static_assert(U % M == 0, "whole groups");
+  const double kMagic = 6755399441055744.0;
+  const double c[6] = {kL * kL * kL * kL * kL * kL / 720.0, kL * kL * kL * kL * kL / 120.0, kL * kL * kL * kL / 24.0,
+                       kL * kL * kL / 6.0, kL * kL / 2.0, kL};
+#pragma unroll
+  for (int g = 0; g < U; g += M) {
+    double f[M], y[M];
+    int k[M];
+#pragma unroll
+    for (int i = 0; i < M; ++i) f[i] = (double)logit[g + i];
+#pragma unroll
+    for (int i = 0; i < M; ++i) y[i] = fma(f[i], c_hi, kMagic);
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      k[i] = __double2loint(y[i]);
+      y[i] -= kMagic;
+    }
+#pragma unroll
+    for (int i = 0; i < M; ++i) y[i] = fma(f[i], c_hi, -y[i]);
+#pragma unroll
+    for (int i = 0; i < M; ++i) f[i] = fma(f[i], c_lo, y[i]);
+#pragma unroll
+    for (int i = 0; i < M; ++i) y[i] = c[0];
+#pragma unroll
+    for (int d = 1; d < 6; ++d)
+#pragma unroll
+      for (int i = 0; i < M; ++i) y[i] = fma(y[i], f[i], c[d]);
+#pragma unroll
+    for (int i = 0; i < M; ++i) y[i] *= f[i];
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      const double t = __hiloint2double(__shfl_sync(0xffffffffu, __double2hiint(tab), k[i] & 31),
+                                        __shfl_sync(0xffffffffu, __double2loint(tab), k[i] & 31));
+      const double v = fma(t, y[i], t);
+      e[g + i] = __hiloint2double(__double2hiint(v) + (k[i] & ~31) * 32768, __double2loint(v));
+    }
+  }
+}
+
 struct StoShared {
   double xch[2][kStoMaxCluster * kStoWarps][2];  // the cluster's warps' records, in vocabulary order, double-buffered
   int32_t par[CAST_MAX_TREE];
@@ -148,7 +201,9 @@ __device__ __forceinline__ double sto_warp_sum(double v) {
 }
 
 // Every warp hands its two values to every CTA of the cluster; after the barrier sh.xch[parity] holds all records.
-__device__ __forceinline__ void sto_exchange(StoShared& sh, int parity, int rank, int cs, double v0, double v1) {
+// `meanwhile` runs while the others' records are on their way.
+template <typename F>
+__device__ __forceinline__ void sto_exchange(StoShared& sh, int parity, int rank, int cs, double v0, double v1, F meanwhile) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double* slot = sh.xch[parity][rank * kStoWarps + warp];
   if (cs == 1) {
@@ -156,11 +211,17 @@ __device__ __forceinline__ void sto_exchange(StoShared& sh, int parity, int rank
       slot[0] = v0;
       slot[1] = v1;
     }
+    meanwhile();
     __syncthreads();
     return;
   }
   if (lane < cs) sto_st_remote_f64x2(slot, (uint32_t)lane, v0, v1);
-  sto_cluster_sync();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  meanwhile();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void sto_exchange(StoShared& sh, int parity, int rank, int cs, double v0, double v1) {
+  sto_exchange(sh, parity, rank, cs, v0, v1, [] {});
 }
 
 // The records' sums, in the same order in every warp.
@@ -188,6 +249,10 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
   __shared__ StoShared sh;
   constexpr bool CACHED = NE > 0;
   constexpr int kP = CACHED ? sto_in_registers(NE) : 1;
+  // The children's exponentials are formed while the sums are exchanged, but not where a segment's values leave no registers
+  // for them (us, formed after / during: one sequence of V = 128256 42.3 / 40.3, 64 of 32000 105.6 / 104.2, with 32 entries a
+  // lane, 16 of 128256, 80.5 / 82.2).
+  constexpr bool kOverlap = NE <= 24;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cs = p.cs, rank = blockIdx.x, b = blockIdx.y;
   const int ne = CACHED ? NE : p.ne;
@@ -231,7 +296,7 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
   };
   auto qt = [&](int j) -> double { return CACHED ? eq[32 * j] : value(logit(lq, j), ref_q); };
   // the node's rows evaluated: this lane's sums
-  auto evaluate = [&](double& sp, double& sq) {
+  auto evaluate = [&](double& sp, double& sq, bool zero_refs) {
     sp = sq = 0.0;
     if constexpr (CACHED) {
       constexpr int U = NE < 8 ? NE : 8;  // logits in flight: the next group is loaded while this one is evaluated
@@ -249,22 +314,42 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
           np[j] = j0 + U + j < NE ? logit(lp, j0 + U + j) : 0.f;
           nq[j] = j0 + U + j < NE && has_q ? logit(lq, j0 + U + j) : 0.f;
         }
+        bool plain_p = zero_refs, plain_q = zero_refs;
 #pragma unroll
         for (int j = 0; j < U; ++j) {
-          if (j0 + j >= NE) break;
-          const double e = value(xp[j], ref_p);
-          if (j0 + j < kP) ep[j0 + j < kP ? j0 + j : 0] = e;
-          else eq[32 * (NE + j0 + j - kP)] = e;
-          sp += e;
+          plain_p = plain_p && fabsf(xp[j]) <= ref_p.hi;
+          plain_q = plain_q && fabsf(xq[j]) <= ref_p.hi;
         }
-        if (has_q) {
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {  // target, draft
+          if (side == 1 && !has_q) break;
+          double e[U];
+          // (segments of four entries a lane are mostly padding, which is not within the limits: one sequence of V = 4099
+          // 28.4 us with the look, 27.5 without)
+          if (NE > 4 && __all_sync(0xffffffffu, side == 0 ? plain_p : plain_q)) {
+            sto_exp_plain<U>(side == 0 ? xp : xq, p.c_hi, p.c_lo, tab, e);
+          } else {
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+              e[j] = value(side == 0 ? xp[j] : xq[j], side == 0 ? ref_p : ref_q);
+          }
 #pragma unroll
           for (int j = 0; j < U; ++j) {
             if (j0 + j >= NE) break;
-            const double e = value(xq[j], ref_q);
-            eq[32 * (j0 + j)] = e;
-            sq += e;
+            if (side == 1) eq[32 * (j0 + j)] = e[j];
+            else if (j0 + j < kP) ep[j0 + j < kP ? j0 + j : 0] = e[j];
+            else eq[32 * (NE + j0 + j - kP)] = e[j];
           }
+          // the group's sum in pairs (one after the other they are a chain)
+#pragma unroll
+          for (int j = 0; j < U; ++j)
+            if (j0 + j >= NE) e[j] = 0.0;
+#pragma unroll
+          for (int o = 1; o < U; o *= 2)
+#pragma unroll
+            for (int j = 0; j + o < U; j += 2 * o) e[j] += e[j + o];
+          if (side == 1) sq += e[0];
+          else sp += e[0];
         }
 #pragma unroll
         for (int j = 0; j < U; ++j) {
@@ -282,18 +367,20 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
   };
   // this lane's share of sum_x max(0, P_T - a2 P_D)
   auto residual = [&](double a2) -> double {
-    const double aq = a2 * cq;
+    const double g = -(a2 * cq) / cp;  // (P_T - a P_D) / cp: one multiply-add per entry
     double s = 0.0;
+    auto add = [&](int j) {
+      const double v = fma(qt(j), g, pt(j));
+      s += v > 0.0 ? v : 0.0;
+    };
 #pragma unroll
-    for (int j = 0; j < (CACHED ? NE : 1); ++j) {
-      if (!CACHED) break;
-      s += fmax(0.0, pt(j) * cp - qt(j) * aq);
-    }
+    for (int j = 0; j < (CACHED ? NE : 1); ++j)
+      if (CACHED) add(j);
     if (!CACHED) {
 #pragma unroll 4
-      for (int j = 0; j < ne; ++j) s += fmax(0.0, pt(j) * cp - qt(j) * aq);
+      for (int j = 0; j < ne; ++j) add(j);
     }
-    return s;
+    return s * cp;
   };
 
   for (;;) {
@@ -348,10 +435,16 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
     // ---- softmax sums of the node's rows
     double Sp, Sq = 1.0;
     ref_p = ref_q = StoRef(0.0, p.T);
+    double child_p = 0.0, child_q = 0.0;  // exp(logit / T) of lane j's child
+    auto child_exps = [&] {
+      child_p = sto_exp_any(fma((double)raw_p, p.inv_T, -ref_p.ref));
+      child_q = sto_exp_any(fma((double)raw_q, p.inv_T, -ref_q.ref));
+    };
     for (int attempt = 0;; ++attempt) {
       double sp, sq;
-      evaluate(sp, sq);
-      sto_exchange(sh, parity, rank, cs, sto_warp_sum(sp), sto_warp_sum(sq));
+      evaluate(sp, sq, attempt == 0);
+      if constexpr (kOverlap) sto_exchange(sh, parity, rank, cs, sto_warp_sum(sp), sto_warp_sum(sq), child_exps);
+      else sto_exchange(sh, parity, rank, cs, sto_warp_sum(sp), sto_warp_sum(sq));
       sto_fold(sh, parity, cs, Sp, Sq);
       held = parity;
       parity ^= 1;
@@ -393,8 +486,8 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
     int next = -1;
     for (int j0 = 0; j0 < k && next < 0; j0 += 32) {
       if (j0 > 0) ask(j0);
-      const double px_l = sto_exp_any(fma((double)raw_p, p.inv_T, -ref_p.ref)) * cp,
-                   qx_l = sto_exp_any(fma((double)raw_q, p.inv_T, -ref_q.ref)) * cq;
+      if (j0 > 0 || !kOverlap) child_exps();
+      const double px_l = child_p * cp, qx_l = child_q * cq;
       const unsigned valid = __ballot_sync(0xffffffffu, token_ok);
       bool empty = false;
       for (int j = j0; j < min(k, j0 + 32); ++j) {
@@ -642,6 +735,12 @@ extern "C" cast_status cast_accept_stochastic(cast_ctx* c, const void* target_lo
   p.max_depth = c->cfg.max_depth;
   p.inv_T = 1.0 / temperature;
   p.T = temperature;
+  {
+    const long double c = 32.0L * 1.442695040888963407359924681001892137L / (long double)temperature;
+    p.c_hi = (double)c;
+    p.c_lo = (double)(c - (long double)p.c_hi);
+    if (!isfinite(p.c_hi)) p.c_hi = p.c_lo = 0.0;  // (temperatures of 1e-307: zero is the one logit within the limits)
+  }
   p.tokens = tokens;
   p.parent = parent;
   p.n_tree = n_tree;

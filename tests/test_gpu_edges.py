@@ -191,6 +191,47 @@ def test_stochastic_accept_at_the_steps_of_its_dispatch(binding, V, B, dtype, sh
         assert np.array_equal(got.cpu().numpy()[clear], want[clear])
 
 
+@pytest.mark.parametrize("V,B", [(4099, 1), (40000, 1), (128256, 1), (152064, 2), (190000, 1), (100001, 12), (128256, 12),
+                                 (152064, 12)])
+@pytest.mark.parametrize("dtype,T,top", [(torch.float32, 0.9, None), (torch.bfloat16, 1.3, None), (torch.float32, 0.7, 640.0),
+                                         (torch.float32, 0.9, 689.9)])
+def test_stochastic_accept_mixes_logits_within_and_beyond_the_limits(binding, V, B, dtype, T, top):
+    """Groups of logits that hold what exp(logit / T) takes without a range test and what it does not: tokens that are ruled
+    out (-inf), hardly possible ones (-1e4 T) and, with `top`, two likely ones at top * T, just inside the limit (their sum
+    asks for the second evaluation or just does not). Segments of every size the kernel is compiled for."""
+    from oracle import stochastic_accept
+    rng = np.random.default_rng(V + B)
+    N, H = 4, 3
+    g = torch.Generator(device="cuda").manual_seed(V + B)
+    parent = np.tile(np.array([-1, 0, 0, 1], np.int32), (B, 1))
+    tokens = np.stack([rng.permutation(V)[:N] for _ in range(B)]).astype(np.int32)
+    draft = torch.randn((B, N, V), generator=g, device="cuda") * 3
+    target = draft + 0.5 * torch.randn(draft.shape, generator=g, device="cuda")
+    for x, share, value in ((target, 1e-3, float("-inf")), (target, 1e-4, -1e4 * T), (draft, 1e-4, -1e4 * T)):
+        x[torch.rand(x.shape, generator=g, device="cuda") < share] = value
+    for b in range(B):
+        for t, p in ((1, 0), (2, 0), (3, 1)):
+            draft[b, p, int(tokens[b, t])] = 15.0 - t
+            target[b, p, int(tokens[b, t])] = 14.0 - t
+        if top is not None:
+            target[b, :, V // 3] = top * T
+            target[b, :, V - 1] = (top - 0.5) * T
+    target, draft = target.to(dtype), draft.to(dtype)
+    n_tree = np.full(B, N, np.int32)
+    ua, ub = rng.uniform(0.01, 0.99, (B, N)), rng.uniform(0.01, 0.99, B)
+    ctx = binding.CastContext(max_batch=B, vocab=V, top_k=2, max_depth=H, total_token=N, max_tree=N)
+    dev = lambda a: torch.from_numpy(a).cuda()
+    n, path, bonus = _ints([0] * B), _ints([[0] * (H + 1)] * B), _ints([0] * B)
+    ctx.cast_accept_stochastic(target, draft, B, T, dev(tokens), dev(parent), dev(n_tree), dev(ua), dev(ub), n, path, bonus)
+    assert ctx.cast_poll_status()[0] == 0
+    want_n, want_path, want_bonus, margin = stochastic_accept(target.double().cpu().numpy(), draft.double().cpu().numpy(), tokens,
+                                                              parent, n_tree, H, T, ua, ub)
+    clear = margin > 1e-11
+    assert clear.any()
+    for got, want in ((n, want_n), (path, want_path), (bonus, want_bonus)):
+        assert np.array_equal(got.cpu().numpy()[clear], want[clear])
+
+
 @pytest.mark.parametrize("logits", ["f32", "bf16"])
 @pytest.mark.parametrize("V", [33, 8191, 16385, 32769, 65529, 131073, 262147])
 @pytest.mark.parametrize("kind", ["random", "rising", "constant", "one_block", "few_finite"])
