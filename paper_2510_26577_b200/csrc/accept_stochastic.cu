@@ -582,9 +582,8 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
     double pick_v = 0.0, pick_at = 0.0;  // this lane's mass in the row that was picked, and the sum before that row
     int pick = -1;
     bool found = false;
-    auto visit = [&](int j) {
-      const double v = fmax(0.0, pt(j) * cp - (has_q ? qt(j) * aq : 0.0));
-      const double row = sto_warp_sum(v);
+    auto mass_of = [&](int j) -> double { return fmax(0.0, pt(j) * cp - (has_q ? qt(j) * aq : 0.0)); };
+    auto visit = [&](int j, double v, double row) {
       if (!found && row > 0.0) {
         pick = j;
         pick_v = v;
@@ -593,11 +592,26 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
       }
       run += row;
     };
+    constexpr int kRows = !CACHED ? 1 : NE < 8 ? NE : 8;  // rows summed side by side (a sum is a chain of five shuffles and additions)
 #pragma unroll
-    for (int j = 0; j < (CACHED ? NE : 1); ++j)
-      if (CACHED) visit(j);
+    for (int j0 = 0; j0 < NE; j0 += kRows) {
+      double v[kRows], row[kRows];
+#pragma unroll
+      for (int i = 0; i < kRows; ++i) row[i] = v[i] = j0 + i < NE ? mass_of(j0 + i) : 0.0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) row[i] += __shfl_xor_sync(0xffffffffu, row[i], o);
+#pragma unroll
+      for (int i = 0; i < kRows; ++i)
+        if (j0 + i < NE) visit(j0 + i, v[i], row[i]);
+      if (found) break;  // (the same in all lanes)
+    }
     if (!CACHED)
-      for (int j = 0; j < ne; ++j) visit(j);
+      for (int j = 0; j < ne; ++j) {
+        const double v = mass_of(j);
+        visit(j, v, sto_warp_sum(v));
+      }
     double incl = pick_v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
