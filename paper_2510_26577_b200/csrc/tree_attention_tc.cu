@@ -988,7 +988,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     if (p.q_tma && ntile > 0) {  // (a split without tiles stages its empty partial in this region right away)
       if (lane == 0) mbar_expect_tx(bar_q, (uint32_t)(kReg * 128 * q_live));
       __syncwarp();
-      const int first = lane / kReg * p.q_box, reg = lane % kReg;  // one (box, half of the dims) per lane: at most 16 boxes
+      const int first = lane / kReg * p.q_box, reg = lane % kReg;  // one (box, half of the dims) per lane: at most 12 boxes
       if (first < q_live)
         tma_load_3d(&map_q, smem + kSmemQ + reg * kRegionQ + first * 128, bar_q, reg * 64, kvh * G, b * p.Ncap + F + ((row0 + first) >> p.g_log2));
     }
@@ -1559,7 +1559,10 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   // back: 235 -> 223 us at 1.3 GHz and above, 197 -> 195 from rest). Not where CTAs are short: the copies are on the chain of a
   // split (six draft windows on 4 sequences 85 -> 90 us) and of sequences under some 1000 positions (48 of 64-512, 17.6 -> 19.1).
   const int max_pos = page_size == 0 ? seq_capacity : seq_capacity * page_size;
-  const bool fine = G < kBM && !(pl.cluster_mode && pl.cs > 1) && max_pos >= 1024;
+  const bool fine = Nmax * G <= kBM * 3 / 4 && !(pl.cluster_mode && pl.cs > 1) && max_pos >= 1024;
+  // Nor where the largest tree leaves less than a quarter of a block dead: there the copies bought nothing and cost a little (16
+  // sequences of 2048, 64 tokens, 43.3 -> 43.9 us per layer; a second descriptor, for the kernel to choose by the live rows,
+  // made short launches of 64-dim heads 2 % slower).
   const int q_tokens = G > kBM ? 0 : !fine ? kBM / G : G < 8 ? 8 / G : 1;  // (G divides 128 where this is used: a power of two)
   CUtensorMap map_q = map_k;  // (a valid descriptor either way; used only when q_tma is set)
   const bool q_tma = G <= kBM && (kBM % G) == 0 && make_q_map(&map_q, q, B, Ncap, Hq, G, D, q_tokens);

@@ -432,11 +432,12 @@ def test_a_list_of_a_shape_outside_the_promise_is_not_trusted_inside(binding):
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("B,Hkv,G,cap,longest", [
     (38, 8, 1, 24, 1100), (40, 8, 2, 17, 1000), (38, 8, 4, 33, 1024), (64, 8, 8, 19, 1030), (64, 5, 16, 9, 1200),
-    (38, 8, 64, 4, 1100), (38, 8, 128, 2, 1100), (3, 2, 4, 40, 9000), (38, 8, 4, 33, 300)])
+    (38, 8, 64, 4, 1100), (38, 8, 128, 2, 1100), (38, 8, 4, 24, 1024), (64, 8, 8, 12, 1030), (64, 5, 16, 6, 1200),
+    (40, 8, 64, 1, 1100), (3, 2, 4, 20, 9000), (3, 2, 4, 40, 9000), (38, 8, 4, 33, 300)])
 def test_query_rows_past_the_tree_are_left_out(binding, D, B, Hkv, G, cap, longest):
     """Many sequences, or pieces of long ones: a row block's queries come eight rows at a time, those with live rows only. The
-    tree sizes run over the edges of the copies; what lies past the trees is NaN. (The last two: pieces of long sequences, and
-    sequences too short for it.) Two bf16 roundings, of the probabilities and of the output: 2^-9 of |v|'s maximum each."""
+    tree sizes run over the edges of the copies; what lies past the trees is NaN. (The last ones: pieces of long sequences; trees
+    too large for it and sequences too short.) Two bf16 roundings, of the probabilities and of the output: 2^-9 of |v|'s maximum each."""
     rng = np.random.default_rng(B + G)
     n_tree = [1 + i % cap for i in range(B)]
     kv = [longest] + [int(x) for x in rng.integers(0, 200, B - 1)]
