@@ -446,3 +446,21 @@ def test_query_rows_past_the_tree_are_left_out(binding, D, B, Hkv, G, cap, longe
         keep = ~want.isnan()
         assert torch.equal(got.isnan(), ~keep)
         assert float((got.double() - want)[keep].abs().max()) < 2.0 ** -8 * 6
+
+
+@pytest.mark.parametrize("B,cap,Hq,Hkv,page,sizes,kv", [
+    (24, 64, 16, 8, 16, None, [6000] * 24),                              # 192 equal items on 296 slots
+    (9, 128, 16, 4, 0, [128] * 9, [9000, 100, 64, 1, 2000, 300, 63, 65, 4000]),  # one sequence much longer than the rest
+    (40, 96, 16, 8, 16, None, [20 + 13 * i for i in range(39)] + [9000]),  # unsplit, the items fill more than a wave
+    (9, 128, 16, 4, 16, [5, 128, 17, 1, 90, 64, 33, 128, 2], [9000, 100, 64, 1, 9000, 300, 63, 8999, 4000]),
+    (16, 64, 32, 8, 16, None, [2048] * 16)])                             # items that are left as they are
+def test_pieces_cut_for_a_wave_more(binding, B, cap, Hq, Hkv, page, sizes, kv):
+    """With the early-read promise the launch has blocks to spare, and the decode may cut the items finer than they need. Two
+    bf16 roundings, of the probabilities and of the output, and the partials' in half precision: 2^-9, 2^-9 and 2^-11 of |v|'s
+    maximum."""
+    rng = np.random.default_rng(B + cap)
+    n_tree = sizes or [cap] * B
+    got, want = _attend(binding, rng, B, cap, n_tree, Hq, Hkv, 128, page, kv, early=True)
+    keep = ~want.isnan()
+    assert torch.equal(got.isnan(), ~keep)
+    assert float((got.double() - want)[keep].abs().max()) < 2.25 * 2.0 ** -9 * 6
