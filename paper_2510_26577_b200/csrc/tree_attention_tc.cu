@@ -653,10 +653,12 @@ __device__ __forceinline__ WorkItem decode_work_chunked(const TcParams& p, int i
   // 221 us per layer; 22 of 7740, 141 -> 130). By 15 % at least: 16 sequences of 512-4096, 12 % by the estimate, gain nothing
   // at a full power draw (69.1 -> 69.7), equal ones of 2048 lose (43 -> 55).
   const int now = max(min(chunk, tmax) + kPieceTiles, (T + items * kPieceTiles) / slots);
-  bool done = false;
-  if (grid > cap && 20 * (T / slots + (W + 1) * kPieceTiles) < 17 * now) {
-    items = splits_at(chunk_for(min((W + 1) * slots, grid)));
+  bool finer = grid > cap && 20 * (T / slots + (W + 1) * kPieceTiles) < 17 * now;
+  if (finer) items = splits_at(chunk_for(min((W + 1) * slots, grid)));
+#pragma unroll 1
+  for (;;) {
     order();
+    if (!finer) break;
     int est = 0;
     for (int first = 0; first < items; first += slots) {
       int len = 0;
@@ -665,10 +667,10 @@ __device__ __forceinline__ WorkItem decode_work_chunked(const TcParams& p, int i
         if (first >= off[k] && first < off[k] + cnt[k]) len = (tl[k] + ns[k] - 1) / ns[k];
       est += warp_sum(len) + kPieceTiles;
     }
-    done = 20 * est < 17 * now;
-    if (!done) splits_at(chunk);
+    if (20 * est < 17 * now) break;
+    finer = false;
+    splits_at(chunk);
   }
-  if (!done) order();
   WorkItem w;
   w.valid = w.active = false;
   w.b = w.kvh = w.rb = w.split = w.N = w.L = w.F = 0;
