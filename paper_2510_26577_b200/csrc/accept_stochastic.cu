@@ -367,10 +367,12 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
   };
   // this lane's share of sum_x max(0, P_T - a2 P_D)
   auto residual = [&](double a2) -> double {
-    const double g = -(a2 * cq) / cp;  // (P_T - a P_D) / cp: one multiply-add per entry
+    // Each row is scaled by its own sum: both products are of order one. (One multiply-add less per entry with the quotient
+    // a2 Sp / Sq of the sums: that leaves fp64 where the rows lie far apart, T = 0.05 and tops of 32 and -4.)
+    const double aq = a2 * cq;
     double s = 0.0;
     auto add = [&](int j) {
-      const double v = fma(qt(j), g, pt(j));
+      const double v = fma(pt(j), cp, -(qt(j) * aq));
       s += v > 0.0 ? v : 0.0;
     };
 #pragma unroll
@@ -380,7 +382,7 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
 #pragma unroll 4
       for (int j = 0; j < ne; ++j) add(j);
     }
-    return s * cp;
+    return s;
   };
 
   for (;;) {

@@ -232,6 +232,48 @@ def test_stochastic_accept_mixes_logits_within_and_beyond_the_limits(binding, V,
         assert np.array_equal(got.cpu().numpy()[clear], want[clear])
 
 
+def _sample_at_root(binding, target, draft, T, tokens, ua, ub):
+    """Trees of a root and tokens.shape[1] - 1 children: accepted lengths, paths and bonus tokens, and the oracle's with margins."""
+    from oracle import stochastic_accept
+    B, N, V = target.shape
+    parent = np.tile(np.array([-1] + [0] * (N - 1), np.int32), (B, 1))
+    n_tree = np.full(B, N, np.int32)
+    ctx = binding.CastContext(max_batch=B, vocab=V, top_k=2, max_depth=2, total_token=N, max_tree=N)
+    dev = lambda a: torch.from_numpy(a).cuda()
+    n, path, bonus = _ints([0] * B), _ints([[0] * 3] * B), _ints([0] * B)
+    ctx.cast_accept_stochastic(target, draft, B, T, dev(tokens), dev(parent), dev(n_tree), dev(ua), dev(ub), n, path, bonus)
+    assert ctx.cast_poll_status()[0] == 0
+    want = stochastic_accept(target.double().cpu().numpy(), draft.double().cpu().numpy(), tokens, parent, n_tree, 2, T, ua, ub)
+    return [x.cpu().numpy() for x in (n, path, bonus)], want[:3], want[3]
+
+
+@pytest.mark.parametrize("V,B", [(4099, 8), (40000, 8), (128256, 5), (128256, 12), (200001, 4)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("top_p,top_q", [(32.0, -7.0), (-7.0, 32.0)])
+def test_stochastic_accept_of_rows_far_apart(binding, V, B, dtype, top_p, top_q):
+    """Temperature 0.05, one row's top logits at 32 (a sum of 1e278) and the other's at -7 (1e-61), each way round: both sums
+    are within fp64's range, their quotient is not. The children are the tokens that the target likes least, to be rejected.
+    The last vocabulary is one whose segments are not cached."""
+    rng = np.random.default_rng(V + B)
+    T, hot = 0.05, np.stack([rng.permutation(V)[:8] for _ in range(B)])
+    rows = np.empty((2, B, 3, V))
+    for x, top in zip(rows, (top_p, top_q)):
+        x[:] = top - rng.uniform(4, 40, x.shape)
+        step = 2.0 ** -2 if top > 0 else 2.0 ** -5  # (as fine as bf16 has them there)
+        for b in range(B):
+            x[b][:, hot[b]] = top - step * (rng.permutation(8) // 3)
+    target, draft = (torch.from_numpy(x).to(dtype).cuda() for x in rows)
+    t0, d0 = (np.take_along_axis(x[:, 0].double().cpu().numpy(), hot, 1) / T for x in (target, draft))
+    worst = np.argsort(t0 - d0, axis=1)[:, :2]
+    tokens = np.concatenate([np.zeros((B, 1)), np.take_along_axis(hot, worst, 1)], 1).astype(np.int32)
+    ua, ub = rng.uniform(0.95, 0.999, (B, 3)), rng.uniform(0.01, 0.99, B)
+    got, want, margin = _sample_at_root(binding, target, draft, T, tokens, ua, ub)
+    clear = margin > 1e-9
+    assert clear.sum() >= B // 2 and (want[0][clear] == 0).any()
+    for g, w in zip(got, want):
+        assert np.array_equal(g[clear], w[clear])
+
+
 @pytest.mark.parametrize("logits", ["f32", "bf16"])
 @pytest.mark.parametrize("V", [33, 8191, 16385, 32769, 65529, 131073, 262147])
 @pytest.mark.parametrize("kind", ["random", "rising", "constant", "one_block", "few_finite"])
