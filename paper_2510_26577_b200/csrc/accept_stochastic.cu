@@ -365,14 +365,17 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
       }
     }
   };
+  // P_T - a P_D at this lane's j-th token, aq = a cq. Each row is scaled by its own sum: both products are of order one. (One
+  // multiply-add less per entry with the quotient a Sp / Sq of the sums: that leaves fp64 where the rows lie far apart, T = 0.05
+  // and tops of 32 and -4.) The residual sums and the search for the bonus token both call this: a residual may be nothing but
+  // the last bits of two equal rows, and a segment whose sum is positive must hold a token of positive mass.
+  auto left = [&](int j, double aq) -> double { return __fma_rn(pt(j), cp, -__dmul_rn(qt(j), aq)); };
   // this lane's share of sum_x max(0, P_T - a2 P_D)
   auto residual = [&](double a2) -> double {
-    // Each row is scaled by its own sum: both products are of order one. (One multiply-add less per entry with the quotient
-    // a2 Sp / Sq of the sums: that leaves fp64 where the rows lie far apart, T = 0.05 and tops of 32 and -4.)
     const double aq = a2 * cq;
     double s = 0.0;
     auto add = [&](int j) {
-      const double v = fma(pt(j), cp, -(qt(j) * aq));
+      const double v = left(j, aq);
       s += v > 0.0 ? v : 0.0;
     };
 #pragma unroll
@@ -584,7 +587,7 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
     double pick_v = 0.0, pick_at = 0.0;  // this lane's mass in the row that was picked, and the sum before that row
     int pick = -1;
     bool found = false;
-    auto mass_of = [&](int j) -> double { return fmax(0.0, pt(j) * cp - (has_q ? qt(j) * aq : 0.0)); };
+    auto mass_of = [&](int j) -> double { return fmax(0.0, has_q ? left(j, aq) : pt(j) * cp); };
     auto visit = [&](int j, double v, double row) {
       if (!found && row > 0.0) {
         pick = j;

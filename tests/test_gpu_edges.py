@@ -274,6 +274,26 @@ def test_stochastic_accept_of_rows_far_apart(binding, V, B, dtype, top_p, top_q)
         assert np.array_equal(g[clear], w[clear])
 
 
+@pytest.mark.parametrize("V,B", [(4099, 64), (40000, 64), (128256, 4), (128256, 24), (200001, 16)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_stochastic_accept_of_rows_with_all_mass_on_one_token(binding, V, B, dtype):
+    """Both rows of the root hold all their mass on the same token; the child is another one, with e^-60 of the draft's mass and
+    none of the target's, and is rejected. What is left of P_T - P_D is 0 or the last bits of it: the bonus token is that token."""
+    for seed in range(6):
+        rng = np.random.default_rng(V + 1000 * seed)
+        target, draft = (torch.full((B, 2, V), float("-inf"), dtype=dtype, device="cuda") for _ in range(2))
+        at = np.stack([1 + rng.permutation(V - 1)[:2] for _ in range(B)])
+        rows, hot, child = torch.arange(B, device="cuda"), torch.from_numpy(at[:, 0]).cuda(), torch.from_numpy(at[:, 1]).cuda()
+        top = torch.from_numpy(rng.uniform(-5, 20, (2, B))).cuda().to(dtype)
+        target[rows, 0, hot], draft[rows, 0, hot] = top[0], top[1]
+        draft[rows, 0, child] = top[1] - 60.0
+        tokens = np.stack([np.zeros(B), at[:, 1]], 1).astype(np.int32)
+        got, want, _ = _sample_at_root(binding, target, draft, 1.0, tokens, rng.uniform(0.1, 0.9, (B, 2)), rng.uniform(0.1, 0.9, B))
+        assert np.array_equal(want[2], at[:, 0])
+        for g, w in zip(got, want):
+            assert np.array_equal(g, w)
+
+
 @pytest.mark.parametrize("logits", ["f32", "bf16"])
 @pytest.mark.parametrize("V", [33, 8191, 16385, 32769, 65529, 131073, 262147])
 @pytest.mark.parametrize("kind", ["random", "rising", "constant", "one_block", "few_finite"])
