@@ -92,7 +92,6 @@ struct TcParams {
   const int32_t* wl_sizes;  // [2][CAST_MAX_BATCH] the n_tree and kv_len that the list was decoded from, or null: it holds
   int early;  // the tree arrays, lengths, page table and prefix rows may be read before the dependency wait
   int tmem_first;  // tensor memory may be taken before the dependency wait (see the kernel)
-  int spare_from;  // CTAs from here on may have no item (0: none is counted on to); the work list says so
   int cs;   // CTAs per cluster (1..8); 0: no clusters, splits sized on the device and merged through global memory
   int rpc;  // cluster mode: row blocks a cluster covers at most (cs is a multiple of it)
   int nsplit_max, num_sms, nrb;  // global-merge mode
@@ -546,8 +545,8 @@ __device__ __forceinline__ void merge_rows(const TcParams& p, uint32_t stage_o_s
 // For launches with long CTAs or many ragged sequences, where an even load matters more than the
 // cost of the merge: no clusters; CTA i takes work item i. Sequence b has Hkv * row_blocks(b) *
 // splits(b) items, splits(b) = ceil(tiles(b) / chunk), chunk (>= 4 tiles) being the smallest piece
-// size for which all items fit into the waves of 2 * num_sms CTAs that they need unsplit; when the unsplit work
-// already fills a wave, nothing is split (but see the estimate below). The pieces are of about equal size whatever the mix of
+// size for which all items fit into the launched waves of 2 * num_sms CTAs; when the unsplit work
+// already fills a wave, nothing is split. The pieces are of about equal size whatever the mix of
 // lengths. Partials go to a workspace; the last CTA of a row block to finish (an atomic ticket,
 // nothing spins) merges them.
 __device__ __forceinline__ int warp_sum(int v) {
@@ -555,7 +554,6 @@ __device__ __forceinline__ int warp_sum(int v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-constexpr int kPieceTiles = 12;  // what a piece costs its slot besides its tiles, in tiles
 __device__ __forceinline__ WorkItem decode_work_chunked(const TcParams& p, int idx, int grid) {
   constexpr int KB = CAST_MAX_BATCH / 32;
   const int lane = threadIdx.x & 31;
@@ -589,87 +587,62 @@ __device__ __forceinline__ WorkItem decode_work_chunked(const TcParams& p, int i
   const int slots = 2 * p.num_sms;
   int W = (base + slots - 1) / slots;
   W = W < 1 ? 1 : W;
-  int ns[KB], cnt[KB], off[KB], key[KB];
-  // Sets the splits of pieces of `chunk` tiles and their order; returns the number of pieces. Pieces are numbered longest
-  // first (the block scheduler hands CTAs out in index order, so the long pieces start first and the short ones fill the
-  // gaps): sequence j precedes sequence b when its pieces are longer, ties by index.
-  auto splits_at = [&](int chunk) {
+  int cap = W * slots;
+  cap = cap > grid ? grid : cap;
+  // smallest chunk (>= 4 tiles) whose item count fits: the count falls as the chunk grows, and a chunk
+  // of tmax tiles (no splits at all) always fits
+  auto items_at = [&](int chunk) {
     int items = 0;
 #pragma unroll
     for (int k = 0; k < KB; ++k) {
       int n = (tl[k] + chunk - 1) / chunk;
       n = n > p.nsplit_max ? p.nsplit_max : n;
-      ns[k] = n < 1 ? 1 : n;
-      cnt[k] = p.Hkv * nr[k] * ns[k];
-      items += cnt[k];
+      items += p.Hkv * nr[k] * n;
     }
     return warp_sum(items);
   };
-  // smallest chunk (>= 4 tiles) whose item count fits: the count falls as the chunk grows, and a chunk
-  // of tmax tiles (no splits at all) always fits
-  auto chunk_for = [&](int cap) {
-    int lo = (T + cap - 1) / cap, hi = tmax < 4 ? 4 : tmax;
-    lo = lo < 4 ? 4 : lo;
-    lo = lo > hi ? hi : lo;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (splits_at(mid) <= cap) hi = mid; else lo = mid + 1;
-    }
-    return lo;
-  };
-  auto order = [&] {
+  int lo = (T + cap - 1) / cap, hi = tmax < 4 ? 4 : tmax;
+  lo = lo < 4 ? 4 : lo;
+  lo = lo > hi ? hi : lo;
+  if (base >= slots) lo = hi;  // the unsplit work fills a wave already: no splits
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (items_at(mid) <= cap) hi = mid; else lo = mid + 1;
+  }
+  const int chunk = lo;
+  int ns[KB], cnt[KB], off[KB];
 #pragma unroll
-    for (int k = 0; k < KB; ++k) {
-      key[k] = tl[k] * 16 / ns[k];
-      off[k] = 0;
-    }
-    if (p.B > 1) {
+  for (int k = 0; k < KB; ++k) {
+    int n = (tl[k] + chunk - 1) / chunk;
+    n = n > p.nsplit_max ? p.nsplit_max : n;
+    ns[k] = n < 1 ? 1 : n;
+    cnt[k] = p.Hkv * nr[k] * ns[k];
+    off[k] = 0;
+  }
+  // items are numbered longest piece first (the block scheduler hands CTAs out in index order, so
+  // the long pieces start first and the short ones fill the gaps): sequence j precedes sequence b
+  // when its pieces are longer, ties by index
+  int key[KB];
+#pragma unroll
+  for (int k = 0; k < KB; ++k) key[k] = tl[k] * 16 / ns[k];
+  if (p.B > 1) {
 #pragma unroll 8
-      for (int j = 0; j < p.B; ++j) {
-        const int src = j & 31;
-        int pj, cj;
-        if (j < 32) {
-          pj = __shfl_sync(0xffffffffu, key[0], src);
-          cj = __shfl_sync(0xffffffffu, cnt[0], src);
-        } else {
-          pj = __shfl_sync(0xffffffffu, key[KB - 1], src);
-          cj = __shfl_sync(0xffffffffu, cnt[KB - 1], src);
-        }
+    for (int j = 0; j < p.B; ++j) {
+      const int src = j & 31;
+      int pj, cj;
+      if (j < 32) {
+        pj = __shfl_sync(0xffffffffu, key[0], src);
+        cj = __shfl_sync(0xffffffffu, cnt[0], src);
+      } else {
+        pj = __shfl_sync(0xffffffffu, key[KB - 1], src);
+        cj = __shfl_sync(0xffffffffu, cnt[KB - 1], src);
+      }
 #pragma unroll
-        for (int k = 0; k < KB; ++k) {
-          const int bm = k * 32 + lane;
-          if (pj > key[k] || (pj == key[k] && j < bm)) off[k] += cj;
-        }
+      for (int k = 0; k < KB; ++k) {
+        const int bm = k * 32 + lane;
+        if (pj > key[k] || (pj == key[k] && j < bm)) off[k] += cj;
       }
     }
-  };
-  const int cap = min(W * slots, grid);
-  // (the unsplit work fills a wave already: no splits, unless the rule below finds them worth it)
-  const int chunk = base >= slots ? max(tmax, 4) : chunk_for(cap);
-  int items = splits_at(chunk);
-  // Items that fill their waves badly - somewhat more than half of the slots, each a long piece, or one sequence much longer
-  // than the rest - are cut for one wave more, where the estimate (in tiles: the longest piece of every wave) says that it
-  // pays and the launch has the blocks for it (8 sequences of 14 000, 64 heads on 8, 46 tokens: 192 items on 296 slots, 251 ->
-  // 221 us per layer; 22 of 7740, 141 -> 130). By 15 % at least: 16 sequences of 512-4096, 12 % by the estimate, gain nothing
-  // at a full power draw (69.1 -> 69.7), equal ones of 2048 lose (43 -> 55).
-  const int now = max(min(chunk, tmax) + kPieceTiles, (T + items * kPieceTiles) / slots);
-  bool finer = grid > cap && 20 * (T / slots + (W + 1) * kPieceTiles) < 17 * now;
-  if (finer) items = splits_at(chunk_for(min((W + 1) * slots, grid)));
-#pragma unroll 1
-  for (;;) {
-    order();
-    if (!finer) break;
-    int est = 0;
-    for (int first = 0; first < items; first += slots) {
-      int len = 0;
-#pragma unroll
-      for (int k = 0; k < KB; ++k)
-        if (first >= off[k] && first < off[k] + cnt[k]) len = (tl[k] + ns[k] - 1) / ns[k];
-      est += warp_sum(len) + kPieceTiles;
-    }
-    if (20 * est < 17 * now) break;
-    finer = false;
-    splits_at(chunk);
   }
   WorkItem w;
   w.valid = w.active = false;
@@ -842,11 +815,6 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   // there is no such predecessor: by the promise of the early mode, or behind this call's own work list. The warp that
   // allocates releases the dependents, after it has, so that it is no such predecessor itself.
   const bool early = p.early != 0;
-  // A spare CTA without an item leaves before it takes anything: the next launch waits for its slot.
-  if (p.spare_from > 0 && (int)blockIdx.x >= p.spare_from) {
-    if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (!load_item(p.worklist + (size_t)blockIdx.x * 8).valid) return;
-  }
   if (p.tmem_first) tmem_take();
   if (!early) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1613,17 +1581,9 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
   p.scale_log2 = scale * 1.4426950408889634f;
   p.st = c->state;
   p.num_sms = c->num_sms; p.nrb = pl.nrb;
-  p.spare_from = 0;
   p.part_o = nullptr; p.part_ml = nullptr; p.ticket = nullptr;
   *status = CAST_OK;
-  // Under the early-read promise, one wave of CTAs more than the items need at least: the decode may cut them finer (see
-  // decode_work_chunked). Spare ones leave at once: no difference at 16 sequences of 2048, 256 items; but 0.5 to 1 % at 96 and
-  // 128 items, so not where the items fill half of the slots or less: those are cut in two or more as it is. And only behind a
-  // work list: CTAs that decode for themselves take 1.5 us longer (12 of 512-6000, 64 dims, 27.6 -> 29.1 per layer).
-  const int slots = 2 * c->num_sms;
-  const bool spare = promised && first_row == nullptr && !pl.cluster_mode && pl.nsplit_max > 1 &&
-                     2ll * B * Hkv * pl.nrb > slots && pl.grid + slots <= kAttnWorkListCap;
-  const long long grid = pl.grid + (spare ? slots : 0);
+  const long long grid = pl.grid;
   const int cs = pl.cs;
   p.rpc = pl.rpc; p.nsplit_max = pl.nsplit_max;
   p.cs = pl.cluster_mode ? cs : 0;
@@ -1663,7 +1623,6 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
     // the sizes and decodes for itself where they differ (64 dims, us per layer, decoding always / comparing / trusting:
     // one sequence of 1024 9.4 / 8.8 / 8.6, 64 of 512-1024 41.0 / 34.0 / 33.3; in early mode comparing would cost 0.3 of 11.9).
     p.wl_sizes = p.tmem_first ? nullptr : c->attn_worklist + (size_t)kAttnWorkListCap * 8;
-    p.spare_from = spare ? (int)pl.grid : 0;  // (promised: the list is trusted)
   }
   auto* const kern = D == 64 ? tree_attn_tc_kernel<64> : tree_attn_tc_kernel<128>;
   const int smem_bytes = D == 64 ? Geo<64>::kSmemBytes : Geo<128>::kSmemBytes;

@@ -113,8 +113,9 @@ def _random_trees(rng, B, cap, n_tree):
 
 
 def _attend(binding, rng, B, cap, n_tree, Hq, Hkv, D, page, kv, dtype=torch.bfloat16, gain=1.0, first=None, early=False,
-            beyond=None):
-    """Device output and fp64 reference of one call. `beyond`: what the query rows past a tree hold."""
+            beyond=None, budget=None):
+    """Device output and fp64 reference of one call. `beyond`: what the query rows past a tree hold; `budget`: total_token, where
+    it is not the trees' capacity."""
     g = torch.Generator(device="cuda").manual_seed(int(rng.integers(1 << 30)))
     unit = page or 1
     seq = -(-(max(kv) + cap) // unit)
@@ -126,7 +127,7 @@ def _attend(binding, rng, B, cap, n_tree, Hq, Hkv, D, page, kv, dtype=torch.bflo
         for b, n in enumerate(n_tree):
             q[b, n:] = beyond
     anc, nt, kv_len = _random_trees(rng, B, cap, n_tree), _ints(n_tree), _ints(kv)
-    ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=cap, max_tree=cap)
+    ctx = binding.CastContext(max_batch=B, vocab=100, top_k=2, max_depth=4, total_token=budget or cap, max_tree=cap)
     ctx.cast_reserve_attention(dtype, B, Hq, Hkv, D, page, seq)
     if early:
         ctx.cast_set_attention_early_reads(True)
@@ -516,13 +517,32 @@ def test_query_rows_past_the_tree_are_left_out(binding, D, B, Hkv, G, cap, longe
     (40, 96, 16, 8, 16, None, [20 + 13 * i for i in range(39)] + [9000]),  # unsplit, the items fill more than a wave
     (9, 128, 16, 4, 16, [5, 128, 17, 1, 90, 64, 33, 128, 2], [9000, 100, 64, 1, 9000, 300, 63, 8999, 4000]),
     (16, 64, 32, 8, 16, None, [2048] * 16)])                             # items that are left as they are
-def test_pieces_cut_for_a_wave_more(binding, B, cap, Hq, Hkv, page, sizes, kv):
-    """With the early-read promise the launch has blocks to spare, and the decode may cut the items finer than they need. Two
-    bf16 roundings, of the probabilities and of the output, and the partials' in half precision: 2^-9, 2^-9 and 2^-11 of |v|'s
-    maximum."""
+def test_items_that_fill_their_waves_badly(binding, B, cap, Hq, Hkv, page, sizes, kv):
+    """Equal long items on too many slots, one long sequence among short ones, more items than a wave, with the early-read
+    promise. Two bf16 roundings, of the probabilities and of the output, and the partials' in half precision where a row block is
+    split: 2^-9, 2^-9 and 2^-11 of |v|'s maximum."""
     rng = np.random.default_rng(B + cap)
     n_tree = sizes or [cap] * B
     got, want = _attend(binding, rng, B, cap, n_tree, Hq, Hkv, 128, page, kv, early=True)
     keep = ~want.isnan()
     assert torch.equal(got.isnan(), ~keep)
     assert float((got.double() - want)[keep].abs().max()) < 2.25 * 2.0 ** -9 * 6
+
+
+@pytest.mark.parametrize("B,cap,Hq,Hkv,largest,kv", [
+    (24, 64, 16, 8, 64, [6000] * 24),                          # 192 equal items on 296 slots, each one piece
+    (8, 48, 64, 8, 46, [14000] * 7 + [9000]),                  # three row blocks per sequence and head
+    (24, 128, 32, 8, 30, [6000 + 20 * i for i in range(24)]),  # trees far under the budget: more waves launched than they need
+    (20, 128, 32, 8, 60, [300 * i + 7 for i in range(20)])])   # the same, ragged, more items than a wave
+def test_launches_without_clusters_cut_by_the_trees_alone(binding, B, cap, Hq, Hkv, largest, kv):
+    """How a row block is split, and so how its sums are rounded (a block in one piece is not, before the output), depends on the
+    trees and lengths, not on the early-read promise or on the waves that the budget has launched: the same bits."""
+    n_tree = [largest - i % 3 for i in range(B)]
+    outs = []
+    for early, budget in ((False, cap), (True, cap), (False, largest), (True, largest)):
+        got, want = _attend(binding, np.random.default_rng(B), B, cap, n_tree, Hq, Hkv, 128, 16, kv, early=early, budget=budget)
+        outs.append(torch.stack([got[b, :largest - 2] for b in range(B)]))
+    keep = ~want.isnan()
+    assert float((got.double() - want)[keep].abs().max()) < 2.25 * 2.0 ** -9 * 6
+    for other in outs[1:]:
+        assert torch.equal(outs[0], other)
