@@ -103,7 +103,7 @@ struct cast_ctx {
   // workspace of the tensor-core attention's global-merge mode: tickets, then split partials
   void* attn_tc_ws;
   size_t attn_tc_ws_bytes;
-  int attn_attr_set[2];  // its kernels' attributes have been set on the context's device (heads of 128 dims, of 64)
+  int attn_attr_set[2][2];  // its kernels' attributes have been set on the context's device (heads of 128 dims, of 64)
 
   // stochastic acceptance, per logits dtype (0 fp32, 1 bf16): cluster size found to be launchable
   // (0: not looked up yet), whether a CTA's vocabulary slice is cached on chip, and how many such clusters run at once

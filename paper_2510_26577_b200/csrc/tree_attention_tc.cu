@@ -49,6 +49,10 @@ constexpr int kBM = 128;          // query rows per CTA (UMMA M)
 constexpr int kBN = 64;           // positions per tile
 constexpr int kSoftmaxThreads = 128;               // one thread per query row
 constexpr int kThreadsTC = 256;  // 4 softmax warps, K producer, MMA issuer, V producer, 1 idle: registers are allotted per 4 warps
+// Rows per copy of Q where live rows alone are copied: a multiple of the swizzle's period of eight. (us, rows 8 / 16 / 32: 48
+// sequences of 64-512 in a cache of 4096 28.0 / 27.7 / 27.6 per layer; 64 of 512-4096 with 6-12 tokens, two layers back to back,
+// 7.0 / 7.5 / 6.5 % off the whole copy's 230.)
+constexpr int kQBox = 16;
 constexpr int kRegionQ = kBM * 128;                // [128 rows][64] bf16, 128-byte rows: 16 KB
 constexpr int kRegionKV = kBN * 128;               // [64 positions][64] bf16: 8 KB
 constexpr int kPartRow = 256;                      // bytes of a partial output row: 128 halves or 64 floats
@@ -85,9 +89,7 @@ struct TcParams {
   const __nv_bfloat16* q;
   __nv_bfloat16* out;
   int B, Ncap, Nmax, Hq, Hkv, G, page_size, seq_capacity, num_pages, words;
-  int q_tma;   // Q row blocks are fetched by TMA (the group size divides 128)
-  int q_box;   // rows of such a copy: the block's 128, or whole tokens, at least 8 rows (a power of two, as G is then)
-  int g_log2;  // log2 of the group size, where it divides 128
+  int q_tma;  // Q row blocks are fetched by TMA (the group size divides 128)
   const int32_t* worklist;  // one decoded work item per CTA (8 ints each), or null: every CTA decodes for itself
   const int32_t* wl_sizes;  // [2][CAST_MAX_BATCH] the n_tree and kv_len that the list was decoded from, or null: it holds
   int early;  // the tree arrays, lengths, page table and prefix rows may be read before the dependency wait
@@ -105,6 +107,7 @@ struct TcParams {
   const uint32_t* anc;
   float scale_log2;
   DevState* st;
+  int q_box, g_log2;  // the kernel that copies live rows of Q only: rows of a copy (whole tokens, a power of two), log2 of G
 };
 
 // ---- PTX wrappers -----------------------------------------------------------
@@ -764,7 +767,7 @@ __global__ void __launch_bounds__(256) attn_worklist_kernel(const TcParams p, in
   if ((threadIdx.x & 31) == 0) store_item(list + (size_t)idx * 8, w);
 }
 
-template <int HD>
+template <int HD, bool FINE>
 __global__ void __launch_bounds__(kThreadsTC, 2)
 tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                     const __grid_constant__ CUtensorMap map_q) {
@@ -871,8 +874,8 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
   const int row = row0 + r;
   const bool row_ok = warp < 4 && row < rows_total;
   const int t_tok = row_ok ? F + row / G : 0, h_q = kvh * G + (row_ok ? row % G : 0);
-  // Rows of Q that come by TMA: the boxes that hold live rows. The rest are zeros.
-  const int q_live = (min(rows_total - row0, kBM) + p.q_box - 1) & -p.q_box;
+  // Rows of Q that are copied: the boxes that hold live rows. The rest are zeros.
+  const int q_live = FINE ? (min(rows_total - row0, kBM) + p.q_box - 1) & -p.q_box : kBM;
 
   uint64_t* bar_fullk = reinterpret_cast<uint64_t*>(smem + GE::kSmemBar);  // [kStagesK]
   uint64_t* bar_fullv = bar_fullk + kStagesK;                              // [kStagesV]
@@ -978,36 +981,45 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     __threadfence_block();
     asm volatile("bar.arrive 2, %0;" ::"n"(kThreadsTC) : "memory");
     // The Q row block: rows are (tree token, head of the group) pairs, so a block is 128 / G consecutive
-    // tokens x the group's G heads x 128 dims: one 3-D box per 64-dim half, 128-byte swizzled like K, or (see the host) boxes of
-    // eight rows. (A box's rows past the tree hold whatever the caller's buffer holds: their P is masked to exact zeros.)
+    // tokens x the group's G heads x 128 dims: one 3-D box per 64-dim half, 128-byte swizzled like K, or (FINE) lower boxes.
+    // (A box's rows past the tree hold whatever the caller's buffer holds: their P is masked to exact zeros.)
     if (early) {  // prefix tiles first, then the wait, then Q (the previous kernel may have written it)
       for (; k_issued < kStagesK && k_issued < ntile && (t0 + k_issued + 1) * kBN <= L; ++k_issued) issue_tile(k_issued, 0);
       asm volatile("griddepcontrol.wait;" ::: "memory");
       asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
-    if (p.q_tma && ntile > 0) {  // (a split without tiles stages its empty partial in this region right away)
+    if (FINE && ntile > 0) {
       if (lane == 0) mbar_expect_tx(bar_q, (uint32_t)(kReg * 128 * q_live));
       __syncwarp();
-      const int first = lane / kReg * p.q_box, reg = lane % kReg;  // one (box, half of the dims) per lane: at most 12 boxes
+      const int first = lane / kReg * p.q_box, reg = lane % kReg;  // one (box, half of the dims) per lane
       if (first < q_live)
         tma_load_3d(&map_q, smem + kSmemQ + reg * kRegionQ + first * 128, bar_q, reg * 64, kvh * G, b * p.Ncap + F + ((row0 + first) >> p.g_log2));
+    } else if (p.q_tma && ntile > 0) {  // (a split without tiles stages its empty partial in this region right away)
+      if (lane == 0) mbar_expect_tx(bar_q, kReg * kRegionQ);
+      __syncwarp();
+      if (lane < kReg)
+        tma_load_3d(&map_q, smem + kSmemQ + lane * kRegionQ, bar_q, lane * 64, kvh * G, b * p.Ncap + F + row0 / G);
     }
     // the first K tiles need no stage wait: the ring fills while Q is on its way
     for (; k_issued < kStagesK && k_issued < ntile; ++k_issued) issue_tile(k_issued, 0);
   } else if (warp < 4) {
+    if (FINE && ntile > 0) {
+      // zeros for the dead rows: the rest of either half's region, consecutive lanes side by side (a lane per row had all
+      // eight lanes of a store on the same banks: 0.9 us of 20 per layer at 48 short sequences). Ahead of the loads below, which
+      // the fence would wait for.
+      for (int at = q_live * 128 + tid * 16; at < kRegionQ; at += kSoftmaxThreads * 16) {
+#pragma unroll
+        for (int reg = 0; reg < kReg; ++reg) *reinterpret_cast<uint4*>(smem + kSmemQ + reg * kRegionQ + at) = make_uint4(0u, 0u, 0u, 0u);
+      }
+      fence_proxy_async();
+    }
     // ancestor mask -> registers; without TMA for Q: the Q row -> swizzled shared memory (rows past the tree zero)
     if (row_ok) {
 #pragma unroll
       for (int w = 0; w < 4; ++w)
         if (w < p.words) aw[w] = p.anc[((size_t)b * p.Ncap + t_tok) * p.words + w];
     }
-    if (p.q_tma && r >= q_live && ntile > 0) {
-#pragma unroll
-      for (int c = 0; c < HD / 8; ++c)
-        *reinterpret_cast<uint4*>(smem + kSmemQ + (c >> 3) * kRegionQ + r * 128 + (c & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
-      fence_proxy_async();
-    }
-    if (!p.q_tma) {
+    if (!FINE && !p.q_tma) {
       const __nv_bfloat16* qrow = p.q + (((size_t)b * p.Ncap + t_tok) * p.Hq + h_q) * HD;
       uint4 qv[HD / 8];
 #pragma unroll
@@ -1074,7 +1086,7 @@ tree_attn_tc_kernel(const TcParams p, const __grid_constant__ CUtensorMap map_k,
     };
     // next scores first: Q K^T of tile it+1 runs while the softmax of tile `it` does; the other CTA on
     // this SM covers the moments when a K tile is late
-    bool ok = ntile_u == 0 || ((!p.q_tma || mbar_wait(bar_q, 0)) && mbar_wait(&bar_fullk[0], 0));
+    bool ok = ntile_u == 0 || ((!(FINE || p.q_tma) || mbar_wait(bar_q, 0)) && mbar_wait(&bar_fullk[0], 0));
     if (ok && ntile_u > 0) {
       tc_fence_after();
       mma_qk(0, 0);
@@ -1553,23 +1565,26 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
     return false;
   const int G = Hq / Hkv, Ncap = c->cfg.max_tree;
   const int Nmax = c->cfg.total_token < Ncap ? c->cfg.total_token : Ncap;
-  // Q comes in one copy per row block and half of the dims, or in copies of eight rows (a period of the swizzle's pattern), only
-  // those with live rows, zeros for the others: products with dead rows are computed all the same, and on other sequences'
-  // queries they cost power, which is what bounds a loaded machine (64 sequences of 512-4096, 12 tokens, two layers back to
-  // back: 235 -> 223 us at 1.3 GHz and above, 197 -> 195 from rest). Not where CTAs are short: the copies are on the chain of a
-  // split (six draft windows on 4 sequences 85 -> 90 us) and of sequences under some 1000 positions (48 of 64-512, 17.6 -> 19.1).
+  // Q comes in one copy per row block and half of the dims, or (fine) in lower ones, only those with live rows, zeros for the
+  // others: products with dead rows are computed all the same, and on other sequences' queries they cost power, which is what
+  // bounds a loaded machine (64 sequences of 512-4096, 12 tokens, two layers back to back: 230 -> 214 us; three layers 97.2 -> 95.0
+  // per layer). The rule looks at what the host knows: trees of this context fit three quarters of one row block at most (above
+  // that there is little to leave out: with copies of eight rows and the earlier fill 16 sequences of 2048, 64 tokens, 43.3 ->
+  // 43.9), no clusters (a cluster's CTA has few tiles and the copies are on its chain: draft windows on 4 sequences 85 -> 90, as
+  // before) and room for 1024 positions (below: 48 of 64-512 18.75 -> 19.0, 64 of 128-900 32.2 -> 31.7). A context with room for
+  // more that holds short sequences pays up to 1.2 % without early reads, nothing with them (48 of 64-512: 27.3 -> 27.65, 19.1 ->
+  // 19.0). A kernel of its own, so that launches without it run the code they had (4 sequences of 32768, a group of seven: with
+  // the copies' code beside the rest 0.8 % slower).
   const int max_pos = page_size == 0 ? seq_capacity : seq_capacity * page_size;
-  const bool fine = Nmax * G <= kBM * 3 / 4 && !(pl.cluster_mode && pl.cs > 1) && max_pos >= 1024;
-  // Nor where the largest tree leaves less than a quarter of a block dead: there the copies bought nothing and cost a little (16
-  // sequences of 2048, 64 tokens, 43.3 -> 43.9 us per layer; a second descriptor, for the kernel to choose by the live rows,
-  // made short launches of 64-dim heads 2 % slower).
-  const int q_tokens = G > kBM ? 0 : !fine ? kBM / G : G < 8 ? 8 / G : 1;  // (G divides 128 where this is used: a power of two)
+  bool fine = Nmax * G <= kBM * 3 / 4 && !(pl.cluster_mode && pl.cs > 1) && max_pos >= 1024;
+  const int q_tokens = G > kBM ? 0 : !fine ? kBM / G : G < kQBox ? kQBox / G : 1;  // (G divides 128 where this is used: a power of two)
   CUtensorMap map_q = map_k;  // (a valid descriptor either way; used only when q_tma is set)
   const bool q_tma = G <= kBM && (kBM % G) == 0 && make_q_map(&map_q, q, B, Ncap, Hq, G, D, q_tokens);
+  fine = fine && q_tma;
   TcParams p;
   p.q_tma = q_tma ? 1 : 0;
-  p.q_box = q_tma ? q_tokens * G : kBM;
-  p.g_log2 = q_tma ? __builtin_ctz((unsigned)G) : 0;
+  p.q_box = fine ? q_tokens * G : kBM;
+  p.g_log2 = fine ? __builtin_ctz((unsigned)G) : 0;
   // the shapes the header names: a caller of others may have set the promise without keeping it
   const bool promised = c->attn_early && D == 128 && q_tma;
   p.early = (promised && !c->tree_inputs_fresh) ? 1 : 0;
@@ -1624,16 +1639,18 @@ bool tree_attention_tc_launch(cast_ctx* c, const void* q, const void* k, const v
     // one sequence of 1024 9.4 / 8.8 / 8.6, 64 of 512-1024 41.0 / 34.0 / 33.3; in early mode comparing would cost 0.3 of 11.9).
     p.wl_sizes = p.tmem_first ? nullptr : c->attn_worklist + (size_t)kAttnWorkListCap * 8;
   }
-  auto* const kern = D == 64 ? tree_attn_tc_kernel<64> : tree_attn_tc_kernel<128>;
+  auto* const kern = D == 64 ? (fine ? tree_attn_tc_kernel<64, true> : tree_attn_tc_kernel<64, false>)
+                             : (fine ? tree_attn_tc_kernel<128, true> : tree_attn_tc_kernel<128, false>);
   const int smem_bytes = D == 64 ? Geo<64>::kSmemBytes : Geo<128>::kSmemBytes;
-  if (!c->attn_attr_set[D == 64]) {  // (a function's attributes belong to the device, as the context does)
+  int& attr_set = c->attn_attr_set[D == 64][fine];
+  if (!attr_set) {  // (a function's attributes belong to the device, as the context does)
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess) {
       *status = CAST_ERR_CUDA;
       return true;
     }
     // two CTAs per SM need the largest shared-memory carve-out
     cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    c->attn_attr_set[D == 64] = 1;
+    attr_set = 1;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);

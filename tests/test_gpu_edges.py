@@ -498,9 +498,10 @@ def test_a_list_of_a_shape_outside_the_promise_is_not_trusted_inside(binding):
     (38, 8, 64, 4, 1100), (38, 8, 128, 2, 1100), (38, 8, 4, 24, 1024), (64, 8, 8, 12, 1030), (64, 5, 16, 6, 1200),
     (40, 8, 64, 1, 1100), (3, 2, 4, 20, 9000), (3, 2, 4, 40, 9000), (38, 8, 4, 33, 300)])
 def test_query_rows_past_the_tree_are_left_out(binding, D, B, Hkv, G, cap, longest):
-    """Many sequences, or pieces of long ones: a row block's queries come eight rows at a time, those with live rows only. The
-    tree sizes run over the edges of the copies; what lies past the trees is NaN. (The last ones: pieces of long sequences; trees
-    too large for it and sequences too short.) Two bf16 roundings, of the probabilities and of the output: 2^-9 of |v|'s maximum each."""
+    """Where the largest tree fills three quarters of a row block at most, launches without clusters copy the boxes of queries
+    that hold live rows and fill the rest with zeros; the tree sizes run over the edges of the boxes, and what lies past the
+    trees is NaN. The cases whose budget is above that, the cluster of (3, 2, 4) and the short sequences of the last one take whole
+    row blocks. Two bf16 roundings, of the probabilities and of the output: 2^-9 of |v|'s maximum each."""
     rng = np.random.default_rng(B + G)
     n_tree = [1 + i % cap for i in range(B)]
     kv = [longest] + [int(x) for x in rng.integers(0, 200, B - 1)]
@@ -509,6 +510,26 @@ def test_query_rows_past_the_tree_are_left_out(binding, D, B, Hkv, G, cap, longe
         keep = ~want.isnan()
         assert torch.equal(got.isnan(), ~keep)
         assert float((got.double() - want)[keep].abs().max()) < 2.0 ** -8 * 6
+
+
+@pytest.mark.parametrize("mode", ["default", "early", "rows"])
+@pytest.mark.parametrize("D,B,Hkv,G,cap,page", [(128, 24, 8, 4, 24, 16), (128, 33, 8, 1, 96, 0), (128, 20, 8, 8, 12, 32),
+                                                (128, 30, 5, 16, 6, 16), (128, 23, 8, 32, 3, 16), (64, 24, 8, 4, 24, 16),
+                                                (64, 38, 4, 2, 48, 0)])
+def test_live_query_rows_of_blocks_in_pieces(binding, D, B, Hkv, G, cap, page, mode):
+    """Ragged sequences with somewhat more row blocks than half of a wave's slots: the long ones are cut and merged through the
+    workspace, every piece with its live query rows alone; with early reads Q comes behind the first tiles, and a window's rows
+    start inside the tree. The partials' half precision adds 2^-11 of |v|'s maximum to two bf16 roundings of 2^-9."""
+    slots = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert slots < 2 * B * Hkv < 2 * slots and cap * G <= 96  # one block each, no clusters
+    n_tree = [1 + (i * 5) % cap for i in range(B)]
+    kv = [100 + 6000 * i // B for i in range(B)]
+    first = [n // 3 for n in n_tree] if mode == "rows" else None
+    got, want = _attend(binding, np.random.default_rng(B + G), B, cap, n_tree, Hkv * G, Hkv, D, page, kv, first=first,
+                        early=mode == "early", beyond=float("nan"))
+    keep = ~want.isnan()
+    assert torch.equal(got.isnan(), ~keep)
+    assert float((got.double() - want)[keep].abs().max()) < 2.25 * 2.0 ** -9 * 6
 
 
 @pytest.mark.parametrize("B,cap,Hq,Hkv,page,sizes,kv", [
