@@ -34,7 +34,7 @@ namespace {
 constexpr int kStoThreads = 512;
 constexpr int kStoWarps = kStoThreads / 32;
 constexpr int kStoMaxCluster = 16;
-constexpr int kStoInFlight = 8;  // exponentials of a lane that are worked on side by side, at most
+constexpr int kStoInFlight = 8;  // logits of a row that a lane has in flight and exponentials that it works on side by side
 // Vocabulary entries per CTA up to which the plan caches segments (196 608 tokens in clusters of 16): the rule that
 // cast_accept_stochastic_plan has always answered by, set when a slice of both rows filled shared memory. The kernels hold
 // up to 38 x 512 entries now, so the times do not cross here: V = 262144, one sequence, 76 us recomputing and 41 cached.
@@ -141,49 +141,45 @@ __device__ __forceinline__ double sto_exp_row(float logit, const StoRef& row, do
 // almost all are. Step by step for M of them side by side: each is a chain of a dozen dependent fp64 instructions, and taken
 // one after the other they left the pipe half idle (cycles of a warp per exponential, V = 128256: 56 before, 48 now, of which
 // the fp64 instructions take 29 and the two shuffles and the conversion, which other pipes run, 8 each). No range tests, and
-// the argument is reduced from the logit itself, t = logit * 32 / (T ln2) = k + f, |f| <= 1/2, by a factor in two parts (f is
-// right to 2^-54 of its own size; through x = logit / T it carried x's rounding). The polynomial of e^r is taken in f.
-// (The conversion by integer instructions: 80.9 -> 83.5 us for the 16 sequences below; M = 2 or 4: 86.1, 82.9.)
-template <int U>
-__device__ __forceinline__ void sto_exp_plain(const float (&logit)[U], double c_hi, double c_lo, double tab, double (&e)[U]) {
+// the argument is reduced from the logit itself, t = logit * 32 / (T ln2) = k + f, |f| <= 1/2, by a factor in two parts: f's two
+// roundings are 2^-54 each, 2e-18 in the result, where x = logit / T carried its own, up to 690 * 2^-53. What is left is the
+// table entry's 2^-52 and the last step's 2^-53. The polynomial of e^r is taken in f.
+// (The conversion by integer instructions: 80.9 -> 83.5 us for 16 sequences of V = 128256; M = 2 or 4: 86.1, 82.9.)
+template <int M>
+__device__ __forceinline__ void sto_exp_plain(const float (&logit)[M], double c_hi, double c_lo, double tab, double (&e)[M]) {
   constexpr double kL = 6.93147180559945309417e-01 / 32.0;
-  constexpr int M = U < kStoInFlight ? U : kStoInFlight;
-  static_assert(U % M == 0, "whole groups");
   const double kMagic = 6755399441055744.0;
   const double c[6] = {kL * kL * kL * kL * kL * kL / 720.0, kL * kL * kL * kL * kL / 120.0, kL * kL * kL * kL / 24.0,
                        kL * kL * kL / 6.0, kL * kL / 2.0, kL};
+  double f[M], y[M];
+  int k[M];
 #pragma unroll
-  for (int g = 0; g < U; g += M) {
-    double f[M], y[M];
-    int k[M];
+  for (int i = 0; i < M; ++i) f[i] = (double)logit[i];
 #pragma unroll
-    for (int i = 0; i < M; ++i) f[i] = (double)logit[g + i];
+  for (int i = 0; i < M; ++i) y[i] = fma(f[i], c_hi, kMagic);
 #pragma unroll
-    for (int i = 0; i < M; ++i) y[i] = fma(f[i], c_hi, kMagic);
+  for (int i = 0; i < M; ++i) {
+    k[i] = __double2loint(y[i]);
+    y[i] -= kMagic;
+  }
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-      k[i] = __double2loint(y[i]);
-      y[i] -= kMagic;
-    }
+  for (int i = 0; i < M; ++i) y[i] = fma(f[i], c_hi, -y[i]);
 #pragma unroll
-    for (int i = 0; i < M; ++i) y[i] = fma(f[i], c_hi, -y[i]);
+  for (int i = 0; i < M; ++i) f[i] = fma(f[i], c_lo, y[i]);
 #pragma unroll
-    for (int i = 0; i < M; ++i) f[i] = fma(f[i], c_lo, y[i]);
+  for (int i = 0; i < M; ++i) y[i] = c[0];
 #pragma unroll
-    for (int i = 0; i < M; ++i) y[i] = c[0];
+  for (int d = 1; d < 6; ++d)
 #pragma unroll
-    for (int d = 1; d < 6; ++d)
+    for (int i = 0; i < M; ++i) y[i] = fma(y[i], f[i], c[d]);
 #pragma unroll
-      for (int i = 0; i < M; ++i) y[i] = fma(y[i], f[i], c[d]);
+  for (int i = 0; i < M; ++i) y[i] *= f[i];
 #pragma unroll
-    for (int i = 0; i < M; ++i) y[i] *= f[i];
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-      const double t = __hiloint2double(__shfl_sync(0xffffffffu, __double2hiint(tab), k[i] & 31),
-                                        __shfl_sync(0xffffffffu, __double2loint(tab), k[i] & 31));
-      const double v = fma(t, y[i], t);
-      e[g + i] = __hiloint2double(__double2hiint(v) + (k[i] & ~31) * 32768, __double2loint(v));
-    }
+  for (int i = 0; i < M; ++i) {
+    const double t = __hiloint2double(__shfl_sync(0xffffffffu, __double2hiint(tab), k[i] & 31),
+                                      __shfl_sync(0xffffffffu, __double2loint(tab), k[i] & 31));
+    const double v = fma(t, y[i], t);
+    e[i] = __hiloint2double(__double2hiint(v) + (k[i] & ~31) * 32768, __double2loint(v));
   }
 }
 
@@ -299,7 +295,7 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
   auto evaluate = [&](double& sp, double& sq, bool zero_refs) {
     sp = sq = 0.0;
     if constexpr (CACHED) {
-      constexpr int U = NE < 8 ? NE : 8;  // logits in flight: the next group is loaded while this one is evaluated
+      constexpr int U = NE < kStoInFlight ? NE : kStoInFlight;  // the next group is loaded while this one is evaluated
       float xp[U], xq[U];
 #pragma unroll
       for (int j = 0; j < U; ++j) {
@@ -324,11 +320,14 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
         for (int side = 0; side < 2; ++side) {  // target, draft
           if (side == 1 && !has_q) break;
           double e[U];
+          bool plain = false;
           // (segments of four entries a lane are mostly padding, which is not within the limits: one sequence of V = 4099
           // 28.4 us with the look, 27.5 without)
-          if (NE > 4 && __all_sync(0xffffffffu, side == 0 ? plain_p : plain_q)) {
-            sto_exp_plain<U>(side == 0 ? xp : xq, p.c_hi, p.c_lo, tab, e);
-          } else {
+          if constexpr (NE > 4) {
+            plain = __all_sync(0xffffffffu, side == 0 ? plain_p : plain_q);
+            if (plain) sto_exp_plain(side == 0 ? xp : xq, p.c_hi, p.c_lo, tab, e);
+          }
+          if (!plain) {
 #pragma unroll
             for (int j = 0; j < U; ++j)
               e[j] = value(side == 0 ? xp[j] : xq[j], side == 0 ? ref_p : ref_q);

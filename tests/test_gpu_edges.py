@@ -295,6 +295,34 @@ def test_stochastic_accept_of_rows_with_all_mass_on_one_token(binding, V, B, dty
             assert np.array_equal(g, w)
 
 
+@pytest.mark.parametrize("V,B", [(65536, 8), (128256, 4), (128256, 24)])
+@pytest.mark.parametrize("T", [0.05, 0.8, 3.0])
+def test_stochastic_accept_exponentials_to_fp64_rounding(binding, V, B, T):
+    """Two tokens of about equal mass, logits up to 600 T on either side of zero, all others 60 nats and more below (1e-22 of the
+    mass): u just below the first one's share gives that token, just above it the second. The share is known to 40 digits. An
+    exponential is off by 2^-52 (its table entry) + 2^-53 (its last step) + 0.011 * 2^-52 (the polynomial), the two sums, their
+    folds, the scale and the goal by some ten roundings of 2^-53: 4e-15 is twice all that. An argument that carries its own
+    rounding, as next to padding (which these vocabularies have at the end only), would be off by up to 600 * 2^-53 = 7e-14."""
+    from decimal import Decimal, getcontext
+    getcontext().prec = 40
+    rng = np.random.default_rng(V + B)
+    top = np.linspace(-600, 600, B) + rng.uniform(-5, 5, B)
+    x = ((top[:, None] - rng.uniform(60, 80, (B, V))) * T).astype(np.float32)
+    at = np.sort(np.stack([1 + rng.permutation(V * 9 // 10)[:2] for _ in range(B)]), axis=1)
+    below, above = np.empty(B), np.empty(B)
+    for b in range(B):
+        x[b, at[b]] = (top[b] + rng.uniform(0, 1, 2)) * T
+        first, second = (Decimal(float(v)) / Decimal(T) for v in x[b, at[b]])
+        share = 1 / (1 + (second - first).exp())
+        below[b], above[b] = (float(share * (1 + s * Decimal(4e-15))) for s in (-1, 1))
+    x = x[:, None]
+    target = torch.from_numpy(x).cuda()
+    tokens, ua = np.zeros((B, 1), np.int32), np.full((B, 1), 0.5)
+    for ub, want in ((below, at[:, 0]), (above, at[:, 1])):
+        got, _, _ = _sample_at_root(binding, target, target, T, tokens, ua, ub)
+        assert np.array_equal(got[2], want)
+
+
 @pytest.mark.parametrize("logits", ["f32", "bf16"])
 @pytest.mark.parametrize("V", [33, 8191, 16385, 32769, 65529, 131073, 262147])
 @pytest.mark.parametrize("kind", ["random", "rising", "constant", "one_block", "few_finite"])
