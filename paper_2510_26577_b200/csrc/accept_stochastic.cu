@@ -18,11 +18,12 @@
 //
 // What bounds it: fp64 issue in the exponentials (64 lanes per SM: 2 V / cluster-size of them per node and CTA at about
 // a dozen fp64 instructions each; with the rest of an exponential 3.1 us a node at V = 128256 and 16 CTAs, 6.4 with 8) and
-// the chain of cluster-wide sums (about 1.2 us each). Hence: no pass for the maximum (fp64 has the exponent range to sum exp(logit / T) as it is; the row is
-// evaluated again against its maximum only if the sum leaves 1e-280 .. 1e280), one exchange per node and per rejection
-// and none for the bonus token, whose segment sums are those of the last exchange.
-// Measured with the compaction behind it (T = 0.8, trees of 24, fp32): V = 128256 1 sequence 46 -> 40 us, 16 87 -> 80 by
-// taking the exponentials side by side; V = 32000 64 sequences 110 -> 104.
+// the chain of cluster-wide sums (about 1.2 us each). Hence: no pass for the maximum (fp64 has the exponent range to sum
+// exp(logit / T) as it is; the row is evaluated again against its maximum only if the sum leaves 1e-280 .. 1e280), one
+// exchange per node and per rejection and none for the bonus token, whose segment sums are those of the last exchange.
+// Measured alone (T = 0.8, trees of 24, fp32, means over three or four sets of trees; before the exponentials went side by
+// side -> now): V = 128256 1 sequence 32.3 -> 28.3 us, 8 67.3 -> 58.2, 16 84.6 -> 74.9; V = 32000 16 sequences 37.7 -> 35.2;
+// all but 50 tokens of a row ruled out, V = 128256, 16 sequences 86.6 -> 87.3.
 #include <math.h>
 
 #include "cast_internal.h"
@@ -247,8 +248,10 @@ __global__ void __launch_bounds__(kStoThreads, 1) accept_stochastic_kernel(const
   constexpr int kP = CACHED ? sto_in_registers(NE) : 1;
   // The children's exponentials are formed while the sums are exchanged, but not where a segment's values leave no registers
   // for them (us, formed after / during: one sequence of V = 128256 42.3 / 40.3, 64 of 32000 105.6 / 104.2, with 32 entries a
-  // lane, 16 of 128256, 80.5 / 82.2).
-  constexpr bool kOverlap = NE <= 24;
+  // lane, 16 of 128256, 80.5 / 82.2), nor where a node is short (up to four entries a lane, fp32, this launch alone, means over
+  // four sets of trees: 16 sequences of V = 4099 30.8 / 32.0, of 1000 31.4 / 32.1, of 16001 30.2 / 30.8, of 32000 35.1 / 35.2,
+  // eight of 4099 in bf16 23.0 / 23.5; one of 1000 22.7 / 22.3).
+  constexpr bool kOverlap = NE > 4 && NE <= 24;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cs = p.cs, rank = blockIdx.x, b = blockIdx.y;
   const int ne = CACHED ? NE : p.ne;
